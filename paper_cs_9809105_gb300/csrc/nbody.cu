@@ -7,8 +7,9 @@
 // instruction, the reciprocal square root per half).
 //
 // Two schedules:
-//  * tiled: each thread owns x bodies; the z array streams through shared memory in tiles
-//    that every CTA reads from L2 (the GPU's own way to share one array among all cells);
+//  * tiled: each lane owns x bodies; the z array streams through shared memory in tiles
+//    that every CTA reads from L2 (the GPU's own way to share one array among all cells), split
+//    over the warps of a CTA and the CTAs of a cluster;
 //  * hyper-systolic (Section 4.1 with the regular bases of Definition REGULARBASE2): a
 //    cluster of p CTAs is the ring of p cells, each owning a block of x; the K replicas of
 //    x (A = (0, 1, ..., 1)) are the blocks of the K-1 right-hand neighbours, read once
@@ -27,8 +28,11 @@
 namespace hsmm {
 namespace {
 
-constexpr int NB_TILE = 256;    // threads and z tile of the tiled kernel
-constexpr int ILP = 2;          // x bodies per thread (tiled, scalar)
+// tiled kernel: warps per CTA (each takes its share of a z tile of NB_THREADS bodies), x bodies
+// per lane and per CTA, z bodies per unrolled step, CTAs of a cluster (the split of z)
+constexpr int NB_WARPS = 8, NB_THREADS = 32 * NB_WARPS;
+constexpr int NB_ILP = 4, NB_XB = 32 * NB_ILP, NB_UNROLL = 8;
+constexpr int NB_ZS = 8;
 constexpr int NB_RING = 128;    // bodies per cell and threads per CTA (hyper-systolic)
 
 // a += f(x, z): m_z d / (|d|^2 + eps2)^(3/2), d = r_z - r_x
@@ -104,60 +108,92 @@ __device__ __forceinline__ float4 ld_peer_f4(uint32_t addr) {
     return v;
 }
 
-// PACKED (eps2 > 0): ILP x bodies per thread as ILP/2 packed pairs; else one body at a time
-// with the r = 0 case handled.  The z array is split over the CTAs of a cluster (4 to 8, the
-// host picks the count that spreads the CTAs evenly over the SMs) that share the same x bodies;
-// their partial sums are added in the fixed order of the cluster ranks through distributed
-// shared memory (deterministic, no workspace).
-template <bool PACKED, int ILPN>
-__global__ void __launch_bounds__(NB_TILE) nbody_tiled(int64_t nx, int64_t nz, const float4* __restrict__ x,
-                                                       const float4* __restrict__ z, float eps2,
-                                                       float4* __restrict__ out) {
-    __shared__ float4 tile[NB_TILE];
-    __shared__ float4 part[ILPN][NB_TILE];
-    const int zs = int(cluster_ctarank());
-    const int ZS = int(cluster_nctarank());
-    const int64_t i0 = int64_t(blockIdx.x / ZS) * NB_TILE * ILPN + threadIdx.x;
-    const int64_t zchunk = ((nz + ZS - 1) / ZS + NB_TILE - 1) / NB_TILE * NB_TILE;
+// Tiled schedule.  A CTA owns NB_XB = 128 x bodies, four per lane, and each of its eight warps
+// works on its own eighth of every z tile; a cluster of NB_ZS = 8 CTAs shares the same x bodies
+// and splits z.  Partial sums are added in the fixed order of warps, then cluster ranks, through
+// shared and distributed shared memory (deterministic, no workspace).
+//   PACKED (eps2 > 0): the four bodies as two packed pairs; else one body at a time with the
+//   r = 0 case handled.
+// Bound by the FP32 pipe: 12 packed instructions per two interactions, so what counts is that
+// every scheduler has warps to hide their latency behind.  The 64-way split of z (eight warps x
+// eight CTAs) gives an x array of 20000 bodies 1256 CTAs, four resident per SM; with 1024 x bodies
+// per CTA it had 140 CTAs on 152 SMs, two warps per scheduler.  z is kept duplicated, (x, x, y, y)
+// and (z, z, m, m), so that both halves of a packed operand come from one 16-byte load without
+// register moves, and the next tile is fetched into registers while one is used.
+// G interactions/s before -> now: 1061 -> 2169 at 20000 bodies, 2236 -> 2490 at 131072; 6.3 us at
+// 1000 bodies.  Also measured: four CTAs per cluster (1991 at 20000, 2461 at 131072), 16 (not
+// portable, equal at 5000), 64 lanes x 4 warps (2011, 2494), unrolled by 4 (2146, 2468) or 16
+// (1989, 2328), two bodies a lane (2011, 2265), six (1776, 2208).
+template <bool PACKED>
+__global__ void __launch_bounds__(NB_THREADS) nbody_tiled(int64_t nx, int64_t nz, const float4* __restrict__ x,
+                                                          const float4* __restrict__ z, float eps2,
+                                                          float4* __restrict__ out) {
+    // two z tiles of NB_THREADS bodies (two float4 each), later the partial sums [warp][body]
+    __shared__ float4 sm[2 * 2 * NB_THREADS];
+    static_assert(2 * 2 * NB_THREADS >= NB_WARPS * NB_XB, "the partial sums reuse the z tiles");
+    const int lane = int(lane_id()), warp = int(warp_id());
+    const int zs = int(cluster_ctarank()), ZS = int(cluster_nctarank());
+    const int64_t xblock = int64_t(blockIdx.x / ZS) * NB_XB;
+    // this CTA's share of z, in multiples of eight bodies per warp
+    constexpr int ZU = NB_UNROLL * NB_WARPS;
+    const int64_t zchunk = ((nz + ZS - 1) / ZS + ZU - 1) / ZU * ZU;
     const int64_t zbeg = int64_t(zs) * zchunk;
     const int64_t zend = min(nz, zbeg + zchunk);
-    float4 xi[ILPN];
+    float4 xi[NB_ILP];
 #pragma unroll
-    for (int k = 0; k < ILPN; ++k) {
-        const int64_t i = i0 + k * NB_TILE;
+    for (int k = 0; k < NB_ILP; ++k) {
+        const int64_t i = xblock + k * 32 + lane;
         xi[k] = i < nx ? x[i] : make_float4(0.f, 0.f, 0.f, 0.f);
     }
-    float3 a[PACKED ? 1 : ILPN];
-    XPair pr[PACKED ? ILPN / 2 : 1];
+    float3 a[PACKED ? 1 : NB_ILP];
+    XPair pr[PACKED ? NB_ILP / 2 : 1];
     if constexpr (PACKED) {
 #pragma unroll
-        for (int k = 0; k < ILPN / 2; ++k) pr[k] = make_pair(xi[2 * k], xi[2 * k + 1]);
+        for (int k = 0; k < NB_ILP / 2; ++k) pr[k] = make_pair(xi[2 * k], xi[2 * k + 1]);
     } else {
 #pragma unroll
-        for (int k = 0; k < ILPN; ++k) a[k] = make_float3(0.f, 0.f, 0.f);
+        for (int k = 0; k < NB_ILP; ++k) a[k] = make_float3(0.f, 0.f, 0.f);
     }
     const uint64_t e2 = pk2(eps2, eps2);
-    for (int64_t j0 = zbeg; j0 < zend; j0 += NB_TILE) {
-        const int64_t j = j0 + threadIdx.x;
-        tile[threadIdx.x] = j < zend ? z[j] : make_float4(0.f, 0.f, 0.f, 0.f);   // padding: zero mass
-        __syncthreads();
+    // padding: zero mass, far from any body (at the origin a body there and a tiny eps2 would
+    // give 0 x infinity)
+    const float4 pad = make_float4(1e18f, 1e18f, 1e18f, 0.f);
+    auto put = [&](int buf, const float4& v) {
+        float4* t = sm + buf * 2 * NB_THREADS + 2 * threadIdx.x;
+        t[0] = make_float4(v.x, v.x, v.y, v.y);
+        t[1] = make_float4(v.z, v.z, v.w, v.w);
+    };
+    put(0, zbeg + threadIdx.x < zend ? z[zbeg + threadIdx.x] : pad);
+    __syncthreads();
+    int buf = 0;
+    for (int64_t j0 = zbeg; j0 < zend; j0 += NB_THREADS) {
+        const bool more = j0 + NB_THREADS < zend;
+        const int64_t jn = j0 + NB_THREADS + threadIdx.x;
+        float4 next = pad;
+        if (more && jn < zend) next = z[jn];
+        // bodies of this tile per warp: 32, fewer (a multiple of eight) in the last one
+        const int64_t rem = zend - j0;
+        const int cnt = rem >= NB_THREADS ? 32 : int((rem + ZU - 1) / ZU) * NB_UNROLL;
+        const float4* t = sm + buf * 2 * NB_THREADS + warp * cnt * 2;
 #pragma unroll 8
-        for (int q = 0; q < NB_TILE; ++q) {
-            const float4 zj = tile[q];
+        for (int q = 0; q < cnt; ++q) {
             if constexpr (PACKED) {
-                const uint64_t zx = pk2(zj.x, zj.x), zy = pk2(zj.y, zj.y), zz = pk2(zj.z, zj.z),
-                               zm = pk2(zj.w, zj.w);
+                const ulonglong2 u = *reinterpret_cast<const ulonglong2*>(t + 2 * q);
+                const ulonglong2 w = *reinterpret_cast<const ulonglong2*>(t + 2 * q + 1);
 #pragma unroll
-                for (int k = 0; k < ILPN / 2; ++k) interact2(pr[k], zx, zy, zz, zm, e2);
+                for (int k = 0; k < NB_ILP / 2; ++k) interact2(pr[k], u.x, u.y, w.x, w.y, e2);
             } else {
+                const float4 u = t[2 * q], w = t[2 * q + 1];
 #pragma unroll
-                for (int k = 0; k < ILPN; ++k) interact(xi[k], zj, eps2, a[k]);
+                for (int k = 0; k < NB_ILP; ++k) interact(xi[k], make_float4(u.x, u.z, w.x, w.z), eps2, a[k]);
             }
         }
+        if (more) put(buf ^ 1, next);
         __syncthreads();
+        buf ^= 1;
     }
 #pragma unroll
-    for (int k = 0; k < ILPN; ++k) {
+    for (int k = 0; k < NB_ILP; ++k) {
         float3 r;
         if constexpr (PACKED) {
             float l0, h0, l1, h1, l2, h2;
@@ -168,25 +204,36 @@ __global__ void __launch_bounds__(NB_TILE) nbody_tiled(int64_t nx, int64_t nz, c
         } else {
             r = a[k];
         }
-        part[k][threadIdx.x] = make_float4(r.x, r.y, r.z, 0.f);
+        sm[warp * NB_XB + k * 32 + lane] = make_float4(r.x, r.y, r.z, 0.f);
     }
-    cluster_sync_all();
-    if (zs == 0) {
+    __syncthreads();
+    if (threadIdx.x < NB_XB) {
+        float4 sum = sm[threadIdx.x];
 #pragma unroll
-        for (int k = 0; k < ILPN; ++k) {
-            float4 sum = part[k][threadIdx.x];
-            for (int q = 1; q < ZS; ++q) {
-                const float4 v = ld_peer_f4(mapa_shared(smem_u32(&part[k][threadIdx.x]), uint32_t(q)));
-                sum.x += v.x;
-                sum.y += v.y;
-                sum.z += v.z;
-            }
-            const int64_t i = i0 + k * NB_TILE;
-            if (i < nx) out[i] = make_float4(sum.x, sum.y, sum.z, 0.f);
+        for (int w = 1; w < NB_WARPS; ++w) {
+            const float4 v = sm[w * NB_XB + threadIdx.x];
+            sum.x += v.x;
+            sum.y += v.y;
+            sum.z += v.z;
         }
+        sm[threadIdx.x] = sum;
     }
     __syncwarp();
-    cluster_sync_all();   // the other ranks keep their partial sums until rank 0 has read them
+    cluster_sync_all();
+    // every rank adds up its 16 bodies of the x block (with eight ranks)
+    const int share = (NB_XB + ZS - 1) / ZS;
+    for (int b = zs * share + int(threadIdx.x); b < min(NB_XB, (zs + 1) * share); b += NB_THREADS) {
+        float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int q = 0; q < ZS; ++q) {
+            const float4 v = ld_peer_f4(mapa_shared(smem_u32(&sm[b]), uint32_t(q)));
+            sum.x += v.x;
+            sum.y += v.y;
+            sum.z += v.z;
+        }
+        if (xblock + b < nx) out[xblock + b] = make_float4(sum.x, sum.y, sum.z, 0.f);
+    }
+    __syncwarp();
+    cluster_sync_all();   // the other ranks keep their partial sums until they have been read
 }
 
 template <int K, bool PACKED>
@@ -287,32 +334,21 @@ hsmm_status_t nbody_forces(int64_t nx, int64_t nz, const float* x, const float* 
     // eps2 > 0: r^2 > 0 for every pair, the packed FP32 pair kernels apply
     const bool packed = eps2 > 0.f;
     if (ring_p == 0) {
-        const int ilp = packed ? 4 : ILP;
-        // z split over zsplit CTAs: the count in 4..8 that spreads the CTAs most evenly over the SMs
-        const int64_t xblocks = (nx + int64_t(NB_TILE) * ilp - 1) / (int64_t(NB_TILE) * ilp);
-        const int sms = num_sms();
-        int zsplit = 4;
-        double best = -1.0;
-        for (int c = 4; c <= 8; ++c) {
-            const double per_sm = double(xblocks * c) / sms;
-            const double eff = per_sm / double(int64_t(per_sm + 0.999999));
-            if (eff > best + 1e-9) { best = eff; zsplit = c; }
-        }
-        const int64_t blocks = xblocks * zsplit;
-        if (blocks > INT32_MAX) return HSMM_STATUS_NOT_SUPPORTED;
+        const int64_t xblocks = (nx + NB_XB - 1) / NB_XB;
+        if (xblocks > INT32_MAX / NB_ZS) return HSMM_STATUS_NOT_SUPPORTED;
         cudaLaunchConfig_t tc = {};
-        tc.gridDim = dim3(unsigned(blocks), 1, 1);
-        tc.blockDim = dim3(NB_TILE, 1, 1);
+        tc.gridDim = dim3(unsigned(xblocks * NB_ZS), 1, 1);
+        tc.blockDim = dim3(NB_THREADS, 1, 1);
         tc.stream = st;
         cudaLaunchAttribute ta[1];
         ta[0].id = cudaLaunchAttributeClusterDimension;
-        ta[0].val.clusterDim.x = unsigned(zsplit);
+        ta[0].val.clusterDim.x = NB_ZS;
         ta[0].val.clusterDim.y = 1;
         ta[0].val.clusterDim.z = 1;
         tc.attrs = ta;
         tc.numAttrs = 1;
-        const cudaError_t te = packed ? cudaLaunchKernelEx(&tc, nbody_tiled<true, 4>, nx, nz, x4, z4, eps2, o4)
-                                      : cudaLaunchKernelEx(&tc, nbody_tiled<false, ILP>, nx, nz, x4, z4, eps2, o4);
+        const cudaError_t te = packed ? cudaLaunchKernelEx(&tc, nbody_tiled<true>, nx, nz, x4, z4, eps2, o4)
+                                      : cudaLaunchKernelEx(&tc, nbody_tiled<false>, nx, nz, x4, z4, eps2, o4);
         count_launches(1);
         if (te != cudaSuccess) return record_cuda(te);
         return check_launch();
