@@ -413,6 +413,14 @@ __global__ void __launch_bounds__(kNumThreads, 1)
 // took about as long; so with beta == 0 and a TMA-able C each warp stages 32 x 32
 // blocks in shared memory and writes them with one TMA store each (clipped at the
 // matrix edge by the TMA unit), which leaves room for six stages.
+//
+// The producer and the MMA role are run by their whole warps, with each asynchronous instruction
+// predicated on one elected lane: loop state and descriptors then live in uniform registers.  A
+// single-lane branch moved every descriptor there first, 253 cycles a k-block for the four MMAs
+// and the commit (125 now, of 512 tensor cycles) and about 470 for the producer's two loads
+// (300).  Before -> now, in a row in a CUDA graph: 8192 x 4096 x 2048 76.2 -> 72.6 us, 2048 x
+// 4096 x 8192 (T, N) 78.8 -> 77.6, 8192 x 2048 x 4096 (N, T) 84.7 -> 79.3, 4096 x 4096 x 1024
+// 27.5 -> 25.0, TF32 4096^3 168 -> 157.
 #ifndef PP_STAGES_CFG
 #define PP_STAGES_CFG 6
 #define PP_EPI_CFG 4
@@ -437,7 +445,7 @@ __global__ void __launch_bounds__(PP_THREADS, 1)
     uint8_t* smem = align1024(smem_raw);
     uint8_t* stage_c = smem + PP_STAGES * PAIR_STAGE_BYTES;
     Bars* bars = reinterpret_cast<Bars*>(stage_c + PP_STAGE_C);
-    const int warp = int(warp_id()), lane = int(lane_id());
+    const int warp = warp_id_uniform(), lane = int(lane_id());
     uint32_t* status = &g_status_gemm_tc;
     const uint32_t rank = cluster_ctarank() & 1u;
     const bool leader = (rank == 0);
@@ -479,53 +487,55 @@ __global__ void __launch_bounds__(PP_THREADS, 1)
     const int nkb = (g.K + C_::BK - 1) / C_::BK;
 
     if (warp == 0) {
-        if (lane == 0) {
-            pdl_wait();   // A and B may be written by the previous kernel
-            int stage = 0;
-            uint32_t phase = 0;
-            int last_parity[8];
-            for (int i = 0; i < 8; ++i) last_parity[i] = -1;
-            bool ok = true;
-            for (int t = pair; t < ntiles && ok && !*abort; t += npairs) {
-                int tm, tn;
-                tile_coords(t, tiles_m, tiles_n, tm, tn);
-                const int arow = tm * 2 * BM + int(rank) * BM;
-                const int brow = tn * PAIR_BN + int(rank) * BM;
-                for (int kb = 0; kb < nkb; ++kb) {
-                    if (!mbar_wait(&bars->empty[stage], phase ^ 1u, g.timeout_ns, status, abort)) { ok = false; break; }
-                    uint8_t* a_dst = smem + stage * PAIR_STAGE_BYTES;
-                    uint8_t* b_dst = a_dst + BM * 128;
-                    const uint32_t full_leader = mapa_shared(smem_u32(&bars->full[stage]), 0);
-                    if (leader) mbar_arrive_expect_tx(&bars->full[stage], 2 * PAIR_STAGE_BYTES);
-                    if (!g.a_mn) {
-                        tma_load_2d_pair(a_dst, &tmA, full_leader, kb * C_::BK, arow);
-                    } else if (g.a_mn3) {
-                        tma_load_3d_pair(a_dst, &tmA, full_leader, 0, kb * C_::BK, arow / C_::MN_CHUNK);
-                    } else {
+        const bool issue = elect_one();
+        pdl_wait();   // A and B may be written by the previous kernel
+        int stage = 0, filled = 0;
+        uint32_t phase = 0;
+        bool ok = true;
+        const uint32_t full0 = mapa_shared(smem_u32(&bars->full[0]), 0);
+        for (int t = pair; t < ntiles && ok && !*abort; t += npairs) {
+            int tm, tn;
+            tile_coords(t, tiles_m, tiles_n, tm, tn);
+            const int arow = tm * 2 * BM + int(rank) * BM;
+            const int brow = tn * PAIR_BN + int(rank) * BM;
+            for (int kb = 0; kb < nkb; ++kb) {
+                // the first round of stages starts empty
+                if (filled >= PP_STAGES &&
+                    !mbar_wait_warp(&bars->empty[stage], phase ^ 1u, g.timeout_ns, status, abort)) { ok = false; break; }
+                uint8_t* a_dst = smem + stage * PAIR_STAGE_BYTES;
+                uint8_t* b_dst = a_dst + BM * 128;
+                const uint32_t full_leader = full0 + uint32_t(stage) * 8u;
+                mbar_arrive_expect_tx_if(issue && leader, &bars->full[stage], 2 * PAIR_STAGE_BYTES);
+                if (!g.a_mn) {
+                    tma_load_2d_pair_if(issue, a_dst, &tmA, full_leader, kb * C_::BK, arow);
+                } else if (g.a_mn3) {
+                    tma_load_3d_pair_if(issue, a_dst, &tmA, full_leader, 0, kb * C_::BK, arow / C_::MN_CHUNK);
+                } else {
 #pragma unroll
-                        for (int c = 0; c < BM / C_::MN_CHUNK; ++c)
-                            tma_load_2d_pair(a_dst + c * C_::BK * 128, &tmA, full_leader, arow + c * C_::MN_CHUNK,
-                                             kb * C_::BK);
-                    }
-                    if (!g.b_mn) {
-                        tma_load_2d_pair(b_dst, &tmB, full_leader, kb * C_::BK, brow);
-                    } else if (g.b_mn3) {
-                        tma_load_3d_pair(b_dst, &tmB, full_leader, 0, kb * C_::BK, brow / C_::MN_CHUNK);
-                    } else {
-#pragma unroll
-                        for (int c = 0; c < BM / C_::MN_CHUNK; ++c)
-                            tma_load_2d_pair(b_dst + c * C_::BK * 128, &tmB, full_leader, brow + c * C_::MN_CHUNK,
-                                             kb * C_::BK);
-                    }
-                    last_parity[stage] = int(phase);
-                    if (++stage == PP_STAGES) { stage = 0; phase ^= 1u; }
+                    for (int c = 0; c < BM / C_::MN_CHUNK; ++c)
+                        tma_load_2d_pair_if(issue, a_dst + c * C_::BK * 128, &tmA, full_leader, arow + c * C_::MN_CHUNK,
+                                            kb * C_::BK);
                 }
+                if (!g.b_mn) {
+                    tma_load_2d_pair_if(issue, b_dst, &tmB, full_leader, kb * C_::BK, brow);
+                } else if (g.b_mn3) {
+                    tma_load_3d_pair_if(issue, b_dst, &tmB, full_leader, 0, kb * C_::BK, brow / C_::MN_CHUNK);
+                } else {
+#pragma unroll
+                    for (int c = 0; c < BM / C_::MN_CHUNK; ++c)
+                        tma_load_2d_pair_if(issue, b_dst + c * C_::BK * 128, &tmB, full_leader, brow + c * C_::MN_CHUNK,
+                                            kb * C_::BK);
+                }
+                ++filled;
+                if (++stage == PP_STAGES) { stage = 0; phase ^= 1u; }
             }
-            for (int i = 0; i < PP_STAGES; ++i)
-                if (last_parity[i] >= 0) mbar_wait(&bars->empty[i], uint32_t(last_parity[i]), g.timeout_ns, status, abort);
         }
+        // every issued stage is released (empty) only after its copies landed and were consumed
+        for (int f = max(0, filled - PP_STAGES); f < filled; ++f)
+            mbar_wait_warp(&bars->empty[f % PP_STAGES], uint32_t(f / PP_STAGES) & 1u, g.timeout_ns, status, abort);
     } else if (warp == 1) {
-        if (lane == 0 && leader) {
+        if (leader) {
+            const bool issue = elect_one();
             const uint32_t idesc = make_idesc(TF32 ? 2u : 1u, g.a_mn != 0, g.b_mn != 0, 2 * BM, PAIR_BN);
             const uint64_t a0 = operand_desc<C_>(smem_u32(smem), 0, g.a_mn != 0);
             const uint64_t b0 = operand_desc<C_>(smem_u32(smem) + BM * 128, 0, g.b_mn != 0);
@@ -537,35 +547,30 @@ __global__ void __launch_bounds__(PP_THREADS, 1)
             uint32_t aphase = 0;
             bool ok = true;
             for (int t = pair; t < ntiles && ok && !*abort; t += npairs) {
-                if (!mbar_wait(&bars->acc_empty[abuf], aphase ^ 1u, g.timeout_ns, status, abort)) break;
+                if (!mbar_wait_warp(&bars->acc_empty[abuf], aphase ^ 1u, g.timeout_ns, status, abort)) break;
                 tc_fence_after();
                 const uint32_t d_tmem = tmem + uint32_t(abuf * PAIR_BN);
-                // lean issue loop (the single issuing thread must keep up with the tensor pipe):
-                // descriptors from the stage index, four k-blocks per unrolled iteration
+                // lean issue loop: descriptors from the stage index, four k-blocks per unrolled iteration
 #pragma unroll 4
                 for (int kb = 0; kb < nkb; ++kb) {
-                    if (!mbar_wait(&bars->full[stage], phase, g.timeout_ns, status, abort)) { ok = false; break; }
+                    if (!mbar_wait_warp(&bars->full[stage], phase, g.timeout_ns, status, abort)) { ok = false; break; }
                     tc_fence_after();
                     const uint64_t ad = a0 + uint64_t(stage) * sstep, bd = b0 + uint64_t(stage) * sstep;
 #pragma unroll
-                    for (int ks = 0; ks < C_::KSTEPS; ++ks) {
-                        const uint32_t acc = ks == 0 ? uint32_t(kb) : 1u;
-                        if (TF32)
-                            umma_tf32_pair(d_tmem, ad + ks * aks, bd + ks * bks, idesc, acc);
-                        else
-                            umma_f16_pair(d_tmem, ad + ks * aks, bd + ks * bks, idesc, acc);
-                    }
-                    umma_commit_pair(&bars->empty[stage], 0x3);
+                    for (int ks = 0; ks < C_::KSTEPS; ++ks)
+                        umma_pair_if<TF32>(issue, d_tmem, ad + ks * aks, bd + ks * bks, idesc,
+                                           ks == 0 ? uint32_t(kb) : 1u);
+                    umma_commit_pair_if(issue, &bars->empty[stage], 0x3);
                     stage = (stage + 1 == PP_STAGES) ? 0 : stage + 1;
                     phase ^= (stage == 0) ? 1u : 0u;
                 }
                 if (!ok) break;
-                umma_commit_pair(&bars->acc_full[abuf], 0x3);
+                umma_commit_pair_if(issue, &bars->acc_full[abuf], 0x3);
                 abuf ^= 1;
                 if (abuf == 0) aphase ^= 1u;
             }
-            umma_commit_pair(&bars->mma_done, 0x1);
-            mbar_wait(&bars->mma_done, 0, g.timeout_ns, status, abort);
+            umma_commit_pair_if(issue, &bars->mma_done, 0x1);
+            mbar_wait_warp(&bars->mma_done, 0, g.timeout_ns, status, abort);
         }
     } else {
         // epilogue: warp w reads TMEM lanes 32*(w%4) .. of this CTA's 128 rows and, with eight
