@@ -750,10 +750,24 @@ hsmm_status_t launch_plain(const CUtensorMap& ta, const CUtensorMap& tb, const C
 
 }  // namespace
 
-// Plain 256-wide tiles run on CTA pairs unless HSMM_GEMM_KERNEL=single selects one CTA per tile.
-static bool gemm_pair_enabled() {
+// HSMM_GEMM_KERNEL chooses the kernel: "single" one CTA per tile, "split" narrow tiles with the
+// contraction split over a cluster (gemm_split_tc.cu), anything else 256-wide tiles on CTA pairs;
+// unset: by the product's size.
+enum class TcKernel { Auto, Pair, Single, Split };
+static TcKernel tc_kernel_choice() {
     const char* v = std::getenv("HSMM_GEMM_KERNEL");
-    return !(v && std::strcmp(v, "single") == 0);
+    if (!v) return TcKernel::Auto;
+    return std::strcmp(v, "single") == 0 ? TcKernel::Single : std::strcmp(v, "split") == 0 ? TcKernel::Split
+                                                                                           : TcKernel::Pair;
+}
+
+// Estimated microseconds of a product on the persistent kernels below: launch and epilogue, then
+// a k-block of the widest tile for every tile of the busiest pair (or CTA).
+static double whole_tiles_cost(int64_t m, int64_t n, int64_t k, bool tf32) {
+    const int64_t nkb = (k + (tf32 ? 31 : 63)) / (tf32 ? 32 : 64);
+    const int64_t rows = m > BM ? 2 * BM : BM, slots = m > BM ? num_sms() / 2 : num_sms();
+    const int64_t tiles = ((m + rows - 1) / rows) * ((n + PAIR_BN - 1) / PAIR_BN);
+    return 6.0 + double((tiles + slots - 1) / slots) * double(nkb) * (m > BM ? 0.27 : 0.35);
 }
 
 hsmm_status_t gemm_tc(hsmm_dtype_t ab, hsmm_dtype_t c, hsmm_op_t ta, hsmm_op_t tb, int64_t m, int64_t n, int64_t k,
@@ -792,6 +806,38 @@ hsmm_status_t gemm_tc(hsmm_dtype_t ab, hsmm_dtype_t c, hsmm_op_t ta, hsmm_op_t t
                           uint64_t(ext / MN_CHUNK), uint64_t(MN_CHUNK), mn_sw, uint32_t(rows / MN_CHUNK));
     };
     const bool out_bf16 = (c == HSMM_R_16BF);
+    if (tf32 && out_bf16) return HSMM_STATUS_NOT_SUPPORTED;
+    // Few tiles: narrow ones with the contraction split over a cluster, wherever the estimate says
+    // so.  Over 120 drawn shapes (8..8192 a side) the kernel taken was the faster one of the two
+    // each time the two were apart, and its tile and split within 5% of the best of fourteen
+    // measured for 104 of them (1.25 at most); e.g. 2304 x 360 x 3000 18.5 us on whole tiles, 12.9
+    // split, 880 x 2864 x 1848 (TF32) 22.8 whole, 25.4 split.
+    const TcKernel choice = tc_kernel_choice();
+    if (tile_n == 0 && (choice == TcKernel::Auto || choice == TcKernel::Split)) {
+        const SplitPlan plan = split_plan(m, n, k, tf32, g.b_mn);
+        if (plan.bn != 0 && (choice == TcKernel::Split || plan.cost < whole_tiles_cost(m, n, k, tf32))) {
+            CUtensorMap sA, sB;
+            bool oks = g.a_mn ? (g.a_mn3 ? enc_mn3(&sA, A, m, lda, BM)
+                                         : encode_map(&sA, dt, esize, A, uint64_t(m), uint64_t(k), uint64_t(lda),
+                                                      MN_CHUNK, BK, 0, 0, mn_sw))
+                              : encode_map(&sA, dt, esize, A, uint64_t(k), uint64_t(m), uint64_t(lda), BK, BM);
+            oks = oks && (g.b_mn ? (g.b_mn3 ? enc_mn3(&sB, B, n, ldb, plan.bn)
+                                            : encode_map(&sB, dt, esize, B, uint64_t(n), uint64_t(k), uint64_t(ldb),
+                                                         MN_CHUNK, BK, 0, 0, mn_sw))
+                                 : encode_map(&sB, dt, esize, B, uint64_t(k), uint64_t(n), uint64_t(ldb), BK,
+                                              uint32_t(plan.bn)));
+            if (!oks) return fail(HSMM_STATUS_NOT_SUPPORTED, "gemm: TMA descriptor encoding failed (CUresult %d)",
+                                  g_last_encode_result);
+            SplitArgs sg{};
+            sg.M = g.M; sg.N = g.N; sg.K = g.K;
+            sg.a_mn = g.a_mn; sg.b_mn = g.b_mn; sg.a_mn3 = g.a_mn3; sg.b_mn3 = g.b_mn3;
+            sg.alpha = alpha; sg.beta = beta; sg.C = C; sg.ldc = ldc;
+            sg.timeout_ns = g.timeout_ns;
+            sg.bn = plan.bn;
+            sg.c_vec = beta == 0.f && ldc % 4 == 0 && aligned_to(C, out_bf16 ? 8 : 16);
+            return gemm_tc_split(tf32, out_bf16, sA, sB, sg, plan, st);
+        }
+    }
     // C through TMA stores of 32 x 32 blocks when beta == 0 and C is TMA-able; the map covers
     // the rows up to the last whole 16-byte unit (a store clips rows only to such units)
     CUtensorMap pC;
@@ -803,7 +849,7 @@ hsmm_status_t gemm_tc(hsmm_dtype_t ab, hsmm_dtype_t c, hsmm_op_t ta, hsmm_op_t t
                           uint64_t(g.m_tma), uint64_t(n), uint64_t(ldc), 32, 32, 0, 0, CU_TENSOR_MAP_SWIZZLE_NONE))
                   ? 1 : 0;
     // CTA pairs for 256-wide tiles whenever M fills more than one 128-row half
-    if (BN == 256 && m > BM && gemm_pair_enabled()) {
+    if (BN == 256 && m > BM && choice != TcKernel::Single) {
         CUtensorMap pA, pB;
         bool okp = g.a_mn ? (g.a_mn3 ? enc_mn3(&pA, A, m, lda, BM)
                                      : encode_map(&pA, dt, esize, A, uint64_t(m), uint64_t(k), uint64_t(lda), MN_CHUNK,

@@ -89,6 +89,28 @@ bool encode_map(CUtensorMap* map, CUtensorMapDataType dt, int esize, const void*
                 uint32_t box_batch = 1);
 int last_encode_result();
 
+// ---- gemm_split_tc.cu ----
+struct SplitArgs {
+    int M, N, K;
+    int a_mn, b_mn;         // operand majorness
+    int a_mn3, b_mn3;       // MN-major operand described as a 3D tensor of chunks (see gemm_tc)
+    float alpha, beta;
+    void* C;
+    int64_t ldc;
+    uint64_t timeout_ns;
+    int c_vec;              // four rows of a column of C can be stored at once (beta == 0)
+    int bn, stages;         // tile width; stages are set by the launch
+};
+// 128 x bn tiles, k split over a cluster of `split` CTAs; cost: estimated microseconds (bn = 0: no plan)
+struct SplitPlan {
+    int bn, split;
+    double cost;
+};
+SplitPlan split_plan(int64_t m, int64_t n, int64_t k, bool tf32, bool b_mn);
+hsmm_status_t gemm_tc_split(bool tf32, bool out_bf16, const CUtensorMap& ta, const CUtensorMap& tb, const SplitArgs& g,
+                            const SplitPlan& plan, cudaStream_t st);
+uint32_t status_take_split();
+
 // ---- gemm_ozaki_tc.cu ----
 // Slice products of the FP64-accurate form: S_d = sum_{t+u=d} Q^A_t (Q^B_u)^T, d = 2..s+1, exact INT32,
 // stored as [d-2][n][m].
