@@ -295,6 +295,9 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
 // Both CTAs' TMA copies complete on the even CTA's `full` barrier; the MMA
 // commits are multicast to both CTAs (stage release, accumulator ready); both
 // CTAs' epilogue warps release an accumulator on the even CTA's `acc_empty`.
+// The producer and MMA roles are run by whole warps (see gemm_tc.cu): 1000 x 1200 x 900 149.9 ->
+// 146.6 us, 4096^3 from host memory 3318 -> 3279, complex 1500 x 1100 x 2301 714 -> 706; 8192^3
+// is bound by the power cap (18.51 -> 18.46 ms).
 
 __global__ void __launch_bounds__(OZ_THREADS, 1)
     gemm_ozaki_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
@@ -303,7 +306,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = align1024(smem_raw);
     Bars* bars = reinterpret_cast<Bars*>(smem + PAIR_STAGES * PAIR_STAGE_BYTES);
-    const int warp = int(warp_id()), lane = int(lane_id());
+    const int warp = warp_id_uniform(), lane = int(lane_id());
     uint32_t* status = &g_status_ozaki_tc;
     const uint32_t rank = cluster_ctarank() & 1u;  // role in the pair
     const bool leader = (rank == 0);
@@ -344,42 +347,43 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
 
     if (warp < 4) regs_dec<OZ_REGS_LOW>();
     if (warp == 0) {
-        if (lane == 0) {
-            int stage = 0;
-            uint32_t phase = 0;
-            int last_parity[8];
-            for (int i = 0; i < 8; ++i) last_parity[i] = -1;
-            bool ok = true;
-            for (int i = 0; i < nitems && ok && !*abort; ++i) {
-                const OzItem it = oz_item(i, ntiles, npairs, pair, s);
-                int tm, tn;
-                tile_coords(it.t, tiles_m, tiles_n, tm, tn);
-                const int arow = tm * 2 * BM + int(rank) * BM;
-                const int brow = tn * PAIR_BN + int(rank) * BM;
-                for (int di = 0; di < oz_item_nd(it, s) && ok; ++di) {
-                    const int d = oz_item_d(it, di, s);
-                    for (int ta = oz_tlo(d, s); ta <= oz_thi(d, s) && ok; ++ta) {
-                        const int ub = d - ta;
-                        for (int kb = 0; kb < nkb; ++kb) {
-                            if (!mbar_wait(&bars->empty[stage], phase ^ 1u, g.timeout_ns, status, abort)) { ok = false; break; }
-                            uint8_t* a_dst = smem + stage * PAIR_STAGE_BYTES;
-                            uint8_t* b_dst = a_dst + BM * 128;
-                            const uint32_t full_leader = mapa_shared(smem_u32(&bars->full[stage]), 0);
-                            if (leader) mbar_arrive_expect_tx(&bars->full[stage], 2 * PAIR_STAGE_BYTES);
-                            tma_load_3d_pair(a_dst, &tmA, full_leader, kb * C_::BK, arow, ta - 1);
-                            tma_load_3d_pair(b_dst, &tmB, full_leader, kb * C_::BK, brow, ub - 1);
-                            last_parity[stage] = int(phase);
-                            if (++stage == PAIR_STAGES) { stage = 0; phase ^= 1u; }
-                        }
+        // both roles are run by their whole warps, one elected lane issues (see elect_one)
+        const bool issue = elect_one();
+        int stage = 0, filled = 0;
+        uint32_t phase = 0;
+        bool ok = true;
+        const uint32_t full0 = mapa_shared(smem_u32(&bars->full[0]), 0);
+        for (int i = 0; i < nitems && ok && !*abort; ++i) {
+            const OzItem it = oz_item(i, ntiles, npairs, pair, s);
+            int tm, tn;
+            tile_coords(it.t, tiles_m, tiles_n, tm, tn);
+            const int arow = tm * 2 * BM + int(rank) * BM;
+            const int brow = tn * PAIR_BN + int(rank) * BM;
+            for (int di = 0; di < oz_item_nd(it, s) && ok; ++di) {
+                const int d = oz_item_d(it, di, s);
+                for (int ta = oz_tlo(d, s); ta <= oz_thi(d, s) && ok; ++ta) {
+                    const int ub = d - ta;
+                    for (int kb = 0; kb < nkb; ++kb) {
+                        // the first round of stages starts empty
+                        if (filled >= PAIR_STAGES &&
+                            !mbar_wait_warp(&bars->empty[stage], phase ^ 1u, g.timeout_ns, status, abort)) { ok = false; break; }
+                        uint8_t* a_dst = smem + stage * PAIR_STAGE_BYTES;
+                        const uint32_t full_leader = full0 + uint32_t(stage) * 8u;
+                        mbar_arrive_expect_tx_if(issue && leader, &bars->full[stage], 2 * PAIR_STAGE_BYTES);
+                        tma_load_3d_pair_if(issue, a_dst, &tmA, full_leader, kb * C_::BK, arow, ta - 1);
+                        tma_load_3d_pair_if(issue, a_dst + BM * 128, &tmB, full_leader, kb * C_::BK, brow, ub - 1);
+                        ++filled;
+                        if (++stage == PAIR_STAGES) { stage = 0; phase ^= 1u; }
                     }
                 }
             }
-            // every issued stage is released (empty) only after its copies landed and were consumed
-            for (int i = 0; i < PAIR_STAGES; ++i)
-                if (last_parity[i] >= 0) mbar_wait(&bars->empty[i], uint32_t(last_parity[i]), g.timeout_ns, status, abort);
         }
+        // every issued stage is released (empty) only after its copies landed and were consumed
+        for (int f = max(0, filled - PAIR_STAGES); f < filled; ++f)
+            mbar_wait_warp(&bars->empty[f % PAIR_STAGES], uint32_t(f / PAIR_STAGES) & 1u, g.timeout_ns, status, abort);
     } else if (warp == 1) {
-        if (lane == 0 && leader) {
+        if (leader) {
+            const bool issue = elect_one();
             const uint32_t idesc = make_idesc(1u, false, false, 2 * BM, PAIR_BN);
             const uint64_t a0 = operand_desc<C_>(smem_u32(smem), 0, false);
             const uint64_t b0 = operand_desc<C_>(smem_u32(smem) + BM * 128, 0, false);
@@ -390,7 +394,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
             int abuf = 0;
             uint32_t aphase = 0;
             bool ok = true;
-            // One thread issues every MMA of the pair, so its own instruction time per k-block
+            // One warp issues every MMA of the pair, so its own instruction time per k-block
             // (one wait, four MMAs, one commit) has to stay below the 512 tensor-pipe cycles
             // the k-block takes.  The loop is kept lean for that: one counter per FP32 chunk,
             // descriptors formed from the stage index (no state carried between k-blocks
@@ -401,33 +405,33 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
                     const int d = oz_item_d(it, di, s);
                     int left_d = (oz_thi(d, s) - oz_tlo(d, s) + 1) * nkb;
                     while (left_d > 0 && ok) {
-                        if (!mbar_wait(&bars->acc_empty[abuf], aphase ^ 1u, g.timeout_ns, status, abort)) { ok = false; break; }
+                        if (!mbar_wait_warp(&bars->acc_empty[abuf], aphase ^ 1u, g.timeout_ns, status, abort)) { ok = false; break; }
                         tc_fence_after();
                         const uint32_t d_tmem = tmem + uint32_t(abuf * PAIR_BN);
                         const int nk = min(kcb, left_d);     // k-blocks of this exact FP32 chunk
 #pragma unroll 4
                         for (int j = 0; j < nk; ++j) {
-                            if (!mbar_wait(&bars->full[stage], phase, g.timeout_ns, status, abort)) { ok = false; break; }
+                            if (!mbar_wait_warp(&bars->full[stage], phase, g.timeout_ns, status, abort)) { ok = false; break; }
                             tc_fence_after();
                             const uint64_t ad = a0 + uint64_t(stage) * sstep, bd = b0 + uint64_t(stage) * sstep;
-                            umma_f16_pair(d_tmem, ad, bd, idesc, uint32_t(j));    // j == 0 starts the chunk
 #pragma unroll
-                            for (int ks = 1; ks < C_::KSTEPS; ++ks)
-                                umma_f16_pair(d_tmem, ad + ks * kstep, bd + ks * kstep, idesc, 1u);
-                            umma_commit_pair(&bars->empty[stage], 0x3);
+                            for (int ks = 0; ks < C_::KSTEPS; ++ks)   // j == 0, ks == 0 starts the chunk
+                                umma_pair_if<false>(issue, d_tmem, ad + ks * kstep, bd + ks * kstep, idesc,
+                                                    ks == 0 ? uint32_t(j) : 1u);
+                            umma_commit_pair_if(issue, &bars->empty[stage], 0x3);
                             stage = (stage + 1 == PAIR_STAGES) ? 0 : stage + 1;
                             phase ^= (stage == 0) ? 1u : 0u;
                         }
                         if (!ok) break;
-                        umma_commit_pair(&bars->acc_full[abuf], 0x3);
+                        umma_commit_pair_if(issue, &bars->acc_full[abuf], 0x3);
                         abuf ^= 1;
                         if (abuf == 0) aphase ^= 1u;
                         left_d -= nk;
                     }
                 }
             }
-            umma_commit_pair(&bars->mma_done, 0x1);
-            mbar_wait(&bars->mma_done, 0, g.timeout_ns, status, abort);
+            umma_commit_pair_if(issue, &bars->mma_done, 0x1);
+            mbar_wait_warp(&bars->mma_done, 0, g.timeout_ns, status, abort);
         }
     } else if (warp >= 4) {
         regs_inc<OZ_REGS_HIGH>();
