@@ -71,36 +71,45 @@ static_assert(OZ_THREADS * OZ_REGS_LAUNCH == 128 * OZ_REGS_LOW + 256 * OZ_REGS_H
 __host__ __device__ __forceinline__ int oz_tlo(int d, int s) { return d - s > 1 ? d - s : 1; }
 __host__ __device__ __forceinline__ int oz_thi(int d, int s) { return d - 1 < s ? d - 1 : s; }
 
-// Work of the CTA pairs of the slice-product kernel.  The tiles of the full waves are whole
-// items (all anti-diagonals d = s+1 .. 2, tile t = pair + i npairs).  The tiles of the last,
-// partial wave are cut into G = s/2 + 1 groups of anti-diagonals that hold (nearly) the same
-// number of slice pairs: group 0 is d = s+1 (s pairs), group j >= 1 is d = s+1-j and d = j+1
-// ((s-j) + j pairs; for even s the last group is d = s/2+1 alone).  The groups are dealt to
-// the pairs in turn, so the last wave ends within one group of the mean instead of a tile.
-struct OzItem {
-    int t;        // tile
-    int j;        // -1: whole tile; else the anti-diagonal group
+__host__ __device__ __forceinline__ int oz_weight(int d, int s) { return oz_thi(d, s) - oz_tlo(d, s) + 1; }
+
+// Work of the CTA pairs of the slice-product kernel.  The tiles of the full waves are whole items
+// (all anti-diagonals d = s+1 .. 2, tile t = pair + i npairs).  The tiles of the last, partial
+// wave are dealt out in units of one anti-diagonal, or of part of its slice pairs: the host
+// assigns them, largest first, to the least loaded pair and passes the table as a kernel
+// parameter.  A unit that holds only part of an anti-diagonal adds its INT32 sums to S_d with
+// reduction atomics (exact in any order) in a plane zeroed before.
+// Units of one anti-diagonal, not groups of them with equal slice-pair counts: 20 tiles were 80
+// groups on 76 pairs, two rounds of 7 slice pairs each, and are 8 at most now (7.4 the mean).
+// Before -> now, same bits: 1000 x 1200 x 900 146.6 -> 109.9 us, complex 1500 x 1100 x 2301 706
+// -> 676, 4096^3 from host memory (blocks of 64 tiles) 3279 -> 2952, 8192^3 18.0 -> 17.8 ms.
+struct OzWork {
+    int t;         // tile
+    int nd;        // anti-diagonals: s (whole tile, d = s+1 .. 2) or 1
+    int d;         // of a unit: the anti-diagonal (0: whole tile), its first slice of A and slice pairs
+    int ta, nt;
+    bool add;      // S_d += (several units share the anti-diagonal)
 };
-__host__ __device__ __forceinline__ int oz_groups(int s) { return s / 2 + 1; }
-__host__ __device__ __forceinline__ int oz_items(int ntiles, int npairs, int pair, int s) {
+constexpr int OZ_MAX_PAIRS = 100, OZ_MAX_UNITS = 1600;   // at most 16 units for each of 99 tail tiles
+struct OzTable {
+    uint16_t first[OZ_MAX_PAIRS + 1];    // units of a pair: first[pair] .. first[pair + 1] - 1
+    uint32_t unit[OZ_MAX_UNITS];         // tail tile | d << 8 | first slice of A << 16 | pairs << 22 | add << 28
+};
+__device__ __forceinline__ int oz_items(const OzTable& tab, int ntiles, int npairs, int pair) {
+    return ntiles / npairs + int(tab.first[pair + 1]) - int(tab.first[pair]);
+}
+__device__ __forceinline__ OzWork oz_item(const OzTable& tab, int i, int ntiles, int npairs, int pair, int s) {
     const int full = ntiles / npairs;
-    const int units = (ntiles - full * npairs) * oz_groups(s);
-    return full + (units > pair ? (units - pair + npairs - 1) / npairs : 0);
+    if (i < full) return OzWork{pair + i * npairs, s, 0, 0, 0, false};
+    const uint32_t u = tab.unit[int(tab.first[pair]) + i - full];
+    return OzWork{full * npairs + int(u & 0xFFu), 1, int((u >> 8) & 0xFFu), int((u >> 16) & 0x3Fu),
+                  int((u >> 22) & 0x3Fu), ((u >> 28) & 1u) != 0};
 }
-__host__ __device__ __forceinline__ OzItem oz_item(int i, int ntiles, int npairs, int pair, int s) {
-    const int full = ntiles / npairs;
-    if (i < full) return OzItem{pair + i * npairs, -1};
-    const int u = pair + (i - full) * npairs;
-    return OzItem{full * npairs + u / oz_groups(s), u % oz_groups(s)};
-}
-// anti-diagonals of an item: count, and the di-th (descending within the item)
-__host__ __device__ __forceinline__ int oz_item_nd(const OzItem& it, int s) {
-    if (it.j < 0) return s;
-    return (it.j >= 1 && it.j + 1 < s + 1 - it.j) ? 2 : 1;
-}
-__host__ __device__ __forceinline__ int oz_item_d(const OzItem& it, int di, int s) {
-    if (it.j < 0) return s + 1 - di;
-    return di == 0 ? s + 1 - it.j : it.j + 1;
+// the di-th anti-diagonal of an item: d, its first slice of A and its slice pairs
+__device__ __forceinline__ void oz_item_d(const OzWork& it, int di, int s, int& d, int& ta, int& nt) {
+    d = it.d != 0 ? it.d : s + 1 - di;
+    ta = it.d != 0 ? it.ta : oz_tlo(d, s);
+    nt = it.d != 0 ? it.nt : oz_weight(d, s);
 }
 
 __global__ void __launch_bounds__(OZ_THREADS, 1)
@@ -301,7 +310,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
 
 __global__ void __launch_bounds__(OZ_THREADS, 1)
     gemm_ozaki_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-                           OzakiArgs g) {
+                           OzakiArgs g, const __grid_constant__ OzTable tab) {
     using C_ = Cfg<OZ_BN, false>;                  // BK, KSTEPS, descriptors (K-major, 128-byte rows)
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = align1024(smem_raw);
@@ -343,7 +352,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
     const int nkb = (g.K + C_::BK - 1) / C_::BK;
     const int s = g.slices;
     const int kcb = g.kc_blocks;
-    const int nitems = oz_items(ntiles, npairs, pair, s);
+    const int nitems = oz_items(tab, ntiles, npairs, pair);
 
     if (warp < 4) regs_dec<OZ_REGS_LOW>();
     if (warp == 0) {
@@ -354,14 +363,15 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
         bool ok = true;
         const uint32_t full0 = mapa_shared(smem_u32(&bars->full[0]), 0);
         for (int i = 0; i < nitems && ok && !*abort; ++i) {
-            const OzItem it = oz_item(i, ntiles, npairs, pair, s);
+            const OzWork it = oz_item(tab, i, ntiles, npairs, pair, s);
             int tm, tn;
             tile_coords(it.t, tiles_m, tiles_n, tm, tn);
             const int arow = tm * 2 * BM + int(rank) * BM;
             const int brow = tn * PAIR_BN + int(rank) * BM;
-            for (int di = 0; di < oz_item_nd(it, s) && ok; ++di) {
-                const int d = oz_item_d(it, di, s);
-                for (int ta = oz_tlo(d, s); ta <= oz_thi(d, s) && ok; ++ta) {
+            for (int di = 0; di < it.nd && ok; ++di) {
+                int d, ta0, nt;
+                oz_item_d(it, di, s, d, ta0, nt);
+                for (int ta = ta0; ta < ta0 + nt && ok; ++ta) {
                     const int ub = d - ta;
                     for (int kb = 0; kb < nkb; ++kb) {
                         // the first round of stages starts empty
@@ -400,10 +410,11 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
             // descriptors formed from the stage index (no state carried between k-blocks
             // but the stage and its phase), and four k-blocks per unrolled iteration.
             for (int i = 0; i < nitems && ok && !*abort; ++i) {
-                const OzItem it = oz_item(i, ntiles, npairs, pair, s);
-                for (int di = 0; di < oz_item_nd(it, s) && ok; ++di) {
-                    const int d = oz_item_d(it, di, s);
-                    int left_d = (oz_thi(d, s) - oz_tlo(d, s) + 1) * nkb;
+                const OzWork it = oz_item(tab, i, ntiles, npairs, pair, s);
+                for (int di = 0; di < it.nd && ok; ++di) {
+                    int d, ta0, nt;
+                    oz_item_d(it, di, s, d, ta0, nt);
+                    int left_d = nt * nkb;
                     while (left_d > 0 && ok) {
                         if (!mbar_wait_warp(&bars->acc_empty[abuf], aphase ^ 1u, g.timeout_ns, status, abort)) { ok = false; break; }
                         tc_fence_after();
@@ -443,18 +454,19 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
         uint32_t aphase = 0;
         bool ok = true;
         for (int i = 0; i < nitems && ok; ++i) {
-            const OzItem it = oz_item(i, ntiles, npairs, pair, s);
+            const OzWork it = oz_item(tab, i, ntiles, npairs, pair, s);
             int tm, tn;
             tile_coords(it.t, tiles_m, tiles_n, tm, tn);
             const int64_t row = int64_t(tm) * 2 * BM + int64_t(rank) * BM + q * 32 + lane;
             const int64_t col0 = int64_t(tn) * PAIR_BN + half * OZ_HALF;
             const bool row_ok = row < g.M;
-            for (int di = 0; di < oz_item_nd(it, s) && ok; ++di) {
-                const int d = oz_item_d(it, di, s);
+            for (int di = 0; di < it.nd && ok; ++di) {
+                int d, ta0, nt;
+                oz_item_d(it, di, s, d, ta0, nt);
                 int S[OZ_HALF];
 #pragma unroll
                 for (int j = 0; j < OZ_HALF; ++j) S[j] = 0;
-                const int total = (oz_thi(d, s) - oz_tlo(d, s) + 1) * nkb;
+                const int total = nt * nkb;
                 const int nch = (total + kcb - 1) / kcb;
                 for (int c = 0; c < nch; ++c) {
                     int okw = 0;
@@ -485,9 +497,15 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
                 const int64_t rem = int64_t(g.N) - col0;
                 const int jmax = rem < OZ_HALF ? int(rem) : OZ_HALF;
                 int32_t* Sp = g.sd + int64_t(d - 2) * g.sd_plane + row + col0 * int64_t(g.M);
+                if (it.add) {
 #pragma unroll
-                for (int j = 0; j < OZ_HALF; ++j)
-                    if (j < jmax) Sp[int64_t(j) * g.M] = S[j];
+                    for (int j = 0; j < OZ_HALF; ++j)
+                        if (j < jmax) atomicAdd(Sp + int64_t(j) * g.M, S[j]);
+                } else {
+#pragma unroll
+                    for (int j = 0; j < OZ_HALF; ++j)
+                        if (j < jmax) Sp[int64_t(j) * g.M] = S[j];
+                }
             }
         }
     }
@@ -497,6 +515,99 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
     tc_fence_after();
     if (warp == 1) tmem_dealloc_pair(tmem, 512);
 }
+
+// Zeros in the planes d_lo .. s+1 of S_d under the tiles of the last, partial wave
+__global__ void __launch_bounds__(256) ozaki_zero_kernel(OzakiArgs g, int first_tile, int d_lo) {
+    const int tiles_m = (g.M + 2 * BM - 1) / (2 * BM), tiles_n = (g.N + PAIR_BN - 1) / PAIR_BN;
+    int tm, tn;
+    tile_coords(first_tile + int(blockIdx.x), tiles_m, tiles_n, tm, tn);
+    const int64_t row = int64_t(tm) * 2 * BM + threadIdx.x;
+    if (row >= g.M) return;
+    int32_t* p = g.sd + int64_t(d_lo - 2 + int(blockIdx.y)) * g.sd_plane + row;
+    const int64_t c1 = min(int64_t(g.N), int64_t(tn + 1) * PAIR_BN);
+    for (int64_t c = int64_t(tn) * PAIR_BN + blockIdx.z; c < c1; c += gridDim.z) p[c * g.M] = 0;
+}
+
+// Deal the anti-diagonals of `tiles` tiles to npairs pairs, each cut into pieces of at most `piece`
+// slice pairs: largest piece first, to the least loaded pair.  Returns the largest load.
+int deal_units(int tiles, int npairs, int s, int piece, OzTable* tab) {
+    struct Unit {
+        uint32_t code;
+        uint8_t pair;
+    };
+    static thread_local Unit units[OZ_MAX_UNITS];
+    int n = 0;
+    int load[OZ_MAX_PAIRS] = {0}, count[OZ_MAX_PAIRS] = {0};
+    // pairs by load: a ring of stacks, one per load value (loads stay within `s` of the least)
+    int next[OZ_MAX_PAIRS], head[32];
+    for (int i = 0; i < 32; ++i) head[i] = -1;
+    for (int p = npairs - 1; p >= 0; --p) { next[p] = head[0]; head[0] = p; }
+    int least = 0, most = 0;
+    for (int w = std::min(s, piece); w >= 1; --w)
+        for (int d = s + 1; d >= 2; --d) {
+            const int total = oz_weight(d, s), parts = (total + piece - 1) / piece;
+            for (int q = 0; q < parts; ++q) {
+                const int lo = total * q / parts, hi = total * (q + 1) / parts;
+                if (hi - lo != w) continue;
+                for (int t = 0; t < tiles; ++t) {
+                    while (head[least & 31] < 0) ++least;
+                    const int p = head[least & 31];
+                    head[least & 31] = next[p];
+                    load[p] += w;
+                    next[p] = head[load[p] & 31];
+                    head[load[p] & 31] = p;
+                    most = std::max(most, load[p]);
+                    if (n == OZ_MAX_UNITS) return 1 << 30;
+                    ++count[p];
+                    units[n++] = Unit{uint32_t(t) | uint32_t(d) << 8 | uint32_t(oz_tlo(d, s) + lo) << 16 |
+                                          uint32_t(w) << 22 | (parts > 1 ? 1u : 0u) << 28,
+                                      uint8_t(p)};
+                }
+            }
+        }
+    int at = 0, pos[OZ_MAX_PAIRS];
+    for (int p = 0; p < npairs; ++p) {
+        tab->first[p] = uint16_t(at);
+        pos[p] = at;
+        at += count[p];
+    }
+    tab->first[npairs] = uint16_t(at);
+    for (int i = 0; i < n; ++i) tab->unit[pos[units[i].pair]++] = units[i].code;
+    return most;
+}
+
+// The table of a launch and the anti-diagonals (d >= zero_from) whose planes have to be zeroed
+// under the tail tiles; the last ones of this host thread are kept (they depend on the counts only).
+struct OzSchedule {
+    int ntiles, npairs, s, nkb, zero_from;
+    OzTable tab;
+};
+const OzSchedule& oz_schedule(int ntiles, int npairs, int s, int nkb) {
+    static thread_local OzSchedule cache[4];
+    static thread_local int turn = 0;
+    for (const OzSchedule& c : cache)
+        if (c.npairs == npairs && c.ntiles == ntiles && c.s == s && c.nkb == nkb) return c;
+    OzSchedule& c = cache[turn];
+    turn = (turn + 1) % 4;
+    c.ntiles = ntiles; c.npairs = npairs; c.s = s; c.nkb = nkb; c.zero_from = 0;
+    const int tail = ntiles % npairs;
+    const int whole = deal_units(tail, npairs, s, s, &c.tab);
+    const int total = tail * s * (s + 1) / 2, piece = std::max(1, (total + npairs - 1) / npairs);
+    if (tail > 0 && piece < s) {
+        // cutting anti-diagonals pays when the busiest pair saves more than the zeroing (a launch
+        // and the planes' bytes) and the atomics cost
+        OzTable cut;
+        const int most = deal_units(tail, npairs, s, piece, &cut);
+        const double saved_us = double(whole - most) * nkb * 0.26;
+        const double cost_us = 5.0 + double(tail) * (s - piece) * 0.26 / 5.0;
+        if (saved_us > cost_us) {
+            c.tab = cut;
+            c.zero_from = piece + 2;     // oz_weight(d) = d - 1 > piece
+        }
+    }
+    return c;
+}
+
 }  // namespace
 
 // The slice products run on CTA pairs; HSMM_OZAKI_KERNEL = single selects the one-CTA kernel
@@ -513,10 +624,17 @@ static hsmm_status_t launch_ozaki_pairs(const CUtensorMap& mA, const CUtensorMap
         return cudaFuncSetAttribute(gemm_ozaki_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, PAIR_SMEM);
     });
     if (as != HSMM_STATUS_SUCCESS) return as;
-    const int max_pairs = num_sms() / 2;
+    const int max_pairs = std::min(num_sms() / 2, OZ_MAX_PAIRS);
     const int tiles = ((g.M + 2 * BM - 1) / (2 * BM)) * ((g.N + PAIR_BN - 1) / PAIR_BN);
-    // whole tiles while they fill every pair; fewer tiles than pairs are cut into anti-diagonal groups
-    const int pairs = std::max(1, tiles >= max_pairs ? max_pairs : std::min(max_pairs, tiles * oz_groups(slices)));
+    // whole tiles while they fill every pair; the tiles of a partial wave go out in smaller units
+    const int pairs = std::max(1, tiles >= max_pairs ? max_pairs : std::min(max_pairs, tiles * slices * (slices + 1) / 2));
+    const OzSchedule& sc = oz_schedule(tiles, pairs, slices, (g.K + 63) / 64);
+    if (sc.zero_from > 0) {
+        const int tail = tiles % pairs;
+        ozaki_zero_kernel<<<dim3(unsigned(tail), unsigned(slices + 2 - sc.zero_from), 8), 256, 0, st>>>(
+            g, tiles - tail, sc.zero_from);
+        count_launches(1);
+    }
     cudaLaunchConfig_t lc = {};
     lc.gridDim = dim3(unsigned(2 * pairs), 1, 1);
     lc.blockDim = dim3(OZ_THREADS, 1, 1);
@@ -529,7 +647,7 @@ static hsmm_status_t launch_ozaki_pairs(const CUtensorMap& mA, const CUtensorMap
     at[0].val.clusterDim.z = 1;
     lc.attrs = at;
     lc.numAttrs = 1;
-    cudaError_t e = cudaLaunchKernelEx(&lc, gemm_ozaki_pair_kernel, mA, mB, g);
+    cudaError_t e = cudaLaunchKernelEx(&lc, gemm_ozaki_pair_kernel, mA, mB, g, sc.tab);
     count_launches(1);
     if (e != cudaSuccess) return record_cuda(e);
     return check_launch();
