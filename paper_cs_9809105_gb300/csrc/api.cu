@@ -110,20 +110,14 @@ OzakiLayout ozaki_layout(int64_t m, int64_t n, int64_t k, int slices) {
     return L;
 }
 
-hsmm_status_t ozaki_split_op_a(bool cplx, hsmm_op_t ta, int64_t m, int64_t k, const void* A, int64_t lda, int bits,
-                               int s, int32_t* ea, void* qa, int64_t ldq, int64_t plane, cudaStream_t st) {
-    if (cplx) return ozaki_zsplit(m, k, A, lda, ta == HSMM_OP_N, ta == HSMM_OP_C, false, bits, s, ea, qa, ldq, plane, st);
-    if (ta == HSMM_OP_N)
-        return ozaki_split(m, k, static_cast<const double*>(A), lda, true, bits, s, ea, qa, ldq, plane, st);
-    return ozaki_split(k, m, static_cast<const double*>(A), lda, false, bits, s, ea, qa, ldq, plane, st);
+SplitOperand split_operand_a(bool cplx, hsmm_op_t ta, int64_t m, int64_t k, const void* A, int64_t lda, int32_t* ea,
+                             void* qa, int64_t ldq, int64_t plane) {
+    return SplitOperand{A, lda, m, k, ta == HSMM_OP_N, cplx && ta == HSMM_OP_C, false, ea, qa, ldq, plane};
 }
 
-hsmm_status_t ozaki_split_op_b(bool cplx, hsmm_op_t tb, int64_t k, int64_t n, const void* B, int64_t ldb, int bits,
-                               int s, int32_t* eb, void* qb, int64_t ldq, int64_t plane, cudaStream_t st) {
-    if (cplx) return ozaki_zsplit(n, k, B, ldb, tb != HSMM_OP_N, tb == HSMM_OP_C, true, bits, s, eb, qb, ldq, plane, st);
-    if (tb == HSMM_OP_N)
-        return ozaki_split(k, n, static_cast<const double*>(B), ldb, false, bits, s, eb, qb, ldq, plane, st);
-    return ozaki_split(n, k, static_cast<const double*>(B), ldb, true, bits, s, eb, qb, ldq, plane, st);
+SplitOperand split_operand_b(bool cplx, hsmm_op_t tb, int64_t k, int64_t n, const void* B, int64_t ldb, int32_t* eb,
+                             void* qb, int64_t ldq, int64_t plane) {
+    return SplitOperand{B, ldb, n, k, tb != HSMM_OP_N, cplx && tb == HSMM_OP_C, true, eb, qb, ldq, plane};
 }
 
 int default_slices(const hsmm_config_t* c) { return c->ozaki_slices > 0 ? c->ozaki_slices : 7; }
@@ -266,9 +260,9 @@ hsmm_status_t hsmm_gemm(const hsmm_config_t* cfg, hsmm_op_t transA, hsmm_op_t tr
         int32_t* ea = reinterpret_cast<int32_t*>(ws + L.ea);
         int32_t* eb = reinterpret_cast<int32_t*>(ws + L.eb);
         int32_t* sd = reinterpret_cast<int32_t*>(ws + L.sd);
-        hsmm_status_t r = ozaki_split_op_a(true, transA, m, k, A, lda, bits, s, ea, ws + L.qa, L.ldq, L.qa_plane, st);
-        if (r == HSMM_STATUS_SUCCESS)
-            r = ozaki_split_op_b(true, transB, k, n, B, ldb, bits, s, eb, ws + L.qb, L.ldq, L.qb_plane, st);
+        const SplitOperand ops[2] = {split_operand_a(true, transA, m, k, A, lda, ea, ws + L.qa, L.ldq, L.qa_plane),
+                                     split_operand_b(true, transB, k, n, B, ldb, eb, ws + L.qb, L.ldq, L.qb_plane)};
+        hsmm_status_t r = ozaki_split(true, ops, 2, bits, s, st);
         if (r == HSMM_STATUS_SUCCESS)
             r = gemm_ozaki_slices(m, 2 * n, 2 * k, L.ldq, s, bits, ws + L.qa, L.qa_plane, ws + L.qb, L.qb_plane, sd,
                                   L.sd_plane, st);
@@ -321,9 +315,9 @@ hsmm_status_t hsmm_gemm(const hsmm_config_t* cfg, hsmm_op_t transA, hsmm_op_t tr
     uint8_t* ws = static_cast<uint8_t*>(c.workspace);
     int32_t* ea = reinterpret_cast<int32_t*>(ws + L.ea);
     int32_t* eb = reinterpret_cast<int32_t*>(ws + L.eb);
-    hsmm_status_t r = ozaki_split_op_a(false, transA, m, k, A, lda, bits, s, ea, ws + L.qa, L.ldq, L.qa_plane, st);
-    if (r != HSMM_STATUS_SUCCESS) return r;
-    r = ozaki_split_op_b(false, transB, k, n, B, ldb, bits, s, eb, ws + L.qb, L.ldq, L.qb_plane, st);
+    const SplitOperand ops[2] = {split_operand_a(false, transA, m, k, A, lda, ea, ws + L.qa, L.ldq, L.qa_plane),
+                                 split_operand_b(false, transB, k, n, B, ldb, eb, ws + L.qb, L.ldq, L.qb_plane)};
+    hsmm_status_t r = ozaki_split(false, ops, 2, bits, s, st);
     if (r != HSMM_STATUS_SUCCESS) return r;
     int32_t* sd = reinterpret_cast<int32_t*>(ws + L.sd);
     r = gemm_ozaki_slices(m, n, k, L.ldq, s, bits, ws + L.qa, L.qa_plane, ws + L.qb, L.qb_plane, sd, L.sd_plane, st);
@@ -379,8 +373,8 @@ hsmm_status_t hsmm_ozaki_split(int64_t rows, int64_t cols, const double* M, int6
     if (plane < nv * ldq || plane % 8 != 0) return fail(HSMM_STATUS_INVALID_VALUE, "ozaki_split: bad slice pitch");
     if (rows == 0 || cols == 0) return HSMM_STATUS_SUCCESS;
     if (!M || !expo || !q) return HSMM_STATUS_INVALID_VALUE;
-    return ozaki_split(rows, cols, M, ld, by_rows != 0, bits, slices, expo, q, ldq, plane,
-                       static_cast<cudaStream_t>(stream));
+    const SplitOperand op{M, ld, nv, len, by_rows != 0, false, false, expo, q, ldq, plane};
+    return ozaki_split(false, &op, 1, bits, slices, static_cast<cudaStream_t>(stream));
 }
 
 hsmm_status_t hsmm_ozaki_slice_products(int64_t m, int64_t n, int64_t k, int slices, int bits, const void* qa,

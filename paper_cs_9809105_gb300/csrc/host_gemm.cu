@@ -251,9 +251,11 @@ extern "C" hsmm_status_t hsmm_gemm_host(const hsmm_config_t* cfg, hsmm_op_t tran
     auto split_a = [&](int I) {
         const int64_t i0 = I * P.mi, h = panel_h(I);
         hsmm_status_t q = record_cuda(cudaStreamWaitEvent(S, evA[I], 0));
-        if (q == HSMM_STATUS_SUCCESS && ozaki_run)
-            q = ozaki_split_op_a(P.cplx, transA, h, k, dA + a_row(i0, P.ldA), P.ldA, P.bits, P.slices, ea + i0,
-                                 qa + i0 * P.L.ldq * 2, P.L.ldq, P.L.qa_plane, S);
+        if (q == HSMM_STATUS_SUCCESS && ozaki_run) {
+            const SplitOperand op = split_operand_a(P.cplx, transA, h, k, dA + a_row(i0, P.ldA), P.ldA, ea + i0,
+                                                    qa + i0 * P.L.ldq * 2, P.L.ldq, P.L.qa_plane);
+            q = ozaki_split(P.cplx, &op, 1, P.bits, P.slices, S);
+        }
         return q;
     };
     r = split_a(0);
@@ -261,9 +263,11 @@ extern "C" hsmm_status_t hsmm_gemm_host(const hsmm_config_t* cfg, hsmm_op_t tran
         const int64_t j0 = J * P.nj, w = panel_w(J);
         r = record_cuda(cudaStreamWaitEvent(S, evB[J], 0));
         const uint8_t* dBp = (transB == HSMM_OP_N) ? dB + j0 * P.ldB * P.eb : dB + j0 * P.eb;
-        if (r == HSMM_STATUS_SUCCESS && ozaki_run)
-            r = ozaki_split_op_b(P.cplx, transB, k, w, dBp, P.ldB, P.bits, P.slices, eb, W + P.L.qb, P.L.ldq,
-                                 P.L.qb_plane, S);
+        if (r == HSMM_STATUS_SUCCESS && ozaki_run) {
+            const SplitOperand op = split_operand_b(P.cplx, transB, k, w, dBp, P.ldB, eb, W + P.L.qb, P.L.ldq,
+                                                    P.L.qb_plane);
+            r = ozaki_split(P.cplx, &op, 1, P.bits, P.slices, S);
+        }
         for (int I = 0; I < P.rpanels && r == HSMM_STATUS_SUCCESS; ++I) {
             const int64_t i0 = I * P.mi, h = panel_h(I);
             const uint8_t* dAp = dA + a_row(i0, P.ldA);

@@ -119,17 +119,25 @@ hsmm_status_t gemm_ozaki_slices(int64_t m, int64_t n, int64_t k, int64_t ldq, in
                                 cudaStream_t st);
 
 // ---- ozaki.cu ----
-// slices written as [t][v][w]: row pitch ldq, slice (plane) pitch `plane` elements (>= lines * ldq)
-hsmm_status_t ozaki_split(int64_t rows, int64_t cols, const double* M, int64_t ld, bool by_rows, int bits,
-                          int slices, int32_t* expo, void* q, int64_t ldq, int64_t plane, cudaStream_t st);
+// One operand to split: nv lines of nw entries, entry (v, w) at M[v + w ld] (v_contig) or
+// M[w + v ld]; slices written as [t][v][w] with row pitch ldq and slice (plane) pitch `plane`
+// elements (>= lines * ldq).  Complex operands go into the real form of the complex product (A' =
+// [Re, Im] rows for role_b = false; B'' = [[Re, Im], [-Im, Re]] columns for role_b = true, 2 nv
+// lines); conj: op = C.
+struct SplitOperand {
+    const void* M;
+    int64_t ld, nv, nw;
+    bool v_contig, conj, role_b;
+    int32_t* expo;
+    void* q;
+    int64_t ldq, plane;
+};
+// Splits one or two operands (count), in one launch if their lines run the same way in memory.
+hsmm_status_t ozaki_split(bool cplx, const SplitOperand* ops, int count, int bits, int slices, cudaStream_t st);
 // C = alpha 2^(ea_i + eb_j) sum_d 2^(-bits d) S_d + beta C
 hsmm_status_t ozaki_recombine(int64_t m, int64_t n, int slices, int bits, const int32_t* sd, int64_t sd_plane,
                               const int32_t* ea, const int32_t* eb, double alpha, double beta, double* C, int64_t ldc,
                               cudaStream_t st);
-// Complex operands into the real form of the complex product (A' = [Re, Im] rows of op(A) for
-// role_b = false; B'' = [[Re, Im], [-Im, Re]] columns of op(B) for role_b = true, 2 nv lines)
-hsmm_status_t ozaki_zsplit(int64_t nv, int64_t nw, const void* M, int64_t ld, bool v_contig, bool conj, bool role_b,
-                           int bits, int slices, int32_t* expo, void* q, int64_t ldq, int64_t plane, cudaStream_t st);
 // C = alpha (Re + i Im) + beta C from the real form's S_d (m x 2n), complex alpha, beta (re, im)
 hsmm_status_t ozaki_zrecombine(int64_t m, int64_t n, int slices, int bits, const int32_t* sd, int64_t sd_plane,
                                const int32_t* ea, const int32_t* eb, const double* alpha, const double* beta, void* C,
@@ -142,12 +150,11 @@ struct OzakiLayout {
 OzakiLayout ozaki_layout(int64_t m, int64_t n, int64_t k, int slices);
 int default_slices(const hsmm_config_t* c);   // cfg->ozaki_slices, or 7
 int default_bits(const hsmm_config_t* c);     // cfg->ozaki_bits, or 7
-// Rows of op(A) (m x k) / columns of op(B) (k x n) into slices; cplx: complex operands into the
-// real form (A' = [Re, Im]; B'' = [[Re, Im], [-Im, Re]], 2n lines)
-hsmm_status_t ozaki_split_op_a(bool cplx, hsmm_op_t ta, int64_t m, int64_t k, const void* A, int64_t lda, int bits,
-                               int s, int32_t* ea, void* qa, int64_t ldq, int64_t plane, cudaStream_t st);
-hsmm_status_t ozaki_split_op_b(bool cplx, hsmm_op_t tb, int64_t k, int64_t n, const void* B, int64_t ldb, int bits,
-                               int s, int32_t* eb, void* qb, int64_t ldq, int64_t plane, cudaStream_t st);
+// Rows of op(A) (m x k) / columns of op(B) (k x n) as operands to split; cplx: complex operands
+SplitOperand split_operand_a(bool cplx, hsmm_op_t ta, int64_t m, int64_t k, const void* A, int64_t lda, int32_t* ea,
+                             void* qa, int64_t ldq, int64_t plane);
+SplitOperand split_operand_b(bool cplx, hsmm_op_t tb, int64_t k, int64_t n, const void* B, int64_t ldb, int32_t* eb,
+                             void* qb, int64_t ldq, int64_t plane);
 // Plane pitch (elements) of the workspace planes of hsmm_gemm's FP64-accurate form: the
 // plane size rounded up to 256 bytes plus 1 KiB, so that the s planes one thread touches
 // are not a power of two apart (such strides land on the same DRAM channels).

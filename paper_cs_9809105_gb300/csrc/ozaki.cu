@@ -10,9 +10,10 @@
 // op(B)), w = the contraction index, contiguous, row pitch ldq (a multiple of 8 so
 // that the TMA row stride is a multiple of 16 bytes).
 //
-// Kernels: (1) exponent init, (2) per-line maximum exponent with atomicMax,
-// (3) slicing (transposing through shared memory when the input has v contiguous),
-// (4) zero-line fix-up of the exponents.  All HBM-bound.
+// One launch splits both operands of a product (or one): every CTA finds the exponents of its
+// lines and slices them while they are still on the chip.
+#include <algorithm>
+#include <atomic>
 #include <climits>
 #include <cstdint>
 #include <cuda_bf16.h>
@@ -41,16 +42,6 @@ int64_t ozaki_plane_pitch(int64_t elems, int64_t elem_bytes) {
 
 namespace {
 
-__global__ void expo_init(int64_t nvec, int32_t* expo) {
-    const int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (i < nvec) expo[i] = INT_MIN;
-}
-
-__global__ void expo_fix(int64_t nvec, int32_t* expo) {
-    const int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (i < nvec && expo[i] == INT_MIN) expo[i] = 0;
-}
-
 __device__ __forceinline__ int line_exponent(double mx) {
     if (mx == 0.0) return INT_MIN;
     int e;
@@ -76,91 +67,6 @@ __device__ __forceinline__ int line_exponent_bits(uint64_t mb) {
     return top == 0 ? INT_MIN : line_exponent(__longlong_as_double(int64_t(top)));
 }
 
-// v contiguous in memory (M(v, w) at v + w*ld): thread per v, w split over blockIdx.y;
-// four independent maxima keep four loads in flight per thread
-__global__ void __launch_bounds__(256) expo_vcontig(int64_t nv, int64_t nw, const double* __restrict__ M, int64_t ld,
-                                                   int64_t w_per_split, int32_t* expo) {
-    const int64_t v = int64_t(blockIdx.x) * 256 + threadIdx.x;
-    if (v >= nv) return;
-    const int64_t w0 = int64_t(blockIdx.y) * w_per_split;
-    const int64_t w1 = min(nw, w0 + w_per_split);
-    const double* p = M + v;
-    uint64_t m0 = 0, m1 = 0, m2 = 0, m3 = 0;
-    int64_t w = w0;
-    for (; w + 4 <= w1; w += 4) {
-        m0 = mag_max(m0, mag_bits(__ldcs(p + (w + 0) * ld)));
-        m1 = mag_max(m1, mag_bits(__ldcs(p + (w + 1) * ld)));
-        m2 = mag_max(m2, mag_bits(__ldcs(p + (w + 2) * ld)));
-        m3 = mag_max(m3, mag_bits(__ldcs(p + (w + 3) * ld)));
-    }
-    for (; w < w1; ++w) m0 = mag_max(m0, mag_bits(__ldcs(p + w * ld)));
-    const int e = line_exponent_bits(mag_max(mag_max(m0, m1), mag_max(m2, m3)));
-    if (e != INT_MIN) atomicMax(&expo[v], e);
-}
-
-// The same with two lines per thread and 16-byte loads (nv even, ld even, M 16-byte aligned):
-// half the load requests
-__global__ void __launch_bounds__(256) expo_vcontig2(int64_t nv, int64_t nw, const double* __restrict__ M, int64_t ld,
-                                                    int64_t w_per_split, int32_t* expo) {
-    const int64_t v = (int64_t(blockIdx.x) * 256 + threadIdx.x) * 2;
-    if (v >= nv) return;
-    const int64_t w0 = int64_t(blockIdx.y) * w_per_split;
-    const int64_t w1 = min(nw, w0 + w_per_split);
-    const double2* p = reinterpret_cast<const double2*>(M + v);
-    const int64_t ld2 = ld / 2;
-    uint64_t a0 = 0, a1 = 0, b0 = 0, b1 = 0;
-    int64_t w = w0;
-    for (; w + 2 <= w1; w += 2) {
-        const double2 x0 = __ldcs(p + w * ld2), x1 = __ldcs(p + (w + 1) * ld2);
-        a0 = mag_max(a0, mag_bits(x0.x));
-        b0 = mag_max(b0, mag_bits(x0.y));
-        a1 = mag_max(a1, mag_bits(x1.x));
-        b1 = mag_max(b1, mag_bits(x1.y));
-    }
-    if (w < w1) {
-        const double2 x0 = __ldcs(p + w * ld2);
-        a0 = mag_max(a0, mag_bits(x0.x));
-        b0 = mag_max(b0, mag_bits(x0.y));
-    }
-    const int ea = line_exponent_bits(mag_max(a0, a1)), eb = line_exponent_bits(mag_max(b0, b1));
-    if (ea != INT_MIN) atomicMax(&expo[v], ea);
-    if (eb != INT_MIN) atomicMax(&expo[v + 1], eb);
-}
-
-// w contiguous in memory (M(w, v) at w + v*ld): block per (v, w-chunk)
-__global__ void __launch_bounds__(256) expo_wcontig(int64_t nv, int64_t nw, const double* __restrict__ M, int64_t ld,
-                                                   int64_t w_per_split, int32_t* expo) {
-    const int64_t v = blockIdx.x;
-    const int64_t w0 = int64_t(blockIdx.y) * w_per_split;
-    const int64_t w1 = min(nw, w0 + w_per_split);
-    uint64_t mx = 0;
-    const double* line = M + v * ld;
-    if ((reinterpret_cast<uintptr_t>(line + w0) & 15u) == 0) {
-        // 16-byte loads: two consecutive entries per thread and step (the line start is aligned)
-        const double2* l2 = reinterpret_cast<const double2*>(line + w0);
-        const int64_t n2 = (w1 - w0) / 2;
-        for (int64_t i = threadIdx.x; i < n2; i += 256) {
-            const double2 x = __ldcs(l2 + i);
-            mx = mag_max(mx, mag_max(mag_bits(x.x), mag_bits(x.y)));
-        }
-        if (threadIdx.x == 0 && ((w1 - w0) & 1)) mx = mag_max(mx, mag_bits(__ldcs(line + w1 - 1)));
-    } else {
-        for (int64_t w = w0 + threadIdx.x; w < w1; w += 256) mx = mag_max(mx, mag_bits(__ldcs(line + w)));
-    }
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) mx = mag_max(mx, __shfl_xor_sync(0xffffffffu, mx, off));
-    __shared__ uint64_t red[8];
-    if (lane_id() == 0) red[warp_id()] = mx;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        uint64_t m2 = red[0];
-        for (int i = 1; i < 8; ++i) m2 = mag_max(m2, red[i]);
-        const int e = line_exponent_bits(m2);
-        if (e != INT_MIN) atomicMax(&expo[v], e);
-    }
-    (void)nv;
-}
-
 // BF16 bit pattern of a small integer q (|q| <= 255: exact), from integer operations only
 __device__ __forceinline__ uint16_t bf16_of_small_int(uint32_t mag, uint32_t neg) {
     if (mag == 0) return 0;
@@ -169,92 +75,11 @@ __device__ __forceinline__ uint16_t bf16_of_small_int(uint32_t mag, uint32_t neg
     return uint16_t((neg << 15) | ((127u + top) << 7) | mant);
 }
 
-// Slice one value into s digits of `bits` bits, truncating toward zero.  With
-// |v| = M 2^(E-1075) (M the 53-bit significand), digit t of |v| 2^(-e) is
-//   floor(M 2^(E - 1075 - e + bits t)) mod 2^bits,
-// read from the significand with integer shifts: the same digits the FP64 steps
-// y = x 2^bits, q = trunc(y), x = y - q produce, without FP64 arithmetic (the FP64
-// pipe of this GPU is narrow).  Each digit carries the sign of v.
-__device__ __forceinline__ void slice_value(double val, int e, int bits, int s, __nv_bfloat16* out,
-                                            int64_t slice_stride) {
-    const uint64_t u = uint64_t(__double_as_longlong(val));
-    const uint32_t neg = uint32_t(u >> 63);
-    int E = int((u >> 52) & 0x7FF);
-    uint64_t M = u & ((uint64_t(1) << 52) - 1);
-    if (E != 0) M |= uint64_t(1) << 52; else E = 1;           // subnormals: no implicit bit
-    const uint32_t mask = (1u << bits) - 1u;
-    uint16_t* o = reinterpret_cast<uint16_t*>(out);
-    if (e == INT_MIN || M == 0) {
-        for (int t = 0; t < s; ++t) o[int64_t(t) * slice_stride] = 0;
-        return;
-    }
-    const int base = E - 1075 - e;                             // <= -53 because |v| < 2^e
-    if (bits * s <= 63) {
-        // all s digits at once: F = floor(|v| 2^(bits s - e)) fits in 63 bits
-        const int sh = base + bits * s;
-        const uint64_t F = sh >= 0 ? (M << sh) : (-sh >= 64 ? 0 : (M >> -sh));
-        for (int t = 1; t <= s; ++t) {
-            const uint32_t d = uint32_t(F >> (bits * (s - t))) & mask;
-            o[int64_t(t - 1) * slice_stride] = bf16_of_small_int(d, neg);
-        }
-    } else {
-        for (int t = 1; t <= s; ++t) {
-            const int sh = base + bits * t;
-            uint32_t d;
-            if (sh < 0) d = (-sh >= 64) ? 0u : uint32_t(M >> -sh) & mask;
-            else d = (sh >= bits) ? 0u : uint32_t(M << sh) & mask;
-            o[int64_t(t - 1) * slice_stride] = bf16_of_small_int(d, neg);
-        }
-    }
-}
-
-// w contiguous: thread per (w, v) element, coalesced in and out
-__global__ void __launch_bounds__(256) slice_wcontig(int64_t nv, int64_t nw, const double* __restrict__ M, int64_t ld,
-                                                    const int32_t* __restrict__ expo, int bits, int s,
-                                                    __nv_bfloat16* __restrict__ q, int64_t ldq, int64_t slice_stride) {
-    const int64_t v = blockIdx.y;
-    const int64_t w = int64_t(blockIdx.x) * 256 + threadIdx.x;
-    if (w >= ldq) return;
-    __nv_bfloat16* out = q + v * ldq + w;
-    if (w >= nw) {
-        for (int t = 0; t < s; ++t) out[int64_t(t) * slice_stride] = __float2bfloat16_rn(0.f);
-        return;
-    }
-    slice_value(M[w + v * ld], expo[v], bits, s, out, slice_stride);
-}
-
-// v contiguous: 32 x 32 tiles transposed through shared memory
-__global__ void __launch_bounds__(256) slice_vcontig(int64_t nv, int64_t nw, const double* __restrict__ M, int64_t ld,
-                                                    const int32_t* __restrict__ expo, int bits, int s,
-                                                    __nv_bfloat16* __restrict__ q, int64_t ldq, int64_t slice_stride) {
-    __shared__ double tile[32][33];
-    const int64_t v0 = int64_t(blockIdx.y) * 32, w0 = int64_t(blockIdx.x) * 32;
-    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;   // 32 x 8
-    // load: threads along v (contiguous)
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const int wl = ty + 8 * i;
-        const int64_t v = v0 + tx, w = w0 + wl;
-        tile[wl][tx] = (v < nv && w < nw) ? M[v + w * ld] : 0.0;
-    }
-    __syncthreads();
-    // store: threads along w (contiguous in the output)
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const int vl = ty + 8 * i;
-        const int64_t v = v0 + vl, w = w0 + tx;
-        if (v >= nv || w >= ldq) continue;
-        __nv_bfloat16* out = q + v * ldq + w;
-        if (w >= nw) {
-            for (int t = 0; t < s; ++t) out[int64_t(t) * slice_stride] = __float2bfloat16_rn(0.f);
-            continue;
-        }
-        slice_value(tile[tx][vl], expo[v], bits, s, out, slice_stride);
-    }
-}
-
-// One value prepared for digit extraction: |v| = mag 2^(base + e), so digit t of
-// |v| 2^(-e) is floor(mag 2^(base + bits t)) mod 2^bits (see slice_value).
+// One value prepared for digit extraction.  With |v| = M 2^(E-1075) (M the 53-bit significand),
+// digit t of |v| 2^(-e) is floor(M 2^(E - 1075 - e + bits t)) mod 2^bits, read from the
+// significand with integer shifts: the same digits the FP64 steps y = x 2^bits, q = trunc(y),
+// x = y - q produce, without FP64 arithmetic (the FP64 pipe of this GPU is narrow).  Each digit
+// carries the sign of v.  Here |v| = mag 2^(base + e).
 struct Digits {
     uint64_t mag;
     int base;
@@ -280,9 +105,21 @@ __device__ __forceinline__ uint32_t digit_bits(const Digits& x, int bits, int t)
     return (sh >= bits) ? 0u : uint32_t(x.mag << sh) & mask;
 }
 
-// Four consecutive values of one line -> for each slice t one 8-byte store of four BF16 digits.
+// four BF16 digits of consecutive entries: one 8-byte store, or 2-byte ones for the first `valid`
+__device__ __forceinline__ void put4(uint16_t* o, uint32_t w01, uint32_t w23, bool vec, int valid) {
+    if (vec && valid == 4) {
+        *reinterpret_cast<uint2*>(o) = make_uint2(w01, w23);
+    } else {
+        o[0] = uint16_t(w01);
+        if (valid > 1) o[1] = uint16_t(w01 >> 16);
+        if (valid > 2) o[2] = uint16_t(w23);
+        if (valid > 3) o[3] = uint16_t(w23 >> 16);
+    }
+}
+
+// Four consecutive values of one line -> four BF16 digits for each slice t.
 __device__ __forceinline__ void slice_store4(const double (&x)[4], int e, int bits, int s, uint16_t* out,
-                                             int64_t slice_stride) {
+                                             int64_t slice_stride, bool vec, int valid = 4) {
     Digits dg[4];
 #pragma unroll
     for (int c = 0; c < 4; ++c) dg[c] = prepare_digits(x[c], e);
@@ -290,10 +127,8 @@ __device__ __forceinline__ void slice_store4(const double (&x)[4], int e, int bi
         uint32_t h[4];
 #pragma unroll
         for (int c = 0; c < 4; ++c) h[c] = bf16_of_small_int(digit_bits(dg[c], bits, t), dg[c].neg);
-        uint2 pk;
-        pk.x = h[0] | (h[1] << 16);
-        pk.y = h[2] | (h[3] << 16);
-        *reinterpret_cast<uint2*>(out + int64_t(t - 1) * slice_stride) = pk;
+        put4(out + int64_t(t - 1) * slice_stride, h[0] | (h[1] << 16), h[2] | (h[3] << 16), vec,
+             valid);
     }
 }
 
@@ -327,7 +162,8 @@ __device__ __forceinline__ uint32_t bf16x2_of_digits(uint32_t d0, uint32_t d1, u
 }
 
 template <int BITS, int S>
-__device__ __forceinline__ void slice_store4_fixed(const double (&x)[4], int e, uint16_t* out, int64_t slice_stride) {
+__device__ __forceinline__ void slice_store4_fixed(const double (&x)[4], int e, uint16_t* out, int64_t slice_stride,
+                                                   bool vec, int valid = 4) {
     constexpr uint32_t MASK = (1u << BITS) - 1u;
     uint64_t F[4];
     uint32_t ng[4];
@@ -341,278 +177,396 @@ __device__ __forceinline__ void slice_store4_fixed(const double (&x)[4], int e, 
         uint32_t d[4];
 #pragma unroll
         for (int c = 0; c < 4; ++c) d[c] = uint32_t(F[c] >> (BITS * (S - t))) & MASK;
-        uint2 pk;
-        pk.x = bf16x2_of_digits(d[0], d[1], b01);
-        pk.y = bf16x2_of_digits(d[2], d[3], b23);
-        *reinterpret_cast<uint2*>(out + int64_t(t - 1) * slice_stride) = pk;
+        put4(out + int64_t(t - 1) * slice_stride, bf16x2_of_digits(d[0], d[1], b01), bf16x2_of_digits(d[2], d[3], b23),
+             vec, valid);
     }
 }
 
 // BITS = 0: digit width and count from the arguments; else the compile-time form
 template <int BITS, int S>
 __device__ __forceinline__ void slice_store4_any(const double (&x)[4], int e, int bits, int s, uint16_t* out,
-                                                 int64_t slice_stride) {
-    if constexpr (BITS > 0) slice_store4_fixed<BITS, S>(x, e, out, slice_stride);
-    else slice_store4(x, e, bits, s, out, slice_stride);
-}
-
-// w contiguous, four consecutive w per thread: 16-byte loads (ld even, M 16-byte aligned)
-// and 8-byte stores (ldq and the slice pitch multiples of 4, q 8-byte aligned)
-template <int BITS, int S>
-__global__ void __launch_bounds__(256) slice_wcontig4(int64_t nv, int64_t nw, const double* __restrict__ M, int64_t ld,
-                                                     const int32_t* __restrict__ expo, int bits, int s,
-                                                     __nv_bfloat16* __restrict__ q, int64_t ldq, int64_t slice_stride) {
-    const int64_t v = blockIdx.y;
-    const int64_t w = (int64_t(blockIdx.x) * 256 + threadIdx.x) * 4;
-    if (w >= ldq) return;
-    const double* row = M + v * ld;
-    double x[4];
-    if (w + 4 <= nw) {
-        const double2 p0 = __ldcs(reinterpret_cast<const double2*>(row + w));
-        const double2 p1 = __ldcs(reinterpret_cast<const double2*>(row + w + 2));
-        x[0] = p0.x; x[1] = p0.y; x[2] = p1.x; x[3] = p1.y;
-    } else {
-#pragma unroll
-        for (int c = 0; c < 4; ++c) x[c] = (w + c < nw) ? row[w + c] : 0.0;
-    }
-    slice_store4_any<BITS, S>(x, expo[v], bits, s, reinterpret_cast<uint16_t*>(q) + v * ldq + w, slice_stride);
-}
-
-// v contiguous: 64 (w) x 32 (v) tiles transposed through shared memory; each thread then
-// slices four consecutive w of two lines
-template <int BITS, int S>
-__global__ void __launch_bounds__(256) slice_vcontig4(int64_t nv, int64_t nw, const double* __restrict__ M, int64_t ld,
-                                                     const int32_t* __restrict__ expo, int bits, int s,
-                                                     __nv_bfloat16* __restrict__ q, int64_t ldq, int64_t slice_stride) {
-    __shared__ double tile[64][33];
-    const int64_t v0 = int64_t(blockIdx.y) * 32, w0 = int64_t(blockIdx.x) * 64;
-    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;   // 32 x 8
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        const int wl = ty + 8 * i;
-        const int64_t v = v0 + tx, w = w0 + wl;
-        tile[wl][tx] = (v < nv && w < nw) ? __ldcs(M + v + w * ld) : 0.0;
-    }
-    __syncthreads();
-    const int wq = threadIdx.x & 15, vh = threadIdx.x >> 4;   // 16 x 16
-    const int64_t w = w0 + 4 * wq;
-    if (w >= ldq) return;
-#pragma unroll
-    for (int r = 0; r < 2; ++r) {
-        const int vl = vh + 16 * r;
-        const int64_t v = v0 + vl;
-        if (v >= nv) continue;
-        double x[4];
-#pragma unroll
-        for (int c = 0; c < 4; ++c) x[c] = tile[4 * wq + c][vl];   // zero beyond nw (loaded as 0)
-        slice_store4_any<BITS, S>(x, expo[v], bits, s, reinterpret_cast<uint16_t*>(q) + v * ldq + w, slice_stride);
-    }
+                                                 int64_t slice_stride, bool vec, int valid = 4) {
+    if constexpr (BITS > 0) slice_store4_fixed<BITS, S>(x, e, out, slice_stride, vec, valid);
+    else slice_store4(x, e, bits, s, out, slice_stride, vec, valid);
 }
 
 // ---------------------------------------------------------------------------
-// Complex operands (Section 7: the method on complex data).  The complex product
-// op(A) op(B) is the real product A' B'' of
+// The split of one operand.  nv lines of nw entries; `v_contig`: entry (v, w) at M[v + w ld],
+// else at M[w + v ld].  Real: slices of line v in row v, entries nw..ldq-1 zero.
+//
+// Complex (Section 7: the method on complex data): the complex product op(A) op(B) is the real
+// product A' B'' of
 //   A'  = [Re op(A), Im op(A)]                              m x 2k
 //   B'' = [[Re op(B), Im op(B)], [-Im op(B), Re op(B)]]     2k x 2n
-// whose first n columns are Re(op(A) op(B)) and last n are Im(op(A) op(B)).  Each
-// line (row of op(A), column of op(B)) gets one exponent from the largest real or
-// imaginary part; each entry is sliced once and its digits are written to the
-// two (A') or four (B'') places it occupies, negated where B'' has -Im.
+// whose first n columns are Re(op(A) op(B)) and last n are Im(op(A) op(B)).  Each line (row of
+// op(A), column of op(B)) gets one exponent from the largest real or imaginary part.  A line of
+// nw entries fills row v with [Re, Im] (A') or row v with [Re, -Im] and row nv + v with [Im, Re]
+// (B''), 2 nw values and zeros up to ldq.
+//
+// Two schedules:
+//  * w contiguous: one to eight warps hold a line in registers (real, up to 8 x 4 values a
+//    thread), or a CTA in shared memory (complex), take its exponent and slice it.  Longer lines
+//    are read again, from L2.
+//  * v contiguous: a cluster of 1 to 8 CTAs shares 32 lines and scans a part of w each; the maxima
+//    meet in distributed shared memory.  A second kernel slices tiles of 64 w x 32 lines, transposed
+//    through shared memory.  (As a programmatic dependent it was slower, 14.2 against 10.4 us at
+//    1000 x 900.  Slicing in the scanning cluster, the lines read again from L2, was slower
+//    from 2048 x 4096 on: 339 against 323 us at 8192^2, four CTAs per SM.)
+// Bound by DRAM at large sizes (8 bytes in, 2 s bytes out for each value) and by launches at small
+// ones: an operand took four launches before (initialise the exponents, scan, slice, fix up), the
+// scan read everything once more, and complex rows of odd length were stored two bytes at a
+// time.  Before -> now, seven slices of seven bits, us in a row in a CUDA graph: w contiguous
+// 8192^2 298 -> 261 (5.6 TB/s), 4096^2 82 -> 71, 1000 x 900 9.2 -> 6.4; v contiguous 1000 x 900
+// 15.5 -> 10.5, 5000 x 300 22.8 -> 15.2, 4096^2 91 -> 92, 8192^2 323 -> 350 (the scan's short
+// pieces of a row); both operands of a complex 1500 x 1100 x 2301 product 190 -> 76.
 // ---------------------------------------------------------------------------
+constexpr int SPLIT_CLUSTER = 8;   // most CTAs that share 32 v-contiguous lines
+constexpr int SPLIT_HELD = 8;      // chunks of four values a thread holds (real, w contiguous)
 
-// complex lines, v contiguous (M(v, w) at v + w*ld): thread per v
-__global__ void __launch_bounds__(256) zexpo_vcontig(int64_t nv, int64_t nw, const double2* __restrict__ M, int64_t ld,
-                                                    int64_t w_per_split, int32_t* expo) {
-    const int64_t v = int64_t(blockIdx.x) * 256 + threadIdx.x;
-    if (v >= nv) return;
-    const int64_t w0 = int64_t(blockIdx.y) * w_per_split;
-    const int64_t w1 = min(nw, w0 + w_per_split);
-    uint64_t m0 = 0, m1 = 0;
-    int64_t w = w0;
-    for (; w + 2 <= w1; w += 2) {
-        const double2 a = M[v + w * ld], b = M[v + (w + 1) * ld];
-        m0 = mag_max(m0, mag_max(mag_bits(a.x), mag_bits(a.y)));
-        m1 = mag_max(m1, mag_max(mag_bits(b.x), mag_bits(b.y)));
-    }
-    for (; w < w1; ++w) {
-        const double2 a = M[v + w * ld];
-        m0 = mag_max(m0, mag_max(mag_bits(a.x), mag_bits(a.y)));
-    }
-    const int e = line_exponent_bits(mag_max(m0, m1));
-    if (e != INT_MIN) atomicMax(&expo[v], e);
-}
+struct SplitJob {
+    const double* M;               // complex: pairs of doubles
+    int64_t ld, nv, nw;
+    int32_t* expo;
+    uint16_t* q;
+    int64_t ldq, plane;
+    int v_contig, conj, role_b;
+    int vec_in, vec_out;           // 16-byte loads (real, w contiguous); 8-byte stores
+    int warps;                     // w contiguous, real: warps per line (1, 2, 4 or 8)
+    int cached;                    // w contiguous, complex: the line fits shared memory
+    unsigned blocks;
+};
 
-// complex lines, w contiguous (M(w, v) at w + v*ld): block per (v, w-chunk)
-__global__ void __launch_bounds__(256) zexpo_wcontig(int64_t nv, int64_t nw, const double2* __restrict__ M, int64_t ld,
-                                                    int64_t w_per_split, int32_t* expo) {
-    const int64_t v = blockIdx.x;
-    const int64_t w0 = int64_t(blockIdx.y) * w_per_split;
-    const int64_t w1 = min(nw, w0 + w_per_split);
-    uint64_t mx = 0;
-    for (int64_t w = w0 + threadIdx.x; w < w1; w += 256) {
-        const double2 a = M[w + v * ld];
-        mx = mag_max(mx, mag_max(mag_bits(a.x), mag_bits(a.y)));
-    }
+__device__ __forceinline__ uint64_t warp_mag_max(uint64_t mx) {
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) mx = mag_max(mx, __shfl_xor_sync(0xffffffffu, mx, off));
+    return mx;
+}
+// exponent of a line as stored: 0 for an all-zero line (its digits are zero for any exponent)
+__device__ __forceinline__ int stored_exponent(uint64_t mx) {
+    const int e = line_exponent_bits(mx);
+    return e == INT_MIN ? 0 : e;
+}
+
+// four values w .. w+3 of a w-contiguous real line, zero from nw on
+__device__ __forceinline__ void load4(const double* line, int64_t w, int64_t nw, bool vec, double (&x)[4]) {
+    if (vec && w + 4 <= nw) {
+        const double2 a = __ldcs(reinterpret_cast<const double2*>(line + w));
+        const double2 b = __ldcs(reinterpret_cast<const double2*>(line + w + 2));
+        x[0] = a.x; x[1] = a.y; x[2] = b.x; x[3] = b.y;
+    } else {
+#pragma unroll
+        for (int c = 0; c < 4; ++c) x[c] = (w + c < nw) ? __ldcs(line + w + c) : 0.0;
+    }
+}
+
+template <int BITS, int S>
+__device__ __forceinline__ void split_w_real(const SplitJob& j, int64_t block, int bits, int s) {
     __shared__ uint64_t red[8];
-    if (lane_id() == 0) red[warp_id()] = mx;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        uint64_t m2 = red[0];
-        for (int i = 1; i < 8; ++i) m2 = mag_max(m2, red[i]);
-        const int e = line_exponent_bits(m2);
-        if (e != INT_MIN) atomicMax(&expo[v], e);
-    }
-    (void)nv;
-}
-
-// The s digits of `valid` (<= 4) consecutive entries of one output line, negated if
-// flip; one 8-byte store per slice when vec (and all four present), else 2-byte stores.
-__device__ __forceinline__ void emit4(const Digits (&dg)[4], int valid, uint32_t flip, int bits, int s, uint16_t* out,
-                                      int64_t slice_stride, bool vec) {
-    for (int t = 1; t <= s; ++t) {
-        uint32_t h[4];
+    const int WL = j.warps, G = 32 * WL, t = int(threadIdx.x) & (G - 1);
+    const int64_t v = block * (8 / WL) + warp_id() / WL;
+    const bool live = v < j.nv;                             // the same in every warp of a line
+    if (WL == 1 && !live) return;
+    const double* line = j.M + (live ? v : 0) * j.ld;
+    const int64_t step = 4 * G;
+    const bool held = j.ldq <= SPLIT_HELD * step, vec = j.vec_in != 0;
+    double x[SPLIT_HELD][4];
+    uint64_t mx = 0;
+    if (held) {
 #pragma unroll
-        for (int c = 0; c < 4; ++c)
-            h[c] = c < valid ? bf16_of_small_int(digit_bits(dg[c], bits, t), dg[c].neg ^ flip) : 0u;
-        uint16_t* o = out + int64_t(t - 1) * slice_stride;
-        if (vec && valid == 4) {
-            uint2 pk;
-            pk.x = h[0] | (h[1] << 16);
-            pk.y = h[2] | (h[3] << 16);
-            *reinterpret_cast<uint2*>(o) = pk;
-        } else {
-            for (int c = 0; c < valid; ++c) o[c] = uint16_t(h[c]);
+        for (int c = 0; c < SPLIT_HELD; ++c)
+            if (c * step < j.nw) load4(line, c * step + 4 * t, j.nw, vec, x[c]);
+#pragma unroll
+        for (int c = 0; c < SPLIT_HELD; ++c)
+            if (c * step < j.nw) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i) mx = mag_max(mx, mag_bits(x[c][i]));
+            }
+    } else {
+#pragma unroll 4
+        for (int64_t w = 4 * t; w < j.nw; w += step) {
+            double y[4];
+            load4(line, w, j.nw, vec, y);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) mx = mag_max(mx, mag_bits(y[i]));
         }
     }
-}
-
-// The compile-time form of emit4 (digits from one 64-bit word per value, see digits_word)
-template <int BITS, int S>
-__device__ __forceinline__ void emit4_fixed(const uint64_t (&F)[4], const uint32_t (&ng)[4], int valid, uint32_t flip,
-                                            uint16_t* out, int64_t slice_stride, bool vec) {
-    constexpr uint32_t MASK = (1u << BITS) - 1u;
-    uint32_t sg[4];
-#pragma unroll
-    for (int c = 0; c < 4; ++c) sg[c] = c < valid ? ((ng[c] ^ flip) << 31) : 0u;
-    const uint64_t b01 = (uint64_t(0x4B000000u | sg[1]) << 32) | (0x4B000000u | sg[0]);
-    const uint64_t b23 = (uint64_t(0x4B000000u | sg[3]) << 32) | (0x4B000000u | sg[2]);
-#pragma unroll
-    for (int t = 1; t <= S; ++t) {
-        uint32_t d[4];
-#pragma unroll
-        for (int c = 0; c < 4; ++c) d[c] = c < valid ? uint32_t(F[c] >> (BITS * (S - t))) & MASK : 0u;
-        const uint32_t w01 = bf16x2_of_digits(d[0], d[1], b01), w23 = bf16x2_of_digits(d[2], d[3], b23);
-        uint16_t* o = out + int64_t(t - 1) * slice_stride;
-        if (vec && valid == 4) {
-            *reinterpret_cast<uint2*>(o) = make_uint2(w01, w23);
-        } else {
-            const uint32_t h[4] = {w01 & 0xFFFFu, w01 >> 16, w23 & 0xFFFFu, w23 >> 16};
-            for (int c = 0; c < valid; ++c) o[c] = uint16_t(h[c]);
-        }
+    mx = warp_mag_max(mx);
+    if (WL > 1) {
+        if (lane_id() == 0) red[warp_id()] = mx;
+        __syncthreads();
+        const int w0 = int(warp_id()) / WL * WL;
+        for (int i = 0; i < WL; ++i) mx = mag_max(mx, red[w0 + i]);
+        if (!live) return;
     }
-}
-
-// Digits of entries w..w+valid-1 of line v (values x, conjugated if conj) into the real form.
-// role_b = false: A' (line v: Re at w, Im at nw + w).  role_b = true: B'' (line v = j < n:
-// Re at w, -Im at nw + w; line n + j: Im at w, Re at nw + w).
-template <int BITS, int S>
-__device__ __forceinline__ void zslice_emit(const double2 (&x)[4], int valid, int e, bool conj, bool role_b,
-                                            int64_t v, int64_t nv, int64_t nw, int64_t w, int bits, int s,
-                                            uint16_t* q, int64_t ldq, int64_t slice_stride, bool vec) {
-    if constexpr (BITS > 0) {
-        uint64_t Fr[4], Fi[4];
-        uint32_t nr[4], ni[4];
+    const int e = stored_exponent(mx);
+    if (t == 0) j.expo[v] = e;
+    uint16_t* out = j.q + v * j.ldq;
+    if (held) {
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            Fr[c] = digits_word<BITS, S>(x[c].x, e, nr[c]);
-            Fi[c] = digits_word<BITS, S>(conj ? -x[c].y : x[c].y, e, ni[c]);
-        }
-        uint16_t* row = q + v * ldq;
-        emit4_fixed<BITS, S>(Fr, nr, valid, 0u, row + w, slice_stride, vec);
-        emit4_fixed<BITS, S>(Fi, ni, valid, role_b ? 1u : 0u, row + nw + w, slice_stride, vec);
-        if (role_b) {
-            uint16_t* row2 = q + (nv + v) * ldq;
-            emit4_fixed<BITS, S>(Fi, ni, valid, 0u, row2 + w, slice_stride, vec);
-            emit4_fixed<BITS, S>(Fr, nr, valid, 0u, row2 + nw + w, slice_stride, vec);
+        for (int c = 0; c < SPLIT_HELD; ++c) {
+            const int64_t w = c * step + 4 * t;
+            if (c * step >= j.nw) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i) x[c][i] = 0.0;
+            }
+            if (w < j.ldq) slice_store4_any<BITS, S>(x[c], e, bits, s, out + w, j.plane, j.vec_out != 0);
         }
     } else {
-        Digits dr[4], di[4];
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            dr[c] = prepare_digits(x[c].x, e);
-            di[c] = prepare_digits(conj ? -x[c].y : x[c].y, e);
-        }
-        uint16_t* row = q + v * ldq;
-        emit4(dr, valid, 0u, bits, s, row + w, slice_stride, vec);
-        emit4(di, valid, role_b ? 1u : 0u, bits, s, row + nw + w, slice_stride, vec);
-        if (role_b) {
-            uint16_t* row2 = q + (nv + v) * ldq;
-            emit4(di, valid, 0u, bits, s, row2 + w, slice_stride, vec);
-            emit4(dr, valid, 0u, bits, s, row2 + nw + w, slice_stride, vec);
+        for (int64_t w = 4 * t; w < j.ldq; w += step) {
+            double y[4];
+            load4(line, w, j.nw, vec, y);
+            slice_store4_any<BITS, S>(y, e, bits, s, out + w, j.plane, j.vec_out != 0);
         }
     }
 }
 
-// w contiguous: four consecutive w of one line per thread
-template <int BITS, int S>
-__global__ void __launch_bounds__(256) zslice_wcontig(int64_t nv, int64_t nw, const double2* __restrict__ M, int64_t ld,
-                                                     const int32_t* __restrict__ expo, bool conj, bool role_b, int bits,
-                                                     int s, __nv_bfloat16* __restrict__ q, int64_t ldq,
-                                                     int64_t slice_stride, bool vec) {
-    const int64_t v = blockIdx.y;
-    const int64_t w = (int64_t(blockIdx.x) * 256 + threadIdx.x) * 4;
-    if (w >= nw) return;
-    const int valid = nw - w < 4 ? int(nw - w) : 4;
-    double2 x[4];
-#pragma unroll
-    for (int c = 0; c < 4; ++c) x[c] = c < valid ? M[w + c + v * ld] : make_double2(0.0, 0.0);
-    zslice_emit<BITS, S>(x, valid, expo[v], conj, role_b, v, nv, nw, w, bits, s, reinterpret_cast<uint16_t*>(q),
-                         ldq, slice_stride, vec);
+// part 0 / 1 of complex entry (v, w): real, imaginary (conjugated for op = C)
+__device__ __forceinline__ double zpart(const SplitJob& j, int64_t idx, int part) {
+    const double y = j.M[2 * idx + part];
+    return part == 1 && j.conj ? -y : y;
+}
+// which part of which entry stands at position p < 2 nw of row kind `second` (B'' rows nv + v)
+__device__ __forceinline__ int zpart_at(const SplitJob& j, int64_t p, bool second, int64_t& w, bool& flip) {
+    const bool right = p >= j.nw;
+    w = right ? p - j.nw : p;
+    flip = right && j.role_b && !second;                    // -Im
+    return int(right) ^ int(second);
 }
 
-// v contiguous: 64 (w) x 32 (v) complex tiles transposed through shared memory
+// place of entry w in a cached line: four consecutive entries per lane without bank conflicts
+__host__ __device__ __forceinline__ int cache_at(int w) { return w + (w >> 4); }
+
 template <int BITS, int S>
-__global__ void __launch_bounds__(256) zslice_vcontig(int64_t nv, int64_t nw, const double2* __restrict__ M, int64_t ld,
-                                                     const int32_t* __restrict__ expo, bool conj, bool role_b, int bits,
-                                                     int s, __nv_bfloat16* __restrict__ q, int64_t ldq,
-                                                     int64_t slice_stride, bool vec) {
-    __shared__ double2 tile[64][33];
-    const int64_t v0 = int64_t(blockIdx.y) * 32, w0 = int64_t(blockIdx.x) * 64;
-    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+__device__ __forceinline__ void split_w_complex(const SplitJob& j, int64_t v, int bits, int s, double* cache) {
+    __shared__ uint64_t red[8];
+    const int t = int(threadIdx.x);
+    const double2* line = reinterpret_cast<const double2*>(j.M) + v * j.ld;
+    const int half = j.cached ? cache_at(int(j.nw)) + 1 : 0;      // imaginary parts from here on
+    uint64_t mx = 0;
+    for (int64_t w0 = t; w0 < j.nw; w0 += 256 * 8) {
+        double2 a[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) a[u] = w0 + 256 * u < j.nw ? line[w0 + 256 * u] : make_double2(0.0, 0.0);
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const int64_t w = w0 + 256 * u;
+            mx = mag_max(mx, mag_max(mag_bits(a[u].x), mag_bits(a[u].y)));
+            if (j.cached && w < j.nw) {
+                cache[cache_at(int(w))] = a[u].x;
+                cache[half + cache_at(int(w))] = j.conj ? -a[u].y : a[u].y;
+            }
+        }
+    }
+    mx = warp_mag_max(mx);
+    if (lane_id() == 0) red[warp_id()] = mx;
+    __syncthreads();
+    mx = red[0];
+#pragma unroll
+    for (int i = 1; i < 8; ++i) mx = mag_max(mx, red[i]);
+    const int e = stored_exponent(mx);
+    if (t == 0) j.expo[v] = e;
+    const int64_t nw = j.nw;
+    for (int second = 0; second <= (j.role_b ? 1 : 0); ++second) {
+        uint16_t* out = j.q + (second ? j.nv + v : v) * j.ldq;
+        for (int64_t p = 4 * t; p < j.ldq; p += 1024) {
+            double x[4];
+            const bool left = p + 4 <= nw, right = p >= nw && p + 4 <= 2 * nw;
+            if (j.cached && (left || right)) {              // all four from one half of the row
+                const int part = int(right) ^ second, w = int(right ? p - nw : p);
+                const bool flip = right && j.role_b && second == 0;
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    const double y = cache[part * half + cache_at(w + c)];
+                    x[c] = flip ? -y : y;
+                }
+            } else {
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    x[c] = 0.0;
+                    if (p + c < 2 * nw) {
+                        int64_t w;
+                        bool flip;
+                        const int part = zpart_at(j, p + c, second != 0, w, flip);
+                        const double y = j.cached ? cache[part * half + cache_at(int(w))] : zpart(j, v * j.ld + w, part);
+                        x[c] = flip ? -y : y;
+                    }
+                }
+            }
+            slice_store4_any<BITS, S>(x, e, bits, s, out + p, j.plane, j.vec_out != 0);
+        }
+    }
+}
+
+// entries [w0, w0 + n) of line vl of a tile (n <= 64, column v of row w at (v + w / 4) % 32) to
+// positions base + w0 .. of its row, four at a time from the first position that is a multiple
+// of four; thread wq of 16.  The entries before it and the last partial group go one by one.
+template <int BITS, int S>
+__device__ __forceinline__ void emit_tile_row(const SplitJob& j, const double (*tile)[32], int vl, int wq, int n,
+                                              int64_t pos, uint16_t* row, int e, bool flip, int bits, int s) {
+    const int lead = j.vec_out ? min(n, int(-pos & 3)) : 0;
+    auto group = [&](int first, int valid) {
+        double x[4];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            const int r = first + c;
+            const double y = c < valid ? tile[r & 63][(vl + ((r & 63) >> 2)) & 31] : 0.0;
+            x[c] = flip ? -y : y;
+        }
+        slice_store4_any<BITS, S>(x, e, bits, s, row + pos + first, j.plane, j.vec_out != 0, valid);
+    };
+    const int first = lead + 4 * wq;
+    if (first < n) group(first, min(4, n - first));
+    if (lead > 0 && wq == 15) group(0, lead);
+}
+
+// Exponents of 2 LX v-contiguous lines: a cluster shares them, each CTA scans its part of w, LX
+// lanes with two lines each by 256 / LX entries at a time.  Loads come in batches, the last one
+// predicated (a remainder loop would take them one by one).
+template <int LX, bool CPLX>
+__device__ __forceinline__ void scan_v(const SplitJob& j, int64_t block) {
+    constexpr int R = 256 / LX, U = CPLX ? 4 : 8;
+    __shared__ uint64_t red[R][2 * LX], cmax[2 * LX];
+    const int rank = int(cluster_ctarank()), CS = int(cluster_nctarank());
+    const int tx = int(threadIdx.x) % LX, ty = int(threadIdx.x) / LX;
+    const int64_t v0 = block / CS * (2 * LX), v = v0 + 2 * tx;
+    const int64_t part = (j.nw + CS - 1) / CS, w0 = rank * part, w1 = min(j.nw, w0 + part);
+    const bool two = v + 1 < j.nv, vec = two && j.vec_in;
+    uint64_t ma = 0, mb = 0;
+    if (v < j.nv) {
+        for (int64_t w = w0 + ty; w < w1; w += R * U) {
+            if constexpr (CPLX) {
+                double2 x[U], y[U];
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const bool in = w + R * u < w1;
+                    const double2* p = reinterpret_cast<const double2*>(j.M) + v + (w + R * u) * j.ld;
+                    x[u] = in ? p[0] : make_double2(0.0, 0.0);
+                    y[u] = in && two ? p[1] : make_double2(0.0, 0.0);
+                }
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    ma = mag_max(ma, mag_max(mag_bits(x[u].x), mag_bits(x[u].y)));
+                    mb = mag_max(mb, mag_max(mag_bits(y[u].x), mag_bits(y[u].y)));
+                }
+            } else {
+                double2 x[U];
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const bool in = w + R * u < w1;
+                    const double* p = j.M + v + (w + R * u) * j.ld;
+                    if (in && vec) x[u] = *reinterpret_cast<const double2*>(p);
+                    else x[u] = make_double2(in ? p[0] : 0.0, in && two ? p[1] : 0.0);
+                }
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    ma = mag_max(ma, mag_bits(x[u].x));
+                    mb = mag_max(mb, mag_bits(x[u].y));
+                }
+            }
+        }
+    }
+    red[ty][2 * tx] = ma;
+    red[ty][2 * tx + 1] = mb;
+    __syncthreads();
+    const int t = int(threadIdx.x);
+    uint64_t mx = 0;
+    if (t < 2 * LX) {
+#pragma unroll
+        for (int i = 0; i < R; ++i) mx = mag_max(mx, red[i][t]);
+        cmax[t] = mx;
+    }
+    __syncwarp();
+    cluster_sync_all();
+    if (rank == 0 && t < 2 * LX) {
+        for (int r = 1; r < CS; ++r) {
+            uint64_t y;
+            asm volatile("ld.shared::cluster.u64 %0, [%1];" : "=l"(y) : "r"(mapa_shared(smem_u32(&cmax[t]), uint32_t(r)))
+                         : "memory");
+            mx = mag_max(mx, y);
+        }
+        if (v0 + t < j.nv) j.expo[v0 + t] = stored_exponent(mx);
+    }
+    __syncwarp();
+    cluster_sync_all();            // no CTA leaves while rank 0 may still read its maxima
+}
+
+// one tile of 64 w x 32 v-contiguous lines, transposed through shared memory
+template <int BITS, int S, bool CPLX>
+__device__ __forceinline__ void slice_v(const SplitJob& j, int64_t block, int bits, int s) {
+    // column v of row w at (v + w / 4) % 32: conflict-free both along v and for the four
+    // consecutive w a thread slices
+    __shared__ double tile[CPLX ? 2 : 1][64][32];
+    const int tx = int(threadIdx.x) & 31, ty = int(threadIdx.x) >> 5;   // 32 x 8
+    const int64_t len = CPLX ? j.nw : j.ldq;        // a real row's padding belongs to its last entries
+    const int64_t tiles_w = (len + 63) / 64;
+    const int64_t w0 = block % tiles_w * 64, v0 = block / tiles_w * 32, v = v0 + tx;
+    const int n = int(min(int64_t(64), len - w0));
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
         const int wl = ty + 8 * i;
-        const int64_t v = v0 + tx, w = w0 + wl;
-        tile[wl][tx] = (v < nv && w < nw) ? M[v + w * ld] : make_double2(0.0, 0.0);
+        const int64_t w = w0 + wl;
+        const bool in = v < j.nv && w < j.nw;
+        const int col = (tx + (wl >> 2)) & 31;
+        if constexpr (CPLX) {
+            const double2 a = in ? __ldcs(reinterpret_cast<const double2*>(j.M) + v + w * j.ld) : make_double2(0.0, 0.0);
+            tile[0][wl][col] = a.x;
+            tile[CPLX ? 1 : 0][wl][col] = j.conj ? -a.y : a.y;
+        } else {
+            tile[0][wl][col] = in ? __ldcs(j.M + v + w * j.ld) : 0.0;
+        }
     }
     __syncthreads();
-    const int wq = threadIdx.x & 15, vh = threadIdx.x >> 4;
-    const int64_t w = w0 + 4 * wq;
-    if (w >= nw) return;
-    const int valid = nw - w < 4 ? int(nw - w) : 4;
-#pragma unroll
+    const int wq = int(threadIdx.x) & 15, vh = int(threadIdx.x) >> 4;   // 16 x 16
+#pragma unroll 1
     for (int r = 0; r < 2; ++r) {
         const int vl = vh + 16 * r;
-        const int64_t v = v0 + vl;
-        if (v >= nv) continue;
-        double2 x[4];
+        if (v0 + vl >= j.nv) continue;
+        const int e = j.expo[v0 + vl];
+        uint16_t* row = j.q + (v0 + vl) * j.ldq;
+        if constexpr (CPLX) {
+            constexpr int IM = CPLX ? 1 : 0;
+            emit_tile_row<BITS, S>(j, tile[0], vl, wq, n, w0, row, e, false, bits, s);
+            emit_tile_row<BITS, S>(j, tile[IM], vl, wq, n, j.nw + w0, row, e, j.role_b != 0, bits, s);
+            if (j.role_b) {
+                uint16_t* row2 = row + j.nv * j.ldq;
+                emit_tile_row<BITS, S>(j, tile[IM], vl, wq, n, w0, row2, e, false, bits, s);
+                emit_tile_row<BITS, S>(j, tile[0], vl, wq, n, j.nw + w0, row2, e, false, bits, s);
+            }
+        } else if (4 * wq < n) {
+            double x[4];
 #pragma unroll
-        for (int c = 0; c < 4; ++c) x[c] = tile[4 * wq + c][vl];
-        zslice_emit<BITS, S>(x, valid, expo[v], conj, role_b, v, nv, nw, w, bits, s, reinterpret_cast<uint16_t*>(q),
-                             ldq, slice_stride, vec);
+            for (int c = 0; c < 4; ++c) x[c] = tile[0][4 * wq + c][(vl + wq) & 31];
+            slice_store4_any<BITS, S>(x, e, bits, s, row + w0 + 4 * wq, j.plane, j.vec_out != 0);
+        }
+    }
+    if constexpr (CPLX) {          // zeros from 2 nw to ldq
+        if (w0 == 0 && v < j.nv)
+            for (int64_t p = 2 * j.nw + ty; p < j.ldq; p += 8)
+                for (int t = 0; t < s; ++t)
+                    for (int second = 0; second <= (j.role_b ? 1 : 0); ++second)
+                        j.q[((second ? j.nv : 0) + v) * j.ldq + p + int64_t(t) * j.plane] = 0;
     }
 }
 
-// zero the padding [from, ldq) of every line of every slice
-__global__ void zpad_kernel(int64_t lines, int64_t from, int64_t ldq, int s, __nv_bfloat16* __restrict__ q,
-                            int64_t slice_stride) {
-    const int64_t line = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (line >= lines) return;
-    uint16_t* o = reinterpret_cast<uint16_t*>(q) + line * ldq;
-    for (int t = 0; t < s; ++t)
-        for (int64_t w = from; w < ldq; ++w) o[int64_t(t) * slice_stride + w] = 0;
+// Blocks 0 .. j0.blocks - 1 split the first operand, the rest the second.
+template <int BITS, int S, bool CPLX>
+__global__ void __launch_bounds__(256, CPLX ? 4 : 2) ozaki_split_w_kernel(SplitJob j0, SplitJob j1, int bits, int s) {
+    extern __shared__ double cache[];
+    const bool first = blockIdx.x < j0.blocks;
+    const SplitJob& j = first ? j0 : j1;
+    const int64_t block = first ? blockIdx.x : blockIdx.x - j0.blocks;
+    if constexpr (CPLX) split_w_complex<BITS, S>(j, block, bits, s, cache);
+    else split_w_real<BITS, S>(j, block, bits, s);
+}
+template <int LX, bool CPLX>
+__global__ void __launch_bounds__(256) ozaki_scan_v_kernel(SplitJob j0, SplitJob j1) {
+    const bool first = blockIdx.x < j0.blocks;
+    scan_v<LX, CPLX>(first ? j0 : j1, first ? blockIdx.x : blockIdx.x - j0.blocks);
+}
+template <int BITS, int S, bool CPLX>
+__global__ void __launch_bounds__(256) ozaki_slice_v_kernel(SplitJob j0, SplitJob j1, int bits, int s) {
+    const bool first = blockIdx.x < j0.blocks;
+    slice_v<BITS, S, CPLX>(first ? j0 : j1, first ? blockIdx.x : blockIdx.x - j0.blocks, bits, s);
 }
 
 }  // namespace
@@ -788,61 +742,103 @@ hsmm_status_t ozaki_recombine(int64_t m, int64_t n, int slices, int bits, const 
     return check_launch();
 }
 
-// rows x cols column-major M; by_rows: v = row (w = column), else v = column (w = row).
-hsmm_status_t ozaki_split(int64_t rows, int64_t cols, const double* M, int64_t ld, bool by_rows, int bits,
-                          int slices, int32_t* expo, void* qv, int64_t ldq, int64_t plane, cudaStream_t st) {
-    const int64_t nv = by_rows ? rows : cols;
-    const int64_t nw = by_rows ? cols : rows;
-    __nv_bfloat16* q = static_cast<__nv_bfloat16*>(qv);
-    if (nv > 65535 * 32LL && by_rows) return HSMM_STATUS_NOT_SUPPORTED;
-    if (nv > 65535 && !by_rows) return HSMM_STATUS_NOT_SUPPORTED;
-    expo_init<<<unsigned((nv + 255) / 256), 256, 0, st>>>(nv, expo);
-    const int sms = num_sms();
-    // four digits per 8-byte store when every slice row starts 8-byte aligned; the default
-    // 7 slices of 7 bits with compile-time digit positions
-    const bool q8 = ldq % 4 == 0 && plane % 4 == 0 && aligned_to(qv, 8);
-    const bool fixed77 = bits == 7 && slices == 7;
-    if (by_rows) {
-        // v = row: contiguous
-        const int64_t vb = (nv + 255) / 256;
-        int64_t splits = (int64_t(sms) * 8 + vb - 1) / vb;
-        splits = splits < 1 ? 1 : (splits > nw ? nw : splits);
-        const int64_t wps = (nw + splits - 1) / splits;
-        if (nv % 2 == 0 && ld % 2 == 0 && aligned_to(M, 16))
-            expo_vcontig2<<<dim3(unsigned((nv / 2 + 255) / 256), unsigned((nw + wps - 1) / wps)), 256, 0, st>>>(
-                nv, nw, M, ld, wps, expo);
-        else
-            expo_vcontig<<<dim3(unsigned(vb), unsigned((nw + wps - 1) / wps)), 256, 0, st>>>(nv, nw, M, ld, wps, expo);
-        if (q8 && fixed77)
-            slice_vcontig4<7, 7><<<dim3(unsigned((ldq + 63) / 64), unsigned((nv + 31) / 32)), 256, 0, st>>>(
-                nv, nw, M, ld, expo, bits, slices, q, ldq, plane);
-        else if (q8)
-            slice_vcontig4<0, 0><<<dim3(unsigned((ldq + 63) / 64), unsigned((nv + 31) / 32)), 256, 0, st>>>(
-                nv, nw, M, ld, expo, bits, slices, q, ldq, plane);
-        else
-            slice_vcontig<<<dim3(unsigned((ldq + 31) / 32), unsigned((nv + 31) / 32)), 256, 0, st>>>(
-                nv, nw, M, ld, expo, bits, slices, q, ldq, plane);
+namespace {
+
+constexpr size_t SPLIT_CACHE = 200 * 1024;     // shared memory for a complex line
+size_t split_cache_bytes(int64_t nw) { return size_t(16) * (size_t(nw) + size_t(nw) / 16 + 1); }
+
+hsmm_status_t make_split_job(const SplitOperand& o, bool cplx, SplitJob* j) {
+    if (o.v_contig && o.nv > 65535 * 32LL) return HSMM_STATUS_NOT_SUPPORTED;
+    if (!o.v_contig && o.nv > 65535) return HSMM_STATUS_NOT_SUPPORTED;
+    j->M = static_cast<const double*>(o.M);
+    j->ld = o.ld; j->nv = o.nv; j->nw = o.nw;
+    j->expo = o.expo;
+    j->q = static_cast<uint16_t*>(o.q);
+    j->ldq = o.ldq; j->plane = o.plane;
+    j->v_contig = o.v_contig; j->conj = o.conj; j->role_b = o.role_b;
+    j->vec_in = o.ld % 2 == 0 && aligned_to(o.M, 16);
+    j->vec_out = o.ldq % 4 == 0 && o.plane % 4 == 0 && aligned_to(o.q, 8);
+    j->warps = 1;                  // as many warps per line as hold it in their registers
+    while (j->warps < 8 && o.ldq > int64_t(SPLIT_HELD) * 128 * j->warps) j->warps *= 2;
+    j->cached = cplx && !o.v_contig && split_cache_bytes(o.nw) <= SPLIT_CACHE;
+    const int lines = cplx ? 1 : 8 / j->warps;     // lines of a CTA (w contiguous)
+    j->blocks = unsigned((o.nv + lines - 1) / lines);
+    return HSMM_STATUS_SUCCESS;
+}
+
+template <int BITS, int S, bool CPLX>
+hsmm_status_t launch_split(SplitJob a, SplitJob b, int bits, int slices, cudaStream_t st) {
+    cudaLaunchConfig_t lc = {};
+    lc.blockDim = dim3(256, 1, 1);
+    lc.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = 1;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cudaError_t e;
+    if (a.v_contig) {
+        // 128 lines per scanning CTA (1 KiB of a row of w), 32 where that leaves SMs idle; clusters
+        // so that a CTA has a batch of loads and more
+        const int64_t nv = std::max(a.nv, b.nv), nw = std::max(a.nw, b.nw);
+        const int lines = (nv + 127) / 128 * SPLIT_CLUSTER >= 2 * num_sms() * 4 / 5 ? 128 : 32;
+        unsigned cs = 1;
+        while (cs < unsigned(SPLIT_CLUSTER) && nw > int64_t(128) * cs) cs *= 2;
+        const auto scan_blocks = [cs, lines](const SplitJob& j) { return unsigned((j.nv + lines - 1) / lines * cs); };
+        const auto slice_blocks = [](const SplitJob& j) {
+            return unsigned((j.nv + 31) / 32 * (((CPLX ? j.nw : j.ldq) + 63) / 64));
+        };
+        a.blocks = scan_blocks(a);
+        b.blocks = scan_blocks(b);
+        at[0].val.clusterDim.x = cs;
+        lc.attrs = at;
+        lc.numAttrs = 1;
+        lc.gridDim = dim3(a.blocks + b.blocks, 1, 1);
+        e = lines == 128 ? cudaLaunchKernelEx(&lc, ozaki_scan_v_kernel<64, CPLX>, a, b)
+                         : cudaLaunchKernelEx(&lc, ozaki_scan_v_kernel<16, CPLX>, a, b);
+        count_launches(1);
+        if (e != cudaSuccess) return record_cuda(e);
+        a.blocks = slice_blocks(a);
+        b.blocks = slice_blocks(b);
+        lc.numAttrs = 0;
+        lc.gridDim = dim3(a.blocks + b.blocks, 1, 1);
+        e = cudaLaunchKernelEx(&lc, ozaki_slice_v_kernel<BITS, S, CPLX>, a, b, bits, slices);
     } else {
-        int64_t splits = (int64_t(sms) * 8 + nv - 1) / nv;
-        const int64_t maxs = (nw + 2047) / 2048;
-        splits = splits < 1 ? 1 : (splits > maxs ? maxs : splits);
-        const int64_t wps = (nw + splits - 1) / splits;
-        expo_wcontig<<<dim3(unsigned(nv), unsigned((nw + wps - 1) / wps)), 256, 0, st>>>(nv, nw, M, ld, wps, expo);
-        if (q8 && ld % 2 == 0 && aligned_to(M, 16) && fixed77)
-            slice_wcontig4<7, 7><<<dim3(unsigned((ldq + 1023) / 1024), unsigned(nv)), 256, 0, st>>>(
-                nv, nw, M, ld, expo, bits, slices, q, ldq, plane);
-        else if (q8 && ld % 2 == 0 && aligned_to(M, 16))
-            slice_wcontig4<0, 0><<<dim3(unsigned((ldq + 1023) / 1024), unsigned(nv)), 256, 0, st>>>(
-                nv, nw, M, ld, expo, bits, slices, q, ldq, plane);
-        else
-            slice_wcontig<<<dim3(unsigned((ldq + 255) / 256), unsigned(nv)), 256, 0, st>>>(nv, nw, M, ld, expo, bits,
-                                                                                           slices, q, ldq, plane);
+        auto kern = ozaki_split_w_kernel<BITS, S, CPLX>;
+        if (CPLX) {
+            static std::atomic<uint64_t> attrs{0};
+            const hsmm_status_t as = attrs_once_per_device(attrs, [kern] {
+                return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(SPLIT_CACHE));
+            });
+            if (as != HSMM_STATUS_SUCCESS) return as;
+            lc.dynamicSmemBytes = std::max(a.cached ? split_cache_bytes(a.nw) : 0, b.cached ? split_cache_bytes(b.nw) : 0);
+        }
+        lc.gridDim = dim3(a.blocks + b.blocks, 1, 1);
+        e = cudaLaunchKernelEx(&lc, kern, a, b, bits, slices);
     }
-    expo_fix<<<unsigned((nv + 255) / 256), 256, 0, st>>>(nv, expo);
-    count_launches(4);
+    count_launches(1);
+    if (e != cudaSuccess) return record_cuda(e);
     return check_launch();
 }
 
+hsmm_status_t launch_split(bool cplx, const SplitJob& a, const SplitJob& b, int bits, int slices, cudaStream_t st) {
+    const bool fixed77 = bits == 7 && slices == 7;
+    if (cplx) return fixed77 ? launch_split<7, 7, true>(a, b, bits, slices, st) : launch_split<0, 0, true>(a, b, bits, slices, st);
+    return fixed77 ? launch_split<7, 7, false>(a, b, bits, slices, st) : launch_split<0, 0, false>(a, b, bits, slices, st);
+}
+
+}  // namespace
+
+hsmm_status_t ozaki_split(bool cplx, const SplitOperand* ops, int count, int bits, int slices, cudaStream_t st) {
+    SplitJob j[2] = {};
+    for (int i = 0; i < count; ++i) {
+        const hsmm_status_t r = make_split_job(ops[i], cplx, &j[i]);
+        if (r != HSMM_STATUS_SUCCESS) return r;
+    }
+    if (count == 1 || j[0].v_contig == j[1].v_contig) return launch_split(cplx, j[0], j[1], bits, slices, st);
+    const hsmm_status_t r = launch_split(cplx, j[0], SplitJob{}, bits, slices, st);
+    return r != HSMM_STATUS_SUCCESS ? r : launch_split(cplx, j[1], SplitJob{}, bits, slices, st);
+}
 
 hsmm_status_t ozaki_zrecombine(int64_t m, int64_t n, int slices, int bits, const int32_t* sd, int64_t sd_plane,
                                const int32_t* ea, const int32_t* eb, const double* alpha, const double* beta, void* C,
@@ -853,57 +849,6 @@ hsmm_status_t ozaki_zrecombine(int64_t m, int64_t n, int slices, int bits, const
         m, n, slices, bits, gsize, sd, sd_plane, ea, eb, make_double2(alpha[0], alpha[1]),
         make_double2(beta[0], beta[1]), static_cast<double2*>(C), ldc);
     count_launches(1);
-    return check_launch();
-}
-
-// Complex operand into the real form (A' for role_b = false, B'' for role_b = true).
-// Lines v (rows of op(A) / columns of op(B)), nv of them, each of nw complex entries;
-// v_contig: entry (v, w) at M[v + w*ld], else at M[w + v*ld]; conj: op = C.
-hsmm_status_t ozaki_zsplit(int64_t nv, int64_t nw, const void* Mv, int64_t ld, bool v_contig, bool conj, bool role_b,
-                           int bits, int slices, int32_t* expo, void* qv, int64_t ldq, int64_t plane, cudaStream_t st) {
-    const double2* M = static_cast<const double2*>(Mv);
-    __nv_bfloat16* q = static_cast<__nv_bfloat16*>(qv);
-    if (v_contig && nv > 65535 * 32LL) return HSMM_STATUS_NOT_SUPPORTED;
-    if (!v_contig && nv > 65535) return HSMM_STATUS_NOT_SUPPORTED;
-    expo_init<<<unsigned((nv + 255) / 256), 256, 0, st>>>(nv, expo);
-    const int sms = num_sms();
-    const bool vec = ldq % 4 == 0 && plane % 4 == 0 && nw % 4 == 0 && aligned_to(qv, 8);
-    const bool fixed77 = bits == 7 && slices == 7;
-    if (v_contig) {
-        const int64_t vb = (nv + 255) / 256;
-        int64_t splits = (int64_t(sms) * 8 + vb - 1) / vb;
-        splits = splits < 1 ? 1 : (splits > nw ? nw : splits);
-        const int64_t wps = (nw + splits - 1) / splits;
-        zexpo_vcontig<<<dim3(unsigned(vb), unsigned((nw + wps - 1) / wps)), 256, 0, st>>>(nv, nw, M, ld, wps, expo);
-        const dim3 grid(unsigned((nw + 63) / 64), unsigned((nv + 31) / 32));
-        if (fixed77)
-            zslice_vcontig<7, 7><<<grid, 256, 0, st>>>(nv, nw, M, ld, expo, conj, role_b, bits, slices, q, ldq, plane,
-                                                       vec);
-        else
-            zslice_vcontig<0, 0><<<grid, 256, 0, st>>>(nv, nw, M, ld, expo, conj, role_b, bits, slices, q, ldq, plane,
-                                                       vec);
-    } else {
-        int64_t splits = (int64_t(sms) * 8 + nv - 1) / nv;
-        const int64_t maxs = (nw + 2047) / 2048;
-        splits = splits < 1 ? 1 : (splits > maxs ? maxs : splits);
-        const int64_t wps = (nw + splits - 1) / splits;
-        zexpo_wcontig<<<dim3(unsigned(nv), unsigned((nw + wps - 1) / wps)), 256, 0, st>>>(nv, nw, M, ld, wps, expo);
-        const dim3 grid(unsigned((nw + 1023) / 1024), unsigned(nv));
-        if (fixed77)
-            zslice_wcontig<7, 7><<<grid, 256, 0, st>>>(nv, nw, M, ld, expo, conj, role_b, bits, slices, q, ldq, plane,
-                                                       vec);
-        else
-            zslice_wcontig<0, 0><<<grid, 256, 0, st>>>(nv, nw, M, ld, expo, conj, role_b, bits, slices, q, ldq, plane,
-                                                       vec);
-    }
-    const int64_t lines = role_b ? 2 * nv : nv;
-    int launches = 4;
-    if (2 * nw < ldq) {
-        zpad_kernel<<<unsigned((lines + 255) / 256), 256, 0, st>>>(lines, 2 * nw, ldq, slices, q, plane);
-        ++launches;
-    }
-    expo_fix<<<unsigned((nv + 255) / 256), 256, 0, st>>>(nv, expo);
-    count_launches(launches);
     return check_launch();
 }
 
