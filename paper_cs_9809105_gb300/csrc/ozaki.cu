@@ -592,131 +592,140 @@ __device__ __forceinline__ double scaled_int(int64_t G, int P) {
 //   G = sum_{d=dl}^{dh} S_d 2^(bits (dh - d)),  |G| < 2^(31 + bits (g-1) + 1) <= 2^53,
 // so G 2^(e_i + f_j - bits dh) is an exact double and each group costs one FP64
 // addition (smallest group first).
-__global__ void __launch_bounds__(256) ozaki_recombine_kernel(int64_t m, int64_t n, int s, int bits, int gsize,
-                                                             const int32_t* __restrict__ sd, int64_t plane,
-                                                             const int32_t* __restrict__ ea,
-                                                             const int32_t* __restrict__ eb, double alpha, double beta,
-                                                             double* __restrict__ C, int64_t ldc) {
-    const int64_t i = int64_t(blockIdx.x) * 256 + threadIdx.x;
-    if (i >= m) return;
-    const int ei = ea[i];
-    for (int64_t j = blockIdx.y; j < n; j += gridDim.y) {
-        const int32_t* p = sd + i + j * m;
-        const int E0 = ei + eb[j];
-        double acc = 0.0;
-        for (int dh = s + 1; dh >= 2; dh -= gsize) {
-            const int dl = dh - gsize + 1 > 2 ? dh - gsize + 1 : 2;
-            int64_t G = 0;
-            for (int d = dl; d <= dh; ++d) G = G * (int64_t(1) << bits) + int64_t(__ldcs(p + int64_t(d - 2) * plane));
-            const double gv = scaled_int(G, E0 - bits * dh);
-            acc = (dh == s + 1) ? gv : acc + gv;      // the first group needs no FP64 addition
-        }
-        double v = (alpha == 1.0) ? acc : alpha * acc;
-        if (beta != 0.0) v = fma(beta, C[i + j * ldc], v);
-        C[i + j * ldc] = v;
+// Complex: Re and Im of op(A) op(B) are columns j and n + j of the real form's S_d; C = alpha
+// (Re + i Im) + beta C, alpha and beta complex.
+//
+// V rows per thread: 4 with 16-byte loads of every S_d plane (m, the plane pitch and ldc suitably
+// aligned; checked by the host), else 1.  F77: s = 7 slices of 7 bits (groups d = 5..8 and d =
+// 2..4), all planes loaded before any arithmetic, the same operations in the same order as the
+// general loop; a loop over the planes keeps one load in flight per thread.  Bound by DRAM (4 s
+// bytes in and 8 out per real element).
+template <int V>
+__device__ __forceinline__ void load_sums(const int32_t* p, int (&v)[V]) {
+    if constexpr (V == 4) {
+        const int4 x = __ldcs(reinterpret_cast<const int4*>(p));
+        v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w;
+    } else {
+        v[0] = __ldcs(p);
     }
 }
 
-// The same for four consecutive rows per thread: 16-byte loads of every S_d plane and
-// 16-byte stores of C (m, the plane pitch and ldc suitably aligned; checked by the host).
-// FIXED77: s = 7 slices of 7 bits (groups d = 5..8 and d = 2..4), all seven planes loaded
-// before any arithmetic, the same operations in the same order as the general loop.
-__device__ __forceinline__ int lane_of(const int4& v, int c) { return c == 0 ? v.x : c == 1 ? v.y : c == 2 ? v.z : v.w; }
-template <bool FIXED77>
-__global__ void __launch_bounds__(256) ozaki_recombine4_kernel(int64_t m, int64_t n, int s, int bits, int gsize,
-                                                              const int32_t* __restrict__ sd, int64_t plane,
-                                                              const int32_t* __restrict__ ea,
-                                                              const int32_t* __restrict__ eb, double alpha,
-                                                              double beta, double* __restrict__ C, int64_t ldc) {
-    const int64_t i = (int64_t(blockIdx.x) * 256 + threadIdx.x) * 4;
-    if (i >= m) return;
-    const int4 ei = *reinterpret_cast<const int4*>(ea + i);
-    for (int64_t j = blockIdx.y; j < n; j += gridDim.y) {
-        const int32_t* p = sd + i + j * m;
-        const int fj = eb[j];
-        const int E0[4] = {ei.x + fj, ei.y + fj, ei.z + fj, ei.w + fj};
-        double acc[4] = {0.0, 0.0, 0.0, 0.0};
-        if constexpr (FIXED77) {
-            int4 v[7];
+// the sums of V rows of one column, scaled by 2^E0[c]
+template <int V, bool F77>
+__device__ __forceinline__ void combine(const int32_t* p, int64_t plane, int s, int bits, int gsize, const int (&E0)[V],
+                                        double (&acc)[V]) {
+    if constexpr (F77) {
+        int v[7][V];
 #pragma unroll
-            for (int d = 2; d <= 8; ++d) v[d - 2] = __ldcs(reinterpret_cast<const int4*>(p + int64_t(d - 2) * plane));
+        for (int d = 2; d <= 8; ++d) load_sums<V>(p + int64_t(d - 2) * plane, v[d - 2]);
 #pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                int64_t G1 = 0, G2 = 0;
+        for (int c = 0; c < V; ++c) {
+            int64_t G1 = 0, G2 = 0;
 #pragma unroll
-                for (int d = 5; d <= 8; ++d) G1 = G1 * 128 + int64_t(lane_of(v[d - 2], c));
+            for (int d = 5; d <= 8; ++d) G1 = G1 * 128 + int64_t(v[d - 2][c]);
 #pragma unroll
-                for (int d = 2; d <= 4; ++d) G2 = G2 * 128 + int64_t(lane_of(v[d - 2], c));
-                acc[c] = scaled_int(G1, E0[c] - 7 * 8) + scaled_int(G2, E0[c] - 7 * 4);
+            for (int d = 2; d <= 4; ++d) G2 = G2 * 128 + int64_t(v[d - 2][c]);
+            acc[c] = scaled_int(G1, E0[c] - 7 * 8) + scaled_int(G2, E0[c] - 7 * 4);
+        }
+    } else {
+        for (int dh = s + 1; dh >= 2; dh -= gsize) {
+            const int dl = dh - gsize + 1 > 2 ? dh - gsize + 1 : 2;
+            int64_t G[V];
+#pragma unroll
+            for (int c = 0; c < V; ++c) G[c] = 0;
+            for (int d = dl; d <= dh; ++d) {
+                int v[V];
+                load_sums<V>(p + int64_t(d - 2) * plane, v);
+#pragma unroll
+                for (int c = 0; c < V; ++c) G[c] = G[c] * (int64_t(1) << bits) + int64_t(v[c]);
+            }
+#pragma unroll
+            for (int c = 0; c < V; ++c) {
+                const double gv = scaled_int(G[c], E0[c] - bits * dh);
+                acc[c] = (dh == s + 1) ? gv : acc[c] + gv;      // the first group needs no FP64 addition
+            }
+        }
+    }
+}
+
+struct RecombineArgs {
+    int64_t m, n;
+    int s, bits, gsize;
+    const int32_t* sd;
+    int64_t plane;
+    const int32_t *ea, *eb;
+    double2 alpha, beta;        // real: the first component
+    double* C;                  // complex: pairs
+    int64_t ldc;
+};
+
+template <int V, bool F77, bool CPLX>
+__global__ void __launch_bounds__(256) ozaki_recombine_kernel(RecombineArgs g) {
+    const int64_t i = (int64_t(blockIdx.x) * 256 + threadIdx.x) * V;
+    if (i >= g.m) return;
+    int ei[V];
+    if constexpr (V == 4) {
+        const int4 e = *reinterpret_cast<const int4*>(g.ea + i);
+        ei[0] = e.x; ei[1] = e.y; ei[2] = e.z; ei[3] = e.w;
+    } else {
+        ei[0] = g.ea[i];
+    }
+    for (int64_t j = blockIdx.y; j < g.n; j += gridDim.y) {
+        const int fj = g.eb[j];
+        int E0[V];
+#pragma unroll
+        for (int c = 0; c < V; ++c) E0[c] = ei[c] + fj;
+        double re[V];
+        combine<V, F77>(g.sd + i + j * g.m, g.plane, g.s, g.bits, g.gsize, E0, re);
+        if constexpr (CPLX) {
+            double im[V];
+            combine<V, F77>(g.sd + i + (g.n + j) * g.m, g.plane, g.s, g.bits, g.gsize, E0, im);
+            double2* cp = reinterpret_cast<double2*>(g.C) + i + j * g.ldc;
+#pragma unroll
+            for (int c = 0; c < V; ++c) {
+                double vr = g.alpha.x * re[c] - g.alpha.y * im[c];
+                double vi = g.alpha.x * im[c] + g.alpha.y * re[c];
+                if (g.beta.x != 0.0 || g.beta.y != 0.0) {
+                    const double2 c0 = cp[c];
+                    vr = fma(g.beta.x, c0.x, fma(-g.beta.y, c0.y, vr));
+                    vi = fma(g.beta.x, c0.y, fma(g.beta.y, c0.x, vi));
+                }
+                cp[c] = make_double2(vr, vi);
             }
         } else {
-        for (int dh = s + 1; dh >= 2; dh -= gsize) {
-            const int dl = dh - gsize + 1 > 2 ? dh - gsize + 1 : 2;
-            int64_t G[4] = {0, 0, 0, 0};
-            for (int d = dl; d <= dh; ++d) {
-                const int4 v = __ldcs(reinterpret_cast<const int4*>(p + int64_t(d - 2) * plane));
-                G[0] = G[0] * (int64_t(1) << bits) + int64_t(v.x);
-                G[1] = G[1] * (int64_t(1) << bits) + int64_t(v.y);
-                G[2] = G[2] * (int64_t(1) << bits) + int64_t(v.z);
-                G[3] = G[3] * (int64_t(1) << bits) + int64_t(v.w);
-            }
+            double* cp = g.C + i + j * g.ldc;
 #pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                const double gv = scaled_int(G[c], E0[c] - bits * dh);
-                acc[c] = (dh == s + 1) ? gv : acc[c] + gv;   // the first group needs no FP64 addition
+            for (int c = 0; c < V; ++c) re[c] = (g.alpha.x == 1.0) ? re[c] : g.alpha.x * re[c];
+            if constexpr (V == 4) {
+                double2* c2 = reinterpret_cast<double2*>(cp);
+                if (g.beta.x != 0.0) {
+                    const double2 a = c2[0], b = c2[1];
+                    re[0] = fma(g.beta.x, a.x, re[0]); re[1] = fma(g.beta.x, a.y, re[1]);
+                    re[2] = fma(g.beta.x, b.x, re[2]); re[3] = fma(g.beta.x, b.y, re[3]);
+                }
+                c2[0] = make_double2(re[0], re[1]);
+                c2[1] = make_double2(re[2], re[3]);
+            } else {
+                if (g.beta.x != 0.0) re[0] = fma(g.beta.x, cp[0], re[0]);
+                cp[0] = re[0];
             }
         }
-        }
-        double* cp = C + i + j * ldc;
-        double v[4];
-#pragma unroll
-        for (int c = 0; c < 4; ++c) v[c] = (alpha == 1.0) ? acc[c] : alpha * acc[c];
-        if (beta != 0.0) {
-            const double2 c0 = reinterpret_cast<const double2*>(cp)[0], c1 = reinterpret_cast<const double2*>(cp)[1];
-            v[0] = fma(beta, c0.x, v[0]); v[1] = fma(beta, c0.y, v[1]);
-            v[2] = fma(beta, c1.x, v[2]); v[3] = fma(beta, c1.y, v[3]);
-        }
-        reinterpret_cast<double2*>(cp)[0] = make_double2(v[0], v[1]);
-        reinterpret_cast<double2*>(cp)[1] = make_double2(v[2], v[3]);
     }
 }
 
-// Complex result: Re and Im of op(A) op(B) are columns j and n + j of the real form's
-// S_d; C = alpha (Re + i Im) + beta C, alpha and beta complex.
-__global__ void __launch_bounds__(256) ozaki_zrecombine_kernel(int64_t m, int64_t n, int s, int bits, int gsize,
-                                                              const int32_t* __restrict__ sd, int64_t plane,
-                                                              const int32_t* __restrict__ ea,
-                                                              const int32_t* __restrict__ eb, double2 alpha,
-                                                              double2 beta, double2* __restrict__ C, int64_t ldc) {
-    const int64_t i = int64_t(blockIdx.x) * 256 + threadIdx.x;
-    if (i >= m) return;
-    const int ei = ea[i];
-    const int64_t m2 = m;   // plane row pitch: S_d is [d-2][column of the real form][i]
-    for (int64_t j = blockIdx.y; j < n; j += gridDim.y) {
-        const int32_t* pr = sd + i + j * m2;
-        const int32_t* pi = sd + i + (n + j) * m2;
-        const int E0 = ei + eb[j];
-        double re = 0.0, im = 0.0;
-        for (int dh = s + 1; dh >= 2; dh -= gsize) {
-            const int dl = dh - gsize + 1 > 2 ? dh - gsize + 1 : 2;
-            int64_t Gr = 0, Gi = 0;
-            for (int d = dl; d <= dh; ++d) {
-                Gr = Gr * (int64_t(1) << bits) + int64_t(__ldcs(pr + int64_t(d - 2) * plane));
-                Gi = Gi * (int64_t(1) << bits) + int64_t(__ldcs(pi + int64_t(d - 2) * plane));
-            }
-            const double gr = scaled_int(Gr, E0 - bits * dh), gi = scaled_int(Gi, E0 - bits * dh);
-            re = (dh == s + 1) ? gr : re + gr;      // the first group needs no FP64 addition
-            im = (dh == s + 1) ? gi : im + gi;
-        }
-        double vr = alpha.x * re - alpha.y * im;
-        double vi = alpha.x * im + alpha.y * re;
-        if (beta.x != 0.0 || beta.y != 0.0) {
-            const double2 c = C[i + j * ldc];
-            vr = fma(beta.x, c.x, fma(-beta.y, c.y, vr));
-            vi = fma(beta.x, c.y, fma(beta.y, c.x, vi));
-        }
-        C[i + j * ldc] = make_double2(vr, vi);
-    }
+template <bool CPLX>
+hsmm_status_t launch_recombine(const RecombineArgs& g, cudaStream_t st) {
+    // complex C is 16-byte aligned by its type; a real one needs an even ldc for 16-byte stores
+    const bool vec4 = g.m % 4 == 0 && g.plane % 4 == 0 && aligned_to(g.sd, 16) && aligned_to(g.ea, 16) &&
+                      aligned_to(g.C, 16) && (CPLX || g.ldc % 2 == 0);
+    const bool f77 = g.s == 7 && g.bits == 7;
+    const dim3 grid(unsigned(((vec4 ? g.m / 4 : g.m) + 255) / 256), unsigned(g.n < 65535 ? g.n : 65535));
+    if (vec4 && f77) ozaki_recombine_kernel<4, true, CPLX><<<grid, 256, 0, st>>>(g);
+    else if (vec4) ozaki_recombine_kernel<4, false, CPLX><<<grid, 256, 0, st>>>(g);
+    else if (f77) ozaki_recombine_kernel<1, true, CPLX><<<grid, 256, 0, st>>>(g);
+    else ozaki_recombine_kernel<1, false, CPLX><<<grid, 256, 0, st>>>(g);
+    count_launches(1);
+    return check_launch();
 }
 
 }  // namespace
@@ -724,22 +733,8 @@ __global__ void __launch_bounds__(256) ozaki_zrecombine_kernel(int64_t m, int64_
 hsmm_status_t ozaki_recombine(int64_t m, int64_t n, int slices, int bits, const int32_t* sd, int64_t sd_plane,
                               const int32_t* ea, const int32_t* eb, double alpha, double beta, double* C, int64_t ldc,
                               cudaStream_t st) {
-    const int gsize = 1 + 21 / bits;
-    const unsigned gy = unsigned(n < 65535 ? n : 65535);
-    const bool vec4 = m % 4 == 0 && sd_plane % 4 == 0 && ldc % 2 == 0 && aligned_to(sd, 16) && aligned_to(ea, 16) &&
-                      aligned_to(C, 16);
-    if (vec4 && slices == 7 && bits == 7)
-        ozaki_recombine4_kernel<true><<<dim3(unsigned((m / 4 + 255) / 256), gy), 256, 0, st>>>(
-            m, n, slices, bits, gsize, sd, sd_plane, ea, eb, alpha, beta, C, ldc);
-    else if (vec4)
-        ozaki_recombine4_kernel<false><<<dim3(unsigned((m / 4 + 255) / 256), gy), 256, 0, st>>>(
-            m, n, slices, bits, gsize, sd, sd_plane, ea, eb, alpha, beta, C, ldc);
-    else
-        ozaki_recombine_kernel<<<dim3(unsigned((m + 255) / 256), gy), 256, 0, st>>>(m, n, slices, bits, gsize, sd,
-                                                                                   sd_plane, ea, eb, alpha, beta, C,
-                                                                                   ldc);
-    count_launches(1);
-    return check_launch();
+    return launch_recombine<false>(RecombineArgs{m, n, slices, bits, 1 + 21 / bits, sd, sd_plane, ea, eb,
+                                                 make_double2(alpha, 0.0), make_double2(beta, 0.0), C, ldc}, st);
 }
 
 namespace {
@@ -843,13 +838,9 @@ hsmm_status_t ozaki_split(bool cplx, const SplitOperand* ops, int count, int bit
 hsmm_status_t ozaki_zrecombine(int64_t m, int64_t n, int slices, int bits, const int32_t* sd, int64_t sd_plane,
                                const int32_t* ea, const int32_t* eb, const double* alpha, const double* beta, void* C,
                                int64_t ldc, cudaStream_t st) {
-    const int gsize = 1 + 21 / bits;
-    const unsigned gy = unsigned(n < 65535 ? n : 65535);
-    ozaki_zrecombine_kernel<<<dim3(unsigned((m + 255) / 256), gy), 256, 0, st>>>(
-        m, n, slices, bits, gsize, sd, sd_plane, ea, eb, make_double2(alpha[0], alpha[1]),
-        make_double2(beta[0], beta[1]), static_cast<double2*>(C), ldc);
-    count_launches(1);
-    return check_launch();
+    return launch_recombine<true>(RecombineArgs{m, n, slices, bits, 1 + 21 / bits, sd, sd_plane, ea, eb,
+                                                make_double2(alpha[0], alpha[1]), make_double2(beta[0], beta[1]),
+                                                static_cast<double*>(C), ldc}, st);
 }
 
 }  // namespace hsmm
