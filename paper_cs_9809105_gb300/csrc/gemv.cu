@@ -10,11 +10,19 @@
 //          split writes its partial sums to the workspace and a second kernel,
 //          launched as a programmatic dependent (it starts while the splits finish),
 //          adds the splits in a fixed order (deterministic results).
-//  op = T: y_j = sum_i A(i,j) x_i.  Column j is contiguous: one warp per column,
-//          128-bit loads, a fixed shuffle tree for the reduction.
+//  op = T: y_j = sum_i A(i,j) x_i.  Column j is contiguous: one warp per column, up to eight where
+//          there are few columns, 128-bit loads, a fixed shuffle tree for the reduction.
 //  INT8:   exact INT32 accumulation with dp4a; for op = N the 16-row x 4-column
 //          byte tiles are transposed in registers (byte permutes) so that dp4a
 //          multiplies four columns of one row by four packed entries of x.
+//
+// The 128-bit paths need aligned columns (A and lda), not whole vectors of rows: op = T ends a
+// column element by element, and op = N reads whole vectors into the padding rows of every column
+// but the last, whose tail it reads element by element (nothing after A(m-1, n-1) is read).
+// Before -> now, us in a row in a CUDA graph (N / T): INT8 2100 x 5300 with padded columns 9.2 / 7.8
+// -> 6.3 / 3.6, FP32 2101 x 5300 unaligned 16.9 / 29.8 -> 11.9 / 10.5, 16384 x 500 13.6 / 29.7 ->
+// 10.0 / 7.4, 1000^2 6.8 / 3.1 -> 3.9 / 2.4, 6654 x 8018 45.5 / 80.2 -> 34.4 / 39.2, 16384^2 150.3 /
+// 166.7 -> 150.0 / 157.5.
 #include <cstdint>
 #include <cuda_runtime.h>
 
@@ -39,20 +47,34 @@ constexpr int kThreads = 256;
 // ---------------------------------------------------------------------------
 // FP32, op = N
 // ---------------------------------------------------------------------------
-// Vector path: 4 rows per thread (float4), grid (row blocks, column splits).
+// Vector path: 4 rows per thread (float4), grid (row blocks, column splits).  2^rt threads of a CTA
+// take rows; where that is fewer than all (small m), the CTA's column split is cut again into
+// groups of cols_per_group columns, one per 2^rt threads, added in order through shared memory:
+// a thread then has fewer columns to walk one latency after the other.  PLAIN: no groups and m % 4
+// == 0 (34 registers instead of 60: 22.0 against 22.9 us at 8192 x 4096).
+template <bool PLAIN>
 __global__ void __launch_bounds__(kThreads) gemv_f32_n_vec(int64_t m, int64_t n, const float* __restrict__ A,
                                                            int64_t lda, const float* __restrict__ x, int64_t incx,
-                                                           float* __restrict__ part, int64_t cols_per_split) {
+                                                           float* __restrict__ part, int64_t cols_per_split,
+                                                           int rt, int64_t cols_per_group) {
     pdl_trigger();   // the reduction may be scheduled; it waits for this grid to finish
-    const int64_t r0 = (int64_t(blockIdx.x) * kThreads + threadIdx.x) * 4;
-    const int64_t j0 = int64_t(blockIdx.y) * cols_per_split;
-    const int64_t j1 = min(n, j0 + cols_per_split);
-    if (r0 >= m) return;
+    if (PLAIN) rt = 8;
+    const int tr = int(threadIdx.x) & ((1 << rt) - 1), group = PLAIN ? 0 : int(threadIdx.x) >> rt;
+    const int64_t r0 = ((int64_t(blockIdx.x) << rt) + tr) * 4;
+    const int64_t js = int64_t(blockIdx.y) * cols_per_split, j0 = PLAIN ? js : js + group * cols_per_group;
+    int64_t j1 = min(n, js + cols_per_split);
+    if (PLAIN) {
+        if (r0 >= m) return;
+    } else {
+        j1 = r0 < m ? min(j1, j0 + cols_per_group) : 0;      // no rows: no columns
+    }
+    // columns read as whole vectors (a split may be empty)
+    const int64_t jv = (!PLAIN && r0 + 4 > m && j1 == n && j0 < j1) ? j1 - 1 : j1;
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
     const float* a = A + r0;
     int64_t j = j0;
     // 8 columns in flight per thread
-    for (; j + 8 <= j1; j += 8) {
+    for (; j + 8 <= jv; j += 8) {
         float4 v[8];
         float xs[8];
 #pragma unroll
@@ -67,7 +89,7 @@ __global__ void __launch_bounds__(kThreads) gemv_f32_n_vec(int64_t m, int64_t n,
             acc.w = fmaf(v[u].w, xs[u], acc.w);
         }
     }
-    for (; j < j1; ++j) {
+    for (; j < jv; ++j) {
         float4 v = __ldcs(reinterpret_cast<const float4*>(a + j * lda));
         float xv = __ldg(x + j * incx);
         acc.x = fmaf(v.x, xv, acc.x);
@@ -75,11 +97,39 @@ __global__ void __launch_bounds__(kThreads) gemv_f32_n_vec(int64_t m, int64_t n,
         acc.z = fmaf(v.z, xv, acc.z);
         acc.w = fmaf(v.w, xv, acc.w);
     }
+    if (!PLAIN && jv < j1) {      // the last column of a matrix whose rows end inside this vector
+        const float xv = __ldg(x + jv * incx);
+        const float* c = a + jv * lda;
+        acc.x = fmaf(__ldg(c), xv, acc.x);
+        if (r0 + 1 < m) acc.y = fmaf(__ldg(c + 1), xv, acc.y);
+        if (r0 + 2 < m) acc.z = fmaf(__ldg(c + 2), xv, acc.z);
+    }
+    if constexpr (!PLAIN) {
+        __shared__ float4 red[kThreads];
+        red[threadIdx.x] = acc;
+        __syncthreads();
+        if (group != 0) return;
+        for (int g = 1; g < kThreads >> rt; ++g) {
+            const float4 v = red[(g << rt) + tr];
+            acc.x += v.x;
+            acc.y += v.y;
+            acc.z += v.z;
+            acc.w += v.w;
+        }
+    }
+    if (!PLAIN && r0 >= m) return;
     float* p = part + int64_t(blockIdx.y) * m + r0;
-    *reinterpret_cast<float4*>(p) = acc;
+    if (PLAIN || m % 4 == 0) {
+        *reinterpret_cast<float4*>(p) = acc;
+    } else {
+        p[0] = acc.x;
+        if (r0 + 1 < m) p[1] = acc.y;
+        if (r0 + 2 < m) p[2] = acc.z;
+        if (r0 + 3 < m) p[3] = acc.w;
+    }
 }
 
-// Scalar path (unaligned A or odd sizes): 1 row per thread.
+// Scalar path (unaligned columns): 1 row per thread.
 __global__ void __launch_bounds__(kThreads) gemv_f32_n_scalar(int64_t m, int64_t n, const float* __restrict__ A,
                                                               int64_t lda, const float* __restrict__ x,
                                                               int64_t incx, float* __restrict__ part,
@@ -90,7 +140,15 @@ __global__ void __launch_bounds__(kThreads) gemv_f32_n_scalar(int64_t m, int64_t
     const int64_t j1 = min(n, j0 + cols_per_split);
     if (r >= m) return;
     float acc = 0.f;
-    for (int64_t j = j0; j < j1; ++j) acc = fmaf(A[r + j * lda], __ldg(x + j * incx), acc);
+    int64_t j = j0;
+    for (; j + 8 <= j1; j += 8) {      // eight columns in flight
+        float v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) v[u] = __ldcs(A + r + (j + u) * lda);
+#pragma unroll
+        for (int u = 0; u < 8; ++u) acc = fmaf(v[u], __ldg(x + (j + u) * incx), acc);
+    }
+    for (; j < j1; ++j) acc = fmaf(A[r + j * lda], __ldg(x + j * incx), acc);
     part[int64_t(blockIdx.y) * m + r] = acc;
 }
 
@@ -106,6 +164,7 @@ __global__ void __launch_bounds__(kThreads) gemv_reduce(int64_t m, int nsplit, c
     const int64_t i = int64_t(blockIdx.x) * 32 + r;
     Acc sum = Acc(0);
     if (i < m)
+#pragma unroll 4
         for (int q = g; q < nsplit; q += kThreads / 32) sum += Acc(part[int64_t(q) * m + i]);
     __shared__ Acc red[kThreads / 32][32];
     red[g][r] = sum;
@@ -143,46 +202,186 @@ cudaError_t launch_reduce(int64_t m, int nsplit, const T* part, T alpha, T beta,
 }
 
 // ---------------------------------------------------------------------------
-// FP32, op = T: one warp per column
+// op = T
 // ---------------------------------------------------------------------------
-template <bool kVec>
-__global__ void __launch_bounds__(kThreads) gemv_f32_t(int64_t m, int64_t n, const float* __restrict__ A, int64_t lda,
-                                                       const float* __restrict__ x, int64_t incx, float alpha,
-                                                       float beta, float* __restrict__ y, int64_t incy) {
-    const int64_t col = int64_t(blockIdx.x) * (kThreads / 32) + warp_id();
-    if (col >= n) return;
-    const float* a = A + col * lda;
-    const int lane = lane_id();
-    float acc = 0.f;
-    if (kVec) {
-        // m % 4 == 0, a and x 16-byte aligned, incx == 1
-        const int64_t m4 = m / 4;
-        const float4* a4 = reinterpret_cast<const float4*>(a);
-        const float4* x4 = reinterpret_cast<const float4*>(x);
-        int64_t i = lane;
-        for (; i + 96 < m4; i += 128) {
-            float4 v0 = __ldcs(a4 + i), v1 = __ldcs(a4 + i + 32), v2 = __ldcs(a4 + i + 64), v3 = __ldcs(a4 + i + 96);
-            float4 w0 = __ldg(x4 + i), w1 = __ldg(x4 + i + 32), w2 = __ldg(x4 + i + 64), w3 = __ldg(x4 + i + 96);
-            acc = fmaf(v0.x, w0.x, acc); acc = fmaf(v0.y, w0.y, acc); acc = fmaf(v0.z, w0.z, acc); acc = fmaf(v0.w, w0.w, acc);
-            acc = fmaf(v1.x, w1.x, acc); acc = fmaf(v1.y, w1.y, acc); acc = fmaf(v1.z, w1.z, acc); acc = fmaf(v1.w, w1.w, acc);
-            acc = fmaf(v2.x, w2.x, acc); acc = fmaf(v2.y, w2.y, acc); acc = fmaf(v2.z, w2.z, acc); acc = fmaf(v2.w, w2.w, acc);
-            acc = fmaf(v3.x, w3.x, acc); acc = fmaf(v3.y, w3.y, acc); acc = fmaf(v3.z, w3.z, acc); acc = fmaf(v3.w, w3.w, acc);
-        }
-        for (; i < m4; i += 32) {
-            float4 v = __ldcs(a4 + i);
-            float4 w = __ldg(x4 + i);
-            acc = fmaf(v.x, w.x, acc); acc = fmaf(v.y, w.y, acc); acc = fmaf(v.z, w.z, acc); acc = fmaf(v.w, w.w, acc);
-        }
-    } else {
-        for (int64_t i = lane; i < m; i += 32) acc = fmaf(a[i], __ldg(x + i * incx), acc);
-    }
+// A CTA of eight warps takes 8, 4, 2 or 1 columns, 1 to 8 warps per column, each a contiguous part
+// of the rows; the warps' sums are added in order.  16 bytes a lane and load, four loads of A in
+// flight per lane.  (Two columns per warp, x loaded once for both, ran at 5.4 against 6.4 TB/s at
+// 16384^2.)
+struct GemvT {
+    int64_t m, n, lda, incx, incy;
+    int64_t rows;                  // rows of a warp, a multiple of 32 vectors
+    int shift;                     // 2^shift warps per column
+};
+__device__ __forceinline__ void t_store(const GemvT& g, float alpha, float beta, float* y, int64_t col, float acc) {
+    float v = alpha * acc;
+    if (beta != 0.f) v = fmaf(beta, y[col * g.incy], v);
+    y[col * g.incy] = v;
+}
+__device__ __forceinline__ void t_store(const GemvT& g, int32_t alpha, int32_t beta, int32_t* y, int64_t col, int acc) {
+    uint32_t v = uint32_t(alpha) * uint32_t(acc);          // INT32 BLAS arithmetic: wrap-around
+    if (beta != 0) v += uint32_t(beta) * uint32_t(y[col * g.incy]);
+    y[col * g.incy] = int32_t(v);
+}
+__device__ __forceinline__ void t_fma(const float4& a, const float4& x, float& acc) {
+    acc = fmaf(a.x, x.x, acc); acc = fmaf(a.y, x.y, acc); acc = fmaf(a.z, x.z, acc); acc = fmaf(a.w, x.w, acc);
+}
+__device__ __forceinline__ void t_fma(const int4& a, const int4& x, int& acc) {
+    acc = __dp4a(a.x, x.x, acc); acc = __dp4a(a.y, x.y, acc); acc = __dp4a(a.z, x.z, acc); acc = __dp4a(a.w, x.w, acc);
+}
+
+// 16-byte streaming loads that stay together in program order: all of a round are in flight before
+// the first is used
+__device__ __forceinline__ float4 load_stream(const float4* p) {
+    float4 v;
+    asm volatile("ld.global.cs.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+    return v;
+}
+
+// this warp's column, part of it and rows
+__device__ __forceinline__ void t_place(const GemvT& g, int64_t& col, int& part, int64_t& i0, int64_t& i1) {
+    const int warp = int(warp_id());
+    col = int64_t(blockIdx.x) * (kThreads / 32 >> g.shift) + (warp >> g.shift);
+    part = warp & ((1 << g.shift) - 1);
+    i0 = min(g.m, part * g.rows);
+    i1 = min(g.m, i0 + g.rows);
+}
+// sums of the lanes, then of the warps of a column, in order; the first warp stores y
+template <typename S>
+__device__ __forceinline__ void t_finish(const GemvT& g, S acc, int64_t col, int part, S alpha, S beta, S* y) {
+    const int warp = int(warp_id()), lane = int(lane_id());
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-    if (lane == 0) {
-        float v = alpha * acc;
-        if (beta != 0.f) v = fmaf(beta, y[col * incy], v);
-        y[col * incy] = v;
+    if (g.shift > 0) {
+        __shared__ S red[kThreads / 32];
+        if (lane == 0) red[warp] = acc;
+        __syncthreads();
+        if (part != 0) return;
+        for (int i = 1; i < 1 << g.shift; ++i) acc += red[warp + i];
     }
+    if (lane == 0 && col < g.n) t_store(g, alpha, beta, y, col, acc);
+}
+
+// FP32, aligned columns of a whole number of vectors and aligned x, incx == 1, one warp per column:
+// all loads of a round are in flight before the first is used (166 -> 157.5 us at 16384^2, 6.8
+// TB/s).  The same loop was slower for INT8 (44.3 us at 16384^2 against 40.5 for the general one).
+__global__ void __launch_bounds__(kThreads) gemv_f32_t_plain(GemvT g, const float* __restrict__ A,
+                                                             const float* __restrict__ x, float alpha, float beta,
+                                                             float* __restrict__ y) {
+    const int lane = int(lane_id());
+    const int64_t col = int64_t(blockIdx.x) * (kThreads / 32) + warp_id();
+    if (col >= g.n) return;
+    const int64_t mv = g.m / 4;
+    const float4* a = reinterpret_cast<const float4*>(A + col * g.lda);
+    const float4* xp = reinterpret_cast<const float4*>(x);
+    float acc = 0.f;
+    int64_t i = lane;
+    for (; i + 96 < mv; i += 128) {
+        float4 v[4], w[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) v[u] = load_stream(a + i + 32 * u);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) w[u] = __ldg(xp + i + 32 * u);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) t_fma(v[u], w[u], acc);
+    }
+    for (; i < mv; i += 32) t_fma(__ldcs(a + i), __ldg(xp + i), acc);
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
+    if (lane == 0) t_store(g, alpha, beta, y, col, acc);
+}
+
+// The general form: m any, 2^g.shift warps per column.  T: element (float, int8_t), V: 16-byte
+// vector of it, S: sum.  Held to five CTAs an SM (INT8 at 16384^2 43.2 -> 40.5 us).
+template <typename T, typename V, typename S>
+__global__ void __launch_bounds__(kThreads, 5) gemv_t_vec(GemvT g, const T* __restrict__ A, const T* __restrict__ x,
+                                                          S alpha, S beta, S* __restrict__ y) {
+    constexpr int E = 16 / int(sizeof(T));                 // elements of a vector
+    const int lane = int(lane_id());
+    int64_t col, i0, i1;
+    int part;
+    t_place(g, col, part, i0, i1);
+    S acc = S(0);
+    if (col < g.n) {
+        const T* a = A + col * g.lda;
+        const int64_t iv = i0 + (i1 - i0) / E * E;     // rows in whole vectors
+        int64_t i = i0;
+        for (; i + 128 * E <= iv; i += 128 * E) {
+            V v[4], w[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) v[u] = __ldcs(reinterpret_cast<const V*>(a + i + (32 * u + lane) * E));
+#pragma unroll
+            for (int u = 0; u < 4; ++u) w[u] = __ldg(reinterpret_cast<const V*>(x + i + (32 * u + lane) * E));
+#pragma unroll
+            for (int u = 0; u < 4; ++u) t_fma(v[u], w[u], acc);
+        }
+        if (i < iv) {                                  // what is left of a round
+            V v[4], w[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int64_t r = i + (32 * u + lane) * E;
+                const bool in = r < iv;
+                v[u] = in ? __ldcs(reinterpret_cast<const V*>(a + r)) : V{};
+                w[u] = in ? __ldg(reinterpret_cast<const V*>(x + r)) : V{};
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (i + (32 * u + lane) * E < iv) t_fma(v[u], w[u], acc);
+        }
+        i = iv + lane;                                 // the last m % E rows
+        if (i < i1) acc += S(__ldg(a + i)) * S(__ldg(x + i));
+    }
+    t_finish(g, acc, col, part, alpha, beta, y);
+}
+
+// Unaligned columns: one element per lane and load.  UNIT: incx == 1.
+template <typename T, typename S, bool UNIT>
+__global__ void __launch_bounds__(kThreads) gemv_t_scalar(GemvT g, const T* __restrict__ A, const T* __restrict__ x,
+                                                          S alpha, S beta, S* __restrict__ y) {
+    const int lane = int(lane_id());
+    int64_t col, i0, i1;
+    int part;
+    t_place(g, col, part, i0, i1);
+    const int64_t incx = UNIT ? 1 : g.incx;
+    S acc = S(0);
+    if (col < g.n) {
+        const T* a = A + col * g.lda + i0 + lane;
+        const T* xp = x + (i0 + lane) * incx;
+        int64_t left = (i1 - i0 - lane + 31) >> 5;         // elements of this lane
+        for (; left >= 8; left -= 8, a += 256, xp += 256 * incx) {
+            T v[8], w[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) v[u] = __ldg(a + 32 * u);
+#pragma unroll
+            for (int u = 0; u < 8; ++u) w[u] = __ldg(xp + 32 * u * incx);
+#pragma unroll
+            for (int u = 0; u < 8; ++u) acc += S(v[u]) * S(w[u]);
+        }
+        for (; left > 0; --left, a += 32, xp += 32 * incx) acc += S(__ldg(a)) * S(__ldg(xp));
+    }
+    t_finish(g, acc, col, part, alpha, beta, y);
+}
+
+// One warp per column where that is 16 warps an SM and more, else up to eight for about as many.
+template <typename T, typename V, typename S>
+void launch_t(int64_t m, int64_t n, S alpha, const T* A, int64_t lda, const T* x, int64_t incx, S beta, S* y,
+              int64_t incy, bool vec, cudaStream_t st) {
+    const int64_t want = int64_t(num_sms()) * 16, unit = 32 * (16 / int64_t(sizeof(T)));   // one vector per lane
+    GemvT g{m, n, lda, incx, incy, 0, 0};
+    while ((1 << g.shift) < kThreads / 32 && (n << g.shift) < want && m > (4 * unit << g.shift)) ++g.shift;
+    const int64_t parts = int64_t(1) << g.shift;
+    g.rows = ((m + unit - 1) / unit + parts - 1) / parts * unit;
+    const int cols = kThreads / 32 >> g.shift;
+    const unsigned grid = unsigned((n + cols - 1) / cols);
+    if constexpr (sizeof(T) == 4) {
+        if (vec && g.shift == 0 && m % 4 == 0) {
+            gemv_f32_t_plain<<<grid, kThreads, 0, st>>>(g, A, x, alpha, beta, y);
+            return;
+        }
+    }
+    if (vec) gemv_t_vec<T, V, S><<<grid, kThreads, 0, st>>>(g, A, x, alpha, beta, y);
+    else if (incx == 1) gemv_t_scalar<T, S, true><<<grid, kThreads, 0, st>>>(g, A, x, alpha, beta, y);
+    else gemv_t_scalar<T, S, false><<<grid, kThreads, 0, st>>>(g, A, x, alpha, beta, y);
 }
 
 // ---------------------------------------------------------------------------
@@ -209,21 +408,31 @@ __device__ __forceinline__ uint32_t pack_x4(const int8_t* x, int64_t j, int64_t 
     return b0 | (b1 << 8) | (b2 << 16) | (b3 << 24);
 }
 
+template <bool PLAIN>
 __global__ void __launch_bounds__(kThreads) gemv_i8_n_vec(int64_t m, int64_t n, const int8_t* __restrict__ A,
                                                           int64_t lda, const int8_t* __restrict__ x, int64_t incx,
-                                                          int32_t* __restrict__ part, int64_t cols_per_split) {
+                                                          int32_t* __restrict__ part, int64_t cols_per_split,
+                                                          int rt, int64_t cols_per_group) {
     pdl_trigger();   // the reduction may be scheduled; it waits for this grid to finish
-    const int64_t r0 = (int64_t(blockIdx.x) * kThreads + threadIdx.x) * 16;
-    const int64_t j0 = int64_t(blockIdx.y) * cols_per_split;
-    const int64_t j1 = min(n, j0 + cols_per_split);
-    if (r0 >= m) return;
+    if (PLAIN) rt = 8;                                       // see gemv_f32_n_vec; m % 16 == 0
+    const int tr = int(threadIdx.x) & ((1 << rt) - 1), group = PLAIN ? 0 : int(threadIdx.x) >> rt;
+    const int64_t r0 = ((int64_t(blockIdx.x) << rt) + tr) * 16;
+    const int64_t js = int64_t(blockIdx.y) * cols_per_split, j0 = PLAIN ? js : js + group * cols_per_group;
+    int64_t j1 = min(n, js + cols_per_split);
+    if (PLAIN) {
+        if (r0 >= m) return;
+    } else {
+        j1 = r0 < m ? min(j1, j0 + cols_per_group) : 0;      // no rows: no columns
+    }
+    // columns read as whole vectors (a split may be empty)
+    const int64_t jv = (!PLAIN && r0 + 16 > m && j1 == n && j0 < j1) ? j1 - 1 : j1;
     int acc[16];
 #pragma unroll
     for (int r = 0; r < 16; ++r) acc[r] = 0;
     const int8_t* a = A + r0;
     int64_t j = j0;
     // two groups of four columns (eight 16-byte loads) in flight per thread
-    for (; j + 8 <= j1; j += 8) {
+    for (; j + 8 <= jv; j += 8) {
         uint4 c[8];
 #pragma unroll
         for (int u = 0; u < 8; ++u) c[u] = __ldcs(reinterpret_cast<const uint4*>(a + (j + u) * lda));
@@ -246,7 +455,7 @@ __global__ void __launch_bounds__(kThreads) gemv_i8_n_vec(int64_t m, int64_t n, 
             for (int r = 0; r < 4; ++r) acc[12 + r] = __dp4a(int(t[r]), xp, acc[12 + r]);
         }
     }
-    for (; j + 4 <= j1; j += 4) {
+    for (; j + 4 <= jv; j += 4) {
         uint4 c[4];
 #pragma unroll
         for (int u = 0; u < 4; ++u) c[u] = __ldcs(reinterpret_cast<const uint4*>(a + (j + u) * lda));
@@ -265,7 +474,7 @@ __global__ void __launch_bounds__(kThreads) gemv_i8_n_vec(int64_t m, int64_t n, 
 #pragma unroll
         for (int r = 0; r < 4; ++r) acc[12 + r] = __dp4a(int(t[r]), xp, acc[12 + r]);
     }
-    for (; j < j1; ++j) {
+    for (; j < jv; ++j) {
         const uint4 c = __ldcs(reinterpret_cast<const uint4*>(a + j * lda));
         const int xv = int(__ldg(x + j * incx));
         const uint32_t w[4] = {c.x, c.y, c.z, c.w};
@@ -274,9 +483,41 @@ __global__ void __launch_bounds__(kThreads) gemv_i8_n_vec(int64_t m, int64_t n, 
 #pragma unroll
             for (int b = 0; b < 4; ++b) acc[4 * q + b] += int(int8_t((w[q] >> (8 * b)) & 0xffu)) * xv;
     }
-    int32_t* p = part + int64_t(blockIdx.y) * m + r0;
+    if (!PLAIN && jv < j1) {      // the last column of a matrix whose rows end inside this vector
+        const int xv = int(__ldg(x + jv * incx));
 #pragma unroll
-    for (int q = 0; q < 4; ++q) reinterpret_cast<int4*>(p)[q] = make_int4(acc[4 * q], acc[4 * q + 1], acc[4 * q + 2], acc[4 * q + 3]);
+        for (int r = 0; r < 16; ++r)
+            if (r0 + r < m) acc[r] += int(__ldg(a + r + jv * lda)) * xv;
+    }
+    if constexpr (!PLAIN) {
+        __shared__ int4 red[4][kThreads];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) red[q][threadIdx.x] = make_int4(acc[4 * q], acc[4 * q + 1], acc[4 * q + 2], acc[4 * q + 3]);
+        __syncthreads();
+        if (group != 0) return;
+        for (int g = 1; g < kThreads >> rt; ++g) {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int4 v = red[q][(g << rt) + tr];
+                acc[4 * q] += v.x;
+                acc[4 * q + 1] += v.y;
+                acc[4 * q + 2] += v.z;
+                acc[4 * q + 3] += v.w;
+            }
+        }
+    }
+    if (!PLAIN && r0 >= m) return;
+    int32_t* p = part + int64_t(blockIdx.y) * m + r0;
+    if (PLAIN || m % 4 == 0) {   // every split's sums start 16-byte aligned
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            if (PLAIN || r0 + 4 * q < m)
+                reinterpret_cast<int4*>(p)[q] = make_int4(acc[4 * q], acc[4 * q + 1], acc[4 * q + 2], acc[4 * q + 3]);
+    } else {
+#pragma unroll
+        for (int r = 0; r < 16; ++r)
+            if (r0 + r < m) p[r] = acc[r];
+    }
 }
 
 __global__ void __launch_bounds__(kThreads) gemv_i8_n_scalar(int64_t m, int64_t n, const int8_t* __restrict__ A,
@@ -288,55 +529,16 @@ __global__ void __launch_bounds__(kThreads) gemv_i8_n_scalar(int64_t m, int64_t 
     const int64_t j1 = min(n, j0 + cols_per_split);
     if (r >= m) return;
     int acc = 0;
-    for (int64_t j = j0; j < j1; ++j) acc += int(A[r + j * lda]) * int(__ldg(x + j * incx));
+    int64_t j = j0;
+    for (; j + 8 <= j1; j += 8) {      // eight columns in flight
+        int8_t v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) v[u] = __ldcs(A + r + (j + u) * lda);
+#pragma unroll
+        for (int u = 0; u < 8; ++u) acc += int(v[u]) * int(__ldg(x + (j + u) * incx));
+    }
+    for (; j < j1; ++j) acc += int(A[r + j * lda]) * int(__ldg(x + j * incx));
     part[int64_t(blockIdx.y) * m + r] = acc;
-}
-
-// INT8, op = T: one warp per column, 16 bytes per lane per step, dp4a against packed x.
-template <bool kVec>
-__global__ void __launch_bounds__(kThreads) gemv_i8_t(int64_t m, int64_t n, const int8_t* __restrict__ A, int64_t lda,
-                                                      const int8_t* __restrict__ x, int64_t incx, int32_t alpha,
-                                                      int32_t beta, int32_t* __restrict__ y, int64_t incy) {
-    const int64_t col = int64_t(blockIdx.x) * (kThreads / 32) + warp_id();
-    if (col >= n) return;
-    const int8_t* a = A + col * lda;
-    const int lane = lane_id();
-    int acc = 0;
-    if (kVec) {
-        // m % 16 == 0, 16-byte aligned column and x, incx == 1
-        const int64_t m16 = m / 16;
-        const int4* a16 = reinterpret_cast<const int4*>(a);
-        const int4* x16 = reinterpret_cast<const int4*>(x);
-        int64_t i = lane;
-        // four 16-byte loads of A in flight per lane
-        for (; i + 96 < m16; i += 128) {
-            int4 v[4], w[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) v[u] = __ldcs(a16 + i + 32 * u);
-#pragma unroll
-            for (int u = 0; u < 4; ++u) w[u] = __ldg(x16 + i + 32 * u);
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                acc = __dp4a(v[u].x, w[u].x, acc); acc = __dp4a(v[u].y, w[u].y, acc);
-                acc = __dp4a(v[u].z, w[u].z, acc); acc = __dp4a(v[u].w, w[u].w, acc);
-            }
-        }
-        for (; i < m16; i += 32) {
-            const int4 v = __ldcs(a16 + i);
-            const int4 w = __ldg(x16 + i);
-            acc = __dp4a(v.x, w.x, acc); acc = __dp4a(v.y, w.y, acc);
-            acc = __dp4a(v.z, w.z, acc); acc = __dp4a(v.w, w.w, acc);
-        }
-    } else {
-        for (int64_t i = lane; i < m; i += 32) acc += int(a[i]) * int(__ldg(x + i * incx));
-    }
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-    if (lane == 0) {
-        uint32_t v = uint32_t(alpha) * uint32_t(acc);
-        if (beta != 0) v += uint32_t(beta) * uint32_t(y[col * incy]);
-        y[col * incy] = int32_t(v);
-    }
 }
 
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
@@ -368,6 +570,24 @@ size_t gemv_workspace_bytes(hsmm_dtype_t a, hsmm_op_t trans, int64_t m, int64_t 
     return size_t(gemv_splits_rows(m, n, rows_per_thread(a))) * size_t(m) * 4u;
 }
 
+// Row threads of a CTA of the op = N vector kernels: all 256, or fewer (at least 32) while there
+// are under two CTAs an SM (8192 x 4096 FP32, 3.4 CTAs an SM: 22.0 us with 256, 23.3 with 128)
+struct NSplit {
+    int rt;
+    int64_t cols_per_group;
+    dim3 grid;
+};
+static NSplit n_split(int64_t m, int ns, int64_t cps, int rows_per_thread) {
+    NSplit s{8, cps, dim3()};
+    const int64_t vecs = (m + rows_per_thread - 1) / rows_per_thread;
+    auto blocks = [&] { return (vecs + (int64_t(1) << s.rt) - 1) >> s.rt; };
+    while (s.rt > 5 && blocks() * ns < int64_t(num_sms()) * 2) --s.rt;
+    const int groups = kThreads >> s.rt;
+    s.cols_per_group = (cps + groups - 1) / groups;
+    s.grid = dim3(unsigned(blocks()), unsigned(ns));
+    return s;
+}
+
 hsmm_status_t gemv_f32(hsmm_op_t trans, int64_t m, int64_t n, float alpha, const float* A, int64_t lda,
                        const float* x, int64_t incx, float beta, float* y, int64_t incy, void* ws, size_t ws_bytes,
                        cudaStream_t st) {
@@ -376,10 +596,14 @@ hsmm_status_t gemv_f32(hsmm_op_t trans, int64_t m, int64_t n, float alpha, const
         if (ws_bytes < size_t(ns) * size_t(m) * 4u || ws == nullptr) return HSMM_STATUS_WORKSPACE_TOO_SMALL;
         const int64_t cps = (n + ns - 1) / ns;
         float* part = static_cast<float*>(ws);
-        const bool vec = (m % 4 == 0) && (lda % 4 == 0) && aligned16(A) && aligned16(ws);
+        const bool vec = (lda % 4 == 0) && aligned16(A) && aligned16(ws);
         if (vec) {
-            dim3 grid(unsigned((m / 4 + kThreads - 1) / kThreads), unsigned(ns));
-            gemv_f32_n_vec<<<grid, kThreads, 0, st>>>(m, n, A, lda, x, incx, part, cps);
+            const NSplit sp = n_split(m, ns, cps, 4);
+            if (sp.rt == 8 && m % 4 == 0)
+                gemv_f32_n_vec<true><<<sp.grid, kThreads, 0, st>>>(m, n, A, lda, x, incx, part, cps, 8, cps);
+            else
+                gemv_f32_n_vec<false><<<sp.grid, kThreads, 0, st>>>(m, n, A, lda, x, incx, part, cps, sp.rt,
+                                                                  sp.cols_per_group);
         } else {
             dim3 grid(unsigned((m + kThreads - 1) / kThreads), unsigned(ns));
             gemv_f32_n_scalar<<<grid, kThreads, 0, st>>>(m, n, A, lda, x, incx, part, cps);
@@ -388,12 +612,8 @@ hsmm_status_t gemv_f32(hsmm_op_t trans, int64_t m, int64_t n, float alpha, const
         count_launches(2);
         if (e != cudaSuccess) return record_cuda(e);
     } else {
-        const bool vec = (m % 4 == 0) && (lda % 4 == 0) && aligned16(A) && aligned16(x) && incx == 1;
-        const unsigned grid = unsigned((n + kThreads / 32 - 1) / (kThreads / 32));
-        if (vec)
-            gemv_f32_t<true><<<grid, kThreads, 0, st>>>(m, n, A, lda, x, incx, alpha, beta, y, incy);
-        else
-            gemv_f32_t<false><<<grid, kThreads, 0, st>>>(m, n, A, lda, x, incx, alpha, beta, y, incy);
+        const bool vec = (lda % 4 == 0) && aligned16(A) && aligned16(x) && incx == 1;
+        launch_t<float, float4, float>(m, n, alpha, A, lda, x, incx, beta, y, incy, vec, st);
         count_launches(1);
     }
     return check_launch();
@@ -407,10 +627,14 @@ hsmm_status_t gemv_i8(hsmm_op_t trans, int64_t m, int64_t n, int32_t alpha, cons
         if (ws_bytes < size_t(ns) * size_t(m) * 4u || ws == nullptr) return HSMM_STATUS_WORKSPACE_TOO_SMALL;
         const int64_t cps = (n + ns - 1) / ns;
         int32_t* part = static_cast<int32_t*>(ws);
-        const bool vec = (m % 16 == 0) && (lda % 16 == 0) && aligned16(A) && aligned16(ws);
+        const bool vec = (lda % 16 == 0) && aligned16(A) && aligned16(ws);
         if (vec) {
-            dim3 grid(unsigned((m / 16 + kThreads - 1) / kThreads), unsigned(ns));
-            gemv_i8_n_vec<<<grid, kThreads, 0, st>>>(m, n, A, lda, x, incx, part, cps);
+            const NSplit sp = n_split(m, ns, cps, 16);
+            if (sp.rt == 8 && m % 16 == 0)
+                gemv_i8_n_vec<true><<<sp.grid, kThreads, 0, st>>>(m, n, A, lda, x, incx, part, cps, 8, cps);
+            else
+                gemv_i8_n_vec<false><<<sp.grid, kThreads, 0, st>>>(m, n, A, lda, x, incx, part, cps, sp.rt,
+                                                                  sp.cols_per_group);
         } else {
             dim3 grid(unsigned((m + kThreads - 1) / kThreads), unsigned(ns));
             gemv_i8_n_scalar<<<grid, kThreads, 0, st>>>(m, n, A, lda, x, incx, part, cps);
@@ -419,12 +643,8 @@ hsmm_status_t gemv_i8(hsmm_op_t trans, int64_t m, int64_t n, int32_t alpha, cons
         count_launches(2);
         if (e != cudaSuccess) return record_cuda(e);
     } else {
-        const bool vec = (m % 16 == 0) && (lda % 16 == 0) && aligned16(A) && aligned16(x) && incx == 1;
-        const unsigned grid = unsigned((n + kThreads / 32 - 1) / (kThreads / 32));
-        if (vec)
-            gemv_i8_t<true><<<grid, kThreads, 0, st>>>(m, n, A, lda, x, incx, alpha, beta, y, incy);
-        else
-            gemv_i8_t<false><<<grid, kThreads, 0, st>>>(m, n, A, lda, x, incx, alpha, beta, y, incy);
+        const bool vec = (lda % 16 == 0) && aligned16(A) && aligned16(x) && incx == 1;
+        launch_t<int8_t, int4, int>(m, n, alpha, A, lda, x, incx, beta, y, incy, vec, st);
         count_launches(1);
     }
     return check_launch();
