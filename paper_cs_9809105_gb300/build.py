@@ -1,4 +1,5 @@
-"""Build libhsmm.so in-tree: every csrc/*.cu compiled for sm_103a in parallel, then linked.
+"""Build libhsmm.so in-tree: every csrc/*.cu compiled for sm_103a in parallel, then linked, and
+beside it the Python binding's call module (csrc/pycall.c) where Python's headers are installed.
 
 Usage: python -m paper_cs_9809105_gb300.build [--force]
 """
@@ -10,12 +11,14 @@ import hashlib
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 OUT = os.path.join(HERE, "_build")
 LIB = os.path.join(OUT, "libhsmm.so")
+CALL = os.path.join(OUT, "_hsmmcall" + (sysconfig.get_config_var("EXT_SUFFIX") or ".so"))
 INCLUDE = os.path.join(ROOT, "include")
 
 NVCC = os.environ.get("NVCC", os.path.join(os.environ.get("CUDA_HOME", "/usr/local/cuda"), "bin", "nvcc"))
@@ -31,12 +34,12 @@ def _sources():
 def _fingerprint() -> str:
     h = hashlib.sha256()
     for p in _sources() + sorted(glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(CSRC, "*.h"))) + \
-            [os.path.join(INCLUDE, "hsmm.h")]:
+            [os.path.join(CSRC, "pycall.c"), os.path.join(INCLUDE, "hsmm.h")]:
         h.update(p.encode())
         with open(p, "rb") as f:
             h.update(f.read())
     h.update(" ".join(ARCH + FLAGS).encode())
-    h.update(os.uname().machine.encode())
+    h.update((os.uname().machine + CALL).encode())
     return h.hexdigest()
 
 
@@ -44,7 +47,10 @@ def build(force: bool = False, verbose: bool = False) -> str:
     os.makedirs(OUT, exist_ok=True)
     fp = _fingerprint()
     stamp = os.path.join(OUT, "fingerprint")
-    if not force and os.path.exists(LIB) and os.path.exists(stamp) and open(stamp).read() == fp:
+    headers = sysconfig.get_paths()["include"]
+    with_call = os.path.exists(os.path.join(headers, "Python.h"))
+    if not force and os.path.exists(LIB) and (os.path.exists(CALL) or not with_call) and \
+            os.path.exists(stamp) and open(stamp).read() == fp:
         return LIB
     srcs = _sources()
     objs = [os.path.join(OUT, os.path.basename(s) + ".o") for s in srcs]
@@ -66,6 +72,14 @@ def build(force: bool = False, verbose: bool = False) -> str:
     if r.returncode != 0:
         raise RuntimeError(f"link failed:\n{r.stderr}")
     os.replace(tmp, LIB)
+    if with_call:
+        tmp = CALL + f".tmp{os.getpid()}"
+        cmd = [os.environ.get("CC", "gcc"), "-O2", "-shared", "-fPIC", f"-I{headers}", f"-I{INCLUDE}",
+               os.path.join(CSRC, "pycall.c"), "-o", tmp]
+        r = subprocess.run(cmd, capture_output=True, text=True)
+        if r.returncode != 0:
+            raise RuntimeError(f"compiling pycall.c failed:\n{r.stderr}")
+        os.replace(tmp, CALL)
     with open(stamp, "w") as f:
         f.write(fp)
     return LIB

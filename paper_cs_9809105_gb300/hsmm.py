@@ -1,7 +1,8 @@
 """ctypes binding of libhsmm (the C ABI declared in include/hsmm.h).
 
 Argument marshalling only: every step of every product runs in the library's
-CUDA kernels.  PyTorch supplies device memory and streams.  If the compiled
+CUDA kernels.  The calls made once per step (gemm, gemv) go through a small CPython
+module instead (csrc/pycall.c) where it was built.  PyTorch supplies device memory and streams.  If the compiled
 library is missing, importing the functions raises -- there is no fallback.
 
 Matrices passed to the column-major calls are torch CUDA tensors whose first
@@ -12,6 +13,8 @@ column-major product C^T = op(B)^T op(A)^T without copies.
 from __future__ import annotations
 
 import ctypes
+import glob
+import importlib.util
 import os
 
 import torch
@@ -102,8 +105,26 @@ def lib():
         if name not in ("hsmm_status_string", "hsmm_last_cuda_error", "hsmm_last_error_detail", "hsmm_version",
                         "hsmm_launch_count"):
             getattr(L, name).restype = ci
+    _bind_calls(L)
     _lib = L
     return L
+
+
+_call = None      # the CPython module of the per-step calls, or None
+
+
+def _bind_calls(L) -> None:
+    global _call
+    for path in glob.glob(os.path.join(os.path.dirname(LIB_PATH), "_hsmmcall*.so")):
+        spec = importlib.util.spec_from_file_location("_hsmmcall", path)
+        try:
+            mod = importlib.util.module_from_spec(spec)
+            spec.loader.exec_module(mod)
+        except ImportError:       # built for another Python
+            continue
+        mod.bind(*(ctypes.cast(f, ctypes.c_void_p).value for f in (L.hsmm_gemm, L.hsmm_gemv)))
+        _call = mod
+        return
 
 
 def status_string(s: int) -> str:
@@ -167,12 +188,13 @@ def _ld(x: torch.Tensor) -> int:
     """Leading dimension of a column-major matrix view (element (i, j) at i + j*ld)."""
     if x.dim() != 2:
         raise ValueError("matrices must be 2-D")
-    rows, cols = x.shape
+    rows = x.shape[0]
+    s0, s1 = x.stride()
     if rows <= 1:
-        return max(1, x.stride(1))
-    if x.stride(0) != 1:
+        return max(1, s1)
+    if s0 != 1:
         raise ValueError("column-major matrix expected (stride(0) == 1)")
-    return max(rows, x.stride(1))
+    return s1 if s1 > rows else rows
 
 
 _SCALARS: dict = {}
@@ -238,13 +260,20 @@ def gemm(A: torch.Tensor, B: torch.Tensor, C: torch.Tensor, transA="N", transB="
         cfg = make_config(*key[:6], None, *key[6:])
         need = workspace_size(cfg, transA, transB, m, n, k)
         workspace = torch.empty(need, dtype=torch.uint8, device=C.device)
+    sc = _SCALAR_CODE.get(C.dtype, R_32F)
+    if _call is not None:
+        ws, wsb = (0, 0) if workspace is None else (workspace.data_ptr(), workspace.numel() * workspace.element_size())
+        st = _call.gemm(*key[:6], ws, wsb, *key[6:], sc, _op(transA), _op(transB), m, n, k, A.data_ptr(), _ld(A),
+                        B.data_ptr(), _ld(B), C.data_ptr(), _ld(C), _stream(stream, C.device.index), alpha, beta)
+        if st != SUCCESS:
+            _check(st, "hsmm_gemm")
+        return C
     if workspace is not None:
         cfg = make_config(*key[:6], workspace, *key[6:])
     else:   # no workspace: a config per key, built once (the library only reads it)
         cfg = _CONFIGS.get(key)
         if cfg is None:
             cfg = _CONFIGS[key] = make_config(*key[:6], None, *key[6:])
-    sc = _SCALAR_CODE.get(C.dtype, R_32F)
     al, be = _scalar_cached(alpha, sc), _scalar_cached(beta, sc)
     st = lib().hsmm_gemm(ctypes.byref(cfg), _op(transA), _op(transB), m, n, k, ctypes.byref(al), A.data_ptr(),
                          _ld(A), B.data_ptr(), _ld(B), ctypes.byref(be), C.data_ptr(), _ld(C),
@@ -308,29 +337,40 @@ def matmul(a: torch.Tensor, b: torch.Tensor, out: torch.Tensor | None = None, tr
     """
     if not (a.is_contiguous() and b.is_contiguous()):
         raise ValueError("matmul expects contiguous row-major operands")
-    m = a.shape[1] if trans_a else a.shape[0]
-    n = b.shape[0] if trans_b else b.shape[1]
-    if out is None:
+    sa, sb = a.shape, b.shape
+    ra, ca, rb, cb = sa[0], sa[1], sb[0], sb[1]
+    m = ca if trans_a else ra
+    n = rb if trans_b else cb
+    fresh = out is None
+    if fresh:
         dt = out_dtype or (torch.float32 if a.dtype == torch.bfloat16 else a.dtype)
         out = torch.empty((m, n), dtype=dt, device=a.device)
-    if kw or a.dtype != torch.bfloat16 or b.dtype != torch.bfloat16 or not out.is_contiguous() or \
-            out.shape != (m, n):
+    if kw or a.dtype != torch.bfloat16 or b.dtype != torch.bfloat16 or \
+            not (fresh or (out.is_contiguous() and out.shape == (m, n))):
         # the column-major views: row-major X (r x c) is X^T (c x r) with ld = c
         Bv, Av, Cv = b.t(), a.t(), out.t()
         gemm(Bv, Av, Cv, "T" if trans_b else "N", "T" if trans_a else "N", **kw)
         return out
     # the same call without building the three views (this is the per-step path of the
     # autograd Function): C^T (n x m, ld n) = op(b)^T (n x k, ld b.shape[1]) op(a)^T (k x m, ld a.shape[1])
-    k = a.shape[0] if trans_a else a.shape[1]
-    key = (_TORCH2H[a.dtype], _TORCH2H[b.dtype], _TORCH2H[out.dtype], COMPUTE_DEFAULT, 0, 0, 0, 0, 0)
-    cfg = _CONFIGS.get(key)
-    if cfg is None:
-        cfg = _CONFIGS[key] = make_config(*key[:6], None, *key[6:])
-    one, zero = _scalar_cached(1.0, R_32F), _scalar_cached(0.0, R_32F)
-    st = lib().hsmm_gemm(ctypes.byref(cfg), _T if trans_b else _N, _T if trans_a else _N, n, m, k, ctypes.byref(one),
-                         b.data_ptr(), max(1, b.shape[1]), a.data_ptr(), max(1, a.shape[1]), ctypes.byref(zero),
-                         out.data_ptr(), max(1, n), _stream(None, out.device.index))
-    _check(st, "hsmm_gemm")
+    k = ra if trans_a else ca
+    code = _TORCH2H[out.dtype]
+    L = lib()
+    if _call is not None:
+        st = _call.gemm(R_16BF, R_16BF, code, COMPUTE_DEFAULT, 0, 0, 0, 0, 0, 0, 0, R_32F, _T if trans_b else _N,
+                        _T if trans_a else _N, n, m, k, b.data_ptr(), cb or 1, a.data_ptr(), ca or 1, out.data_ptr(),
+                        n or 1, _stream(None, out.device.index), 1.0, 0.0)
+    else:
+        key = (R_16BF, R_16BF, code, COMPUTE_DEFAULT, 0, 0, 0, 0, 0)
+        cfg = _CONFIGS.get(key)
+        if cfg is None:
+            cfg = _CONFIGS[key] = make_config(*key[:6], None, *key[6:])
+        one, zero = _scalar_cached(1.0, R_32F), _scalar_cached(0.0, R_32F)
+        st = L.hsmm_gemm(ctypes.byref(cfg), _T if trans_b else _N, _T if trans_a else _N, n, m, k, ctypes.byref(one),
+                         b.data_ptr(), cb or 1, a.data_ptr(), ca or 1, ctypes.byref(zero), out.data_ptr(), n or 1,
+                         _stream(None, out.device.index))
+    if st != SUCCESS:
+        _check(st, "hsmm_gemm")
     return out
 
 
@@ -348,14 +388,21 @@ def gemv(A: torch.Tensor, x: torch.Tensor, y: torch.Tensor, trans="N", alpha=1, 
     m, n = A.shape
     a = _TORCH2H[A.dtype]
     c = _TORCH2H[y.dtype]
-    cfg = make_config(a, a, c)
     if workspace is None:
         need = gemv_workspace_size(a, trans, m, n)
         workspace = torch.empty(max(need, 16), dtype=torch.uint8, device=A.device)
+    L = lib()
+    if _call is not None:
+        st = _call.gemv(a, c, workspace.data_ptr(), workspace.numel(), _op(trans), m, n, A.data_ptr(), _ld(A),
+                        x.data_ptr(), incx, y.data_ptr(), incy, _stream(stream), alpha, beta)
+        if st != SUCCESS:
+            _check(st, "hsmm_gemv")
+        return y
+    cfg = make_config(a, a, c)
     cfg.workspace = workspace.data_ptr()
     cfg.workspace_bytes = workspace.numel()
     al, be = _scalar(alpha, c), _scalar(beta, c)
-    st = lib().hsmm_gemv(ctypes.byref(cfg), _op(trans), m, n, ctypes.byref(al), A.data_ptr(), _ld(A), x.data_ptr(),
+    st = L.hsmm_gemv(ctypes.byref(cfg), _op(trans), m, n, ctypes.byref(al), A.data_ptr(), _ld(A), x.data_ptr(),
                          incx, ctypes.byref(be), y.data_ptr(), incy, _stream(stream))
     _check(st, "hsmm_gemv")
     return y
