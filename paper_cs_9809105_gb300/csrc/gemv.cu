@@ -20,9 +20,9 @@
 // column element by element, and op = N reads whole vectors into the padding rows of every column
 // but the last, whose tail it reads element by element (nothing after A(m-1, n-1) is read).
 // Before -> now, us in a row in a CUDA graph (N / T): INT8 2100 x 5300 with padded columns 9.2 / 7.8
-// -> 6.3 / 3.6, FP32 2101 x 5300 unaligned 16.9 / 29.8 -> 11.9 / 10.5, 16384 x 500 13.6 / 29.7 ->
-// 10.0 / 7.4, 1000^2 6.8 / 3.1 -> 3.9 / 2.4, 6654 x 8018 45.5 / 80.2 -> 34.4 / 39.2, 16384^2 150.3 /
-// 166.7 -> 150.0 / 157.5.
+// -> 5.9 / 3.2, FP32 2101 x 5300 unaligned 16.9 / 29.8 -> 11.9 / 10.5, 16384 x 500 13.6 / 29.7 ->
+// 10.0 / 7.4, 1000^2 6.8 / 3.1 -> 3.6 / 2.0, 6654 x 8018 45.5 / 80.2 -> 34.4 / 39.2, 16384^2 150.3 /
+// 166.7 -> 150.1 / 156.9.
 #include <cstdint>
 #include <cuda_runtime.h>
 
@@ -44,6 +44,26 @@ namespace {
 
 constexpr int kThreads = 256;
 
+// Every kernel of this file is launched as a programmatic dependent: its CTAs are placed while the
+// kernel before it drains, wait on the device for its end (pdl_wait, the first instruction, before
+// any access to memory) and only then let the next one be placed.  The only exception is the PLAIN
+// form of op = N, where a wait costs more than the gap it hides (16384 x 16384 FP32: 155.8 us with
+// it, 150.0 without).  Between others the gap is 0.3 to 2.4 us: FP32 1000 x 1000 N 3.96 -> 3.58 us and
+// T 2.40 -> 2.02, INT8 2100 x 5300 N then T 14.35 -> 9.58.
+template <typename... P, typename... Q>
+cudaError_t pdl_launch(void (*kern)(P...), dim3 grid, cudaStream_t st, Q... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(kThreads, 1, 1);
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, P(args)...);
+}
+
 // ---------------------------------------------------------------------------
 // FP32, op = N
 // ---------------------------------------------------------------------------
@@ -57,6 +77,7 @@ __global__ void __launch_bounds__(kThreads) gemv_f32_n_vec(int64_t m, int64_t n,
                                                            int64_t lda, const float* __restrict__ x, int64_t incx,
                                                            float* __restrict__ part, int64_t cols_per_split,
                                                            int rt, int64_t cols_per_group) {
+    if (!PLAIN) pdl_wait();   // see pdl_launch
     pdl_trigger();   // the reduction may be scheduled; it waits for this grid to finish
     if (PLAIN) rt = 8;
     const int tr = int(threadIdx.x) & ((1 << rt) - 1), group = PLAIN ? 0 : int(threadIdx.x) >> rt;
@@ -134,6 +155,7 @@ __global__ void __launch_bounds__(kThreads) gemv_f32_n_scalar(int64_t m, int64_t
                                                               int64_t lda, const float* __restrict__ x,
                                                               int64_t incx, float* __restrict__ part,
                                                               int64_t cols_per_split) {
+    pdl_wait();
     pdl_trigger();   // the reduction may be scheduled; it waits for this grid to finish
     const int64_t r = int64_t(blockIdx.x) * kThreads + threadIdx.x;
     const int64_t j0 = int64_t(blockIdx.y) * cols_per_split;
@@ -160,6 +182,7 @@ template <typename T, typename Acc>
 __global__ void __launch_bounds__(kThreads) gemv_reduce(int64_t m, int nsplit, const T* __restrict__ part, T alpha,
                                                         T beta, T* __restrict__ y, int64_t incy) {
     pdl_wait();
+    pdl_trigger();
     const int r = int(lane_id()), g = int(warp_id());
     const int64_t i = int64_t(blockIdx.x) * 32 + r;
     Acc sum = Acc(0);
@@ -185,20 +208,10 @@ __global__ void __launch_bounds__(kThreads) gemv_reduce(int64_t m, int nsplit, c
     }
 }
 
-// launch the reduction as a programmatic dependent of the kernel just launched on st
 template <typename T, typename Acc>
 cudaError_t launch_reduce(int64_t m, int nsplit, const T* part, T alpha, T beta, T* y, int64_t incy,
                           cudaStream_t st) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(unsigned((m + 31) / 32), 1, 1);
-    cfg.blockDim = dim3(kThreads, 1, 1);
-    cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, gemv_reduce<T, Acc>, m, nsplit, part, alpha, beta, y, incy);
+    return pdl_launch(gemv_reduce<T, Acc>, dim3(unsigned((m + 31) / 32)), st, m, nsplit, part, alpha, beta, y, incy);
 }
 
 // ---------------------------------------------------------------------------
@@ -268,6 +281,8 @@ __device__ __forceinline__ void t_finish(const GemvT& g, S acc, int64_t col, int
 __global__ void __launch_bounds__(kThreads) gemv_f32_t_plain(GemvT g, const float* __restrict__ A,
                                                              const float* __restrict__ x, float alpha, float beta,
                                                              float* __restrict__ y) {
+    pdl_wait();
+    pdl_trigger();
     const int lane = int(lane_id());
     const int64_t col = int64_t(blockIdx.x) * (kThreads / 32) + warp_id();
     if (col >= g.n) return;
@@ -298,6 +313,8 @@ __global__ void __launch_bounds__(kThreads, 5) gemv_t_vec(GemvT g, const T* __re
                                                           S alpha, S beta, S* __restrict__ y) {
     constexpr int E = 16 / int(sizeof(T));                 // elements of a vector
     const int lane = int(lane_id());
+    pdl_wait();
+    pdl_trigger();
     int64_t col, i0, i1;
     int part;
     t_place(g, col, part, i0, i1);
@@ -339,6 +356,8 @@ template <typename T, typename S, bool UNIT>
 __global__ void __launch_bounds__(kThreads) gemv_t_scalar(GemvT g, const T* __restrict__ A, const T* __restrict__ x,
                                                           S alpha, S beta, S* __restrict__ y) {
     const int lane = int(lane_id());
+    pdl_wait();
+    pdl_trigger();
     int64_t col, i0, i1;
     int part;
     t_place(g, col, part, i0, i1);
@@ -364,7 +383,7 @@ __global__ void __launch_bounds__(kThreads) gemv_t_scalar(GemvT g, const T* __re
 
 // One warp per column where that is 16 warps an SM and more, else up to eight for about as many.
 template <typename T, typename V, typename S>
-void launch_t(int64_t m, int64_t n, S alpha, const T* A, int64_t lda, const T* x, int64_t incx, S beta, S* y,
+cudaError_t launch_t(int64_t m, int64_t n, S alpha, const T* A, int64_t lda, const T* x, int64_t incx, S beta, S* y,
               int64_t incy, bool vec, cudaStream_t st) {
     const int64_t want = int64_t(num_sms()) * 16, unit = 32 * (16 / int64_t(sizeof(T)));   // one vector per lane
     GemvT g{m, n, lda, incx, incy, 0, 0};
@@ -374,14 +393,12 @@ void launch_t(int64_t m, int64_t n, S alpha, const T* A, int64_t lda, const T* x
     const int cols = kThreads / 32 >> g.shift;
     const unsigned grid = unsigned((n + cols - 1) / cols);
     if constexpr (sizeof(T) == 4) {
-        if (vec && g.shift == 0 && m % 4 == 0) {
-            gemv_f32_t_plain<<<grid, kThreads, 0, st>>>(g, A, x, alpha, beta, y);
-            return;
-        }
+        if (vec && g.shift == 0 && m % 4 == 0)
+            return pdl_launch(gemv_f32_t_plain, dim3(grid), st, g, A, x, alpha, beta, y);
     }
-    if (vec) gemv_t_vec<T, V, S><<<grid, kThreads, 0, st>>>(g, A, x, alpha, beta, y);
-    else if (incx == 1) gemv_t_scalar<T, S, true><<<grid, kThreads, 0, st>>>(g, A, x, alpha, beta, y);
-    else gemv_t_scalar<T, S, false><<<grid, kThreads, 0, st>>>(g, A, x, alpha, beta, y);
+    if (vec) return pdl_launch(gemv_t_vec<T, V, S>, dim3(grid), st, g, A, x, alpha, beta, y);
+    if (incx == 1) return pdl_launch(gemv_t_scalar<T, S, true>, dim3(grid), st, g, A, x, alpha, beta, y);
+    return pdl_launch(gemv_t_scalar<T, S, false>, dim3(grid), st, g, A, x, alpha, beta, y);
 }
 
 // ---------------------------------------------------------------------------
@@ -413,6 +430,7 @@ __global__ void __launch_bounds__(kThreads) gemv_i8_n_vec(int64_t m, int64_t n, 
                                                           int64_t lda, const int8_t* __restrict__ x, int64_t incx,
                                                           int32_t* __restrict__ part, int64_t cols_per_split,
                                                           int rt, int64_t cols_per_group) {
+    if (!PLAIN) pdl_wait();   // see pdl_launch
     pdl_trigger();   // the reduction may be scheduled; it waits for this grid to finish
     if (PLAIN) rt = 8;                                       // see gemv_f32_n_vec; m % 16 == 0
     const int tr = int(threadIdx.x) & ((1 << rt) - 1), group = PLAIN ? 0 : int(threadIdx.x) >> rt;
@@ -523,6 +541,7 @@ __global__ void __launch_bounds__(kThreads) gemv_i8_n_vec(int64_t m, int64_t n, 
 __global__ void __launch_bounds__(kThreads) gemv_i8_n_scalar(int64_t m, int64_t n, const int8_t* __restrict__ A,
                                                              int64_t lda, const int8_t* __restrict__ x, int64_t incx,
                                                              int32_t* __restrict__ part, int64_t cols_per_split) {
+    pdl_wait();
     pdl_trigger();   // the reduction may be scheduled; it waits for this grid to finish
     const int64_t r = int64_t(blockIdx.x) * kThreads + threadIdx.x;
     const int64_t j0 = int64_t(blockIdx.y) * cols_per_split;
@@ -597,24 +616,26 @@ hsmm_status_t gemv_f32(hsmm_op_t trans, int64_t m, int64_t n, float alpha, const
         const int64_t cps = (n + ns - 1) / ns;
         float* part = static_cast<float*>(ws);
         const bool vec = (lda % 4 == 0) && aligned16(A) && aligned16(ws);
+        cudaError_t e = cudaSuccess;
         if (vec) {
             const NSplit sp = n_split(m, ns, cps, 4);
             if (sp.rt == 8 && m % 4 == 0)
                 gemv_f32_n_vec<true><<<sp.grid, kThreads, 0, st>>>(m, n, A, lda, x, incx, part, cps, 8, cps);
             else
-                gemv_f32_n_vec<false><<<sp.grid, kThreads, 0, st>>>(m, n, A, lda, x, incx, part, cps, sp.rt,
-                                                                  sp.cols_per_group);
+                e = pdl_launch(gemv_f32_n_vec<false>, sp.grid, st, m, n, A, lda, x, incx, part, cps, sp.rt,
+                               sp.cols_per_group);
         } else {
             dim3 grid(unsigned((m + kThreads - 1) / kThreads), unsigned(ns));
-            gemv_f32_n_scalar<<<grid, kThreads, 0, st>>>(m, n, A, lda, x, incx, part, cps);
+            e = pdl_launch(gemv_f32_n_scalar, grid, st, m, n, A, lda, x, incx, part, cps);
         }
-        const cudaError_t e = launch_reduce<float, float>(m, ns, part, alpha, beta, y, incy, st);
+        if (e == cudaSuccess) e = launch_reduce<float, float>(m, ns, part, alpha, beta, y, incy, st);
         count_launches(2);
         if (e != cudaSuccess) return record_cuda(e);
     } else {
         const bool vec = (lda % 4 == 0) && aligned16(A) && aligned16(x) && incx == 1;
-        launch_t<float, float4, float>(m, n, alpha, A, lda, x, incx, beta, y, incy, vec, st);
+        const cudaError_t e = launch_t<float, float4, float>(m, n, alpha, A, lda, x, incx, beta, y, incy, vec, st);
         count_launches(1);
+        if (e != cudaSuccess) return record_cuda(e);
     }
     return check_launch();
 }
@@ -628,24 +649,26 @@ hsmm_status_t gemv_i8(hsmm_op_t trans, int64_t m, int64_t n, int32_t alpha, cons
         const int64_t cps = (n + ns - 1) / ns;
         int32_t* part = static_cast<int32_t*>(ws);
         const bool vec = (lda % 16 == 0) && aligned16(A) && aligned16(ws);
+        cudaError_t e = cudaSuccess;
         if (vec) {
             const NSplit sp = n_split(m, ns, cps, 16);
             if (sp.rt == 8 && m % 16 == 0)
                 gemv_i8_n_vec<true><<<sp.grid, kThreads, 0, st>>>(m, n, A, lda, x, incx, part, cps, 8, cps);
             else
-                gemv_i8_n_vec<false><<<sp.grid, kThreads, 0, st>>>(m, n, A, lda, x, incx, part, cps, sp.rt,
-                                                                  sp.cols_per_group);
+                e = pdl_launch(gemv_i8_n_vec<false>, sp.grid, st, m, n, A, lda, x, incx, part, cps, sp.rt,
+                               sp.cols_per_group);
         } else {
             dim3 grid(unsigned((m + kThreads - 1) / kThreads), unsigned(ns));
-            gemv_i8_n_scalar<<<grid, kThreads, 0, st>>>(m, n, A, lda, x, incx, part, cps);
+            e = pdl_launch(gemv_i8_n_scalar, grid, st, m, n, A, lda, x, incx, part, cps);
         }
-        const cudaError_t e = launch_reduce<int32_t, uint32_t>(m, ns, part, alpha, beta, y, incy, st);
+        if (e == cudaSuccess) e = launch_reduce<int32_t, uint32_t>(m, ns, part, alpha, beta, y, incy, st);
         count_launches(2);
         if (e != cudaSuccess) return record_cuda(e);
     } else {
         const bool vec = (lda % 16 == 0) && aligned16(A) && aligned16(x) && incx == 1;
-        launch_t<int8_t, int4, int>(m, n, alpha, A, lda, x, incx, beta, y, incy, vec, st);
+        const cudaError_t e = launch_t<int8_t, int4, int>(m, n, alpha, A, lda, x, incx, beta, y, incy, vec, st);
         count_launches(1);
+        if (e != cudaSuccess) return record_cuda(e);
     }
     return check_launch();
 }
