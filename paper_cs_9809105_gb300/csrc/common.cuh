@@ -123,6 +123,24 @@ __device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, u
     }
 }
 
+// Named barriers of some of a CTA's warps (ids 1..15; 0 is __syncthreads), and one that also tells
+// every thread whether `ok` holds in all of them.
+__device__ __forceinline__ void named_barrier(int id, int threads) {
+    asm volatile("barrier.cta.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+__device__ __forceinline__ bool named_barrier_all(int id, int threads, bool ok) {
+    uint32_t all;
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t"
+        "setp.ne.b32 p, %3, 0;\n\t"
+        "barrier.cta.red.and.pred q, %1, %2, p;\n\t"
+        "selp.u32 %0, 1, 0, q;\n\t}"
+        : "=r"(all)
+        : "r"(id), "r"(threads), "r"(uint32_t(ok))
+        : "memory");
+    return all != 0;
+}
+
 // ---------------------------------------------------------------------------
 // TMA (cp.async.bulk.tensor), tensor maps passed as __grid_constant__ params
 // or kept in global memory
@@ -174,6 +192,9 @@ __device__ __forceinline__ void tma_load_3d_if(uint32_t issue, void* dst, const 
         ::"r"(smem_u32(dst)), "l"(map), "r"(smem_u32(bar)), "r"(c0), "r"(c1), "r"(c2), "r"(issue)
         : "memory");
 }
+
+// bring the sector of p into L2
+__device__ __forceinline__ void l2_prefetch(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p) : "memory"); }
 
 // TMA store of a shared-memory box to global memory (bulk async-group of the issuing thread)
 __device__ __forceinline__ void tma_store_2d(const void* map, const void* src, int32_t c0, int32_t c1) {

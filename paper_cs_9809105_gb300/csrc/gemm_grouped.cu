@@ -72,9 +72,10 @@ struct GroupedArgs {
 };
 
 // Flattened tile record (16 bytes, one load): x problem, y tile row | tile column << 16,
-// z k-blocks, w tile width / 128 (bits 0-1) | A MN-major (2) | B MN-major (3) | C by TMA
-// stores (4) | valid rows (8-16, 1..256) | valid columns (17-25, 1..256).  A tile row is
-// 128 rows for the one-CTA kernel and 256 for the CTA-pair kernel.
+// z k-blocks, w columns of C begin or end inside a 32-byte sector and k is short (0) | A MN-major
+// (2) | B MN-major (3) | C by TMA stores (4) | valid rows (8-16, 1..256) | valid columns (17-25,
+// 1..256) | tile width / 32 - 1 (26-28).  A tile row is 128 rows for the one-CTA kernel and 256 for
+// the CTA-pair kernel.
 __device__ __forceinline__ int rec_bn(const uint4& r) { return int((r.w >> 26) & 7u) * 32 + 32; }
 
 // A TMA store clips the row (inner) dimension of C only to whole 16-byte units, so a grouped
@@ -99,6 +100,7 @@ __device__ __forceinline__ void store_tail_row(const TailC& T, int64_t row, int6
     }
 }
 __host__ __device__ constexpr int c_rows_unit(bool out_bf16) { return out_bf16 ? 8 : 4; }   // rows per 16-byte unit of C
+__device__ __forceinline__ bool rec_edges(const uint4& r) { return r.w & 1u; }
 __device__ __forceinline__ bool rec_amn(const uint4& r) { return (r.w >> 2) & 1u; }
 __device__ __forceinline__ bool rec_bmn(const uint4& r) { return (r.w >> 3) & 1u; }
 __device__ __forceinline__ bool rec_ctma(const uint4& r) { return (r.w >> 4) & 1u; }
@@ -353,28 +355,32 @@ __global__ void __launch_bounds__(kNumThreads, 1) gemm_grouped_kernel(GroupedArg
 // halves, and the even CTA issues M = 256, N = BN_p MMAs that write each CTA's 128 rows
 // into its own TMEM.  Per tile and SM that stages (128 + BN_p/2) instead of 128 + BN_p
 // rows of operands per k-block: the one-CTA kernel is bound by the bytes its SMs can
-// stage, not by the MMAs.  Six 32 KiB stages leave room for the C staging buffers
-// (eight epilogue warps with one 4 KiB buffer each).
-#ifndef GP_STAGES_CFG
-#define GP_STAGES_CFG 6
-#define GP_EPI_CFG 8
-#define GP_CBUF_CFG 1
-#define GP_PRODUCERS_CFG 2
-#endif
-constexpr int GP_STAGES = GP_STAGES_CFG;
-constexpr int GP_EPI_WARPS = GP_EPI_CFG;                   // 4, 8 or 16: 1, 2 or 4 per TMEM lane quarter
-constexpr int GP_EPI_PARTS = GP_EPI_WARPS / 4;              // column parts of a tile, one per warp of a quarter
-constexpr int GP_CBUF = GP_CBUF_CFG;
-constexpr int GP_PRODUCERS = GP_PRODUCERS_CFG;             // warps 0 and (with two) 2
-constexpr int GP_THREADS = 96 + 32 * GP_EPI_WARPS;         // producer, MMA issuer, producer or idle, epilogue
-constexpr int GP_STAGE_C = GP_EPI_WARPS * GP_CBUF * 32 * 32 * 4;  // 32 x 32 FP32 staging buffers per epilogue warp
-constexpr int GP_SMEM = GP_STAGES * PAIR_STAGE_BYTES + GP_STAGE_C + 1024 + 256;
-static_assert(GP_SMEM <= 227 * 1024, "grouped pair kernel shared memory");
-// The two producers take alternate k-blocks, so with an even stage count each stage always
-// belongs to the same producer; with an odd one both would refill it, and a producer's final
-// wait for its last use of a stage could name a phase that has already been passed twice.
-static_assert(GP_PRODUCERS == 1 || GP_STAGES % 2 == 0, "grouped pair kernel: two producers need an even number of stages");
-static_assert(GP_EPI_WARPS == 4 || GP_EPI_WARPS == 8 || GP_EPI_WARPS == 16, "grouped pair kernel: epilogue warps");
+// stage, not by the MMAs.
+//
+// C leaves in one of two ways (grouped_tall decides which, from both sides measured):
+// * TALL: blocks of the CTA's 128 rows x 32 columns; the four epilogue warps of a column half fill a
+//   block together and one thread stores it.  Two 16 KiB blocks per half leave five 32 KiB stages.
+// * otherwise one 32 x 32 block per warp, and six stages.
+// Where C's columns start inside a 32-byte sector (leading dimension or base an odd multiple of 16
+// bytes), a block begins and ends with part of a sector, and a part written to a sector that L2 does
+// not hold is dear: tall blocks have a quarter of them.  What parts are left (edges of 128 rows, ends
+// of columns) are fetched into L2 ahead of the tile's stores where the stores bound the launch
+// (rec_edges).  Us, 32 x 32 blocks -> tall -> with the edges fetched: 17 products 2048 x 2048 x 64,
+// FP32 C with ldc 2052, 83.2 -> 73.7 -> 62.1; 295 of 508 x 500 x 64, ldc 508, 88.8 -> 76.8 -> 68.8;
+// k = 256: 102.5 -> 91.9 -> 86.5; k = 384: 111.0 -> 100.6 -> 98.4; k = 512: 111.4 -> 107.1 -> 108.7.
+constexpr int GP_EPI_WARPS = 8;                            // two per TMEM lane quarter
+constexpr int GP_EPI_PARTS = GP_EPI_WARPS / 4;             // column parts of a tile, four warps each
+constexpr int GP_THREADS = 96 + 32 * GP_EPI_WARPS;         // producer, MMA issuer, producer, epilogue
+constexpr int GP_EDGE_KB = 6;                              // k-blocks up to which the edges are fetched
+template <bool TALL>
+struct GroupedPairCfg {
+    static constexpr int STAGES = TALL ? 5 : 6;
+    static constexpr int CBUF = 2;                          // TALL: blocks staged per part
+    static constexpr int CBLOCK = TALL ? BM * 32 * 4 : 32 * 32 * 4;   // bytes; TALL: 32 FP32 or 64 BF16 columns
+    static constexpr int STAGE_C = TALL ? GP_EPI_PARTS * CBUF * CBLOCK : GP_EPI_WARPS * CBLOCK;
+    static constexpr int SMEM = STAGES * PAIR_STAGE_BYTES + STAGE_C + 1024 + 256;
+    static_assert(SMEM <= 227 * 1024, "grouped pair kernel shared memory");
+};
 
 // Tile records are read two tiles ahead, so that no role waits on a global load at a tile
 // boundary (the producer needs the next record at once, to prefetch its descriptors).
@@ -385,14 +391,22 @@ __device__ __forceinline__ uint4 rec_at(const GroupedArgs& g, int64_t t, const u
     return t < g.total_tiles ? g.tiles[t] : fallback;
 }
 
-template <bool TF32, bool OUT_BF16>
+// the same record as a value the compiler can keep in uniform registers
+__device__ __forceinline__ uint4 rec_uniform(const uint4& r) {
+    return make_uint4(__shfl_sync(0xffffffffu, r.x, 0), __shfl_sync(0xffffffffu, r.y, 0),
+                      __shfl_sync(0xffffffffu, r.z, 0), __shfl_sync(0xffffffffu, r.w, 0));
+}
+
+template <bool TF32, bool OUT_BF16, bool TALL>
 __global__ void __launch_bounds__(GP_THREADS, 1) gemm_grouped_pair_kernel(GroupedArgs g) {
     using C_ = Cfg<256, TF32>;
+    using P_ = GroupedPairCfg<TALL>;
+    constexpr int GP_STAGES = P_::STAGES, GP_CBLOCK = P_::CBLOCK;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = align1024(smem_raw);
     uint8_t* stage_c = smem + GP_STAGES * PAIR_STAGE_BYTES;
-    Bars* bars = reinterpret_cast<Bars*>(stage_c + GP_STAGE_C);
-    const int warp = int(warp_id()), lane = int(lane_id());
+    Bars* bars = reinterpret_cast<Bars*>(stage_c + P_::STAGE_C);
+    const int warp = warp_id_uniform(), lane = int(lane_id());
     uint32_t* status = &g_status_grouped;
     const uint32_t rank = cluster_ctarank() & 1u;
     const bool leader = (rank == 0);
@@ -421,71 +435,78 @@ __global__ void __launch_bounds__(GP_THREADS, 1) gemm_grouped_pair_kernel(Groupe
     volatile int* abort = &bars->abort;
     const int64_t pair = int64_t(blockIdx.x >> 1), npairs = int64_t(gridDim.x >> 1);
 
-    if (warp == 0 || (warp == 2 && GP_PRODUCERS == 2)) {
-        // two producers (warps 0 and 2), each for every other k-block of the CTA's stream: the
-        // TMA loads of a grouped launch name descriptors in global memory, and one issuing
-        // thread cannot keep the MMAs fed with them
-        if (lane == 0) {
-            const int pid = warp == 0 ? 0 : 1;
-            int64_t gk = 0;                  // k-blocks of this CTA so far (both producers count all)
-            int last_parity[8];
-            for (int i = 0; i < 8; ++i) last_parity[i] = -1;
-            bool ok = true;
-            RecPipe rp;
-            rp.cur = g.tiles[pair];
-            rp.next = rec_at(g, pair + npairs, rp.cur);
-            for (int64_t t = pair; t < g.total_tiles && ok && !*abort; t += npairs) {
-                const int64_t tnext = t + npairs;
-                rp.next2 = rec_at(g, tnext + npairs, rp.next);
-                const uint4 rec = rp.cur, rec_next = rp.next;
-                const int pi = int(rec.x);
-                const int tm = int(rec.y & 0xFFFFu), tn = int(rec.y >> 16);
-                const int bn = rec_bn(rec), nkb = int(rec.z);
-                const bool a_mn = rec_amn(rec), b_mn = rec_bmn(rec);
-                const CUtensorMap* mA = g.maps + 3 * pi;
-                const CUtensorMap* mB = mA + 1;
-                if (tnext < g.total_tiles && rec_next.x != rec.x) {
-                    tma_prefetch_desc(g.maps + 3 * rec_next.x);
-                    tma_prefetch_desc(g.maps + 3 * rec_next.x + 1);
-                }
-                const int arow = tm * 2 * BM + int(rank) * BM;
-                const int bhalf = bn / 2;
-                const int brow = tn * bn + int(rank) * bhalf;
-                const uint32_t bytes = 2u * uint32_t(BM + bhalf) * 128u;   // both CTAs' copies
-                for (int kb = 0; kb < nkb; ++kb, ++gk) {
-                    if (GP_PRODUCERS == 2 && int(gk & 1) != pid) continue;
-                    const int stage = int(gk % GP_STAGES);
-                    const uint32_t phase = uint32_t((gk / GP_STAGES) & 1);
-                    if (!mbar_wait(&bars->empty[stage], phase ^ 1u, g.timeout_ns, status, abort)) { ok = false; break; }
-                    uint8_t* a_dst = smem + stage * PAIR_STAGE_BYTES;
-                    uint8_t* b_dst = a_dst + BM * 128;
-                    const uint32_t full_leader = mapa_shared(smem_u32(&bars->full[stage]), 0);
-                    if (leader) mbar_arrive_expect_tx(&bars->full[stage], bytes);
-                    if (!a_mn) {
-                        tma_load_2d_pair(a_dst, mA, full_leader, kb * C_::BK, arow);
-                    } else {
-                        for (int c = 0; c < BM / C_::MN_CHUNK; ++c)
-                            tma_load_2d_pair(a_dst + c * C_::BK * 128, mA, full_leader, arow + c * C_::MN_CHUNK,
-                                             kb * C_::BK);
-                    }
-                    if (!b_mn) {
-                        tma_load_2d_pair(b_dst, mB, full_leader, kb * C_::BK, brow);
-                    } else {
-                        for (int c = 0; c < bhalf / C_::MN_CHUNK; ++c)
-                            tma_load_2d_pair(b_dst + c * C_::BK * 128, mB, full_leader, brow + c * C_::MN_CHUNK,
-                                             kb * C_::BK);
-                    }
-                    last_parity[stage] = int(phase);
-                }
-                rp.cur = rp.next;
-                rp.next = rp.next2;
+    if (warp == 0 || warp == 2) {
+        // two producers (warps 0 and 2), each for every other k-block of the CTA's stream: the TMA
+        // loads of a grouped launch name descriptors in global memory, and one issuing warp cannot
+        // keep the MMAs fed with them where k is short
+        const bool issue = elect_one();
+        const int pid = warp == 0 ? 0 : 1;
+        int total = 0;                       // k-blocks of the tiles so far, both producers'
+        int stage = pid;                     // stage and phase of this producer's next k-block
+        uint32_t phase = 0;
+        bool ok = true;
+        const uint32_t full0 = mapa_shared(smem_u32(&bars->full[0]), 0);
+        RecPipe rp;
+        rp.cur = g.tiles[pair];
+        rp.next = rec_at(g, pair + npairs, rp.cur);
+        for (int64_t t = pair; t < g.total_tiles && ok && !*abort; t += npairs) {
+            const int64_t tnext = t + npairs;
+            rp.next2 = rec_at(g, tnext + npairs, rp.next);
+            const uint4 rec = rec_uniform(rp.cur);
+            const int tm = int(rec.y & 0xFFFFu), tn = int(rec.y >> 16);
+            const int bn = rec_bn(rec), nkb = int(rec.z);
+            const bool a_mn = rec_amn(rec), b_mn = rec_bmn(rec);
+            const CUtensorMap* mA = g.maps + 3 * rec.x;
+            const CUtensorMap* mB = mA + 1;
+            if (issue && tnext < g.total_tiles && rp.next.x != rec.x) {
+                tma_prefetch_desc(g.maps + 3 * rp.next.x);
+                tma_prefetch_desc(g.maps + 3 * rp.next.x + 1);
             }
-            // the leader's MMAs read both CTAs' stages: a stage is free only once they completed
-            for (int i = 0; i < GP_STAGES; ++i)
-                if (last_parity[i] >= 0) mbar_wait(&bars->empty[i], uint32_t(last_parity[i]), g.timeout_ns, status, abort);
+            __syncwarp();
+            const int arow = tm * 2 * BM + int(rank) * BM;
+            const int bhalf = bn / 2;
+            const int brow = tn * bn + int(rank) * bhalf;
+            const uint32_t bytes = 2u * uint32_t(BM + bhalf) * 128u;   // both CTAs' copies
+            for (int kb = (total ^ pid) & 1; kb < nkb; kb += 2) {
+                // The first round of stages starts empty.  With an odd number of stages the block
+                // before this one in its stage is the other producer's, but the one two before it
+                // has been consumed (this producer's last wait was for a later block), so the
+                // parity cannot be mistaken.
+                if (total + kb >= GP_STAGES &&
+                    !mbar_wait_warp(&bars->empty[stage], phase ^ 1u, g.timeout_ns, status, abort)) { ok = false; break; }
+                uint8_t* a_dst = smem + stage * PAIR_STAGE_BYTES;
+                uint8_t* b_dst = a_dst + BM * 128;
+                const uint32_t full_leader = full0 + uint32_t(stage) * 8u;
+                mbar_arrive_expect_tx_if(issue && leader, &bars->full[stage], bytes);
+                if (!a_mn) {
+                    tma_load_2d_pair_if(issue, a_dst, mA, full_leader, kb * C_::BK, arow);
+                } else {
+#pragma unroll
+                    for (int c = 0; c < BM / C_::MN_CHUNK; ++c)
+                        tma_load_2d_pair_if(issue, a_dst + c * C_::BK * 128, mA, full_leader, arow + c * C_::MN_CHUNK,
+                                            kb * C_::BK);
+                }
+                if (!b_mn) {
+                    tma_load_2d_pair_if(issue, b_dst, mB, full_leader, kb * C_::BK, brow);
+                } else {
+                    for (int c = 0; c < bhalf / C_::MN_CHUNK; ++c)
+                        tma_load_2d_pair_if(issue, b_dst + c * C_::BK * 128, mB, full_leader, brow + c * C_::MN_CHUNK,
+                                            kb * C_::BK);
+                }
+                stage += 2;
+                if (stage >= GP_STAGES) { stage -= GP_STAGES; phase ^= 1u; }
+            }
+            total += nkb;
+            rp.cur = rp.next;
+            rp.next = rp.next2;
         }
+        // the leader's MMAs read both CTAs' stages: a stage is free only once they completed
+        // (one warp waits for the last round, in order)
+        for (int f = max(0, total - GP_STAGES); pid == 0 && f < total; ++f)
+            mbar_wait_warp(&bars->empty[f % GP_STAGES], uint32_t(f / GP_STAGES) & 1u, g.timeout_ns, status, abort);
     } else if (warp == 1) {
-        if (lane == 0 && leader) {
+        if (leader) {
+            const bool issue = elect_one();
             int stage = 0;
             uint32_t phase = 0;
             int abuf = 0;
@@ -497,10 +518,10 @@ __global__ void __launch_bounds__(GP_THREADS, 1) gemm_grouped_pair_kernel(Groupe
             rp.next = rec_at(g, pair + npairs, rp.cur);
             for (int64_t t = pair; t < g.total_tiles && ok && !*abort; t += npairs) {
                 rp.next2 = rec_at(g, t + 2 * npairs, rp.next);
-                const uint4 rec = rp.cur;
+                const uint4 rec = rec_uniform(rp.cur);
                 const int nkb = int(rec.z), bn = rec_bn(rec);
                 const bool a_mn = rec_amn(rec), b_mn = rec_bmn(rec);
-                if (!mbar_wait(&bars->acc_empty[abuf], aphase ^ 1u, g.timeout_ns, status, abort)) break;
+                if (!mbar_wait_warp(&bars->acc_empty[abuf], aphase ^ 1u, g.timeout_ns, status, abort)) break;
                 tc_fence_after();
                 const uint32_t d_tmem = tmem + uint32_t(abuf * 256);
                 const uint32_t idesc = make_idesc(TF32 ? 2u : 1u, a_mn, b_mn, 2 * BM, uint32_t(bn));
@@ -509,37 +530,34 @@ __global__ void __launch_bounds__(GP_THREADS, 1) gemm_grouped_pair_kernel(Groupe
                 const uint64_t aks = ks_step<C_>(a_mn), bks = ks_step<C_>(b_mn);
 #pragma unroll 4
                 for (int kb = 0; kb < nkb; ++kb) {
-                    if (!mbar_wait(&bars->full[stage], phase, g.timeout_ns, status, abort)) { ok = false; break; }
+                    if (!mbar_wait_warp(&bars->full[stage], phase, g.timeout_ns, status, abort)) { ok = false; break; }
                     tc_fence_after();
                     const uint64_t ad = a0 + uint64_t(stage) * sstep, bd = b0 + uint64_t(stage) * sstep;
 #pragma unroll
-                    for (int ks = 0; ks < C_::KSTEPS; ++ks) {
-                        const uint32_t acc = ks == 0 ? uint32_t(kb) : 1u;
-                        if (TF32)
-                            umma_tf32_pair(d_tmem, ad + ks * aks, bd + ks * bks, idesc, acc);
-                        else
-                            umma_f16_pair(d_tmem, ad + ks * aks, bd + ks * bks, idesc, acc);
-                    }
-                    umma_commit_pair(&bars->empty[stage], 0x3);
+                    for (int ks = 0; ks < C_::KSTEPS; ++ks)
+                        umma_pair_if<TF32>(issue, d_tmem, ad + ks * aks, bd + ks * bks, idesc,
+                                           ks == 0 ? uint32_t(kb) : 1u);
+                    umma_commit_pair_if(issue, &bars->empty[stage], 0x3);
                     stage = (stage + 1 == GP_STAGES) ? 0 : stage + 1;
                     phase ^= (stage == 0) ? 1u : 0u;
                 }
                 if (!ok) break;
-                umma_commit_pair(&bars->acc_full[abuf], 0x3);
+                umma_commit_pair_if(issue, &bars->acc_full[abuf], 0x3);
                 abuf ^= 1;
                 if (abuf == 0) aphase ^= 1u;
                 rp.cur = rp.next;
                 rp.next = rp.next2;
             }
-            umma_commit_pair(&bars->mma_done, 0x1);
-            mbar_wait(&bars->mma_done, 0, g.timeout_ns, status, abort);
+            umma_commit_pair_if(issue, &bars->mma_done, 0x1);
+            mbar_wait_warp(&bars->mma_done, 0, g.timeout_ns, status, abort);
         }
     } else if (warp >= 3) {
         // epilogue: warp w reads TMEM lanes 32*(w%4) .. of this CTA's 128 rows of the tile and
         // the column part (w-3)/4 of them
         const int q = warp & 3;
         const int part = (warp - 3) >> 2;
-        float* stage_w = reinterpret_cast<float*>(stage_c) + (warp - 3) * GP_CBUF * 32 * 32;
+        const bool storer = (warp - 3) % 4 == 0 && lane == 0;   // issues the stores of its part
+        uint8_t* stage_w = stage_c + (TALL ? part * P_::CBUF : warp - 3) * GP_CBLOCK;
         const uint32_t acc_empty_leader0 = mapa_shared(smem_u32(&bars->acc_empty[0]), 0);
         const uint32_t acc_empty_leader1 = mapa_shared(smem_u32(&bars->acc_empty[1]), 0);
         int abuf = 0;
@@ -552,9 +570,22 @@ __global__ void __launch_bounds__(GP_THREADS, 1) gemm_grouped_pair_kernel(Groupe
             const int64_t tnext = t + npairs;
             rp.next2 = rec_at(g, tnext + npairs, rp.next);
             const uint4 rec = rp.cur, rec_next = rp.next;
+            if (rec_edges(rec) && g.beta == 0.f && (warp - 3) * 32 + lane < rec_cols(rec)) {
+                // one column per thread: its first and last sector of the CTA's rows, if only partly written
+                const GroupedProblem& P = g.probs[rec.x];
+                constexpr int esz = OUT_BF16 ? 2 : 4;
+                const int64_t col = int64_t(rec.y >> 16) * rec_bn(rec) + (warp - 3) * 32 + lane;
+                const int64_t r0 = int64_t(rec.y & 0xFFFFu) * 2 * BM + int(rank) * BM, r1 = min(int64_t(P.M), r0 + BM);
+                const char* c = static_cast<const char*>(P.C) + (col * P.ldc + r0) * esz;
+                const char* e = c + (r1 - r0) * esz;
+                if (r0 < r1 && (reinterpret_cast<uintptr_t>(c) & 31)) l2_prefetch(c);
+                if (r0 < r1 && (reinterpret_cast<uintptr_t>(e) & 31)) l2_prefetch(e - 1);
+            }
             int done = 0;
             if (lane == 0) done = mbar_wait(&bars->acc_full[abuf], aphase, g.timeout_ns, status, abort) ? 1 : 0;
             done = __shfl_sync(0xffffffffu, done, 0);
+            // the four warps of a part share its tall blocks: they go on, or give up, together
+            if (TALL) done = named_barrier_all(1 + part, 128, done != 0);
             if (!done) break;
             tc_fence_after();
             const int tm = int(rec.y & 0xFFFFu), tn = int(rec.y >> 16);
@@ -567,7 +598,7 @@ __global__ void __launch_bounds__(GP_THREADS, 1) gemm_grouped_pair_kernel(Groupe
             const int cbeg = min(bn, part * pcut), cend = part + 1 == GP_EPI_PARTS ? bn : min(bn, (part + 1) * pcut);
             const bool c_tma = rec_ctma(rec) && g.beta == 0.f;
             const int rows = rec_rows(rec);
-            if (c_tma && row_base < rows) {
+            if (c_tma && (TALL ? int(rank) * BM : row_base) < rows) {
                 const int cols = min(rec_cols(rec), cend);
                 const CUtensorMap* mC = g.maps + 3 * rec.x + 2;
                 const int rows_tma = rows & ~(c_rows_unit(OUT_BF16) - 1);
@@ -577,38 +608,79 @@ __global__ void __launch_bounds__(GP_THREADS, 1) gemm_grouped_pair_kernel(Groupe
                     const GroupedProblem& P = g.probs[rec.x];
                     tc_ = TailC{P.C, P.ldc, P.N};
                 }
+                if constexpr (TALL) {
+                    constexpr int step = OUT_BF16 ? 64 : 32;     // columns of a staged block
+                    static_assert(step * BM * (OUT_BF16 ? 2 : 4) <= GP_CBLOCK, "a staged block holds its columns");
+                    const bool store = int(rank) * BM < rows_tma;
 #pragma unroll 1
-                for (int c0 = cbeg; c0 < cols; c0 += 32) {
-                    uint32_t r[32];
-                    tmem_ld32(t_base + uint32_t(c0), r);
-                    tmem_ld_wait();
-                    if (row_base < rows_tma) {
-                        float* sb = stage_w + (cbuf % GP_CBUF) * 32 * 32;
-                        if (lane == 0) {    // the store that last used this buffer has read it
-                            if (GP_CBUF == 2) bulk_wait_group_read<1>();
-                            else bulk_wait_group_read<0>();
-                        }
-                        __syncwarp();
-                        if (OUT_BF16) {
-                            __nv_bfloat16* sh = reinterpret_cast<__nv_bfloat16*>(sb);
+                    for (int c0 = cbeg; c0 < cols; c0 += step) {
+                        uint8_t* sb = stage_w + (cbuf % P_::CBUF) * GP_CBLOCK;
+                        uint32_t acc[step / 32][32];
 #pragma unroll
-                            for (int j = 0; j < 32; ++j)
-                                sh[j * 32 + lane] = __float2bfloat16_rn(g.alpha * __uint_as_float(r[j]));
-                        } else {
+                        for (int s = 0; s < step; s += 32)
+                            if (c0 + s < cols) tmem_ld32(t_base + uint32_t(c0 + s), acc[s / 32]);
+                        tmem_ld_wait();
 #pragma unroll
-                            for (int j = 0; j < 32; ++j) sb[j * 32 + lane] = g.alpha * __uint_as_float(r[j]);
+                        for (int s = 0; s < step; s += 32) {
+                            if (c0 + s >= cols) break;
+                            const uint32_t(&r)[32] = acc[s / 32];
+                            if (OUT_BF16) {
+                                __nv_bfloat16* sh = reinterpret_cast<__nv_bfloat16*>(sb) + s * BM + q * 32 + lane;
+#pragma unroll
+                                for (int j = 0; j < 32; ++j) sh[j * BM] = __float2bfloat16_rn(g.alpha * __uint_as_float(r[j]));
+                            } else {
+                                float* sh = reinterpret_cast<float*>(sb) + q * 32 + lane;
+#pragma unroll
+                                for (int j = 0; j < 32; ++j) sh[j * BM] = g.alpha * __uint_as_float(r[j]);
+                            }
+                            if (tail_lane)
+                                store_tail_row<OUT_BF16>(tc_, int64_t(tm) * 2 * BM + row_base + lane,
+                                                         int64_t(tn) * bn + c0 + s, r, g.alpha);
                         }
+                        if (!store) continue;
                         fence_proxy_async_smem();
-                        __syncwarp();
-                        if (lane == 0) {
-                            tma_store_2d(mC, sb, tm * 2 * BM + row_base, tn * bn + c0);
+                        // after the barrier the other block may be filled again: its store has read it
+                        if (storer) bulk_wait_group_read<0>();
+                        named_barrier(1 + part, 128);
+                        if (storer) {
+#pragma unroll
+                            for (int s = 0; s < step; s += 32)
+                                if (c0 + s < cols)
+                                    tma_store_2d(mC, sb + s * BM * 2, tm * 2 * BM + int(rank) * BM, tn * bn + c0 + s);
                             bulk_commit_group();
                         }
                         ++cbuf;
                     }
-                    if (tail_lane)
-                        store_tail_row<OUT_BF16>(tc_, int64_t(tm) * 2 * BM + row_base + lane, int64_t(tn) * bn + c0, r,
-                                                 g.alpha);
+                } else {
+#pragma unroll 1
+                    for (int c0 = cbeg; c0 < cols; c0 += 32) {
+                        uint32_t r[32];
+                        tmem_ld32(t_base + uint32_t(c0), r);
+                        tmem_ld_wait();
+                        if (row_base < rows_tma) {
+                            if (lane == 0) bulk_wait_group_read<0>();   // the last store has read this block
+                            __syncwarp();
+                            if (OUT_BF16) {
+                                __nv_bfloat16* sh = reinterpret_cast<__nv_bfloat16*>(stage_w);
+#pragma unroll
+                                for (int j = 0; j < 32; ++j)
+                                    sh[j * 32 + lane] = __float2bfloat16_rn(g.alpha * __uint_as_float(r[j]));
+                            } else {
+                                float* sh = reinterpret_cast<float*>(stage_w);
+#pragma unroll
+                                for (int j = 0; j < 32; ++j) sh[j * 32 + lane] = g.alpha * __uint_as_float(r[j]);
+                            }
+                            fence_proxy_async_smem();
+                            __syncwarp();
+                            if (lane == 0) {
+                                tma_store_2d(mC, stage_w, tm * 2 * BM + row_base, tn * bn + c0);
+                                bulk_commit_group();
+                            }
+                        }
+                        if (tail_lane)
+                            store_tail_row<OUT_BF16>(tc_, int64_t(tm) * 2 * BM + row_base + lane, int64_t(tn) * bn + c0, r,
+                                                     g.alpha);
+                    }
                 }
             } else if (!c_tma) {
                 const GroupedProblem P = g.probs[rec.x];
@@ -671,6 +743,7 @@ __global__ void __launch_bounds__(GP_THREADS, 1) gemm_grouped_pair_kernel(Groupe
 struct GroupedImage {
     bool tf32 = false, out_bf16 = false;
     bool pairs = true;                   // 256-row tiles on CTA pairs, else 128-row tiles on one CTA
+    bool tall = true;                    // CTA pairs: C in blocks of 128 rows (grouped_tall)
     int count = 0;                       // problems with work
     int64_t total_tiles = 0;
     std::vector<int> bn_per_problem;     // in the caller's order
@@ -706,6 +779,23 @@ static bool grouped_pairs_enabled() {
     return !(v && std::strcmp(v, "single") == 0);
 }
 
+// Whether C leaves by tall blocks (GroupedPairCfg): yes unless more than half of it, in elements, is
+// in problems whose columns begin and end with whole 32-byte sectors.  Us, tall / 32 x 32: the 512
+// mixed products (one in eight such) 298 / 303, with sector-aligned columns but ragged rows 281 / 285;
+// with rows in multiples of 8 274 / 267, of 32 263 / 255; equal products on sectors 0.95 to 1.04 times.
+static bool whole_sectors(const hsmm_gemm_desc_t& d, int esc) {
+    return reinterpret_cast<uintptr_t>(d.C) % 32 == 0 && d.ldc * esc % 32 == 0 && d.m * esc % 32 == 0;
+}
+static bool grouped_tall(const std::vector<int64_t>& order, const hsmm_gemm_desc_t* descs, int esc) {
+    double all = 0, whole = 0;
+    for (const int64_t i : order) {
+        const double size = double(descs[i].m) * double(descs[i].n);
+        all += size;
+        if (whole_sectors(descs[i], esc)) whole += size;
+    }
+    return whole <= 0.5 * all;
+}
+
 static hsmm_status_t grouped_build_image(hsmm_dtype_t ab, hsmm_dtype_t c, int64_t count, const hsmm_gemm_desc_t* descs,
                                          int tile_n, const int* tile_n_per_problem, int schedule, GroupedImage* img) {
     const bool tf32 = (ab == HSMM_R_32F);
@@ -724,6 +814,7 @@ static hsmm_status_t grouped_build_image(hsmm_dtype_t ab, hsmm_dtype_t c, int64_
         if (descs[i].m > 0 && descs[i].n > 0 && descs[i].k > 0) order.push_back(i);
     if (schedule == 1)
         std::stable_sort(order.begin(), order.end(), [&](int64_t a, int64_t b) { return descs[a].k > descs[b].k; });
+    img->tall = img->pairs && grouped_tall(order, descs, img->out_bf16 ? 2 : 4);
     std::vector<CUtensorMap> maps(order.size() * 3);
     std::vector<uint8_t> c_tma(order.size(), 0);
     const int esc = img->out_bf16 ? 2 : 4;
@@ -759,14 +850,15 @@ static hsmm_status_t grouped_build_image(hsmm_dtype_t ab, hsmm_dtype_t c, int64_
                            : encode_map(&maps[3 * q + 1], dt, esize, d.B, uint64_t(d.k), uint64_t(d.n),
                                         uint64_t(d.ldb), BK, uint32_t(img->pairs ? bn / 2 : bn)));
         if (!ok) return HSMM_STATUS_NOT_SUPPORTED;
-        // C by TMA stores of 32 x 32 blocks when its base and columns are 16-byte aligned; the map
+        // C by TMA stores of blocks (128 x 32 if tall, else 32 x 32) when its base and
+        // columns are 16-byte aligned; the map
         // covers the rows up to the last whole 16-byte unit (a store clips to such units), the
         // epilogue stores the rows after them directly
         std::memset(&maps[3 * q + 2], 0, sizeof(CUtensorMap));
         const int64_t m_tma = d.m - d.m % (16 / esc);
         if (m_tma > 0 && tma_operand_ok(d.C, d.ldc, size_t(esc)) &&
-            encode_map(&maps[3 * q + 2], dtc, esc, d.C, uint64_t(m_tma), uint64_t(d.n), uint64_t(d.ldc), 32, 32, 0, 0,
-                       CU_TENSOR_MAP_SWIZZLE_NONE))
+            encode_map(&maps[3 * q + 2], dtc, esc, d.C, uint64_t(m_tma), uint64_t(d.n), uint64_t(d.ldc),
+                       img->tall ? BM : 32, 32, 0, 0, CU_TENSOR_MAP_SWIZZLE_NONE))
             c_tma[q] = 1;
     }
     img->count = int(order.size());
@@ -778,12 +870,15 @@ static hsmm_status_t grouped_build_image(hsmm_dtype_t ab, hsmm_dtype_t c, int64_
         const GroupedProblem& P = probs[q];
         if (P.tiles_m > 65535 || P.tiles_n > 65535) return HSMM_STATUS_NOT_SUPPORTED;
         const uint32_t nkb = uint32_t((int64_t(P.K) + BK - 1) / BK);
+        const bool edges = img->tall && c_tma[q] && nkb <= uint32_t(GP_EDGE_KB) &&
+                           !whole_sectors(descs[order[q]], esc);
         for (int tn = 0; tn < P.tiles_n; ++tn)
             for (int tm = 0; tm < P.tiles_m; ++tm) {
                 const uint32_t rows = uint32_t(std::min<int64_t>(TM, int64_t(P.M) - int64_t(tm) * TM));
                 const uint32_t cols = uint32_t(std::min<int64_t>(P.bn, int64_t(P.N) - int64_t(tn) * P.bn));
-                const uint32_t w = (uint32_t(P.bn / 32 - 1) << 26) | (uint32_t(P.a_mn) << 2) | (uint32_t(P.b_mn) << 3) |
-                                   (uint32_t(c_tma[q]) << 4) | (rows << 8) | (cols << 17);
+                const uint32_t w = uint32_t(edges) | (uint32_t(P.a_mn) << 2) | (uint32_t(P.b_mn) << 3) |
+                                   (uint32_t(c_tma[q]) << 4) | (rows << 8) | (cols << 17) |
+                                   (uint32_t(P.bn / 32 - 1) << 26);
                 tile_tab[size_t(P.tile_start + int64_t(tn) * P.tiles_m + tm)] =
                     make_uint4(uint32_t(q), uint32_t(tm) | (uint32_t(tn) << 16), nkb, w);
             }
@@ -836,18 +931,19 @@ static hsmm_status_t launch_grouped(const GroupedArgs& a, cudaStream_t st) {
     return check_launch();
 }
 
-template <bool TF32, bool OUT_BF16>
+template <bool TF32, bool OUT_BF16, bool TALL>
 static hsmm_status_t launch_grouped_pair(const GroupedArgs& a, cudaStream_t st) {
-    auto kern = gemm_grouped_pair_kernel<TF32, OUT_BF16>;
+    constexpr int smem = GroupedPairCfg<TALL>::SMEM;
+    auto kern = gemm_grouped_pair_kernel<TF32, OUT_BF16, TALL>;
     static std::atomic<uint64_t> attrs{0};
     const hsmm_status_t as = attrs_once_per_device(
-        attrs, [kern] { return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, GP_SMEM); });
+        attrs, [kern] { return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem); });
     if (as != HSMM_STATUS_SUCCESS) return as;
     const int64_t pairs = std::max<int64_t>(1, std::min<int64_t>(a.total_tiles, num_sms() / 2));
     cudaLaunchConfig_t lc = {};
     lc.gridDim = dim3(unsigned(2 * pairs), 1, 1);
     lc.blockDim = dim3(GP_THREADS, 1, 1);
-    lc.dynamicSmemBytes = GP_SMEM;
+    lc.dynamicSmemBytes = smem;
     lc.stream = st;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
@@ -878,10 +974,13 @@ static hsmm_status_t grouped_launch_image(const GroupedImage& img, const void* d
     a.timeout_ns = wait_timeout_ns();
     if (img.tf32) {
         if (img.out_bf16) return HSMM_STATUS_NOT_SUPPORTED;
-        return img.pairs ? launch_grouped_pair<true, false>(a, st) : launch_grouped<true, false>(a, st);
+        if (!img.pairs) return launch_grouped<true, false>(a, st);
+        return img.tall ? launch_grouped_pair<true, false, true>(a, st) : launch_grouped_pair<true, false, false>(a, st);
     }
+    if (img.pairs && img.out_bf16)
+        return img.tall ? launch_grouped_pair<false, true, true>(a, st) : launch_grouped_pair<false, true, false>(a, st);
     if (img.pairs)
-        return img.out_bf16 ? launch_grouped_pair<false, true>(a, st) : launch_grouped_pair<false, false>(a, st);
+        return img.tall ? launch_grouped_pair<false, false, true>(a, st) : launch_grouped_pair<false, false, false>(a, st);
     return img.out_bf16 ? launch_grouped<false, true>(a, st) : launch_grouped<false, false>(a, st);
 }
 
