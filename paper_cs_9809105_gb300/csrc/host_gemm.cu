@@ -78,6 +78,41 @@ struct HostPlan {
     OzakiLayout L;
 };
 
+// rows (or columns) of a panel when `size` is cut into `panels`: whole 256-row tiles
+int64_t panel_size(int64_t size, int panels) {
+    return panels == 1 ? (size > 1 ? size : 1) : ((size + panels - 1) / panels + 255) / 256 * 256;
+}
+
+// Estimated time of the FP64-accurate form with row panels of mi rows and column panels of nj
+// columns, by the order in which the call below queues its copies, splits, blocks and returns.  The
+// rates are rounded measurements: 205 GB/s a copy, 22 bytes an entry split at 3.5 TB/s, the slice
+// products at 2.0 PFLOP/s of whole tiles, and 26 us a block for its launches and its last wave.
+double ozaki_host_time(int64_t m, int64_t n, int64_t k, int slices, bool cplx, int64_t mi, int64_t nj) {
+    const double e = cplx ? 16 : 8, z = cplx ? 2 : 1, dk = double(k);
+    auto tiles = [](double v) { return double((int64_t(v) + 255) / 256 * 256); };
+    auto copy = [&](double entries) { return 6e-6 + entries * e / 205e9; };
+    auto split = [&](double entries) { return 8e-6 + entries * 22 * z / 3.5e12; };
+    const int rp = int((m + mi - 1) / mi), p = int((n + nj - 1) / nj);
+    auto h = [&](int I) { return double(m - I * mi < mi ? m - I * mi : mi); };
+    auto w = [&](int J) { return double(n - J * nj < nj ? n - J * nj : nj); };
+    double a[8], b[8], x = 0, s = 0, y = 0;
+    for (int I = 0; I < rp; ++I) {
+        a[I] = x += copy(h(I) * dk);
+        if (I == 0) b[0] = x += copy(w(0) * dk);
+    }
+    for (int J = 1; J < p; ++J) b[J] = x += copy(w(J) * dk);
+    s = a[0] + split(h(0) * dk);
+    for (int J = 0; J < p; ++J) {
+        s = (s > b[J] ? s : b[J]) + split(w(J) * dk);
+        for (int I = 0; I < rp; ++I) {
+            if (J == 0 && I > 0) s = (s > a[I] ? s : a[I]) + split(h(I) * dk);
+            s += 26e-6 + slices * (slices + 1) * tiles(h(I)) * tiles(z * w(J)) * z * dk / 2.0e15 + h(I) * w(J) * 36 * z / 5e12;
+            y = (y > s ? y : s) + copy(h(I) * w(J));
+        }
+    }
+    return y;
+}
+
 HostPlan host_plan(const hsmm_config_t& c, hsmm_op_t ta, hsmm_op_t tb, int64_t m, int64_t n, int64_t k) {
     HostPlan P{};
     P.rowsA = (ta == HSMM_OP_N) ? m : k;
@@ -92,27 +127,53 @@ HostPlan host_plan(const hsmm_config_t& c, hsmm_op_t ta, hsmm_op_t tb, int64_t m
     P.ec = elem_bytes(c.c);
     P.cplx = (c.a == HSMM_C_64F);
     P.ozaki = (c.compute == HSMM_COMPUTE_64F_OZAKI);
-    // two panels once each holds at least 2048 columns (whole 256-column tiles)
+    P.slices = default_slices(&c);
+    P.bits = default_bits(&c);
+    // two column panels once each holds at least 2048 columns, and two or four row panels once
+    // each holds at least 2048 rows
     P.panels = n >= 4096 ? 2 : 1;
-    P.nj = P.panels == 1 ? n : ((n + P.panels - 1) / P.panels + 255) / 256 * 256;
-    P.panels = int((n + P.nj - 1) / P.nj);
-    // and two or four row panels once each holds at least 2048 rows (whole 256-row pair
-    // tiles).  A block of 2048 x 4096 is 128 pair tiles, 96% of whole waves of the product
-    // kernel (as for 4096 x 4096); four column panels as well would leave 64 tiles a block,
-    // cut into 256 quarter-tile items for 76 pairs, 84% busy.
     P.rpanels = m >= 8192 ? 4 : (m >= 4096 ? 2 : 1);
-    P.mi = P.rpanels == 1 ? m : ((m + P.rpanels - 1) / P.rpanels + 255) / 256 * 256;
+    const int64_t ws_nj = panel_size(n, P.panels);      // the workspace is sized by this rule
+    // The FP64-accurate form is worth more panels, and from smaller sizes on: its time per block is
+    // estimated for each choice, and the fewest blocks within 3.5% of the best are taken.  Us before ->
+    // now: 1500^3 495 -> 427, 2048^3 813 -> 634, 3000^3 2295 -> 1743, 2048 x 2048 x 8192 2519 -> 1977,
+    // 4096^3 2990 -> 2935, 5000 x 3000 x 4000 3142 -> 2713, 8192^3 19.0 -> 18.6 ms; 1024^3 stays at one
+    // block (206; 223 with two).
+    if (P.ozaki && m > 0 && n > 0) {
+        double t[9];
+        int at = 0;
+        double best = 0;
+        const int pmin = P.panels;
+        for (int i = 0; i < 9; ++i) {
+            const int rp = 1 << (i / 3), p = 1 << (i % 3);
+            t[i] = p < pmin ? 0.0 : ozaki_host_time(m, n, k, P.slices, P.cplx, panel_size(m, rp), panel_size(n, p));
+            if (t[i] > 0 && (best == 0 || t[i] < best)) best = t[i];
+        }
+        auto blocks = [](int i) { return (1 << (i / 3)) * (1 << (i % 3)); };
+        for (int i = 0, found = 0; i < 9; ++i) {
+            if (t[i] == 0 || t[i] > 1.035 * best) continue;
+            if (!found || blocks(i) < blocks(at) || (blocks(i) == blocks(at) && t[i] < t[at])) at = i;
+            found = 1;
+        }
+        P.rpanels = 1 << (at / 3);
+        P.panels = 1 << (at % 3);
+    }
+    P.nj = panel_size(n, P.panels);
+    P.panels = int((n + P.nj - 1) / P.nj);
+    P.mi = panel_size(m, P.rpanels);
     P.rpanels = int((m + P.mi - 1) / P.mi);
     size_t off = 0;
     P.offA = off; off += up256(size_t(P.ldA) * size_t(P.colsA) * P.ea);
     P.offB = off; off += up256(size_t(P.ldB) * size_t(P.colsB) * P.eb);
     P.offC = off; off += up256(size_t(P.ldC) * size_t(n) * P.ec);
     P.offW = off;
-    P.slices = default_slices(&c);
-    P.bits = default_bits(&c);
     if (P.ozaki) {
-        P.L = P.cplx ? ozaki_layout(m, 2 * P.nj, 2 * k, P.slices) : ozaki_layout(m, P.nj, k, P.slices);
-        off += P.L.total;
+        auto layout = [&](int64_t w) {
+            return P.cplx ? ozaki_layout(m, 2 * w, 2 * k, P.slices) : ozaki_layout(m, w, k, P.slices);
+        };
+        P.L = layout(P.nj);
+        const size_t sized = layout(ws_nj < n ? ws_nj : n).total;
+        off += P.L.total > sized ? P.L.total : sized;    // no panel is wider than ws_nj
     }
     P.total = off;
     return P;
