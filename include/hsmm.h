@@ -124,6 +124,8 @@ typedef struct {
  *  bytes) is carved, each piece starting on a 256-byte boundary, into
  *    QA  s planes of m x kq BF16   slices of op(A), [t][i][k] (as hsmm_ozaki_split, by rows)
  *    QB  s planes of n x kq BF16   slices of op(B), [u][j][k] (by columns)
+ *        (where kq is not a multiple of 64, in blocks of 64 columns: [t][k / 64][i][k % 64],
+ *        the last block kq % 64 wide)
  *    EA  m INT32, EB n INT32       exponents of rows / columns
  *    SD  s planes of m x n INT32   S_d = sum_{t+u=d} QA_t QB_u^T, d = 2..s+1, [d-2][j][i]
  *  where a plane of E elements of size z bytes has the pitch (round_up(E z, 256) + 1024) / z
@@ -145,7 +147,8 @@ hsmm_status_t hsmm_gemm(const hsmm_config_t* cfg, hsmm_op_t transA, hsmm_op_t tr
  * Section 3.1, and its complex and transposed forms as in hsmm_gemm; same cfg, ops,
  * scalars and leading dimensions, here of the host arrays).  C is computed in blocks:
  * row panels of op(A) (two once m >= 4096, four once m >= 8192) times column panels of
- * op(B) (two once n >= 4096).  The first panel of each operand is copied first, the later panels while
+ * op(B) (two once n >= 4096); the FP64-accurate forms choose one to four of each by the
+ * estimated time.  The first panel of each operand is copied first, the later panels while
  * the first blocks are computed, and every finished block of C returns to the host while
  * the next one is computed.  The FP64-accurate forms split each panel of op(A) and of
  * op(B) once (the result equals that of hsmm_gemm on the same data).  Copies run on two

@@ -111,13 +111,13 @@ OzakiLayout ozaki_layout(int64_t m, int64_t n, int64_t k, int slices) {
 }
 
 SplitOperand split_operand_a(bool cplx, hsmm_op_t ta, int64_t m, int64_t k, const void* A, int64_t lda, int32_t* ea,
-                             void* qa, int64_t ldq, int64_t plane) {
-    return SplitOperand{A, lda, m, k, ta == HSMM_OP_N, cplx && ta == HSMM_OP_C, false, ea, qa, ldq, plane};
+                             const Slices& qa) {
+    return SplitOperand{A, lda, m, k, ta == HSMM_OP_N, cplx && ta == HSMM_OP_C, false, ea, qa};
 }
 
 SplitOperand split_operand_b(bool cplx, hsmm_op_t tb, int64_t k, int64_t n, const void* B, int64_t ldb, int32_t* eb,
-                             void* qb, int64_t ldq, int64_t plane) {
-    return SplitOperand{B, ldb, n, k, tb != HSMM_OP_N, cplx && tb == HSMM_OP_C, true, eb, qb, ldq, plane};
+                             const Slices& qb) {
+    return SplitOperand{B, ldb, n, k, tb != HSMM_OP_N, cplx && tb == HSMM_OP_C, true, eb, qb};
 }
 
 int default_slices(const hsmm_config_t* c) { return c->ozaki_slices > 0 ? c->ozaki_slices : 7; }
@@ -260,12 +260,13 @@ hsmm_status_t hsmm_gemm(const hsmm_config_t* cfg, hsmm_op_t transA, hsmm_op_t tr
         int32_t* ea = reinterpret_cast<int32_t*>(ws + L.ea);
         int32_t* eb = reinterpret_cast<int32_t*>(ws + L.eb);
         int32_t* sd = reinterpret_cast<int32_t*>(ws + L.sd);
-        const SplitOperand ops[2] = {split_operand_a(true, transA, m, k, A, lda, ea, ws + L.qa, L.ldq, L.qa_plane),
-                                     split_operand_b(true, transB, k, n, B, ldb, eb, ws + L.qb, L.ldq, L.qb_plane)};
+        const Slices qa = workspace_slices(ws + L.qa, L.ldq, L.qa_plane, m);
+        const Slices qb = workspace_slices(ws + L.qb, L.ldq, L.qb_plane, 2 * n);
+        const SplitOperand ops[2] = {split_operand_a(true, transA, m, k, A, lda, ea, qa),
+                                     split_operand_b(true, transB, k, n, B, ldb, eb, qb)};
         hsmm_status_t r = ozaki_split(true, ops, 2, bits, s, st);
         if (r == HSMM_STATUS_SUCCESS)
-            r = gemm_ozaki_slices(m, 2 * n, 2 * k, L.ldq, s, bits, ws + L.qa, L.qa_plane, ws + L.qb, L.qb_plane, sd,
-                                  L.sd_plane, st);
+            r = gemm_ozaki_slices(m, 2 * n, 2 * k, s, bits, qa, qb, sd, L.sd_plane, st);
         if (r != HSMM_STATUS_SUCCESS) return r;
         return ozaki_zrecombine(m, n, s, bits, sd, L.sd_plane, ea, eb, al, be, C, ldc, st);
     }
@@ -315,12 +316,14 @@ hsmm_status_t hsmm_gemm(const hsmm_config_t* cfg, hsmm_op_t transA, hsmm_op_t tr
     uint8_t* ws = static_cast<uint8_t*>(c.workspace);
     int32_t* ea = reinterpret_cast<int32_t*>(ws + L.ea);
     int32_t* eb = reinterpret_cast<int32_t*>(ws + L.eb);
-    const SplitOperand ops[2] = {split_operand_a(false, transA, m, k, A, lda, ea, ws + L.qa, L.ldq, L.qa_plane),
-                                 split_operand_b(false, transB, k, n, B, ldb, eb, ws + L.qb, L.ldq, L.qb_plane)};
+    const Slices qa = workspace_slices(ws + L.qa, L.ldq, L.qa_plane, m);
+    const Slices qb = workspace_slices(ws + L.qb, L.ldq, L.qb_plane, n);
+    const SplitOperand ops[2] = {split_operand_a(false, transA, m, k, A, lda, ea, qa),
+                                 split_operand_b(false, transB, k, n, B, ldb, eb, qb)};
     hsmm_status_t r = ozaki_split(false, ops, 2, bits, s, st);
     if (r != HSMM_STATUS_SUCCESS) return r;
     int32_t* sd = reinterpret_cast<int32_t*>(ws + L.sd);
-    r = gemm_ozaki_slices(m, n, k, L.ldq, s, bits, ws + L.qa, L.qa_plane, ws + L.qb, L.qb_plane, sd, L.sd_plane, st);
+    r = gemm_ozaki_slices(m, n, k, s, bits, qa, qb, sd, L.sd_plane, st);
     if (r != HSMM_STATUS_SUCCESS) return r;
     return ozaki_recombine(m, n, s, bits, sd, L.sd_plane, ea, eb, al, be, static_cast<double*>(C), ldc, st);
 }
@@ -373,7 +376,7 @@ hsmm_status_t hsmm_ozaki_split(int64_t rows, int64_t cols, const double* M, int6
     if (plane < nv * ldq || plane % 8 != 0) return fail(HSMM_STATUS_INVALID_VALUE, "ozaki_split: bad slice pitch");
     if (rows == 0 || cols == 0) return HSMM_STATUS_SUCCESS;
     if (!M || !expo || !q) return HSMM_STATUS_INVALID_VALUE;
-    const SplitOperand op{M, ld, nv, len, by_rows != 0, false, false, expo, q, ldq, plane};
+    const SplitOperand op{M, ld, nv, len, by_rows != 0, false, false, expo, Slices{q, ldq, plane, 0, 0}};
     return ozaki_split(false, &op, 1, bits, slices, static_cast<cudaStream_t>(stream));
 }
 
@@ -401,7 +404,8 @@ hsmm_status_t hsmm_ozaki_slice_products(int64_t m, int64_t n, int64_t k, int sli
         }
         return HSMM_STATUS_SUCCESS;
     }
-    return gemm_ozaki_slices(m, n, k, ldq, slices, bits, qa, qa_plane, qb, qb_plane, sd, sd_plane,
+    return gemm_ozaki_slices(m, n, k, slices, bits, Slices{const_cast<void*>(qa), ldq, qa_plane, 0, 0},
+                             Slices{const_cast<void*>(qb), ldq, qb_plane, 0, 0}, sd, sd_plane,
                              static_cast<cudaStream_t>(stream));
 }
 

@@ -163,6 +163,13 @@ __device__ __forceinline__ void tma_load_3d(void* dst, const void* map, uint64_t
         ::"r"(smem_u32(dst)), "l"(map), "r"(smem_u32(bar)), "r"(c0), "r"(c1), "r"(c2)
         : "memory");
 }
+__device__ __forceinline__ void tma_load_4d(void* dst, const void* map, uint64_t* bar, int32_t c0, int32_t c1,
+                                            int32_t c2, int32_t c3) {
+    asm volatile(
+        "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], [%2];"
+        ::"r"(smem_u32(dst)), "l"(map), "r"(smem_u32(bar)), "r"(c0), "r"(c1), "r"(c2), "r"(c3)
+        : "memory");
+}
 
 // The same loads and the expected-bytes arrival, predicated on `issue` inside the instruction
 // stream (see umma_if below): called by a converged warp with one lane's `issue` set.
@@ -415,6 +422,17 @@ __device__ __forceinline__ void tma_load_3d_pair_if(uint32_t issue, void* dst, c
         "@q cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes "
         "[%0], [%1, {%3, %4, %5}], [%2];\n\t}"
         ::"r"(smem_u32(dst)), "l"(map), "r"(bar_cluster_addr), "r"(c0), "r"(c1), "r"(c2), "r"(issue)
+        : "memory");
+}
+__device__ __forceinline__ void tma_load_4d_pair_if(uint32_t issue, void* dst, const void* map,
+                                                    uint32_t bar_cluster_addr, int32_t c0, int32_t c1, int32_t c2,
+                                                    int32_t c3) {
+    asm volatile(
+        "{\n\t.reg .pred q;\n\t"
+        "setp.ne.b32 q, %6, 0;\n\t"
+        "@q cp.async.bulk.tensor.4d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes "
+        "[%0], [%1, {%3, %4, %5, %7}], [%2];\n\t}"
+        ::"r"(smem_u32(dst)), "l"(map), "r"(bar_cluster_addr), "r"(c0), "r"(c1), "r"(c2), "r"(issue), "r"(c3)
         : "memory");
 }
 __device__ __forceinline__ void tmem_alloc_pair(uint32_t* dst_smem, uint32_t ncols) {

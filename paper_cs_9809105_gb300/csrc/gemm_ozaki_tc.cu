@@ -91,6 +91,17 @@ struct OzWork {
     bool add;      // S_d += (several units share the anti-diagonal)
 };
 constexpr int OZ_MAX_PAIRS = 100, OZ_MAX_UNITS = 1600;   // at most 16 units for each of 99 tail tiles
+
+// The slices of one operand as k-blocks of 64 columns (box 64 x rows x 1 x 1 at column 0, row, block,
+// slice), and what remains of k after them (one block, zero-filled); see Slices for the two layouts.
+// Blocks of whole lines are what the tensor cores can be fed from: rows of a pitch of 8 to 56 columns
+// more than a multiple of 64 cross a line with every 64 columns, and an odd multiple of 8 a sector,
+// and the products then waited for loads (690 cycles a k-block instead of 523).  2048 x 2048 x 4100:
+// 814 -> 592 us, 2048 x 2048 x 2056 406 -> 328, 1000 x 1200 x 900 78 -> 69 (whole product).
+struct SliceMaps {
+    CUtensorMap blocks, rest;
+};
+
 struct OzTable {
     uint16_t first[OZ_MAX_PAIRS + 1];    // units of a pair: first[pair] .. first[pair + 1] - 1
     uint32_t unit[OZ_MAX_UNITS];         // tail tile | d << 8 | first slice of A << 16 | pairs << 22 | add << 28
@@ -113,7 +124,7 @@ __device__ __forceinline__ void oz_item_d(const OzWork& it, int di, int s, int& 
 }
 
 __global__ void __launch_bounds__(OZ_THREADS, 1)
-    gemm_ozaki_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, OzakiArgs g) {
+    gemm_ozaki_kernel(const __grid_constant__ SliceMaps mA, const __grid_constant__ SliceMaps mB, OzakiArgs g) {
     using C_ = Cfg<OZ_BN, false>;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = align1024(smem_raw);
@@ -133,8 +144,10 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
         mbar_init(&bars->mma_done, 1);
         bars->abort = 0;
         fence_mbar_init();
-        tma_prefetch_desc(&tmA);
-        tma_prefetch_desc(&tmB);
+        tma_prefetch_desc(&mA.blocks);
+        tma_prefetch_desc(&mB.blocks);
+        tma_prefetch_desc(&mA.rest);
+        tma_prefetch_desc(&mB.rest);
     }
     if (warp == 1) {
         tmem_alloc(&bars->tmem_base, C_::TMEM_COLS);
@@ -149,7 +162,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
     const int tiles_m = (g.M + BM - 1) / BM;
     const int tiles_n = (g.N + OZ_BN - 1) / OZ_BN;
     const int ntiles = tiles_m * tiles_n;
-    const int nkb = (g.K + C_::BK - 1) / C_::BK;
+    const int nkb = (g.K + C_::BK - 1) / C_::BK, nfull = g.K / C_::BK;
     const int s = g.slices;
     const int kcb = g.kc_blocks;
 
@@ -172,8 +185,11 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
                             uint8_t* a_dst = smem + stage * C_::STAGE_BYTES;
                             uint8_t* b_dst = a_dst + C_::A_BYTES;
                             mbar_arrive_expect_tx(&bars->full[stage], C_::STAGE_BYTES);
-                            tma_load_3d(a_dst, &tmA, &bars->full[stage], kb * C_::BK, tm * BM, ta - 1);
-                            tma_load_3d(b_dst, &tmB, &bars->full[stage], kb * C_::BK, tn * OZ_BN, ub - 1);
+                            const bool rest = kb >= nfull;
+                            const int block = rest ? 0 : kb;
+                            tma_load_4d(a_dst, rest ? &mA.rest : &mA.blocks, &bars->full[stage], 0, tm * BM, block, ta - 1);
+                            tma_load_4d(b_dst, rest ? &mB.rest : &mB.blocks, &bars->full[stage], 0, tn * OZ_BN, block,
+                                        ub - 1);
                             last_parity[stage] = int(phase);
                             if (++stage == C_::STAGES) { stage = 0; phase ^= 1u; }
                         }
@@ -309,7 +325,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
 // is bound by the power cap (18.51 -> 18.46 ms).
 
 __global__ void __launch_bounds__(OZ_THREADS, 1)
-    gemm_ozaki_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
+    gemm_ozaki_pair_kernel(const __grid_constant__ SliceMaps mA, const __grid_constant__ SliceMaps mB,
                            OzakiArgs g, const __grid_constant__ OzTable tab) {
     using C_ = Cfg<OZ_BN, false>;                  // BK, KSTEPS, descriptors (K-major, 128-byte rows)
     extern __shared__ uint8_t smem_raw[];
@@ -332,8 +348,10 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
         mbar_init(&bars->mma_done, 1);
         bars->abort = 0;
         fence_mbar_init();
-        tma_prefetch_desc(&tmA);
-        tma_prefetch_desc(&tmB);
+        tma_prefetch_desc(&mA.blocks);
+        tma_prefetch_desc(&mB.blocks);
+        tma_prefetch_desc(&mA.rest);
+        tma_prefetch_desc(&mB.rest);
     }
     if (warp == 1) {
         tmem_alloc_pair(&bars->tmem_base, 512);
@@ -349,7 +367,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
     const int tiles_n = (g.N + PAIR_BN - 1) / PAIR_BN;
     const int ntiles = tiles_m * tiles_n;
     const int pair = int(blockIdx.x >> 1), npairs = int(gridDim.x >> 1);
-    const int nkb = (g.K + C_::BK - 1) / C_::BK;
+    const int nkb = (g.K + C_::BK - 1) / C_::BK, nfull = g.K / C_::BK;
     const int s = g.slices;
     const int kcb = g.kc_blocks;
     const int nitems = oz_items(tab, ntiles, npairs, pair);
@@ -380,8 +398,12 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
                         uint8_t* a_dst = smem + stage * PAIR_STAGE_BYTES;
                         const uint32_t full_leader = full0 + uint32_t(stage) * 8u;
                         mbar_arrive_expect_tx_if(issue && leader, &bars->full[stage], 2 * PAIR_STAGE_BYTES);
-                        tma_load_3d_pair_if(issue, a_dst, &tmA, full_leader, kb * C_::BK, arow, ta - 1);
-                        tma_load_3d_pair_if(issue, a_dst + BM * 128, &tmB, full_leader, kb * C_::BK, brow, ub - 1);
+                        const bool rest = kb >= nfull;
+                        const int block = rest ? 0 : kb;
+                        tma_load_4d_pair_if(issue, a_dst, rest ? &mA.rest : &mA.blocks, full_leader, 0, arow, block,
+                                            ta - 1);
+                        tma_load_4d_pair_if(issue, a_dst + BM * 128, rest ? &mB.rest : &mB.blocks, full_leader, 0, brow,
+                                            block, ub - 1);
                         ++filled;
                         if (++stage == PAIR_STAGES) { stage = 0; phase ^= 1u; }
                     }
@@ -617,7 +639,7 @@ static bool ozaki_pairs_enabled() {
     return !(v && std::strcmp(v, "single") == 0);
 }
 
-static hsmm_status_t launch_ozaki_pairs(const CUtensorMap& mA, const CUtensorMap& mB, const OzakiArgs& g, int slices,
+static hsmm_status_t launch_ozaki_pairs(const SliceMaps& mA, const SliceMaps& mB, const OzakiArgs& g, int slices,
                                         cudaStream_t st) {
     static std::atomic<uint64_t> attrs{0};
     hsmm_status_t as = attrs_once_per_device(attrs, [] {
@@ -653,9 +675,33 @@ static hsmm_status_t launch_ozaki_pairs(const CUtensorMap& mA, const CUtensorMap
     return check_launch();
 }
 
-hsmm_status_t gemm_ozaki_slices(int64_t m, int64_t n, int64_t k, int64_t ldq, int slices, int bits, const void* qa,
-                                int64_t qa_plane, const void* qb, int64_t qb_plane, int32_t* sd, int64_t sd_plane,
-                                cudaStream_t st) {
+// maps of the slices of `rows` rows and k columns, boxes of box_rows x 64
+static bool slice_maps(const Slices& q, int64_t rows, int64_t k, int slices, uint32_t box_rows, SliceMaps* m) {
+    const uint16_t* base = static_cast<const uint16_t*>(q.q);
+    const int64_t full = k / 64, rem = k % 64;
+    // row pitch and start of the blocks of 64 columns, and of the columns after them
+    int64_t pitch = q.ldq, step = 64, at = q.row0 * q.ldq, rest_pitch = q.ldq, rest_at = at + full * 64;
+    if (q.block_rows > 0) {                       // ldq / 64 == full: ldq is k rounded up to 8, and not to 64
+        pitch = 64;
+        step = q.block_rows * 64;
+        at = q.row0 * 64;
+        rest_pitch = q.ldq % 64;
+        rest_at = full * step + q.row0 * rest_pitch;
+    }
+    auto encode = [&](CUtensorMap* map, int64_t from, int64_t cols, int64_t ld, int64_t blocks) {
+        return encode_map(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, base + from, uint64_t(cols), uint64_t(rows),
+                          uint64_t(ld), 64, box_rows, uint64_t(slices), uint64_t(q.plane), CU_TENSOR_MAP_SWIZZLE_128B, 1,
+                          uint64_t(blocks), uint64_t(step));
+    };
+    if (full > 0 && !encode(&m->blocks, at, 64, pitch, full)) return false;
+    if (rem > 0 && !encode(&m->rest, rest_at, rem, rest_pitch, 1)) return false;
+    if (full == 0) m->blocks = m->rest;
+    if (rem == 0) m->rest = m->blocks;
+    return true;
+}
+
+hsmm_status_t gemm_ozaki_slices(int64_t m, int64_t n, int64_t k, int slices, int bits, const Slices& qa,
+                                const Slices& qb, int32_t* sd, int64_t sd_plane, cudaStream_t st) {
     using C_ = Cfg<OZ_BN, false>;
     // exactness of the FP32 chunks and of the INT32 anti-diagonal sums
     const double qmax = double((1 << bits) - 1);
@@ -672,20 +718,14 @@ hsmm_status_t gemm_ozaki_slices(int64_t m, int64_t n, int64_t k, int64_t ldq, in
     g.timeout_ns = wait_timeout_ns();
     if (ozaki_pairs_enabled()) {
         // pair kernel: boxes of 128 rows (each CTA stages its half of the 256 x 256 tile's A and B)
-        CUtensorMap mA2, mB2;
-        if (!encode_map(&mA2, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, qa, uint64_t(k), uint64_t(m), uint64_t(ldq), C_::BK,
-                        BM, uint64_t(slices), uint64_t(qa_plane)) ||
-            !encode_map(&mB2, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, qb, uint64_t(k), uint64_t(n), uint64_t(ldq), C_::BK,
-                        BM, uint64_t(slices), uint64_t(qb_plane)))
+        SliceMaps mA2, mB2;
+        if (!slice_maps(qa, m, k, slices, BM, &mA2) || !slice_maps(qb, n, k, slices, BM, &mB2))
             return HSMM_STATUS_NOT_SUPPORTED;
         return launch_ozaki_pairs(mA2, mB2, g, slices, st);
     }
-    CUtensorMap mA, mB;
-    bool ok = encode_map(&mA, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, qa, uint64_t(k), uint64_t(m), uint64_t(ldq), C_::BK,
-                         BM, uint64_t(slices), uint64_t(qa_plane));
-    ok = ok && encode_map(&mB, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, qb, uint64_t(k), uint64_t(n), uint64_t(ldq), C_::BK,
-                          OZ_BN, uint64_t(slices), uint64_t(qb_plane));
-    if (!ok) return HSMM_STATUS_NOT_SUPPORTED;
+    SliceMaps mA, mB;
+    if (!slice_maps(qa, m, k, slices, BM, &mA) || !slice_maps(qb, n, k, slices, OZ_BN, &mB))
+        return HSMM_STATUS_NOT_SUPPORTED;
     static std::atomic<uint64_t> attrs{0};
     hsmm_status_t as = attrs_once_per_device(attrs, [] {
         return cudaFuncSetAttribute(gemm_ozaki_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, C_::SMEM_BYTES);

@@ -85,7 +85,7 @@ int last_encode_result() { return g_last_encode_result; }
 // instead of encoding again.  A map depends on nothing but these arguments.
 namespace {
 struct MapKey {
-    uint64_t base, inner, outer, ld, batch, batch_stride;
+    uint64_t base, inner, outer, ld, batch, batch_stride, blocks, block_stride;
     uint32_t box_inner, box_outer, box_batch;
     int32_t dt, esize, swizzle;
 };
@@ -99,14 +99,15 @@ thread_local MapCacheEntry t_map_cache[kMapCache];
 thread_local int t_map_next = 0;
 }  // namespace
 
-// 2D (or 3D with a batch dimension) tiled map with 128-byte swizzle.
+// 2D (3D with a batch dimension, 4D with a dimension of blocks before it) tiled map.
 bool encode_map(CUtensorMap* map, CUtensorMapDataType dt, int esize, const void* base, uint64_t inner, uint64_t outer,
                 uint64_t ld, uint32_t box_inner, uint32_t box_outer, uint64_t batch, uint64_t batch_stride_elems,
-                CUtensorMapSwizzle swizzle, uint32_t box_batch) {
+                CUtensorMapSwizzle swizzle, uint32_t box_batch, uint64_t blocks, uint64_t block_stride_elems) {
     MapKey key;
     std::memset(&key, 0, sizeof(key));
     key.base = reinterpret_cast<uintptr_t>(base); key.inner = inner; key.outer = outer; key.ld = ld;
     key.batch = batch; key.batch_stride = batch_stride_elems;
+    key.blocks = blocks; key.block_stride = block_stride_elems;
     key.box_inner = box_inner; key.box_outer = box_outer; key.box_batch = box_batch;
     key.dt = int32_t(dt); key.esize = esize; key.swizzle = int32_t(swizzle);
     for (int i = 0; i < kMapCache; ++i)
@@ -117,11 +118,17 @@ bool encode_map(CUtensorMap* map, CUtensorMapDataType dt, int esize, const void*
         }
     EncodeTiledFn fn = encode_fn();
     if (!fn) return false;
-    cuuint64_t dims[3] = {inner, outer, batch};
-    cuuint64_t strides[2] = {ld * uint64_t(esize), batch_stride_elems * uint64_t(esize)};
-    cuuint32_t box[3] = {box_inner, box_outer, box_batch};
-    cuuint32_t estr[3] = {1, 1, 1};
-    const cuuint32_t rank = batch ? 3 : 2;
+    cuuint64_t dims[4] = {inner, outer, batch, 0};
+    cuuint64_t strides[3] = {ld * uint64_t(esize), batch_stride_elems * uint64_t(esize), 0};
+    cuuint32_t box[4] = {box_inner, box_outer, box_batch, 1};
+    cuuint32_t estr[4] = {1, 1, 1, 1};
+    cuuint32_t rank = batch ? 3 : 2;
+    if (blocks) {
+        dims[2] = blocks; dims[3] = batch;
+        strides[2] = strides[1]; strides[1] = block_stride_elems * uint64_t(esize);
+        box[2] = 1;
+        rank = 4;
+    }
     CUresult r = fn(map, dt, rank, const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
                     swizzle, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) {

@@ -306,7 +306,7 @@ extern "C" hsmm_status_t hsmm_gemm_host(const hsmm_config_t* cfg, hsmm_op_t tran
     int32_t* ea = reinterpret_cast<int32_t*>(W + P.L.ea);
     int32_t* eb = reinterpret_cast<int32_t*>(W + P.L.eb);
     int32_t* sd = reinterpret_cast<int32_t*>(W + P.L.sd);
-    uint8_t* qa = W + P.L.qa;
+    auto slices_a = [&](int64_t i0) { return workspace_slices(W + P.L.qa, P.L.ldq, P.L.qa_plane, m, i0); };
     const bool ozaki_run = P.ozaki && k > 0 && !is_zero_scalar(c.c, alpha);
     // the first row panel of op(A) arrives first: its split runs while op(B)'s first panel is copied
     auto split_a = [&](int I) {
@@ -314,7 +314,7 @@ extern "C" hsmm_status_t hsmm_gemm_host(const hsmm_config_t* cfg, hsmm_op_t tran
         hsmm_status_t q = record_cuda(cudaStreamWaitEvent(S, evA[I], 0));
         if (q == HSMM_STATUS_SUCCESS && ozaki_run) {
             const SplitOperand op = split_operand_a(P.cplx, transA, h, k, dA + a_row(i0, P.ldA), P.ldA, ea + i0,
-                                                    qa + i0 * P.L.ldq * 2, P.L.ldq, P.L.qa_plane);
+                                                    slices_a(i0));
             q = ozaki_split(P.cplx, &op, 1, P.bits, P.slices, S);
         }
         return q;
@@ -323,10 +323,10 @@ extern "C" hsmm_status_t hsmm_gemm_host(const hsmm_config_t* cfg, hsmm_op_t tran
     for (int J = 0; J < P.panels && r == HSMM_STATUS_SUCCESS; ++J) {
         const int64_t j0 = J * P.nj, w = panel_w(J);
         r = record_cuda(cudaStreamWaitEvent(S, evB[J], 0));
+        const Slices qb = workspace_slices(W + P.L.qb, P.L.ldq, P.L.qb_plane, P.cplx ? 2 * w : w);
         const uint8_t* dBp = (transB == HSMM_OP_N) ? dB + j0 * P.ldB * P.eb : dB + j0 * P.eb;
         if (r == HSMM_STATUS_SUCCESS && ozaki_run) {
-            const SplitOperand op = split_operand_b(P.cplx, transB, k, w, dBp, P.ldB, eb, W + P.L.qb, P.L.ldq,
-                                                    P.L.qb_plane);
+            const SplitOperand op = split_operand_b(P.cplx, transB, k, w, dBp, P.ldB, eb, qb);
             r = ozaki_split(P.cplx, &op, 1, P.bits, P.slices, S);
         }
         for (int I = 0; I < P.rpanels && r == HSMM_STATUS_SUCCESS; ++I) {
@@ -336,8 +336,8 @@ extern "C" hsmm_status_t hsmm_gemm_host(const hsmm_config_t* cfg, hsmm_op_t tran
             if (J == 0 && I > 0) r = split_a(I);
             if (r != HSMM_STATUS_SUCCESS) break;
             if (ozaki_run) {
-                r = gemm_ozaki_slices(h, P.cplx ? 2 * w : w, P.cplx ? 2 * k : k, P.L.ldq, P.slices, P.bits,
-                                      qa + i0 * P.L.ldq * 2, P.L.qa_plane, W + P.L.qb, P.L.qb_plane, sd, P.L.sd_plane, S);
+                r = gemm_ozaki_slices(h, P.cplx ? 2 * w : w, P.cplx ? 2 * k : k, P.slices, P.bits, slices_a(i0), qb, sd,
+                                      P.L.sd_plane, S);
                 if (r == HSMM_STATUS_SUCCESS) {
                     if (P.cplx)
                         r = ozaki_zrecombine(h, w, P.slices, P.bits, sd, P.L.sd_plane, ea + i0, eb,

@@ -86,7 +86,8 @@ bool tma_operand_ok(const void* p, int64_t ld, size_t esize);
 bool encode_map(CUtensorMap* map, CUtensorMapDataType dt, int esize, const void* base, uint64_t inner, uint64_t outer,
                 uint64_t ld, uint32_t box_inner, uint32_t box_outer, uint64_t batch = 0,
                 uint64_t batch_stride_elems = 0, CUtensorMapSwizzle swizzle = CU_TENSOR_MAP_SWIZZLE_128B,
-                uint32_t box_batch = 1);
+                uint32_t box_batch = 1,
+                uint64_t blocks = 0, uint64_t block_stride_elems = 0);
 int last_encode_result();
 
 // ---- gemm_split_tc.cu ----
@@ -111,17 +112,25 @@ hsmm_status_t gemm_tc_split(bool tf32, bool out_bf16, const CUtensorMap& ta, con
                             const SplitPlan& plan, cudaStream_t st);
 uint32_t status_take_split();
 
+// Slices of an operand, from row `row0` of its planes on.  block_rows = 0: [t][v][w], row pitch ldq.
+// Otherwise a plane holds its columns in blocks of 64, [t][w / 64][v][w % 64] with block_rows rows v
+// (the last block ldq % 64 wide): the same bytes, but every 64 columns of a row are one 128-byte line,
+// which is what a TMA box reads of it.
+struct Slices {
+    void* q;
+    int64_t ldq, plane;            // elements; plane >= rows * ldq
+    int64_t block_rows, row0;
+};
+
 // ---- gemm_ozaki_tc.cu ----
 // Slice products of the FP64-accurate form: S_d = sum_{t+u=d} Q^A_t (Q^B_u)^T, d = 2..s+1, exact INT32,
 // stored as [d-2][n][m].
-hsmm_status_t gemm_ozaki_slices(int64_t m, int64_t n, int64_t k, int64_t ldq, int slices, int bits, const void* qa,
-                                int64_t qa_plane, const void* qb, int64_t qb_plane, int32_t* sd, int64_t sd_plane,
-                                cudaStream_t st);
+hsmm_status_t gemm_ozaki_slices(int64_t m, int64_t n, int64_t k, int slices, int bits, const Slices& qa,
+                                const Slices& qb, int32_t* sd, int64_t sd_plane, cudaStream_t st);
 
 // ---- ozaki.cu ----
 // One operand to split: nv lines of nw entries, entry (v, w) at M[v + w ld] (v_contig) or
-// M[w + v ld]; slices written as [t][v][w] with row pitch ldq and slice (plane) pitch `plane`
-// elements (>= lines * ldq).  Complex operands go into the real form of the complex product (A' =
+// M[w + v ld]; the slices of line v are row row0 + v of q.  Complex operands go into the real form of the complex product (A' =
 // [Re, Im] rows for role_b = false; B'' = [[Re, Im], [-Im, Re]] columns for role_b = true, 2 nv
 // lines); conj: op = C.
 struct SplitOperand {
@@ -129,8 +138,7 @@ struct SplitOperand {
     int64_t ld, nv, nw;
     bool v_contig, conj, role_b;
     int32_t* expo;
-    void* q;
-    int64_t ldq, plane;
+    Slices q;
 };
 // Splits one or two operands (count), in one launch if their lines run the same way in memory.
 hsmm_status_t ozaki_split(bool cplx, const SplitOperand* ops, int count, int bits, int slices, cudaStream_t st);
@@ -152,9 +160,14 @@ int default_slices(const hsmm_config_t* c);   // cfg->ozaki_slices, or 7
 int default_bits(const hsmm_config_t* c);     // cfg->ozaki_bits, or 7
 // Rows of op(A) (m x k) / columns of op(B) (k x n) as operands to split; cplx: complex operands
 SplitOperand split_operand_a(bool cplx, hsmm_op_t ta, int64_t m, int64_t k, const void* A, int64_t lda, int32_t* ea,
-                             void* qa, int64_t ldq, int64_t plane);
+                             const Slices& qa);
 SplitOperand split_operand_b(bool cplx, hsmm_op_t tb, int64_t k, int64_t n, const void* B, int64_t ldb, int32_t* eb,
-                             void* qb, int64_t ldq, int64_t plane);
+                             const Slices& qb);
+// The slices at `q` of a workspace: `rows` rows in a plane, the operand's from row0 on.  Rows of whole
+// 128-byte lines are kept as they are, others in blocks of 64 columns.
+inline Slices workspace_slices(void* q, int64_t ldq, int64_t plane, int64_t rows, int64_t row0 = 0) {
+    return Slices{q, ldq, plane, ldq % 64 == 0 ? 0 : rows, row0};
+}
 // Plane pitch (elements) of the workspace planes of hsmm_gemm's FP64-accurate form: the
 // plane size rounded up to 256 bytes plus 1 KiB, so that the s planes one thread touches
 // are not a power of two apart (such strides land on the same DRAM channels).

@@ -192,7 +192,7 @@ __device__ __forceinline__ void slice_store4_any(const double (&x)[4], int e, in
 
 // ---------------------------------------------------------------------------
 // The split of one operand.  nv lines of nw entries; `v_contig`: entry (v, w) at M[v + w ld],
-// else at M[w + v ld].  Real: slices of line v in row v, entries nw..ldq-1 zero.
+// else at M[w + v ld].  Real: slices of line v in row v (SliceRow), entries nw..ldq-1 zero.
 //
 // Complex (Section 7: the method on complex data): the complex product op(A) op(B) is the real
 // product A' B'' of
@@ -227,13 +227,33 @@ struct SplitJob {
     const double* M;               // complex: pairs of doubles
     int64_t ld, nv, nw;
     int32_t* expo;
-    uint16_t* q;
+    uint16_t* q;                   // of line 0
     int64_t ldq, plane;
+    int64_t wt, block, tail;       // columns in blocks of 64, pitch of those, pitch of rows in the rest
+    int64_t tail_at;               // the rest from here
+    bool blocked;                  // else row-major, pitch ldq
     int v_contig, conj, role_b;
     int vec_in, vec_out;           // 16-byte loads (real, w contiguous); 8-byte stores
     int warps;                     // w contiguous, real: warps per line (1, 2, 4 or 8)
     int cached;                    // w contiguous, complex: the line fits shared memory
     unsigned blocks;
+};
+
+// Row v of slice 1 (see Slices; BLOCKED: in blocks of 64 columns), whose entries up to the next
+// multiple of 64 are consecutive.  A kernel of its own for each: the address arithmetic of the blocks
+// cost 2 to 7% (complex 4096^2, v contiguous, 481 -> 510 us with the product by 16 columns).
+template <bool BLOCKED>
+struct SliceRow {
+    uint16_t *blocks, *tail;       // tail: where entry 0 would be if the row had the tail's pitch throughout
+    int64_t block;
+    int wt;
+    __device__ __forceinline__ SliceRow(const SplitJob& j, int64_t v)
+        : blocks(j.q + v * (BLOCKED ? 64 : j.ldq)), tail(j.q + j.tail_at + v * j.tail - j.wt), block(j.block),
+          wt(int(j.wt)) {}
+    __device__ __forceinline__ uint16_t* at(int64_t w) const {
+        if constexpr (BLOCKED) return int(w) < wt ? blocks + (int(w) >> 6) * block + (int(w) & 63) : tail + int(w);
+        else return blocks + w;
+    }
 };
 
 __device__ __forceinline__ uint64_t warp_mag_max(uint64_t mx) {
@@ -259,7 +279,7 @@ __device__ __forceinline__ void load4(const double* line, int64_t w, int64_t nw,
     }
 }
 
-template <int BITS, int S>
+template <int BITS, int S, bool BLOCKED>
 __device__ __forceinline__ void split_w_real(const SplitJob& j, int64_t block, int bits, int s) {
     __shared__ uint64_t red[8];
     const int WL = j.warps, G = 32 * WL, t = int(threadIdx.x) & (G - 1);
@@ -300,7 +320,7 @@ __device__ __forceinline__ void split_w_real(const SplitJob& j, int64_t block, i
     }
     const int e = stored_exponent(mx);
     if (t == 0) j.expo[v] = e;
-    uint16_t* out = j.q + v * j.ldq;
+    const SliceRow<BLOCKED> out(j, v);
     if (held) {
 #pragma unroll
         for (int c = 0; c < SPLIT_HELD; ++c) {
@@ -309,13 +329,13 @@ __device__ __forceinline__ void split_w_real(const SplitJob& j, int64_t block, i
 #pragma unroll
                 for (int i = 0; i < 4; ++i) x[c][i] = 0.0;
             }
-            if (w < j.ldq) slice_store4_any<BITS, S>(x[c], e, bits, s, out + w, j.plane, j.vec_out != 0);
+            if (w < j.ldq) slice_store4_any<BITS, S>(x[c], e, bits, s, out.at(w), j.plane, j.vec_out != 0);
         }
     } else {
         for (int64_t w = 4 * t; w < j.ldq; w += step) {
             double y[4];
             load4(line, w, j.nw, vec, y);
-            slice_store4_any<BITS, S>(y, e, bits, s, out + w, j.plane, j.vec_out != 0);
+            slice_store4_any<BITS, S>(y, e, bits, s, out.at(w), j.plane, j.vec_out != 0);
         }
     }
 }
@@ -336,7 +356,7 @@ __device__ __forceinline__ int zpart_at(const SplitJob& j, int64_t p, bool secon
 // place of entry w in a cached line: four consecutive entries per lane without bank conflicts
 __host__ __device__ __forceinline__ int cache_at(int w) { return w + (w >> 4); }
 
-template <int BITS, int S>
+template <int BITS, int S, bool BLOCKED>
 __device__ __forceinline__ void split_w_complex(const SplitJob& j, int64_t v, int bits, int s, double* cache) {
     __shared__ uint64_t red[8];
     const int t = int(threadIdx.x);
@@ -367,7 +387,7 @@ __device__ __forceinline__ void split_w_complex(const SplitJob& j, int64_t v, in
     if (t == 0) j.expo[v] = e;
     const int64_t nw = j.nw;
     for (int second = 0; second <= (j.role_b ? 1 : 0); ++second) {
-        uint16_t* out = j.q + (second ? j.nv + v : v) * j.ldq;
+        const SliceRow<BLOCKED> out(j, second ? j.nv + v : v);
         for (int64_t p = 4 * t; p < j.ldq; p += 1024) {
             double x[4];
             const bool left = p + 4 <= nw, right = p >= nw && p + 4 <= 2 * nw;
@@ -392,7 +412,7 @@ __device__ __forceinline__ void split_w_complex(const SplitJob& j, int64_t v, in
                     }
                 }
             }
-            slice_store4_any<BITS, S>(x, e, bits, s, out + p, j.plane, j.vec_out != 0);
+            slice_store4_any<BITS, S>(x, e, bits, s, out.at(p), j.plane, j.vec_out != 0);
         }
     }
 }
@@ -400,9 +420,9 @@ __device__ __forceinline__ void split_w_complex(const SplitJob& j, int64_t v, in
 // entries [w0, w0 + n) of line vl of a tile (n <= 64, column v of row w at (v + w / 4) % 32) to
 // positions base + w0 .. of its row, four at a time from the first position that is a multiple
 // of four; thread wq of 16.  The entries before it and the last partial group go one by one.
-template <int BITS, int S>
+template <int BITS, int S, bool BLOCKED>
 __device__ __forceinline__ void emit_tile_row(const SplitJob& j, const double (*tile)[32], int vl, int wq, int n,
-                                              int64_t pos, uint16_t* row, int e, bool flip, int bits, int s) {
+                                              int64_t pos, const SliceRow<BLOCKED>& row, int e, bool flip, int bits, int s) {
     const int lead = j.vec_out ? min(n, int(-pos & 3)) : 0;
     auto group = [&](int first, int valid) {
         double x[4];
@@ -412,7 +432,7 @@ __device__ __forceinline__ void emit_tile_row(const SplitJob& j, const double (*
             const double y = c < valid ? tile[r & 63][(vl + ((r & 63) >> 2)) & 31] : 0.0;
             x[c] = flip ? -y : y;
         }
-        slice_store4_any<BITS, S>(x, e, bits, s, row + pos + first, j.plane, j.vec_out != 0, valid);
+        slice_store4_any<BITS, S>(x, e, bits, s, row.at(pos + first), j.plane, j.vec_out != 0, valid);
     };
     const int first = lead + 4 * wq;
     if (first < n) group(first, min(4, n - first));
@@ -491,7 +511,7 @@ __device__ __forceinline__ void scan_v(const SplitJob& j, int64_t block) {
 }
 
 // one tile of 64 w x 32 v-contiguous lines, transposed through shared memory
-template <int BITS, int S, bool CPLX>
+template <int BITS, int S, bool CPLX, bool BLOCKED>
 __device__ __forceinline__ void slice_v(const SplitJob& j, int64_t block, int bits, int s) {
     // column v of row w at (v + w / 4) % 32: conflict-free both along v and for the four
     // consecutive w a thread slices
@@ -522,21 +542,21 @@ __device__ __forceinline__ void slice_v(const SplitJob& j, int64_t block, int bi
         const int vl = vh + 16 * r;
         if (v0 + vl >= j.nv) continue;
         const int e = j.expo[v0 + vl];
-        uint16_t* row = j.q + (v0 + vl) * j.ldq;
+        const SliceRow<BLOCKED> row(j, v0 + vl);
         if constexpr (CPLX) {
             constexpr int IM = CPLX ? 1 : 0;
-            emit_tile_row<BITS, S>(j, tile[0], vl, wq, n, w0, row, e, false, bits, s);
-            emit_tile_row<BITS, S>(j, tile[IM], vl, wq, n, j.nw + w0, row, e, j.role_b != 0, bits, s);
+            emit_tile_row<BITS, S, BLOCKED>(j, tile[0], vl, wq, n, w0, row, e, false, bits, s);
+            emit_tile_row<BITS, S, BLOCKED>(j, tile[IM], vl, wq, n, j.nw + w0, row, e, j.role_b != 0, bits, s);
             if (j.role_b) {
-                uint16_t* row2 = row + j.nv * j.ldq;
-                emit_tile_row<BITS, S>(j, tile[IM], vl, wq, n, w0, row2, e, false, bits, s);
-                emit_tile_row<BITS, S>(j, tile[0], vl, wq, n, j.nw + w0, row2, e, false, bits, s);
+                const SliceRow<BLOCKED> row2(j, j.nv + v0 + vl);
+                emit_tile_row<BITS, S, BLOCKED>(j, tile[IM], vl, wq, n, w0, row2, e, false, bits, s);
+                emit_tile_row<BITS, S, BLOCKED>(j, tile[0], vl, wq, n, j.nw + w0, row2, e, false, bits, s);
             }
         } else if (4 * wq < n) {
             double x[4];
 #pragma unroll
             for (int c = 0; c < 4; ++c) x[c] = tile[0][4 * wq + c][(vl + wq) & 31];
-            slice_store4_any<BITS, S>(x, e, bits, s, row + w0 + 4 * wq, j.plane, j.vec_out != 0);
+            slice_store4_any<BITS, S>(x, e, bits, s, row.at(w0 + 4 * wq), j.plane, j.vec_out != 0);
         }
     }
     if constexpr (CPLX) {          // zeros from 2 nw to ldq
@@ -544,29 +564,29 @@ __device__ __forceinline__ void slice_v(const SplitJob& j, int64_t block, int bi
             for (int64_t p = 2 * j.nw + ty; p < j.ldq; p += 8)
                 for (int t = 0; t < s; ++t)
                     for (int second = 0; second <= (j.role_b ? 1 : 0); ++second)
-                        j.q[((second ? j.nv : 0) + v) * j.ldq + p + int64_t(t) * j.plane] = 0;
+                        SliceRow<BLOCKED>(j, (second ? j.nv : 0) + v).at(p)[int64_t(t) * j.plane] = 0;
     }
 }
 
 // Blocks 0 .. j0.blocks - 1 split the first operand, the rest the second.
-template <int BITS, int S, bool CPLX>
+template <int BITS, int S, bool CPLX, bool BLOCKED>
 __global__ void __launch_bounds__(256, CPLX ? 4 : 2) ozaki_split_w_kernel(SplitJob j0, SplitJob j1, int bits, int s) {
     extern __shared__ double cache[];
     const bool first = blockIdx.x < j0.blocks;
     const SplitJob& j = first ? j0 : j1;
     const int64_t block = first ? blockIdx.x : blockIdx.x - j0.blocks;
-    if constexpr (CPLX) split_w_complex<BITS, S>(j, block, bits, s, cache);
-    else split_w_real<BITS, S>(j, block, bits, s);
+    if constexpr (CPLX) split_w_complex<BITS, S, BLOCKED>(j, block, bits, s, cache);
+    else split_w_real<BITS, S, BLOCKED>(j, block, bits, s);
 }
 template <int LX, bool CPLX>
 __global__ void __launch_bounds__(256) ozaki_scan_v_kernel(SplitJob j0, SplitJob j1) {
     const bool first = blockIdx.x < j0.blocks;
     scan_v<LX, CPLX>(first ? j0 : j1, first ? blockIdx.x : blockIdx.x - j0.blocks);
 }
-template <int BITS, int S, bool CPLX>
-__global__ void __launch_bounds__(256) ozaki_slice_v_kernel(SplitJob j0, SplitJob j1, int bits, int s) {
+template <int BITS, int S, bool CPLX, bool BLOCKED>
+__global__ void __launch_bounds__(256, CPLX ? 5 : BITS > 0 ? 8 : 6) ozaki_slice_v_kernel(SplitJob j0, SplitJob j1, int bits, int s) {
     const bool first = blockIdx.x < j0.blocks;
-    slice_v<BITS, S, CPLX>(first ? j0 : j1, first ? blockIdx.x : blockIdx.x - j0.blocks, bits, s);
+    slice_v<BITS, S, CPLX, BLOCKED>(first ? j0 : j1, first ? blockIdx.x : blockIdx.x - j0.blocks, bits, s);
 }
 
 }  // namespace
@@ -748,20 +768,32 @@ hsmm_status_t make_split_job(const SplitOperand& o, bool cplx, SplitJob* j) {
     j->M = static_cast<const double*>(o.M);
     j->ld = o.ld; j->nv = o.nv; j->nw = o.nw;
     j->expo = o.expo;
-    j->q = static_cast<uint16_t*>(o.q);
-    j->ldq = o.ldq; j->plane = o.plane;
+    const Slices& q = o.q;
+    j->ldq = q.ldq; j->plane = q.plane;
+    j->q = static_cast<uint16_t*>(q.q);
+    j->wt = 0; j->block = 0; j->tail = 0; j->tail_at = 0;
+    j->blocked = q.block_rows > 0;
+    if (!j->blocked) {
+        j->q += q.row0 * q.ldq;
+    } else {
+        j->wt = q.ldq / 64 * 64;
+        j->block = q.block_rows * 64;
+        j->tail = q.ldq - j->wt;
+        j->tail_at = j->wt * q.block_rows + q.row0 * (j->tail - 64);   // from q, which starts 64 row0 later
+        j->q += q.row0 * 64;
+    }
     j->v_contig = o.v_contig; j->conj = o.conj; j->role_b = o.role_b;
     j->vec_in = o.ld % 2 == 0 && aligned_to(o.M, 16);
-    j->vec_out = o.ldq % 4 == 0 && o.plane % 4 == 0 && aligned_to(o.q, 8);
+    j->vec_out = q.ldq % 4 == 0 && q.plane % 4 == 0 && aligned_to(q.q, 8);
     j->warps = 1;                  // as many warps per line as hold it in their registers
-    while (j->warps < 8 && o.ldq > int64_t(SPLIT_HELD) * 128 * j->warps) j->warps *= 2;
+    while (j->warps < 8 && q.ldq > int64_t(SPLIT_HELD) * 128 * j->warps) j->warps *= 2;
     j->cached = cplx && !o.v_contig && split_cache_bytes(o.nw) <= SPLIT_CACHE;
     const int lines = cplx ? 1 : 8 / j->warps;     // lines of a CTA (w contiguous)
     j->blocks = unsigned((o.nv + lines - 1) / lines);
     return HSMM_STATUS_SUCCESS;
 }
 
-template <int BITS, int S, bool CPLX>
+template <int BITS, int S, bool CPLX, bool BLOCKED>
 hsmm_status_t launch_split(SplitJob a, SplitJob b, int bits, int slices, cudaStream_t st) {
     cudaLaunchConfig_t lc = {};
     lc.blockDim = dim3(256, 1, 1);
@@ -797,9 +829,9 @@ hsmm_status_t launch_split(SplitJob a, SplitJob b, int bits, int slices, cudaStr
         b.blocks = slice_blocks(b);
         lc.numAttrs = 0;
         lc.gridDim = dim3(a.blocks + b.blocks, 1, 1);
-        e = cudaLaunchKernelEx(&lc, ozaki_slice_v_kernel<BITS, S, CPLX>, a, b, bits, slices);
+        e = cudaLaunchKernelEx(&lc, ozaki_slice_v_kernel<BITS, S, CPLX, BLOCKED>, a, b, bits, slices);
     } else {
-        auto kern = ozaki_split_w_kernel<BITS, S, CPLX>;
+        auto kern = ozaki_split_w_kernel<BITS, S, CPLX, BLOCKED>;
         if (CPLX) {
             static std::atomic<uint64_t> attrs{0};
             const hsmm_status_t as = attrs_once_per_device(attrs, [kern] {
@@ -818,8 +850,12 @@ hsmm_status_t launch_split(SplitJob a, SplitJob b, int bits, int slices, cudaStr
 
 hsmm_status_t launch_split(bool cplx, const SplitJob& a, const SplitJob& b, int bits, int slices, cudaStream_t st) {
     const bool fixed77 = bits == 7 && slices == 7;
-    if (cplx) return fixed77 ? launch_split<7, 7, true>(a, b, bits, slices, st) : launch_split<0, 0, true>(a, b, bits, slices, st);
-    return fixed77 ? launch_split<7, 7, false>(a, b, bits, slices, st) : launch_split<0, 0, false>(a, b, bits, slices, st);
+    using Fn = hsmm_status_t (*)(SplitJob, SplitJob, int, int, cudaStream_t);
+    static constexpr Fn fn[8] = {launch_split<0, 0, false, false>, launch_split<0, 0, false, true>,
+                                 launch_split<0, 0, true, false>,  launch_split<0, 0, true, true>,
+                                 launch_split<7, 7, false, false>, launch_split<7, 7, false, true>,
+                                 launch_split<7, 7, true, false>,  launch_split<7, 7, true, true>};
+    return fn[fixed77 * 4 + cplx * 2 + a.blocked](a, b, bits, slices, st);
 }
 
 }  // namespace
@@ -830,7 +866,7 @@ hsmm_status_t ozaki_split(bool cplx, const SplitOperand* ops, int count, int bit
         const hsmm_status_t r = make_split_job(ops[i], cplx, &j[i]);
         if (r != HSMM_STATUS_SUCCESS) return r;
     }
-    if (count == 1 || j[0].v_contig == j[1].v_contig) return launch_split(cplx, j[0], j[1], bits, slices, st);
+    if (count == 1 || (j[0].v_contig == j[1].v_contig && j[0].blocked == j[1].blocked)) return launch_split(cplx, j[0], j[1], bits, slices, st);
     const hsmm_status_t r = launch_split(cplx, j[0], SplitJob{}, bits, slices, st);
     return r != HSMM_STATUS_SUCCESS ? r : launch_split(cplx, j[1], SplitJob{}, bits, slices, st);
 }
