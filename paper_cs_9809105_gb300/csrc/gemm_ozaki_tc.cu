@@ -362,6 +362,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
     tc_fence_after();
     const uint32_t tmem = bars->tmem_base;
     volatile int* abort = &bars->abort;
+    pdl_wait();                    // the setup above overlaps the end of the split (or of the zeroing)
 
     const int tiles_m = (g.M + 2 * BM - 1) / (2 * BM);
     const int tiles_n = (g.N + PAIR_BN - 1) / PAIR_BN;
@@ -544,6 +545,8 @@ __global__ void __launch_bounds__(256) ozaki_zero_kernel(OzakiArgs g, int first_
     int tm, tn;
     tile_coords(first_tile + int(blockIdx.x), tiles_m, tiles_n, tm, tn);
     const int64_t row = int64_t(tm) * 2 * BM + threadIdx.x;
+    pdl_wait();
+    pdl_trigger();
     if (row >= g.M) return;
     int32_t* p = g.sd + int64_t(d_lo - 2 + int(blockIdx.y)) * g.sd_plane + row;
     const int64_t c1 = min(int64_t(g.N), int64_t(tn + 1) * PAIR_BN);
@@ -653,23 +656,13 @@ static hsmm_status_t launch_ozaki_pairs(const SliceMaps& mA, const SliceMaps& mB
     const OzSchedule& sc = oz_schedule(tiles, pairs, slices, (g.K + 63) / 64);
     if (sc.zero_from > 0) {
         const int tail = tiles % pairs;
-        ozaki_zero_kernel<<<dim3(unsigned(tail), unsigned(slices + 2 - sc.zero_from), 8), 256, 0, st>>>(
-            g, tiles - tail, sc.zero_from);
+        const cudaError_t ez = pdl_launch(ozaki_zero_kernel, dim3(unsigned(tail), unsigned(slices + 2 - sc.zero_from), 8),
+                                          256, 0, 1, st, g, tiles - tail, sc.zero_from);
         count_launches(1);
+        if (ez != cudaSuccess) return record_cuda(ez);
     }
-    cudaLaunchConfig_t lc = {};
-    lc.gridDim = dim3(unsigned(2 * pairs), 1, 1);
-    lc.blockDim = dim3(OZ_THREADS, 1, 1);
-    lc.dynamicSmemBytes = PAIR_SMEM;
-    lc.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = 2;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
-    lc.attrs = at;
-    lc.numAttrs = 1;
-    cudaError_t e = cudaLaunchKernelEx(&lc, gemm_ozaki_pair_kernel, mA, mB, g, sc.tab);
+    const cudaError_t e = pdl_launch(gemm_ozaki_pair_kernel, dim3(unsigned(2 * pairs)), OZ_THREADS, PAIR_SMEM, 2, st, mA, mB,
+                                     g, sc.tab);
     count_launches(1);
     if (e != cudaSuccess) return record_cuda(e);
     return check_launch();

@@ -50,18 +50,9 @@ constexpr int kThreads = 256;
 // form of op = N, where a wait costs more than the gap it hides (16384 x 16384 FP32: 155.8 us with
 // it, 150.0 without).  Between others the gap is 0.3 to 2.4 us: FP32 1000 x 1000 N 3.96 -> 3.58 us and
 // T 2.40 -> 2.02, INT8 2100 x 5300 N then T 14.35 -> 9.58.
-template <typename... P, typename... Q>
-cudaError_t pdl_launch(void (*kern)(P...), dim3 grid, cudaStream_t st, Q... args) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid;
-    cfg.blockDim = dim3(kThreads, 1, 1);
-    cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kern, P(args)...);
+template <typename K, typename... Q>
+cudaError_t launch(K kern, dim3 grid, cudaStream_t st, const Q&... args) {
+    return pdl_launch(kern, grid, kThreads, 0, 1, st, args...);
 }
 
 // ---------------------------------------------------------------------------
@@ -77,7 +68,7 @@ __global__ void __launch_bounds__(kThreads) gemv_f32_n_vec(int64_t m, int64_t n,
                                                            int64_t lda, const float* __restrict__ x, int64_t incx,
                                                            float* __restrict__ part, int64_t cols_per_split,
                                                            int rt, int64_t cols_per_group) {
-    if (!PLAIN) pdl_wait();   // see pdl_launch
+    if (!PLAIN) pdl_wait();   // see launch
     pdl_trigger();   // the reduction may be scheduled; it waits for this grid to finish
     if (PLAIN) rt = 8;
     const int tr = int(threadIdx.x) & ((1 << rt) - 1), group = PLAIN ? 0 : int(threadIdx.x) >> rt;
@@ -211,7 +202,7 @@ __global__ void __launch_bounds__(kThreads) gemv_reduce(int64_t m, int nsplit, c
 template <typename T, typename Acc>
 cudaError_t launch_reduce(int64_t m, int nsplit, const T* part, T alpha, T beta, T* y, int64_t incy,
                           cudaStream_t st) {
-    return pdl_launch(gemv_reduce<T, Acc>, dim3(unsigned((m + 31) / 32)), st, m, nsplit, part, alpha, beta, y, incy);
+    return launch(gemv_reduce<T, Acc>, dim3(unsigned((m + 31) / 32)), st, m, nsplit, part, alpha, beta, y, incy);
 }
 
 // ---------------------------------------------------------------------------
@@ -394,11 +385,11 @@ cudaError_t launch_t(int64_t m, int64_t n, S alpha, const T* A, int64_t lda, con
     const unsigned grid = unsigned((n + cols - 1) / cols);
     if constexpr (sizeof(T) == 4) {
         if (vec && g.shift == 0 && m % 4 == 0)
-            return pdl_launch(gemv_f32_t_plain, dim3(grid), st, g, A, x, alpha, beta, y);
+            return launch(gemv_f32_t_plain, dim3(grid), st, g, A, x, alpha, beta, y);
     }
-    if (vec) return pdl_launch(gemv_t_vec<T, V, S>, dim3(grid), st, g, A, x, alpha, beta, y);
-    if (incx == 1) return pdl_launch(gemv_t_scalar<T, S, true>, dim3(grid), st, g, A, x, alpha, beta, y);
-    return pdl_launch(gemv_t_scalar<T, S, false>, dim3(grid), st, g, A, x, alpha, beta, y);
+    if (vec) return launch(gemv_t_vec<T, V, S>, dim3(grid), st, g, A, x, alpha, beta, y);
+    if (incx == 1) return launch(gemv_t_scalar<T, S, true>, dim3(grid), st, g, A, x, alpha, beta, y);
+    return launch(gemv_t_scalar<T, S, false>, dim3(grid), st, g, A, x, alpha, beta, y);
 }
 
 // ---------------------------------------------------------------------------
@@ -430,7 +421,7 @@ __global__ void __launch_bounds__(kThreads) gemv_i8_n_vec(int64_t m, int64_t n, 
                                                           int64_t lda, const int8_t* __restrict__ x, int64_t incx,
                                                           int32_t* __restrict__ part, int64_t cols_per_split,
                                                           int rt, int64_t cols_per_group) {
-    if (!PLAIN) pdl_wait();   // see pdl_launch
+    if (!PLAIN) pdl_wait();   // see launch
     pdl_trigger();   // the reduction may be scheduled; it waits for this grid to finish
     if (PLAIN) rt = 8;                                       // see gemv_f32_n_vec; m % 16 == 0
     const int tr = int(threadIdx.x) & ((1 << rt) - 1), group = PLAIN ? 0 : int(threadIdx.x) >> rt;
@@ -622,11 +613,11 @@ hsmm_status_t gemv_f32(hsmm_op_t trans, int64_t m, int64_t n, float alpha, const
             if (sp.rt == 8 && m % 4 == 0)
                 gemv_f32_n_vec<true><<<sp.grid, kThreads, 0, st>>>(m, n, A, lda, x, incx, part, cps, 8, cps);
             else
-                e = pdl_launch(gemv_f32_n_vec<false>, sp.grid, st, m, n, A, lda, x, incx, part, cps, sp.rt,
+                e = launch(gemv_f32_n_vec<false>, sp.grid, st, m, n, A, lda, x, incx, part, cps, sp.rt,
                                sp.cols_per_group);
         } else {
             dim3 grid(unsigned((m + kThreads - 1) / kThreads), unsigned(ns));
-            e = pdl_launch(gemv_f32_n_scalar, grid, st, m, n, A, lda, x, incx, part, cps);
+            e = launch(gemv_f32_n_scalar, grid, st, m, n, A, lda, x, incx, part, cps);
         }
         if (e == cudaSuccess) e = launch_reduce<float, float>(m, ns, part, alpha, beta, y, incy, st);
         count_launches(2);
@@ -655,11 +646,11 @@ hsmm_status_t gemv_i8(hsmm_op_t trans, int64_t m, int64_t n, int32_t alpha, cons
             if (sp.rt == 8 && m % 16 == 0)
                 gemv_i8_n_vec<true><<<sp.grid, kThreads, 0, st>>>(m, n, A, lda, x, incx, part, cps, 8, cps);
             else
-                e = pdl_launch(gemv_i8_n_vec<false>, sp.grid, st, m, n, A, lda, x, incx, part, cps, sp.rt,
+                e = launch(gemv_i8_n_vec<false>, sp.grid, st, m, n, A, lda, x, incx, part, cps, sp.rt,
                                sp.cols_per_group);
         } else {
             dim3 grid(unsigned((m + kThreads - 1) / kThreads), unsigned(ns));
-            e = pdl_launch(gemv_i8_n_scalar, grid, st, m, n, A, lda, x, incx, part, cps);
+            e = launch(gemv_i8_n_scalar, grid, st, m, n, A, lda, x, incx, part, cps);
         }
         if (e == cudaSuccess) e = launch_reduce<int32_t, uint32_t>(m, ns, part, alpha, beta, y, incy, st);
         count_launches(2);

@@ -212,6 +212,10 @@ __device__ __forceinline__ void slice_store4_any(const double (&x)[4], int e, in
 //    through shared memory.  (As a programmatic dependent it was slower, 14.2 against 10.4 us at
 //    1000 x 900.  Slicing in the scanning cluster, the lines read again from L2, was slower
 //    from 2048 x 4096 on: 339 against 323 us at 8192^2, four CTAs per SM.)
+// All kernels of the form but the slicing one are programmatic dependents of the one before them
+// (pdl_launch), and the products let theirs start only at their end (from the start on: 2 us more at
+// 300 x 400 x 500).  Us a call, eager, before -> now: 128^3 23.2 -> 17.4 (op(A) = T) and 37.4 -> 25.7
+// (N), 300 x 400 x 500 33.3 -> 25.4 and 46.0 -> 34, 1000 x 1200 x 900 77.6 -> 69.5 and 89.8 -> 79.
 // Bound by DRAM at large sizes (8 bytes in, 2 s bytes out for each value) and by launches at small
 // ones: an operand took four launches before (initialise the exponents, scan, slice, fix up), the
 // scan read everything once more, and complex rows of odd length were stored two bytes at a
@@ -572,6 +576,8 @@ __device__ __forceinline__ void slice_v(const SplitJob& j, int64_t block, int bi
 template <int BITS, int S, bool CPLX, bool BLOCKED>
 __global__ void __launch_bounds__(256, CPLX ? 4 : 2) ozaki_split_w_kernel(SplitJob j0, SplitJob j1, int bits, int s) {
     extern __shared__ double cache[];
+    pdl_wait();
+    pdl_trigger();
     const bool first = blockIdx.x < j0.blocks;
     const SplitJob& j = first ? j0 : j1;
     const int64_t block = first ? blockIdx.x : blockIdx.x - j0.blocks;
@@ -580,11 +586,13 @@ __global__ void __launch_bounds__(256, CPLX ? 4 : 2) ozaki_split_w_kernel(SplitJ
 }
 template <int LX, bool CPLX>
 __global__ void __launch_bounds__(256) ozaki_scan_v_kernel(SplitJob j0, SplitJob j1) {
+    pdl_wait();
     const bool first = blockIdx.x < j0.blocks;
     scan_v<LX, CPLX>(first ? j0 : j1, first ? blockIdx.x : blockIdx.x - j0.blocks);
 }
 template <int BITS, int S, bool CPLX, bool BLOCKED>
 __global__ void __launch_bounds__(256, CPLX ? 5 : BITS > 0 ? 8 : 6) ozaki_slice_v_kernel(SplitJob j0, SplitJob j1, int bits, int s) {
+    pdl_trigger();
     const bool first = blockIdx.x < j0.blocks;
     slice_v<BITS, S, CPLX, BLOCKED>(first ? j0 : j1, first ? blockIdx.x : blockIdx.x - j0.blocks, bits, s);
 }
@@ -681,6 +689,8 @@ struct RecombineArgs {
 
 template <int V, bool F77, bool CPLX>
 __global__ void __launch_bounds__(256) ozaki_recombine_kernel(RecombineArgs g) {
+    pdl_wait();
+    pdl_trigger();
     const int64_t i = (int64_t(blockIdx.x) * 256 + threadIdx.x) * V;
     if (i >= g.m) return;
     int ei[V];
@@ -740,11 +750,13 @@ hsmm_status_t launch_recombine(const RecombineArgs& g, cudaStream_t st) {
                       aligned_to(g.C, 16) && (CPLX || g.ldc % 2 == 0);
     const bool f77 = g.s == 7 && g.bits == 7;
     const dim3 grid(unsigned(((vec4 ? g.m / 4 : g.m) + 255) / 256), unsigned(g.n < 65535 ? g.n : 65535));
-    if (vec4 && f77) ozaki_recombine_kernel<4, true, CPLX><<<grid, 256, 0, st>>>(g);
-    else if (vec4) ozaki_recombine_kernel<4, false, CPLX><<<grid, 256, 0, st>>>(g);
-    else if (f77) ozaki_recombine_kernel<1, true, CPLX><<<grid, 256, 0, st>>>(g);
-    else ozaki_recombine_kernel<1, false, CPLX><<<grid, 256, 0, st>>>(g);
+    auto kern = vec4 && f77 ? ozaki_recombine_kernel<4, true, CPLX>
+                : vec4      ? ozaki_recombine_kernel<4, false, CPLX>
+                : f77       ? ozaki_recombine_kernel<1, true, CPLX>
+                            : ozaki_recombine_kernel<1, false, CPLX>;
+    const cudaError_t e = pdl_launch(kern, grid, 256, 0, 1, st, g);
     count_launches(1);
+    if (e != cudaSuccess) return record_cuda(e);
     return check_launch();
 }
 
@@ -795,14 +807,6 @@ hsmm_status_t make_split_job(const SplitOperand& o, bool cplx, SplitJob* j) {
 
 template <int BITS, int S, bool CPLX, bool BLOCKED>
 hsmm_status_t launch_split(SplitJob a, SplitJob b, int bits, int slices, cudaStream_t st) {
-    cudaLaunchConfig_t lc = {};
-    lc.blockDim = dim3(256, 1, 1);
-    lc.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = 1;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
     cudaError_t e;
     if (a.v_contig) {
         // 128 lines per scanning CTA (1 KiB of a row of w), 32 where that leaves SMs idle; clusters
@@ -817,31 +821,25 @@ hsmm_status_t launch_split(SplitJob a, SplitJob b, int bits, int slices, cudaStr
         };
         a.blocks = scan_blocks(a);
         b.blocks = scan_blocks(b);
-        at[0].val.clusterDim.x = cs;
-        lc.attrs = at;
-        lc.numAttrs = 1;
-        lc.gridDim = dim3(a.blocks + b.blocks, 1, 1);
-        e = lines == 128 ? cudaLaunchKernelEx(&lc, ozaki_scan_v_kernel<64, CPLX>, a, b)
-                         : cudaLaunchKernelEx(&lc, ozaki_scan_v_kernel<16, CPLX>, a, b);
+        e = pdl_launch(lines == 128 ? ozaki_scan_v_kernel<64, CPLX> : ozaki_scan_v_kernel<16, CPLX>,
+                       dim3(a.blocks + b.blocks), 256, 0, cs, st, a, b);
         count_launches(1);
         if (e != cudaSuccess) return record_cuda(e);
         a.blocks = slice_blocks(a);
         b.blocks = slice_blocks(b);
-        lc.numAttrs = 0;
-        lc.gridDim = dim3(a.blocks + b.blocks, 1, 1);
-        e = cudaLaunchKernelEx(&lc, ozaki_slice_v_kernel<BITS, S, CPLX, BLOCKED>, a, b, bits, slices);
+        ozaki_slice_v_kernel<BITS, S, CPLX, BLOCKED><<<a.blocks + b.blocks, 256, 0, st>>>(a, b, bits, slices);
     } else {
         auto kern = ozaki_split_w_kernel<BITS, S, CPLX, BLOCKED>;
+        size_t smem = 0;
         if (CPLX) {
             static std::atomic<uint64_t> attrs{0};
             const hsmm_status_t as = attrs_once_per_device(attrs, [kern] {
                 return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(SPLIT_CACHE));
             });
             if (as != HSMM_STATUS_SUCCESS) return as;
-            lc.dynamicSmemBytes = std::max(a.cached ? split_cache_bytes(a.nw) : 0, b.cached ? split_cache_bytes(b.nw) : 0);
+            smem = std::max(a.cached ? split_cache_bytes(a.nw) : 0, b.cached ? split_cache_bytes(b.nw) : 0);
         }
-        lc.gridDim = dim3(a.blocks + b.blocks, 1, 1);
-        e = cudaLaunchKernelEx(&lc, kern, a, b, bits, slices);
+        e = pdl_launch(kern, dim3(a.blocks + b.blocks), 256, smem, 1, st, a, b, bits, slices);
     }
     count_launches(1);
     if (e != cudaSuccess) return record_cuda(e);
