@@ -50,7 +50,10 @@ __device__ __forceinline__ bool elect_one() {
 // Programmatic dependent launch: a kernel launched with programmatic stream serialization
 // may start while the previous kernel of the stream still runs; pdl_wait() blocks until
 // that kernel has completed and its memory operations are visible.  pdl_trigger() lets
-// the dependent kernel be scheduled once every CTA of this grid has issued it.
+// the dependent kernel be scheduled once every CTA of this grid has issued it.  Without it the
+// next kernel is placed as this one's CTAs leave, which already saves most of the gap between two
+// launches (2 to 3 us a call: native FP64 64^3 8.5 -> 5.9, n-body 1000 6.8 -> 5.4, 30 grouped
+// products 15.0 -> 12.9).
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 // launch such a kernel, in clusters of `cluster` CTAs (1: none)

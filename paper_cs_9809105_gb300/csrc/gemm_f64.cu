@@ -61,6 +61,7 @@ __global__ void __launch_bounds__(Tile<T>::NT, Tile<T>::OCC)
     constexpr int TH = Tile<T>::TH, RB = Tile<T>::RB;
     __shared__ double As[BK][T + 1];
     __shared__ double Bs[BK][T + 1];
+    pdl_wait();
     const int64_t m0 = int64_t(blockIdx.x) * T, n0 = int64_t(blockIdx.y) * T;
     const int tx = threadIdx.x % TH, ty = threadIdx.x / TH;
     double acc[RB][RB];
@@ -160,6 +161,7 @@ __global__ void __launch_bounds__(Tile<T>::NT) gemm_z64_kernel(int64_t m, int64_
     constexpr int TH = Tile<T>::TH, RB = Tile<T>::RB;
     __shared__ double2 As[ZK][T + 1];
     __shared__ double2 Bs[ZK][T + 1];     // Bs[kk][c] = op(B)(k0 + kk, n0 + c)
+    pdl_wait();
     const int64_t m0 = int64_t(blockIdx.x) * T, n0 = int64_t(blockIdx.y) * T;
     const int tx = threadIdx.x % TH, ty = threadIdx.x / TH;
     double accr[RB][RB], acci[RB][RB];
@@ -250,16 +252,18 @@ hsmm_status_t gemm_f64_native(hsmm_op_t ta, hsmm_op_t tb, int64_t m, int64_t n, 
     const int t = pick_tile(m, n, 64);
     const dim3 grid(unsigned((m + t - 1) / t), unsigned((n + t - 1) / t));
     if (grid.y > 65535u) return HSMM_STATUS_NOT_SUPPORTED;
+    cudaError_t e = cudaSuccess;
     auto launch = [&](auto tile) {
         constexpr int T = decltype(tile)::value;
-        gemm_f64_kernel<T><<<grid, Tile<T>::NT, 0, st>>>(m, n, k, alpha, A, lda, ta == HSMM_OP_T, B, ldb,
-                                                         tb == HSMM_OP_T, beta, C, ldc);
+        e = pdl_launch(gemm_f64_kernel<T>, grid, Tile<T>::NT, 0, 1, st, m, n, k, alpha, A, lda, ta == HSMM_OP_T, B, ldb,
+                       tb == HSMM_OP_T, beta, C, ldc);
     };
     if (t == 64) launch(std::integral_constant<int, 64>{});
     else if (t == 32) launch(std::integral_constant<int, 32>{});
     else if (t == 16) launch(std::integral_constant<int, 16>{});
     else launch(std::integral_constant<int, 8>{});
     count_launches(1);
+    if (e != cudaSuccess) return record_cuda(e);
     return check_launch();
 }
 
@@ -269,16 +273,18 @@ hsmm_status_t gemm_z64_native(hsmm_op_t ta, hsmm_op_t tb, int64_t m, int64_t n, 
     const int t = pick_tile(m, n, 32);
     const dim3 grid(unsigned((m + t - 1) / t), unsigned((n + t - 1) / t));
     if (grid.y > 65535u) return HSMM_STATUS_NOT_SUPPORTED;
+    cudaError_t e = cudaSuccess;
     auto launch = [&](auto tile) {
         constexpr int T = decltype(tile)::value;
-        gemm_z64_kernel<T><<<grid, Tile<T>::NT, 0, st>>>(
-            m, n, k, make_double2(alpha[0], alpha[1]), static_cast<const double2*>(A), lda, char(ta),
-            static_cast<const double2*>(B), ldb, char(tb), make_double2(beta[0], beta[1]), static_cast<double2*>(C), ldc);
+        e = pdl_launch(gemm_z64_kernel<T>, grid, Tile<T>::NT, 0, 1, st, m, n, k, make_double2(alpha[0], alpha[1]),
+                       static_cast<const double2*>(A), lda, char(ta), static_cast<const double2*>(B), ldb, char(tb),
+                       make_double2(beta[0], beta[1]), static_cast<double2*>(C), ldc);
     };
     if (t == 32) launch(std::integral_constant<int, 32>{});
     else if (t == 16) launch(std::integral_constant<int, 16>{});
     else launch(std::integral_constant<int, 8>{});
     count_launches(1);
+    if (e != cudaSuccess) return record_cuda(e);
     return check_launch();
 }
 

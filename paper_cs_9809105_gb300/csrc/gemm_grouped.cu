@@ -433,6 +433,7 @@ __global__ void __launch_bounds__(GP_THREADS, 1) gemm_grouped_pair_kernel(Groupe
     tc_fence_after();
     const uint32_t tmem = bars->tmem_base;
     volatile int* abort = &bars->abort;
+    pdl_wait();                    // launched as a programmatic dependent: the setup overlaps the kernel before
     const int64_t pair = int64_t(blockIdx.x >> 1), npairs = int64_t(gridDim.x >> 1);
 
     if (warp == 0 || warp == 2) {
@@ -940,19 +941,7 @@ static hsmm_status_t launch_grouped_pair(const GroupedArgs& a, cudaStream_t st) 
         attrs, [kern] { return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem); });
     if (as != HSMM_STATUS_SUCCESS) return as;
     const int64_t pairs = std::max<int64_t>(1, std::min<int64_t>(a.total_tiles, num_sms() / 2));
-    cudaLaunchConfig_t lc = {};
-    lc.gridDim = dim3(unsigned(2 * pairs), 1, 1);
-    lc.blockDim = dim3(GP_THREADS, 1, 1);
-    lc.dynamicSmemBytes = smem;
-    lc.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = 2;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
-    lc.attrs = at;
-    lc.numAttrs = 1;
-    cudaError_t e = cudaLaunchKernelEx(&lc, kern, a);
+    const cudaError_t e = pdl_launch(kern, dim3(unsigned(2 * pairs)), GP_THREADS, smem, 2, st, a);
     count_launches(1);
     if (e != cudaSuccess) return record_cuda(e);
     return check_launch();

@@ -131,6 +131,7 @@ __global__ void __launch_bounds__(NB_THREADS) nbody_tiled(int64_t nx, int64_t nz
     // two z tiles of NB_THREADS bodies (two float4 each), later the partial sums [warp][body]
     __shared__ float4 sm[2 * 2 * NB_THREADS];
     static_assert(2 * 2 * NB_THREADS >= NB_WARPS * NB_XB, "the partial sums reuse the z tiles");
+    pdl_wait();
     const int lane = int(lane_id()), warp = int(warp_id());
     const int zs = int(cluster_ctarank()), ZS = int(cluster_nctarank());
     const int64_t xblock = int64_t(blockIdx.x / ZS) * NB_XB;
@@ -336,19 +337,8 @@ hsmm_status_t nbody_forces(int64_t nx, int64_t nz, const float* x, const float* 
     if (ring_p == 0) {
         const int64_t xblocks = (nx + NB_XB - 1) / NB_XB;
         if (xblocks > INT32_MAX / NB_ZS) return HSMM_STATUS_NOT_SUPPORTED;
-        cudaLaunchConfig_t tc = {};
-        tc.gridDim = dim3(unsigned(xblocks * NB_ZS), 1, 1);
-        tc.blockDim = dim3(NB_THREADS, 1, 1);
-        tc.stream = st;
-        cudaLaunchAttribute ta[1];
-        ta[0].id = cudaLaunchAttributeClusterDimension;
-        ta[0].val.clusterDim.x = NB_ZS;
-        ta[0].val.clusterDim.y = 1;
-        ta[0].val.clusterDim.z = 1;
-        tc.attrs = ta;
-        tc.numAttrs = 1;
-        const cudaError_t te = packed ? cudaLaunchKernelEx(&tc, nbody_tiled<true>, nx, nz, x4, z4, eps2, o4)
-                                      : cudaLaunchKernelEx(&tc, nbody_tiled<false>, nx, nz, x4, z4, eps2, o4);
+        const cudaError_t te = pdl_launch(packed ? nbody_tiled<true> : nbody_tiled<false>, dim3(unsigned(xblocks * NB_ZS)),
+                                          NB_THREADS, 0, NB_ZS, st, nx, nz, x4, z4, eps2, o4);
         count_launches(1);
         if (te != cudaSuccess) return record_cuda(te);
         return check_launch();
