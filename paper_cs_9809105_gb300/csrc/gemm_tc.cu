@@ -165,6 +165,7 @@ struct GemmArgs {
     uint64_t timeout_ns;
     int c_tma;              // pair kernel: beta == 0 and C written by TMA stores through tmC
     int m_tma;              // rows of C that tmC covers: M rounded down to whole 16-byte units
+    int bn;                 // pair kernel: tile columns (a multiple of 32; 256 with an MN-major B)
 };
 
 // ---------------------------------------------------------------------------
@@ -488,7 +489,8 @@ __global__ void __launch_bounds__(PP_THREADS, 1)
     pdl_trigger();
 
     const int tiles_m = (g.M + 2 * BM - 1) / (2 * BM);
-    const int tiles_n = (g.N + PAIR_BN - 1) / PAIR_BN;
+    const int bn = g.bn, bhalf = bn / 2;          // columns of a tile, and those whose rows of B this CTA stages
+    const int tiles_n = (g.N + bn - 1) / bn;
     const int ntiles = tiles_m * tiles_n;
     const int pair = int(blockIdx.x >> 1), npairs = int(gridDim.x >> 1);
     const int nkb = (g.K + C_::BK - 1) / C_::BK;
@@ -500,11 +502,12 @@ __global__ void __launch_bounds__(PP_THREADS, 1)
         uint32_t phase = 0;
         bool ok = true;
         const uint32_t full0 = mapa_shared(smem_u32(&bars->full[0]), 0);
+        const uint32_t bytes = 2u * uint32_t(BM + bhalf) * 128u;      // both CTAs' copies
         for (int t = pair; t < ntiles && ok && !*abort; t += npairs) {
             int tm, tn;
             tile_coords(t, tiles_m, tiles_n, tm, tn);
             const int arow = tm * 2 * BM + int(rank) * BM;
-            const int brow = tn * PAIR_BN + int(rank) * BM;
+            const int brow = tn * bn + int(rank) * bhalf;
             for (int kb = 0; kb < nkb; ++kb) {
                 // the first round of stages starts empty
                 if (filled >= PP_STAGES &&
@@ -512,7 +515,7 @@ __global__ void __launch_bounds__(PP_THREADS, 1)
                 uint8_t* a_dst = smem + stage * PAIR_STAGE_BYTES;
                 uint8_t* b_dst = a_dst + BM * 128;
                 const uint32_t full_leader = full0 + uint32_t(stage) * 8u;
-                mbar_arrive_expect_tx_if(issue && leader, &bars->full[stage], 2 * PAIR_STAGE_BYTES);
+                mbar_arrive_expect_tx_if(issue && leader, &bars->full[stage], bytes);
                 if (!g.a_mn) {
                     tma_load_2d_pair_if(issue, a_dst, &tmA, full_leader, kb * C_::BK, arow);
                 } else if (g.a_mn3) {
@@ -528,8 +531,7 @@ __global__ void __launch_bounds__(PP_THREADS, 1)
                 } else if (g.b_mn3) {
                     tma_load_3d_pair_if(issue, b_dst, &tmB, full_leader, 0, kb * C_::BK, brow / C_::MN_CHUNK);
                 } else {
-#pragma unroll
-                    for (int c = 0; c < BM / C_::MN_CHUNK; ++c)
+                    for (int c = 0; c < bhalf / C_::MN_CHUNK; ++c)
                         tma_load_2d_pair_if(issue, b_dst + c * C_::BK * 128, &tmB, full_leader, brow + c * C_::MN_CHUNK,
                                             kb * C_::BK);
                 }
@@ -543,7 +545,7 @@ __global__ void __launch_bounds__(PP_THREADS, 1)
     } else if (warp == 1) {
         if (leader) {
             const bool issue = elect_one();
-            const uint32_t idesc = make_idesc(TF32 ? 2u : 1u, g.a_mn != 0, g.b_mn != 0, 2 * BM, PAIR_BN);
+            const uint32_t idesc = make_idesc(TF32 ? 2u : 1u, g.a_mn != 0, g.b_mn != 0, 2 * BM, uint32_t(bn));
             const uint64_t a0 = operand_desc<C_>(smem_u32(smem), 0, g.a_mn != 0);
             const uint64_t b0 = operand_desc<C_>(smem_u32(smem) + BM * 128, 0, g.b_mn != 0);
             const uint64_t aks = ks_step<C_>(g.a_mn != 0), bks = ks_step<C_>(g.b_mn != 0);
@@ -584,8 +586,9 @@ __global__ void __launch_bounds__(PP_THREADS, 1)
         // epilogue warps, the column half (w-2)/4 of them
         const int q = warp & 3;
         const int half = PP_EPI_WARPS == 8 ? (warp - 2) >> 2 : 0;
-        const int cbeg = PP_EPI_WARPS == 8 ? half * (PAIR_BN / 2) : 0;
-        const int cend = PP_EPI_WARPS == 8 ? cbeg + PAIR_BN / 2 : PAIR_BN;
+        const int cut = (bn / 2 + 31) / 32 * 32;
+        const int cbeg = PP_EPI_WARPS == 8 ? half * cut : 0;
+        const int cend = PP_EPI_WARPS == 8 && half == 0 ? cut : bn;
         float* stage_w = reinterpret_cast<float*>(stage_c) + (warp - 2) * PP_CBUF * 32 * 32;
         const uint32_t acc_empty_leader0 = mapa_shared(smem_u32(&bars->acc_empty[0]), 0);
         const uint32_t acc_empty_leader1 = mapa_shared(smem_u32(&bars->acc_empty[1]), 0);
@@ -606,7 +609,7 @@ __global__ void __launch_bounds__(PP_THREADS, 1)
             if (g.c_tma && row0 < g.M) {
                 // a TMA store clips the row (inner) dimension only to whole 16-byte units, so tmC
                 // covers the first m_tma rows; the (at most 7) rows after them are stored by their lanes
-                const int cols = min(cend, g.N - tn * PAIR_BN);
+                const int cols = min(cend, g.N - tn * bn);
                 const int64_t row = int64_t(row0) + lane;
                 const bool tail_lane = row >= g.m_tma && row < g.M;
 #pragma unroll 1
@@ -633,13 +636,13 @@ __global__ void __launch_bounds__(PP_THREADS, 1)
                         fence_proxy_async_smem();
                         __syncwarp();
                         if (lane == 0) {
-                            tma_store_2d(&tmC, sb, row0, tn * PAIR_BN + c0);
+                            tma_store_2d(&tmC, sb, row0, tn * bn + c0);
                             bulk_commit_group();
                         }
                         ++cbuf;
                     }
                     if (tail_lane) {
-                        const int64_t col0 = int64_t(tn) * PAIR_BN + c0;
+                        const int64_t col0 = int64_t(tn) * bn + c0;
 #pragma unroll
                         for (int j = 0; j < 32; ++j) {
                             if (col0 + j < g.N) {
@@ -659,7 +662,7 @@ __global__ void __launch_bounds__(PP_THREADS, 1)
                     uint32_t r[32];
                     tmem_ld32(t_base + uint32_t(c0), r);
                     tmem_ld_wait();
-                    const int64_t col0 = int64_t(tn) * PAIR_BN + c0;
+                    const int64_t col0 = int64_t(tn) * bn + c0;
                     if (row < g.M) {
 #pragma unroll
                         for (int j = 0; j < 32; ++j) {
@@ -706,7 +709,7 @@ hsmm_status_t launch_pair(const CUtensorMap& ta, const CUtensorMap& tb, const CU
     const hsmm_status_t as = attrs_once_per_device(
         attrs, [kern] { return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, PP_SMEM); });
     if (as != HSMM_STATUS_SUCCESS) return as;
-    const int ptiles = ((g.M + 2 * BM - 1) / (2 * BM)) * ((g.N + PAIR_BN - 1) / PAIR_BN);
+    const int ptiles = ((g.M + 2 * BM - 1) / (2 * BM)) * ((g.N + g.bn - 1) / g.bn);
     const int pairs = std::max(1, std::min(ptiles, num_sms() / 2));
     cudaLaunchConfig_t lc = {};
     lc.gridDim = dim3(unsigned(2 * pairs), 1, 1);
@@ -768,13 +771,33 @@ static TcKernel tc_kernel_choice() {
                                                                                            : TcKernel::Pair;
 }
 
+// Tile columns of the pair kernel.  256, or with a K-major B 224 or 192 where narrower tiles save
+// part of a last, half empty round over the pairs; `cost`: rounds, in those of 256-wide tiles.  A
+// round of 224 columns takes 0.94 of one of 256 and one of 192 0.82 (4096^3: 19.3, 18.1 and 15.8 us;
+// of 160 and of 128, which stage more bytes than L2 gives, 14.9).  Us, 256 -> chosen: 4096^3 77.1 ->
+// 72.5, 2048 x 4096 x 8192 78.0 -> 74.3, 5120 x 4096 x 1280 33.5 -> 31.5, 4392 x 1384 x 4152 53.8 ->
+// 47.1 (192); 8192 x 4096 x 2048 stays (73.9, 76.3 with 224).
+struct PairTile {
+    int bn;
+    double cost;
+};
+static PairTile pair_tile(int64_t m, int64_t n, bool b_mn) {
+    const int64_t pairs = num_sms() / 2, tiles_m = (m + 2 * BM - 1) / (2 * BM);
+    auto rounds = [&](int bn) { return double((tiles_m * ((n + bn - 1) / bn) + pairs - 1) / pairs); };
+    PairTile best{PAIR_BN, rounds(PAIR_BN)};
+    if (b_mn) return best;                        // chunks of 64 columns, two a CTA
+    for (const PairTile c : {PairTile{224, 0.94 * rounds(224)}, PairTile{192, 0.82 * rounds(192)}})
+        if (c.cost < 0.98 * best.cost) best = c;
+    return best;
+}
+
 // Estimated microseconds of a product on the persistent kernels below: launch and epilogue, then
 // a k-block of the widest tile for every tile of the busiest pair (or CTA).
-static double whole_tiles_cost(int64_t m, int64_t n, int64_t k, bool tf32) {
+static double whole_tiles_cost(int64_t m, int64_t n, int64_t k, bool tf32, bool b_mn) {
     const int64_t nkb = (k + (tf32 ? 31 : 63)) / (tf32 ? 32 : 64);
-    const int64_t rows = m > BM ? 2 * BM : BM, slots = m > BM ? num_sms() / 2 : num_sms();
-    const int64_t tiles = ((m + rows - 1) / rows) * ((n + PAIR_BN - 1) / PAIR_BN);
-    return 6.0 + double((tiles + slots - 1) / slots) * double(nkb) * (m > BM ? 0.27 : 0.35);
+    if (m > BM) return 6.0 + pair_tile(m, n, b_mn).cost * double(nkb) * 0.27;
+    const int64_t tiles = (n + PAIR_BN - 1) / PAIR_BN, slots = num_sms();
+    return 6.0 + double((tiles + slots - 1) / slots) * double(nkb) * 0.35;
 }
 
 hsmm_status_t gemm_tc(hsmm_dtype_t ab, hsmm_dtype_t c, hsmm_op_t ta, hsmm_op_t tb, int64_t m, int64_t n, int64_t k,
@@ -822,7 +845,7 @@ hsmm_status_t gemm_tc(hsmm_dtype_t ab, hsmm_dtype_t c, hsmm_op_t ta, hsmm_op_t t
     const TcKernel choice = tc_kernel_choice();
     if (tile_n == 0 && (choice == TcKernel::Auto || choice == TcKernel::Split)) {
         const SplitPlan plan = split_plan(m, n, k, tf32, g.b_mn);
-        if (plan.bn != 0 && (choice == TcKernel::Split || plan.cost < whole_tiles_cost(m, n, k, tf32))) {
+        if (plan.bn != 0 && (choice == TcKernel::Split || plan.cost < whole_tiles_cost(m, n, k, tf32, g.b_mn))) {
             CUtensorMap sA, sB;
             bool oks = g.a_mn ? (g.a_mn3 ? enc_mn3(&sA, A, m, lda, BM)
                                          : encode_map(&sA, dt, esize, A, uint64_t(m), uint64_t(k), uint64_t(lda),
@@ -862,10 +885,12 @@ hsmm_status_t gemm_tc(hsmm_dtype_t ab, hsmm_dtype_t c, hsmm_op_t ta, hsmm_op_t t
                                      : encode_map(&pA, dt, esize, A, uint64_t(m), uint64_t(k), uint64_t(lda), MN_CHUNK,
                                                   BK, 0, 0, mn_sw))
                           : encode_map(&pA, dt, esize, A, uint64_t(k), uint64_t(m), uint64_t(lda), BK, BM);
+        g.bn = tile_n == 0 ? pair_tile(m, n, g.b_mn).bn : PAIR_BN;
         okp = okp && (g.b_mn ? (g.b_mn3 ? enc_mn3(&pB, B, n, ldb, BM)
                                         : encode_map(&pB, dt, esize, B, uint64_t(n), uint64_t(k), uint64_t(ldb),
                                                      MN_CHUNK, BK, 0, 0, mn_sw))
-                             : encode_map(&pB, dt, esize, B, uint64_t(k), uint64_t(n), uint64_t(ldb), BK, BM));
+                             : encode_map(&pB, dt, esize, B, uint64_t(k), uint64_t(n), uint64_t(ldb), BK,
+                                          uint32_t(g.bn / 2)));
         if (!okp) return fail(HSMM_STATUS_NOT_SUPPORTED, "gemm: TMA descriptor encoding failed (CUresult %d)",
                               g_last_encode_result);
         if (tf32) {
