@@ -397,7 +397,7 @@ def run_precise(args, world, rank, local):
         serial_ms = _time_loop(torch, e2e_serial_step, e2e_reps)
         e2e = {"value": world * flops / (e2e_ms / 1e3) / 1e12, "unit": "TFLOP/s", "ms_per_step": e2e_ms,
                "h2d_bytes_per_step": 2 * M * K * 8, "d2h_bytes_per_step": M * N * 8,
-               "api": "hsmm_gemm_host (page-locked host buffers; C in 4 x 2 blocks of 2048 x 4096)",
+               "api": "hsmm_gemm_host (page-locked host buffers; C in blocks of row and column panels)",
                "serial_copies_ms_per_step": serial_ms}
 
     line = None

@@ -56,25 +56,35 @@ __device__ __forceinline__ bool elect_one() {
 // products 15.0 -> 12.9).
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-// launch such a kernel, in clusters of `cluster` CTAs (1: none)
+// launch a kernel in clusters of `cluster` CTAs (1: none), as a programmatic dependent or not
 template <typename... P, typename... Q>
-cudaError_t pdl_launch(void (*kern)(P...), dim3 grid, int threads, size_t smem, unsigned cluster, cudaStream_t st,
-                       const Q&... args) {
+cudaError_t cluster_launch(bool dependent, void (*kern)(P...), dim3 grid, int threads, size_t smem, unsigned cluster,
+                           cudaStream_t st, const Q&... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = dim3(unsigned(threads), 1, 1);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cudaLaunchAttribute at[2];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    at[1].id = cudaLaunchAttributeClusterDimension;
-    at[1].val.clusterDim.x = cluster;
-    at[1].val.clusterDim.y = 1;
-    at[1].val.clusterDim.z = 1;
+    unsigned n = 0;
+    if (dependent) {
+        at[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[n++].val.programmaticStreamSerializationAllowed = 1;
+    }
+    if (cluster > 1) {
+        at[n].id = cudaLaunchAttributeClusterDimension;
+        at[n].val.clusterDim.x = cluster;
+        at[n].val.clusterDim.y = 1;
+        at[n++].val.clusterDim.z = 1;
+    }
     cfg.attrs = at;
-    cfg.numAttrs = cluster > 1 ? 2 : 1;
+    cfg.numAttrs = n;
     return cudaLaunchKernelEx(&cfg, kern, P(args)...);
+}
+template <typename... P, typename... Q>
+cudaError_t pdl_launch(void (*kern)(P...), dim3 grid, int threads, size_t smem, unsigned cluster, cudaStream_t st,
+                       const Q&... args) {
+    return cluster_launch(true, kern, grid, threads, smem, cluster, st, args...);
 }
 
 // ---------------------------------------------------------------------------

@@ -59,6 +59,7 @@ struct OzakiArgs {
     int32_t* sd;        // S_d, d = 2..s+1, as [d-2][N][M] INT32 (column-major per anti-diagonal)
     int64_t sd_plane;   // elements between consecutive anti-diagonal planes
     uint64_t timeout_ns;
+    int blocked;            // the slices are in blocks of 64 columns
 };
 
 constexpr int OZ_BN = 256;
@@ -92,8 +93,9 @@ struct OzWork {
 };
 constexpr int OZ_MAX_PAIRS = 100, OZ_MAX_UNITS = 1600;   // at most 16 units for each of 99 tail tiles
 
-// The slices of one operand as k-blocks of 64 columns (box 64 x rows x 1 x 1 at column 0, row, block,
-// slice), and what remains of k after them (one block, zero-filled); see Slices for the two layouts.
+// The slices of one operand.  Row-major: `blocks` is all of them, boxes at (column, row, 0, slice).  In
+// blocks of 64 columns (see Slices): `blocks` the whole ones, boxes at (0, row, block, slice), and
+// `rest` the columns after them, zero-filled.
 // Blocks of whole lines are what the tensor cores can be fed from: rows of a pitch of 8 to 56 columns
 // more than a multiple of 64 cross a line with every 64 columns, and an odd multiple of 8 a sector,
 // and the products then waited for loads (690 cycles a k-block instead of 523).  2048 x 2048 x 4100:
@@ -186,9 +188,9 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
                             uint8_t* b_dst = a_dst + C_::A_BYTES;
                             mbar_arrive_expect_tx(&bars->full[stage], C_::STAGE_BYTES);
                             const bool rest = kb >= nfull;
-                            const int block = rest ? 0 : kb;
-                            tma_load_4d(a_dst, rest ? &mA.rest : &mA.blocks, &bars->full[stage], 0, tm * BM, block, ta - 1);
-                            tma_load_4d(b_dst, rest ? &mB.rest : &mB.blocks, &bars->full[stage], 0, tn * OZ_BN, block,
+                            const int col = g.blocked ? 0 : kb * C_::BK, block = g.blocked && !rest ? kb : 0;
+                            tma_load_4d(a_dst, rest ? &mA.rest : &mA.blocks, &bars->full[stage], col, tm * BM, block, ta - 1);
+                            tma_load_4d(b_dst, rest ? &mB.rest : &mB.blocks, &bars->full[stage], col, tn * OZ_BN, block,
                                         ub - 1);
                             last_parity[stage] = int(phase);
                             if (++stage == C_::STAGES) { stage = 0; phase ^= 1u; }
@@ -400,10 +402,10 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
                         const uint32_t full_leader = full0 + uint32_t(stage) * 8u;
                         mbar_arrive_expect_tx_if(issue && leader, &bars->full[stage], 2 * PAIR_STAGE_BYTES);
                         const bool rest = kb >= nfull;
-                        const int block = rest ? 0 : kb;
-                        tma_load_4d_pair_if(issue, a_dst, rest ? &mA.rest : &mA.blocks, full_leader, 0, arow, block,
+                        const int col = g.blocked ? 0 : kb * C_::BK, block = g.blocked && !rest ? kb : 0;
+                        tma_load_4d_pair_if(issue, a_dst, rest ? &mA.rest : &mA.blocks, full_leader, col, arow, block,
                                             ta - 1);
-                        tma_load_4d_pair_if(issue, a_dst + BM * 128, rest ? &mB.rest : &mB.blocks, full_leader, 0, brow,
+                        tma_load_4d_pair_if(issue, a_dst + BM * 128, rest ? &mB.rest : &mB.blocks, full_leader, col, brow,
                                             block, ub - 1);
                         ++filled;
                         if (++stage == PAIR_STAGES) { stage = 0; phase ^= 1u; }
@@ -661,33 +663,36 @@ static hsmm_status_t launch_ozaki_pairs(const SliceMaps& mA, const SliceMaps& mB
         count_launches(1);
         if (ez != cudaSuccess) return record_cuda(ez);
     }
-    const cudaError_t e = pdl_launch(gemm_ozaki_pair_kernel, dim3(unsigned(2 * pairs)), OZ_THREADS, PAIR_SMEM, 2, st, mA, mB,
-                                     g, sc.tab);
+    // A programmatic dependent is placed as SMs come free, not in order, and tiles that share operands
+    // then sit on different halves of the chip: 8192^3 in a row, power-capped, 19.35 -> 19.95 ms.  The 2 us
+    // it saves are worth that only while the products are short (1000 k-blocks a pair, 270 us; 2048^3,
+    // 754, 307.6 -> 303.8 us a call).
+    const bool is_short = double(tiles) * slices * (slices + 1) / 2 * ((g.K + 63) / 64) < 1000.0 * pairs;
+    const cudaError_t e = cluster_launch(is_short, gemm_ozaki_pair_kernel, dim3(unsigned(2 * pairs)), OZ_THREADS, PAIR_SMEM, 2,
+                                         st, mA, mB, g, sc.tab);
     count_launches(1);
     if (e != cudaSuccess) return record_cuda(e);
     return check_launch();
 }
 
-// maps of the slices of `rows` rows and k columns, boxes of box_rows x 64
+// Maps of the slices of `rows` rows and k columns, boxes of box_rows x 64.  Row-major slices are one
+// tensor with all of k inside, so that an L2 fetch may take two neighbouring lines of a row.
 static bool slice_maps(const Slices& q, int64_t rows, int64_t k, int slices, uint32_t box_rows, SliceMaps* m) {
     const uint16_t* base = static_cast<const uint16_t*>(q.q);
-    const int64_t full = k / 64, rem = k % 64;
-    // row pitch and start of the blocks of 64 columns, and of the columns after them
-    int64_t pitch = q.ldq, step = 64, at = q.row0 * q.ldq, rest_pitch = q.ldq, rest_at = at + full * 64;
-    if (q.block_rows > 0) {                       // ldq / 64 == full: ldq is k rounded up to 8, and not to 64
-        pitch = 64;
-        step = q.block_rows * 64;
-        at = q.row0 * 64;
-        rest_pitch = q.ldq % 64;
-        rest_at = full * step + q.row0 * rest_pitch;
-    }
-    auto encode = [&](CUtensorMap* map, int64_t from, int64_t cols, int64_t ld, int64_t blocks) {
+    auto encode = [&](CUtensorMap* map, int64_t from, int64_t cols, int64_t ld, int64_t blocks, int64_t step) {
         return encode_map(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, base + from, uint64_t(cols), uint64_t(rows),
                           uint64_t(ld), 64, box_rows, uint64_t(slices), uint64_t(q.plane), CU_TENSOR_MAP_SWIZZLE_128B, 1,
                           uint64_t(blocks), uint64_t(step));
     };
-    if (full > 0 && !encode(&m->blocks, at, 64, pitch, full)) return false;
-    if (rem > 0 && !encode(&m->rest, rest_at, rem, rest_pitch, 1)) return false;
+    if (q.block_rows == 0) {
+        if (!encode(&m->blocks, q.row0 * q.ldq, k, q.ldq, 1, 64)) return false;
+        m->rest = m->blocks;
+        return true;
+    }
+    const int64_t full = k / 64, rem = k % 64;    // ldq / 64 == full: ldq is k rounded up to 8, and not to 64
+    const int64_t step = q.block_rows * 64, rest_pitch = q.ldq % 64;
+    if (full > 0 && !encode(&m->blocks, q.row0 * 64, 64, 64, full, step)) return false;
+    if (rem > 0 && !encode(&m->rest, full * step + q.row0 * rest_pitch, rem, rest_pitch, 1, 64)) return false;
     if (full == 0) m->blocks = m->rest;
     if (rem == 0) m->rest = m->blocks;
     return true;
@@ -707,6 +712,7 @@ hsmm_status_t gemm_ozaki_slices(int64_t m, int64_t n, int64_t k, int slices, int
     g.M = int(m); g.N = int(n); g.K = int(k);
     g.slices = slices; g.kc_blocks = kc_blocks;
     g.sd = sd;
+    g.blocked = qa.block_rows > 0;      // A and B alike: it follows from ldq
     g.sd_plane = sd_plane;
     g.timeout_ns = wait_timeout_ns();
     if (ozaki_pairs_enabled()) {

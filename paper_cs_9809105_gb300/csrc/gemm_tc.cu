@@ -761,7 +761,7 @@ hsmm_status_t launch_plain(const CUtensorMap& ta, const CUtensorMap& tb, const C
 }  // namespace
 
 // HSMM_GEMM_KERNEL chooses the kernel: "single" one CTA per tile, "split" narrow tiles with the
-// contraction split over a cluster (gemm_split_tc.cu), anything else 256-wide tiles on CTA pairs;
+// contraction split over a cluster (gemm_split_tc.cu), anything else wide tiles on CTA pairs;
 // unset: by the product's size.
 enum class TcKernel { Auto, Pair, Single, Split };
 static TcKernel tc_kernel_choice() {

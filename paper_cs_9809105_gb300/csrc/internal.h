@@ -193,7 +193,7 @@ size_t ring_workspace_bytes(int p, int K, int64_t n);
 hsmm_status_t ring_gemm_f64(int p, int K, int64_t n, const double* A, int64_t lda, const double* B, int64_t ldb,
                             double* C, int64_t ldc, void* workspace, size_t workspace_bytes, cudaStream_t st);
 
-// ---- grouped (gemm_tc.cu) ----
+// ---- gemm_grouped.cu ----
 struct GroupedPlan;
 hsmm_status_t grouped_plan_create(hsmm_dtype_t ab, hsmm_dtype_t c, int64_t count, const hsmm_gemm_desc_t* descs,
                                   int tile_n, GroupedPlan** out);

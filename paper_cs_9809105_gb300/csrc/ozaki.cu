@@ -212,9 +212,9 @@ __device__ __forceinline__ void slice_store4_any(const double (&x)[4], int e, in
 //    through shared memory.  (As a programmatic dependent it was slower, 14.2 against 10.4 us at
 //    1000 x 900.  Slicing in the scanning cluster, the lines read again from L2, was slower
 //    from 2048 x 4096 on: 339 against 323 us at 8192^2, four CTAs per SM.)
-// All kernels of the form but the slicing one are programmatic dependents of the one before them
-// (pdl_launch), and the products let theirs start only at their end (from the start on: 2 us more at
-// 300 x 400 x 500).  Us a call, eager, before -> now: 128^3 23.2 -> 17.4 (op(A) = T) and 37.4 -> 25.7
+// All kernels of the form but the slicing one and long products are programmatic dependents of the one
+// before them (pdl_launch), and the products let theirs start only at their end (from the start on:
+// 2 us more at 300 x 400 x 500).  Us a call, eager, before -> now: 128^3 23.2 -> 17.4 (op(A) = T) and 37.4 -> 25.7
 // (N), 300 x 400 x 500 33.3 -> 25.4 and 46.0 -> 34, 1000 x 1200 x 900 77.6 -> 69.5 and 89.8 -> 79.
 // Bound by DRAM at large sizes (8 bytes in, 2 s bytes out for each value) and by launches at small
 // ones: an operand took four launches before (initialise the exponents, scan, slice, fix up), the
