@@ -87,6 +87,29 @@ cudaError_t pdl_launch(void (*kern)(P...), dim3 grid, int threads, size_t smem, 
     return cluster_launch(true, kern, grid, threads, smem, cluster, st, args...);
 }
 
+// Ordinary (coherent) loads that keep their place among each other and after pdl_wait, so that a round
+// of them stays in flight together
+__device__ __forceinline__ float load(const float* p) {
+    float v;
+    asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ int8_t load(const int8_t* p) {
+    int v;
+    asm volatile("ld.global.s8 %0, [%1];" : "=r"(v) : "l"(p));
+    return int8_t(v);
+}
+__device__ __forceinline__ float4 load(const float4* p) {
+    float4 v;
+    asm volatile("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ int4 load(const int4* p) {
+    int4 v;
+    asm volatile("ld.global.v4.s32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+    return v;
+}
+
 // ---------------------------------------------------------------------------
 // mbarrier
 // ---------------------------------------------------------------------------

@@ -28,6 +28,9 @@ namespace {
 
 constexpr int BK = 16;
 
+// The product kernels are launched as programmatic dependents: resident while the kernel before still
+// writes what they read, so their operands are not const __restrict__ (read-only data).
+
 // T x T tiles on TH x TH threads, a (T / TH)^2 register block each
 template <int T>
 struct Tile {
@@ -40,7 +43,7 @@ struct Tile {
 // Load the T x BK tile of op(M) at (r0, k0) into s[k][r] (zero outside); along_k: op(M)(r, kk) =
 // M[kk + r ld] (kk contiguous), else M[r + kk ld].
 template <int T>
-__device__ __forceinline__ void load_tile(double (*s)[T + 1], const double* __restrict__ M, int64_t ld, bool along_k,
+__device__ __forceinline__ void load_tile(double (*s)[T + 1], const double* M, int64_t ld, bool along_k,
                                           int64_t rows, int64_t kdim, int64_t r0, int64_t k0) {
     constexpr int NT = Tile<T>::NT;
     const int t = threadIdx.x;
@@ -55,8 +58,8 @@ __device__ __forceinline__ void load_tile(double (*s)[T + 1], const double* __re
 
 template <int T>
 __global__ void __launch_bounds__(Tile<T>::NT, Tile<T>::OCC)
-    gemm_f64_kernel(int64_t m, int64_t n, int64_t k, double alpha, const double* __restrict__ A, int64_t lda, bool ta,
-                    const double* __restrict__ B, int64_t ldb, bool tb, double beta, double* __restrict__ C,
+    gemm_f64_kernel(int64_t m, int64_t n, int64_t k, double alpha, const double* A, int64_t lda, bool ta,
+                    const double* B, int64_t ldb, bool tb, double beta, double* C,
                     int64_t ldc) {
     constexpr int TH = Tile<T>::TH, RB = Tile<T>::RB;
     __shared__ double As[BK][T + 1];
@@ -135,7 +138,7 @@ constexpr int ZK = 16;
 
 // Load the T x ZK tile of op(M) at (r0, k0) into s[k][r] (zero outside, conjugated for conj)
 template <int T>
-__device__ __forceinline__ void load_ztile(double2 (*s)[T + 1], const double2* __restrict__ M, int64_t ld, bool along_k,
+__device__ __forceinline__ void load_ztile(double2 (*s)[T + 1], const double2* M, int64_t ld, bool along_k,
                                            bool conj, int64_t rows, int64_t kdim, int64_t r0, int64_t k0) {
     constexpr int NT = Tile<T>::NT;
     const int t = threadIdx.x;
@@ -155,9 +158,9 @@ __device__ __forceinline__ void load_ztile(double2 (*s)[T + 1], const double2* _
 
 template <int T>
 __global__ void __launch_bounds__(Tile<T>::NT) gemm_z64_kernel(int64_t m, int64_t n, int64_t k, double2 alpha,
-                                                              const double2* __restrict__ A, int64_t lda, char ta,
-                                                              const double2* __restrict__ B, int64_t ldb, char tb,
-                                                              double2 beta, double2* __restrict__ C, int64_t ldc) {
+                                                              const double2* A, int64_t lda, char ta,
+                                                              const double2* B, int64_t ldb, char tb,
+                                                              double2 beta, double2* C, int64_t ldc) {
     constexpr int TH = Tile<T>::TH, RB = Tile<T>::RB;
     __shared__ double2 As[ZK][T + 1];
     __shared__ double2 Bs[ZK][T + 1];     // Bs[kk][c] = op(B)(k0 + kk, n0 + c)

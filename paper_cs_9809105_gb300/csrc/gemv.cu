@@ -50,6 +50,9 @@ constexpr int kThreads = 256;
 // form of op = N, where a wait costs more than the gap it hides (16384 x 16384 FP32: 155.8 us with
 // it, 150.0 without).  Between others the gap is 0.3 to 2.4 us: FP32 1000 x 1000 N 3.96 -> 3.58 us and
 // T 2.40 -> 2.02, INT8 2100 x 5300 N then T 14.35 -> 9.58.
+// They are resident while that kernel still writes what they read, so nothing is loaded as read-only
+// data: no __ldg, no const __restrict__ (which the compiler turns into the same non-coherent loads and
+// may move above the wait), but load() (INT8 14580 x 24 T 3.1 us, 4.4 with plain dereferences).
 template <typename K, typename... Q>
 cudaError_t launch(K kern, dim3 grid, cudaStream_t st, const Q&... args) {
     return pdl_launch(kern, grid, kThreads, 0, 1, st, args...);
@@ -64,9 +67,9 @@ cudaError_t launch(K kern, dim3 grid, cudaStream_t st, const Q&... args) {
 // a thread then has fewer columns to walk one latency after the other.  PLAIN: no groups and m % 4
 // == 0 (34 registers instead of 60: 22.0 against 22.9 us at 8192 x 4096).
 template <bool PLAIN>
-__global__ void __launch_bounds__(kThreads) gemv_f32_n_vec(int64_t m, int64_t n, const float* __restrict__ A,
-                                                           int64_t lda, const float* __restrict__ x, int64_t incx,
-                                                           float* __restrict__ part, int64_t cols_per_split,
+__global__ void __launch_bounds__(kThreads) gemv_f32_n_vec(int64_t m, int64_t n, const float* A,
+                                                           int64_t lda, const float* x, int64_t incx,
+                                                           float* part, int64_t cols_per_split,
                                                            int rt, int64_t cols_per_group) {
     if (!PLAIN) pdl_wait();   // see launch
     pdl_trigger();   // the reduction may be scheduled; it waits for this grid to finish
@@ -92,7 +95,7 @@ __global__ void __launch_bounds__(kThreads) gemv_f32_n_vec(int64_t m, int64_t n,
 #pragma unroll
         for (int u = 0; u < 8; ++u) v[u] = __ldcs(reinterpret_cast<const float4*>(a + (j + u) * lda));
 #pragma unroll
-        for (int u = 0; u < 8; ++u) xs[u] = __ldg(x + (j + u) * incx);
+        for (int u = 0; u < 8; ++u) xs[u] = load(x + (j + u) * incx);
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
             acc.x = fmaf(v[u].x, xs[u], acc.x);
@@ -103,18 +106,18 @@ __global__ void __launch_bounds__(kThreads) gemv_f32_n_vec(int64_t m, int64_t n,
     }
     for (; j < jv; ++j) {
         float4 v = __ldcs(reinterpret_cast<const float4*>(a + j * lda));
-        float xv = __ldg(x + j * incx);
+        float xv = load(x + j * incx);
         acc.x = fmaf(v.x, xv, acc.x);
         acc.y = fmaf(v.y, xv, acc.y);
         acc.z = fmaf(v.z, xv, acc.z);
         acc.w = fmaf(v.w, xv, acc.w);
     }
     if (!PLAIN && jv < j1) {      // the last column of a matrix whose rows end inside this vector
-        const float xv = __ldg(x + jv * incx);
+        const float xv = load(x + jv * incx);
         const float* c = a + jv * lda;
-        acc.x = fmaf(__ldg(c), xv, acc.x);
-        if (r0 + 1 < m) acc.y = fmaf(__ldg(c + 1), xv, acc.y);
-        if (r0 + 2 < m) acc.z = fmaf(__ldg(c + 2), xv, acc.z);
+        acc.x = fmaf(load(c), xv, acc.x);
+        if (r0 + 1 < m) acc.y = fmaf(load(c + 1), xv, acc.y);
+        if (r0 + 2 < m) acc.z = fmaf(load(c + 2), xv, acc.z);
     }
     if constexpr (!PLAIN) {
         __shared__ float4 red[kThreads];
@@ -142,9 +145,9 @@ __global__ void __launch_bounds__(kThreads) gemv_f32_n_vec(int64_t m, int64_t n,
 }
 
 // Scalar path (unaligned columns): 1 row per thread.
-__global__ void __launch_bounds__(kThreads) gemv_f32_n_scalar(int64_t m, int64_t n, const float* __restrict__ A,
-                                                              int64_t lda, const float* __restrict__ x,
-                                                              int64_t incx, float* __restrict__ part,
+__global__ void __launch_bounds__(kThreads) gemv_f32_n_scalar(int64_t m, int64_t n, const float* A,
+                                                              int64_t lda, const float* x,
+                                                              int64_t incx, float* part,
                                                               int64_t cols_per_split) {
     pdl_wait();
     pdl_trigger();   // the reduction may be scheduled; it waits for this grid to finish
@@ -159,9 +162,9 @@ __global__ void __launch_bounds__(kThreads) gemv_f32_n_scalar(int64_t m, int64_t
 #pragma unroll
         for (int u = 0; u < 8; ++u) v[u] = __ldcs(A + r + (j + u) * lda);
 #pragma unroll
-        for (int u = 0; u < 8; ++u) acc = fmaf(v[u], __ldg(x + (j + u) * incx), acc);
+        for (int u = 0; u < 8; ++u) acc = fmaf(v[u], load(x + (j + u) * incx), acc);
     }
-    for (; j < j1; ++j) acc = fmaf(A[r + j * lda], __ldg(x + j * incx), acc);
+    for (; j < j1; ++j) acc = fmaf(A[r + j * lda], load(x + j * incx), acc);
     part[int64_t(blockIdx.y) * m + r] = acc;
 }
 
@@ -170,8 +173,8 @@ __global__ void __launch_bounds__(kThreads) gemv_f32_n_scalar(int64_t m, int64_t
 // order, so the result is deterministic.  Launched as a programmatic dependent of the split
 // kernel: the CTAs start while the splits finish and wait for them on the device.
 template <typename T, typename Acc>
-__global__ void __launch_bounds__(kThreads) gemv_reduce(int64_t m, int nsplit, const T* __restrict__ part, T alpha,
-                                                        T beta, T* __restrict__ y, int64_t incy) {
+__global__ void __launch_bounds__(kThreads) gemv_reduce(int64_t m, int nsplit, const T* part, T alpha,
+                                                        T beta, T* y, int64_t incy) {
     pdl_wait();
     pdl_trigger();
     const int r = int(lane_id()), g = int(warp_id());
@@ -269,9 +272,9 @@ __device__ __forceinline__ void t_finish(const GemvT& g, S acc, int64_t col, int
 // FP32, aligned columns of a whole number of vectors and aligned x, incx == 1, one warp per column:
 // all loads of a round are in flight before the first is used (166 -> 157.5 us at 16384^2, 6.8
 // TB/s).  The same loop was slower for INT8 (44.3 us at 16384^2 against 40.5 for the general one).
-__global__ void __launch_bounds__(kThreads) gemv_f32_t_plain(GemvT g, const float* __restrict__ A,
-                                                             const float* __restrict__ x, float alpha, float beta,
-                                                             float* __restrict__ y) {
+__global__ void __launch_bounds__(kThreads) gemv_f32_t_plain(GemvT g, const float* A,
+                                                             const float* x, float alpha, float beta,
+                                                             float* y) {
     pdl_wait();
     pdl_trigger();
     const int lane = int(lane_id());
@@ -287,11 +290,11 @@ __global__ void __launch_bounds__(kThreads) gemv_f32_t_plain(GemvT g, const floa
 #pragma unroll
         for (int u = 0; u < 4; ++u) v[u] = load_stream(a + i + 32 * u);
 #pragma unroll
-        for (int u = 0; u < 4; ++u) w[u] = __ldg(xp + i + 32 * u);
+        for (int u = 0; u < 4; ++u) w[u] = load(xp + i + 32 * u);
 #pragma unroll
         for (int u = 0; u < 4; ++u) t_fma(v[u], w[u], acc);
     }
-    for (; i < mv; i += 32) t_fma(__ldcs(a + i), __ldg(xp + i), acc);
+    for (; i < mv; i += 32) t_fma(__ldcs(a + i), load(xp + i), acc);
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
     if (lane == 0) t_store(g, alpha, beta, y, col, acc);
@@ -300,8 +303,8 @@ __global__ void __launch_bounds__(kThreads) gemv_f32_t_plain(GemvT g, const floa
 // The general form: m any, 2^g.shift warps per column.  T: element (float, int8_t), V: 16-byte
 // vector of it, S: sum.  Held to five CTAs an SM (INT8 at 16384^2 43.2 -> 40.5 us).
 template <typename T, typename V, typename S>
-__global__ void __launch_bounds__(kThreads, 5) gemv_t_vec(GemvT g, const T* __restrict__ A, const T* __restrict__ x,
-                                                          S alpha, S beta, S* __restrict__ y) {
+__global__ void __launch_bounds__(kThreads, 5) gemv_t_vec(GemvT g, const T* A, const T* x,
+                                                          S alpha, S beta, S* y) {
     constexpr int E = 16 / int(sizeof(T));                 // elements of a vector
     const int lane = int(lane_id());
     pdl_wait();
@@ -319,7 +322,7 @@ __global__ void __launch_bounds__(kThreads, 5) gemv_t_vec(GemvT g, const T* __re
 #pragma unroll
             for (int u = 0; u < 4; ++u) v[u] = __ldcs(reinterpret_cast<const V*>(a + i + (32 * u + lane) * E));
 #pragma unroll
-            for (int u = 0; u < 4; ++u) w[u] = __ldg(reinterpret_cast<const V*>(x + i + (32 * u + lane) * E));
+            for (int u = 0; u < 4; ++u) w[u] = load(reinterpret_cast<const V*>(x + i + (32 * u + lane) * E));
 #pragma unroll
             for (int u = 0; u < 4; ++u) t_fma(v[u], w[u], acc);
         }
@@ -330,22 +333,22 @@ __global__ void __launch_bounds__(kThreads, 5) gemv_t_vec(GemvT g, const T* __re
                 const int64_t r = i + (32 * u + lane) * E;
                 const bool in = r < iv;
                 v[u] = in ? __ldcs(reinterpret_cast<const V*>(a + r)) : V{};
-                w[u] = in ? __ldg(reinterpret_cast<const V*>(x + r)) : V{};
+                w[u] = in ? load(reinterpret_cast<const V*>(x + r)) : V{};
             }
 #pragma unroll
             for (int u = 0; u < 4; ++u)
                 if (i + (32 * u + lane) * E < iv) t_fma(v[u], w[u], acc);
         }
         i = iv + lane;                                 // the last m % E rows
-        if (i < i1) acc += S(__ldg(a + i)) * S(__ldg(x + i));
+        if (i < i1) acc += S(load(a + i)) * S(load(x + i));
     }
     t_finish(g, acc, col, part, alpha, beta, y);
 }
 
 // Unaligned columns: one element per lane and load.  UNIT: incx == 1.
 template <typename T, typename S, bool UNIT>
-__global__ void __launch_bounds__(kThreads) gemv_t_scalar(GemvT g, const T* __restrict__ A, const T* __restrict__ x,
-                                                          S alpha, S beta, S* __restrict__ y) {
+__global__ void __launch_bounds__(kThreads) gemv_t_scalar(GemvT g, const T* A, const T* x,
+                                                          S alpha, S beta, S* y) {
     const int lane = int(lane_id());
     pdl_wait();
     pdl_trigger();
@@ -361,13 +364,13 @@ __global__ void __launch_bounds__(kThreads) gemv_t_scalar(GemvT g, const T* __re
         for (; left >= 8; left -= 8, a += 256, xp += 256 * incx) {
             T v[8], w[8];
 #pragma unroll
-            for (int u = 0; u < 8; ++u) v[u] = __ldg(a + 32 * u);
+            for (int u = 0; u < 8; ++u) v[u] = load(a + 32 * u);
 #pragma unroll
-            for (int u = 0; u < 8; ++u) w[u] = __ldg(xp + 32 * u * incx);
+            for (int u = 0; u < 8; ++u) w[u] = load(xp + 32 * u * incx);
 #pragma unroll
             for (int u = 0; u < 8; ++u) acc += S(v[u]) * S(w[u]);
         }
-        for (; left > 0; --left, a += 32, xp += 32 * incx) acc += S(__ldg(a)) * S(__ldg(xp));
+        for (; left > 0; --left, a += 32, xp += 32 * incx) acc += S(load(a)) * S(load(xp));
     }
     t_finish(g, acc, col, part, alpha, beta, y);
 }
@@ -409,17 +412,17 @@ __device__ __forceinline__ void transpose4x4_bytes(uint32_t w0, uint32_t w1, uin
 }
 
 __device__ __forceinline__ uint32_t pack_x4(const int8_t* x, int64_t j, int64_t incx) {
-    const uint32_t b0 = uint8_t(__ldg(x + (j + 0) * incx));
-    const uint32_t b1 = uint8_t(__ldg(x + (j + 1) * incx));
-    const uint32_t b2 = uint8_t(__ldg(x + (j + 2) * incx));
-    const uint32_t b3 = uint8_t(__ldg(x + (j + 3) * incx));
+    const uint32_t b0 = uint8_t(load(x + (j + 0) * incx));
+    const uint32_t b1 = uint8_t(load(x + (j + 1) * incx));
+    const uint32_t b2 = uint8_t(load(x + (j + 2) * incx));
+    const uint32_t b3 = uint8_t(load(x + (j + 3) * incx));
     return b0 | (b1 << 8) | (b2 << 16) | (b3 << 24);
 }
 
 template <bool PLAIN>
-__global__ void __launch_bounds__(kThreads) gemv_i8_n_vec(int64_t m, int64_t n, const int8_t* __restrict__ A,
-                                                          int64_t lda, const int8_t* __restrict__ x, int64_t incx,
-                                                          int32_t* __restrict__ part, int64_t cols_per_split,
+__global__ void __launch_bounds__(kThreads) gemv_i8_n_vec(int64_t m, int64_t n, const int8_t* A,
+                                                          int64_t lda, const int8_t* x, int64_t incx,
+                                                          int32_t* part, int64_t cols_per_split,
                                                           int rt, int64_t cols_per_group) {
     if (!PLAIN) pdl_wait();   // see launch
     pdl_trigger();   // the reduction may be scheduled; it waits for this grid to finish
@@ -485,7 +488,7 @@ __global__ void __launch_bounds__(kThreads) gemv_i8_n_vec(int64_t m, int64_t n, 
     }
     for (; j < jv; ++j) {
         const uint4 c = __ldcs(reinterpret_cast<const uint4*>(a + j * lda));
-        const int xv = int(__ldg(x + j * incx));
+        const int xv = int(load(x + j * incx));
         const uint32_t w[4] = {c.x, c.y, c.z, c.w};
 #pragma unroll
         for (int q = 0; q < 4; ++q)
@@ -493,10 +496,10 @@ __global__ void __launch_bounds__(kThreads) gemv_i8_n_vec(int64_t m, int64_t n, 
             for (int b = 0; b < 4; ++b) acc[4 * q + b] += int(int8_t((w[q] >> (8 * b)) & 0xffu)) * xv;
     }
     if (!PLAIN && jv < j1) {      // the last column of a matrix whose rows end inside this vector
-        const int xv = int(__ldg(x + jv * incx));
+        const int xv = int(load(x + jv * incx));
 #pragma unroll
         for (int r = 0; r < 16; ++r)
-            if (r0 + r < m) acc[r] += int(__ldg(a + r + jv * lda)) * xv;
+            if (r0 + r < m) acc[r] += int(load(a + r + jv * lda)) * xv;
     }
     if constexpr (!PLAIN) {
         __shared__ int4 red[4][kThreads];
@@ -529,9 +532,9 @@ __global__ void __launch_bounds__(kThreads) gemv_i8_n_vec(int64_t m, int64_t n, 
     }
 }
 
-__global__ void __launch_bounds__(kThreads) gemv_i8_n_scalar(int64_t m, int64_t n, const int8_t* __restrict__ A,
-                                                             int64_t lda, const int8_t* __restrict__ x, int64_t incx,
-                                                             int32_t* __restrict__ part, int64_t cols_per_split) {
+__global__ void __launch_bounds__(kThreads) gemv_i8_n_scalar(int64_t m, int64_t n, const int8_t* A,
+                                                             int64_t lda, const int8_t* x, int64_t incx,
+                                                             int32_t* part, int64_t cols_per_split) {
     pdl_wait();
     pdl_trigger();   // the reduction may be scheduled; it waits for this grid to finish
     const int64_t r = int64_t(blockIdx.x) * kThreads + threadIdx.x;
@@ -545,9 +548,9 @@ __global__ void __launch_bounds__(kThreads) gemv_i8_n_scalar(int64_t m, int64_t 
 #pragma unroll
         for (int u = 0; u < 8; ++u) v[u] = __ldcs(A + r + (j + u) * lda);
 #pragma unroll
-        for (int u = 0; u < 8; ++u) acc += int(v[u]) * int(__ldg(x + (j + u) * incx));
+        for (int u = 0; u < 8; ++u) acc += int(v[u]) * int(load(x + (j + u) * incx));
     }
-    for (; j < j1; ++j) acc += int(A[r + j * lda]) * int(__ldg(x + j * incx));
+    for (; j < j1; ++j) acc += int(A[r + j * lda]) * int(load(x + j * incx));
     part[int64_t(blockIdx.y) * m + r] = acc;
 }
 

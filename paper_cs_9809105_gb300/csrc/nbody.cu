@@ -124,10 +124,12 @@ __device__ __forceinline__ float4 ld_peer_f4(uint32_t addr) {
 // 1000 bodies.  Also measured: four CTAs per cluster (1991 at 20000, 2461 at 131072), 16 (not
 // portable, equal at 5000), 64 lanes x 4 warps (2011, 2494), unrolled by 4 (2146, 2468) or 16
 // (1989, 2328), two bodies a lane (2011, 2265), six (1776, 2208).
+// Launched as a programmatic dependent: resident while the kernel before still writes x or z, which are
+// not const __restrict__ for that reason.
 template <bool PACKED>
-__global__ void __launch_bounds__(NB_THREADS) nbody_tiled(int64_t nx, int64_t nz, const float4* __restrict__ x,
-                                                          const float4* __restrict__ z, float eps2,
-                                                          float4* __restrict__ out) {
+__global__ void __launch_bounds__(NB_THREADS) nbody_tiled(int64_t nx, int64_t nz, const float4* x,
+                                                          const float4* z, float eps2,
+                                                          float4* out) {
     // two z tiles of NB_THREADS bodies (two float4 each), later the partial sums [warp][body]
     __shared__ float4 sm[2 * 2 * NB_THREADS];
     static_assert(2 * 2 * NB_THREADS >= NB_WARPS * NB_XB, "the partial sums reuse the z tiles");
@@ -144,7 +146,7 @@ __global__ void __launch_bounds__(NB_THREADS) nbody_tiled(int64_t nx, int64_t nz
 #pragma unroll
     for (int k = 0; k < NB_ILP; ++k) {
         const int64_t i = xblock + k * 32 + lane;
-        xi[k] = i < nx ? x[i] : make_float4(0.f, 0.f, 0.f, 0.f);
+        xi[k] = i < nx ? load(x + i) : make_float4(0.f, 0.f, 0.f, 0.f);
     }
     float3 a[PACKED ? 1 : NB_ILP];
     XPair pr[PACKED ? NB_ILP / 2 : 1];
@@ -164,14 +166,14 @@ __global__ void __launch_bounds__(NB_THREADS) nbody_tiled(int64_t nx, int64_t nz
         t[0] = make_float4(v.x, v.x, v.y, v.y);
         t[1] = make_float4(v.z, v.z, v.w, v.w);
     };
-    put(0, zbeg + threadIdx.x < zend ? z[zbeg + threadIdx.x] : pad);
+    put(0, zbeg + threadIdx.x < zend ? load(z + zbeg + threadIdx.x) : pad);
     __syncthreads();
     int buf = 0;
     for (int64_t j0 = zbeg; j0 < zend; j0 += NB_THREADS) {
         const bool more = j0 + NB_THREADS < zend;
         const int64_t jn = j0 + NB_THREADS + threadIdx.x;
         float4 next = pad;
-        if (more && jn < zend) next = z[jn];
+        if (more && jn < zend) next = load(z + jn);
         // bodies of this tile per warp: 32, fewer (a multiple of eight) in the last one
         const int64_t rem = zend - j0;
         const int cnt = rem >= NB_THREADS ? 32 : int((rem + ZU - 1) / ZU) * NB_UNROLL;
