@@ -146,7 +146,9 @@ HostPlan host_plan(const hsmm_config_t& c, hsmm_op_t ta, hsmm_op_t tb, int64_t m
         const int pmin = P.panels;
         for (int i = 0; i < 9; ++i) {
             const int rp = 1 << (i / 3), p = 1 << (i % 3);
-            t[i] = p < pmin ? 0.0 : ozaki_host_time(m, n, k, P.slices, P.cplx, panel_size(m, rp), panel_size(n, p));
+            // four row panels where fewer would be taller than the split takes
+            const bool skip = p < pmin || (rp < 4 && panel_size(m, rp) > SPLIT_MAX_LINES);
+            t[i] = skip ? 0.0 : ozaki_host_time(m, n, k, P.slices, P.cplx, panel_size(m, rp), panel_size(n, p));
             if (t[i] > 0 && (best == 0 || t[i] < best)) best = t[i];
         }
         auto blocks = [](int i) { return (1 << (i / 3)) * (1 << (i % 3)); };

@@ -140,6 +140,8 @@ struct SplitOperand {
     int32_t* expo;
     Slices q;
 };
+// Lines of one operand that ozaki_split takes (2097120); more are refused.
+constexpr int64_t SPLIT_MAX_LINES = int64_t(65535) * 32;
 // Splits one or two operands (count), in one launch if their lines run the same way in memory.
 hsmm_status_t ozaki_split(bool cplx, const SplitOperand* ops, int count, int bits, int slices, cudaStream_t st);
 // C = alpha 2^(ea_i + eb_j) sum_d 2^(-bits d) S_d + beta C

@@ -775,8 +775,8 @@ constexpr size_t SPLIT_CACHE = 200 * 1024;     // shared memory for a complex li
 size_t split_cache_bytes(int64_t nw) { return size_t(16) * (size_t(nw) + size_t(nw) / 16 + 1); }
 
 hsmm_status_t make_split_job(const SplitOperand& o, bool cplx, SplitJob* j) {
-    if (o.v_contig && o.nv > 65535 * 32LL) return HSMM_STATUS_NOT_SUPPORTED;
-    if (!o.v_contig && o.nv > 65535) return HSMM_STATUS_NOT_SUPPORTED;
+    if (o.nv > SPLIT_MAX_LINES) return fail(HSMM_STATUS_NOT_SUPPORTED, "ozaki: an operand of more than %lld lines",
+                                            static_cast<long long>(SPLIT_MAX_LINES));
     j->M = static_cast<const double*>(o.M);
     j->ld = o.ld; j->nv = o.nv; j->nw = o.nw;
     j->expo = o.expo;
@@ -816,17 +816,16 @@ hsmm_status_t launch_split(SplitJob a, SplitJob b, int bits, int slices, cudaStr
         unsigned cs = 1;
         while (cs < unsigned(SPLIT_CLUSTER) && nw > int64_t(128) * cs) cs *= 2;
         const auto scan_blocks = [cs, lines](const SplitJob& j) { return unsigned((j.nv + lines - 1) / lines * cs); };
-        const auto slice_blocks = [](const SplitJob& j) {
-            return unsigned((j.nv + 31) / 32 * (((CPLX ? j.nw : j.ldq) + 63) / 64));
-        };
+        const auto slice_blocks = [](const SplitJob& j) { return (j.nv + 31) / 32 * (((CPLX ? j.nw : j.ldq) + 63) / 64); };
+        if (slice_blocks(a) + slice_blocks(b) > INT32_MAX) return HSMM_STATUS_NOT_SUPPORTED;
         a.blocks = scan_blocks(a);
         b.blocks = scan_blocks(b);
         e = pdl_launch(lines == 128 ? ozaki_scan_v_kernel<64, CPLX> : ozaki_scan_v_kernel<16, CPLX>,
                        dim3(a.blocks + b.blocks), 256, 0, cs, st, a, b);
         count_launches(1);
         if (e != cudaSuccess) return record_cuda(e);
-        a.blocks = slice_blocks(a);
-        b.blocks = slice_blocks(b);
+        a.blocks = unsigned(slice_blocks(a));
+        b.blocks = unsigned(slice_blocks(b));
         ozaki_slice_v_kernel<BITS, S, CPLX, BLOCKED><<<a.blocks + b.blocks, 256, 0, st>>>(a, b, bits, slices);
     } else {
         auto kern = ozaki_split_w_kernel<BITS, S, CPLX, BLOCKED>;
