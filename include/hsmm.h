@@ -268,7 +268,7 @@ hsmm_status_t hsmm_grouped_plan_destroy(hsmm_grouped_plan_t plan);
 /*
  * hsmm_nbody: the two-array n^2 problem of Section 4, F_i = sum_j f(x_i, z_j) for i < nx,
  * j < nz, with the gravitational interaction Section 2 names as the prototype application,
- *     f(x, z) = m_z (r_z - r_x) / (|r_z - r_x|^2 + eps2)^(3/2)    (0 for r = 0, eps2 = 0).
+ *     f(x, z) = m_z (r_z - r_x) / (|r_z - r_x|^2 + eps2)^(3/2)    (0 for r = 0, any eps2).
  * x: nx bodies, z: nz bodies, each 4 floats (px, py, pz, m; the mass of x is not used),
  * out: nx x 4 floats (ax, ay, az, 0); device pointers, 16-byte aligned, caller-owned.  FP32
  * arithmetic with the hardware reciprocal square root.  x and z may be the same array.

@@ -2,7 +2,7 @@
 // gravitational interaction Section 2 cites as the prototype hyper-systolic application:
 //   f(x, z) = m_z (r_z - r_x) / (|r_z - r_x|^2 + eps2)^(3/2)   (0 for coincident bodies).
 // Bodies are float4 (px, py, pz, m), results float4 (ax, ay, az, 0); FP32 arithmetic with the
-// hardware reciprocal square root.  With eps2 > 0 the kernels work on pairs of x bodies with
+// hardware reciprocal square root.  From eps2 = 2^-66 on the kernels work on pairs of x bodies with
 // the packed FP32 instructions of this GPU (sub/mul/fma .f32x2: two interactions per
 // instruction, the reciprocal square root per half).
 //
@@ -46,6 +46,30 @@ __device__ __forceinline__ void interact(const float4& x, const float4& z, float
     a.z = fmaf(s, dz, a.z);
 }
 
+// The forms of the interaction.  The cube of 1/r overflows below r^2 = 2^-85 and one body's pair with
+// itself is then infinity times zero; so the packed form is taken for eps2 from 2^-66 on (1/r^3 <= 2^99,
+// masses to 2^28), and smaller positive ones multiply in another order, one body at a time.
+enum class Form { Zero, Small, Packed };
+constexpr float PACKED_EPS2 = 1.3552527e-20f;      // 2^-66
+__host__ __device__ __forceinline__ Form form_of(float eps2) {
+    return eps2 >= PACKED_EPS2 ? Form::Packed : eps2 > 0.f ? Form::Small : Form::Zero;
+}
+
+// a += f(x, z) for any eps2 > 0: m / r and d / r, which stay finite (and 0 for d = 0), before the last 1/r
+__device__ __forceinline__ void interact_small(const float4& x, const float4& z, float eps2, float3& a) {
+    const float dx = z.x - x.x, dy = z.y - x.y, dz = z.z - x.z;
+    const float inv = rsqrtf(fmaf(dx, dx, fmaf(dy, dy, fmaf(dz, dz, eps2))));
+    const float m = z.w * inv;
+    a.x = fmaf(m * (dx * inv), inv, a.x);
+    a.y = fmaf(m * (dy * inv), inv, a.y);
+    a.z = fmaf(m * (dz * inv), inv, a.z);
+}
+template <Form F>
+__device__ __forceinline__ void interact_one(const float4& x, const float4& z, float eps2, float3& a) {
+    if constexpr (F == Form::Small) interact_small(x, z, eps2, a);
+    else interact(x, z, eps2, a);
+}
+
 // ---- packed FP32 pairs (f32x2): two x bodies against one z body per instruction ----
 __device__ __forceinline__ uint64_t pk2(float lo, float hi) {
     uint64_t r;
@@ -77,7 +101,7 @@ __device__ __forceinline__ float rsqrt_approx(float v) {
 }
 
 // two x bodies (packed coordinates X, Y, Z) against z (coordinates and mass broadcast to both
-// halves); eps2 > 0, so r^2 > 0 and no pair needs the r = 0 case
+// halves); Form::Packed: r^2 >= eps2, no pair needs the r = 0 case
 struct XPair {
     uint64_t X, Y, Z, ax, ay, az;
 };
@@ -112,8 +136,7 @@ __device__ __forceinline__ float4 ld_peer_f4(uint32_t addr) {
 // works on its own eighth of every z tile; a cluster of NB_ZS = 8 CTAs shares the same x bodies
 // and splits z.  Partial sums are added in the fixed order of warps, then cluster ranks, through
 // shared and distributed shared memory (deterministic, no workspace).
-//   PACKED (eps2 > 0): the four bodies as two packed pairs; else one body at a time with the
-//   r = 0 case handled.
+//   Form::Packed: the four bodies as two packed pairs; else one body at a time.
 // Bound by the FP32 pipe: 12 packed instructions per two interactions, so what counts is that
 // every scheduler has warps to hide their latency behind.  The 64-way split of z (eight warps x
 // eight CTAs) gives an x array of 20000 bodies 1256 CTAs, four resident per SM; with 1024 x bodies
@@ -126,13 +149,14 @@ __device__ __forceinline__ float4 ld_peer_f4(uint32_t addr) {
 // (1989, 2328), two bodies a lane (2011, 2265), six (1776, 2208).
 // Launched as a programmatic dependent: resident while the kernel before still writes x or z, which are
 // not const __restrict__ for that reason.
-template <bool PACKED>
+template <Form F>
 __global__ void __launch_bounds__(NB_THREADS) nbody_tiled(int64_t nx, int64_t nz, const float4* x,
                                                           const float4* z, float eps2,
                                                           float4* out) {
     // two z tiles of NB_THREADS bodies (two float4 each), later the partial sums [warp][body]
     __shared__ float4 sm[2 * 2 * NB_THREADS];
     static_assert(2 * 2 * NB_THREADS >= NB_WARPS * NB_XB, "the partial sums reuse the z tiles");
+    constexpr bool PACKED = F == Form::Packed;
     pdl_wait();
     const int lane = int(lane_id()), warp = int(warp_id());
     const int zs = int(cluster_ctarank()), ZS = int(cluster_nctarank());
@@ -188,7 +212,7 @@ __global__ void __launch_bounds__(NB_THREADS) nbody_tiled(int64_t nx, int64_t nz
             } else {
                 const float4 u = t[2 * q], w = t[2 * q + 1];
 #pragma unroll
-                for (int k = 0; k < NB_ILP; ++k) interact(xi[k], make_float4(u.x, u.z, w.x, w.z), eps2, a[k]);
+                for (int k = 0; k < NB_ILP; ++k) interact_one<F>(xi[k], make_float4(u.x, u.z, w.x, w.z), eps2, a[k]);
             }
         }
         if (more) put(buf ^ 1, next);
@@ -239,10 +263,11 @@ __global__ void __launch_bounds__(NB_THREADS) nbody_tiled(int64_t nx, int64_t nz
     cluster_sync_all();   // the other ranks keep their partial sums until they have been read
 }
 
-template <int K, bool PACKED>
+template <int K, Form F>
 __global__ void __launch_bounds__(NB_RING) nbody_hsys(int64_t nx, int64_t nz, const float4* __restrict__ x,
                                                       const float4* __restrict__ z, float eps2,
                                                       float4* __restrict__ out, int P) {
+    constexpr bool PACKED = F == Form::Packed;
     static_assert(!PACKED || K % 2 == 0, "packed replicas come in pairs");
     __shared__ float4 xs[NB_RING];          // this cell's block of x
     __shared__ float4 zb[2][NB_RING];       // the z block held in step s (buffer s % 2) and the next
@@ -286,7 +311,7 @@ __global__ void __launch_bounds__(NB_RING) nbody_hsys(int64_t nx, int64_t nz, co
                     for (int r = 0; r < K / 2; ++r) interact2(pr[r], zx, zy, zz, zm, e2);
                 } else {
 #pragma unroll
-                    for (int r = 0; r < K; ++r) interact(xr[r], zq, eps2, acc[r]);
+                    for (int r = 0; r < K; ++r) interact_one<F>(xr[r], zq, eps2, acc[r]);
                 }
             }
             if (s + 1 < Kt) {
@@ -334,13 +359,14 @@ hsmm_status_t nbody_forces(int64_t nx, int64_t nz, const float* x, const float* 
     const float4* x4 = reinterpret_cast<const float4*>(x);
     const float4* z4 = reinterpret_cast<const float4*>(z);
     float4* o4 = reinterpret_cast<float4*>(out);
-    // eps2 > 0: r^2 > 0 for every pair, the packed FP32 pair kernels apply
-    const bool packed = eps2 > 0.f;
+    const Form form = form_of(eps2);
     if (ring_p == 0) {
         const int64_t xblocks = (nx + NB_XB - 1) / NB_XB;
         if (xblocks > INT32_MAX / NB_ZS) return HSMM_STATUS_NOT_SUPPORTED;
-        const cudaError_t te = pdl_launch(packed ? nbody_tiled<true> : nbody_tiled<false>, dim3(unsigned(xblocks * NB_ZS)),
-                                          NB_THREADS, 0, NB_ZS, st, nx, nz, x4, z4, eps2, o4);
+        const cudaError_t te = pdl_launch(form == Form::Packed  ? nbody_tiled<Form::Packed>
+                                          : form == Form::Small ? nbody_tiled<Form::Small>
+                                                                : nbody_tiled<Form::Zero>,
+                                          dim3(unsigned(xblocks * NB_ZS)), NB_THREADS, 0, NB_ZS, st, nx, nz, x4, z4, eps2, o4);
         count_launches(1);
         if (te != cudaSuccess) return record_cuda(te);
         return check_launch();
@@ -359,32 +385,23 @@ hsmm_status_t nbody_forces(int64_t nx, int64_t nz, const float* x, const float* 
     at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    cudaError_t e = cudaSuccess;
+    // by K = 1, 2, 4 and form; one replica has no packed pair
+    using Kern = void (*)(int64_t, int64_t, const float4*, const float4*, float, float4*, int);
+    static constexpr Kern kerns[3][3] = {
+        {nbody_hsys<1, Form::Zero>, nbody_hsys<1, Form::Small>, nbody_hsys<1, Form::Zero>},
+        {nbody_hsys<2, Form::Zero>, nbody_hsys<2, Form::Small>, nbody_hsys<2, Form::Packed>},
+        {nbody_hsys<4, Form::Zero>, nbody_hsys<4, Form::Small>, nbody_hsys<4, Form::Packed>}};
     static std::atomic<uint64_t> attrs{0};
     const hsmm_status_t as = attrs_once_per_device(attrs, [] {
-        const void* kerns[5] = {reinterpret_cast<const void*>(nbody_hsys<1, false>),
-                                reinterpret_cast<const void*>(nbody_hsys<2, false>),
-                                reinterpret_cast<const void*>(nbody_hsys<4, false>),
-                                reinterpret_cast<const void*>(nbody_hsys<2, true>),
-                                reinterpret_cast<const void*>(nbody_hsys<4, true>)};
         cudaError_t r = cudaSuccess;
-        for (int i = 0; i < 5 && r == cudaSuccess; ++i)
-            r = cudaFuncSetAttribute(kerns[i], cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        for (const auto& row : kerns)
+            for (const Kern kern : row)
+                if (r == cudaSuccess) r = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
         return r;
     });
     if (as != HSMM_STATUS_SUCCESS) return as;
-    switch (K) {
-        case 1: e = cudaLaunchKernelEx(&cfg, nbody_hsys<1, false>, nx, nz, x4, z4, eps2, o4, P); break;
-        case 2:
-            e = packed ? cudaLaunchKernelEx(&cfg, nbody_hsys<2, true>, nx, nz, x4, z4, eps2, o4, P)
-                       : cudaLaunchKernelEx(&cfg, nbody_hsys<2, false>, nx, nz, x4, z4, eps2, o4, P);
-            break;
-        case 4:
-            e = packed ? cudaLaunchKernelEx(&cfg, nbody_hsys<4, true>, nx, nz, x4, z4, eps2, o4, P)
-                       : cudaLaunchKernelEx(&cfg, nbody_hsys<4, false>, nx, nz, x4, z4, eps2, o4, P);
-            break;
-        default: return HSMM_STATUS_INVALID_VALUE;
-    }
+    if (K != 1 && K != 2 && K != 4) return HSMM_STATUS_INVALID_VALUE;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kerns[K / 2][int(form)], nx, nz, x4, z4, eps2, o4, P);
     count_launches(1);
     if (e != cudaSuccess) return record_cuda(e);
     return check_launch();
