@@ -32,7 +32,7 @@ namespace {
 // per lane and per CTA, z bodies per unrolled step, CTAs of a cluster (the split of z)
 constexpr int NB_WARPS = 8, NB_THREADS = 32 * NB_WARPS;
 constexpr int NB_ILP = 4, NB_XB = 32 * NB_ILP, NB_UNROLL = 8;
-constexpr int NB_ZS = 8;
+constexpr int NB_ZS = 8, NB_ZS_WIDE = 4;   // see nbody_forces
 constexpr int NB_RING = 128;    // bodies per cell and threads per CTA (hyper-systolic)
 
 // a += f(x, z): m_z d / (|d|^2 + eps2)^(3/2), d = r_z - r_x
@@ -133,7 +133,7 @@ __device__ __forceinline__ float4 ld_peer_f4(uint32_t addr) {
 }
 
 // Tiled schedule.  A CTA owns NB_XB = 128 x bodies, four per lane, and each of its eight warps
-// works on its own eighth of every z tile; a cluster of NB_ZS = 8 CTAs shares the same x bodies
+// works on its own eighth of every z tile; a cluster of eight CTAs, or four, shares the same x bodies
 // and splits z.  Partial sums are added in the fixed order of warps, then cluster ranks, through
 // shared and distributed shared memory (deterministic, no workspace).
 //   Form::Packed: the four bodies as two packed pairs; else one body at a time.
@@ -363,10 +363,17 @@ hsmm_status_t nbody_forces(int64_t nx, int64_t nz, const float* x, const float* 
     if (ring_p == 0) {
         const int64_t xblocks = (nx + NB_XB - 1) / NB_XB;
         if (xblocks > INT32_MAX / NB_ZS) return HSMM_STATUS_NOT_SUPPORTED;
+        // Eight CTAs share an x block, four where those alone fill the SMs one and a half times over (four
+        // CTAs an SM) and z is at most a tile for each, or the bodies go one by one: a CTA then has
+        // twice the z bodies to set up and add up for.  Us, four / eight: 70000 x 900 34.4 / 41.3, 30000 x
+        // 1000 17.5 / 19.5, but 50000^2 1038 / 1034 and 20000^2 196 / 178; eps2 = 0: 70000 x 900 53.7 / 69.1,
+        // 40000 x 10000 282 / 295, 131072^2 10665 / 11484.
+        const bool few = nz <= NB_ZS_WIDE * NB_THREADS || form != Form::Packed;
+        const int zs = few && xblocks * NB_ZS_WIDE >= int64_t(num_sms()) * 6 ? NB_ZS_WIDE : NB_ZS;
         const cudaError_t te = pdl_launch(form == Form::Packed  ? nbody_tiled<Form::Packed>
                                           : form == Form::Small ? nbody_tiled<Form::Small>
                                                                 : nbody_tiled<Form::Zero>,
-                                          dim3(unsigned(xblocks * NB_ZS)), NB_THREADS, 0, NB_ZS, st, nx, nz, x4, z4, eps2, o4);
+                                          dim3(unsigned(xblocks * zs)), NB_THREADS, 0, unsigned(zs), st, nx, nz, x4, z4, eps2, o4);
         count_launches(1);
         if (te != cudaSuccess) return record_cuda(te);
         return check_launch();
