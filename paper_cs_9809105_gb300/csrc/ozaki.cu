@@ -16,6 +16,7 @@
 #include <atomic>
 #include <climits>
 #include <cstdint>
+#include <type_traits>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -67,14 +68,6 @@ __device__ __forceinline__ int line_exponent_bits(uint64_t mb) {
     return top == 0 ? INT_MIN : line_exponent(__longlong_as_double(int64_t(top)));
 }
 
-// BF16 bit pattern of a small integer q (|q| <= 255: exact), from integer operations only
-__device__ __forceinline__ uint16_t bf16_of_small_int(uint32_t mag, uint32_t neg) {
-    if (mag == 0) return 0;
-    const uint32_t top = 31u - uint32_t(__clz(mag));          // 0..7
-    const uint32_t mant = (mag << (7u - top)) & 0x7Fu;
-    return uint16_t((neg << 15) | ((127u + top) << 7) | mant);
-}
-
 // One value prepared for digit extraction.  With |v| = M 2^(E-1075) (M the 53-bit significand),
 // digit t of |v| 2^(-e) is floor(M 2^(E - 1075 - e + bits t)) mod 2^bits, read from the
 // significand with integer shifts: the same digits the FP64 steps y = x 2^bits, q = trunc(y),
@@ -105,9 +98,25 @@ __device__ __forceinline__ uint32_t digit_bits(const Digits& x, int bits, int t)
     return (sh >= bits) ? 0u : uint32_t(x.mag << sh) & mask;
 }
 
-// four BF16 digits of consecutive entries: one 8-byte store, or 2-byte ones for the first `valid`
-__device__ __forceinline__ void put4(uint16_t* o, uint32_t w01, uint32_t w23, bool vec, int valid) {
-    if (vec && valid == 4) {
+// BF16 patterns of two digits d in [0, 255], each with the sign n of its value (none for d = 0):
+// the FP32 number (-1)^n (2^23 + d) holds d in its low significand bits, and minus (-1)^n 2^23
+// it is exactly (-1)^n d (+0 for d = 0); one packed subtraction makes both, and the upper halves
+// of the two results, gathered by one byte permutation, are the two BF16 patterns (float(d)
+// has at most 8 significant bits).  Full-rate FP32 and integer operations only.
+__device__ __forceinline__ uint32_t bf16x2_of_digits(uint32_t d0, uint32_t d1, uint64_t bias) {
+    const uint64_t a = (uint64_t(uint32_t(bias >> 32) | d1) << 32) | (uint32_t(bias) | d0);
+    uint64_t y;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(y) : "l"(a), "l"(bias));
+    return __byte_perm(uint32_t(y), uint32_t(y >> 32), 0x7632);
+}
+// (-1)^n 2^23 of two values, n their signs
+__device__ __forceinline__ uint64_t signed_bias(uint32_t n0, uint32_t n1) {
+    return (uint64_t(0x4B000000u | (n1 << 31)) << 32) | (0x4B000000u | (n0 << 31));
+}
+
+// four BF16 digits of consecutive entries: one 8-byte store (full), or 2-byte ones for the first `valid`
+__device__ __forceinline__ void put4(uint16_t* o, uint32_t w01, uint32_t w23, bool full, int valid) {
+    if (full) {
         *reinterpret_cast<uint2*>(o) = make_uint2(w01, w23);
     } else {
         o[0] = uint16_t(w01);
@@ -119,16 +128,17 @@ __device__ __forceinline__ void put4(uint16_t* o, uint32_t w01, uint32_t w23, bo
 
 // Four consecutive values of one line -> four BF16 digits for each slice t.
 __device__ __forceinline__ void slice_store4(const double (&x)[4], int e, int bits, int s, uint16_t* out,
-                                             int64_t slice_stride, bool vec, int valid = 4) {
+                                             int64_t slice_stride, bool full, int valid) {
     Digits dg[4];
 #pragma unroll
     for (int c = 0; c < 4; ++c) dg[c] = prepare_digits(x[c], e);
+    const uint64_t b01 = signed_bias(dg[0].neg, dg[1].neg), b23 = signed_bias(dg[2].neg, dg[3].neg);
     for (int t = 1; t <= s; ++t) {
-        uint32_t h[4];
+        uint32_t d[4];
 #pragma unroll
-        for (int c = 0; c < 4; ++c) h[c] = bf16_of_small_int(digit_bits(dg[c], bits, t), dg[c].neg);
-        put4(out + int64_t(t - 1) * slice_stride, h[0] | (h[1] << 16), h[2] | (h[3] << 16), vec,
-             valid);
+        for (int c = 0; c < 4; ++c) d[c] = digit_bits(dg[c], bits, t);
+        put4(out, bf16x2_of_digits(d[0], d[1], b01), bf16x2_of_digits(d[2], d[3], b23), full, valid);
+        out += slice_stride;
     }
 }
 
@@ -149,45 +159,39 @@ __device__ __forceinline__ uint64_t digits_word(double val, int e, uint32_t& neg
     return -sh >= 64 ? 0 : (mag >> -sh);
 }
 
-// BF16 patterns of two digits d in [0, 255], each with the sign n of its value (none for d = 0):
-// the FP32 number (-1)^n (2^23 + d) holds d in its low significand bits, and minus (-1)^n 2^23
-// it is exactly (-1)^n d (+0 for d = 0); one packed subtraction makes both, and the upper halves
-// of the two results, gathered by one byte permutation, are the two BF16 patterns (float(d)
-// has at most 8 significant bits).  Full-rate FP32 and integer operations only.
-__device__ __forceinline__ uint32_t bf16x2_of_digits(uint32_t d0, uint32_t d1, uint64_t signed_bias) {
-    const uint64_t a = (uint64_t(uint32_t(signed_bias >> 32) | d1) << 32) | (uint32_t(signed_bias) | d0);
-    uint64_t y;
-    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(y) : "l"(a), "l"(signed_bias));
-    return __byte_perm(uint32_t(y), uint32_t(y >> 32), 0x7632);
-}
-
 template <int BITS, int S>
 __device__ __forceinline__ void slice_store4_fixed(const double (&x)[4], int e, uint16_t* out, int64_t slice_stride,
-                                                   bool vec, int valid = 4) {
+                                                   bool full, int valid) {
     constexpr uint32_t MASK = (1u << BITS) - 1u;
     uint64_t F[4];
     uint32_t ng[4];
 #pragma unroll
     for (int c = 0; c < 4; ++c) F[c] = digits_word<BITS, S>(x[c], e, ng[c]);
-    // (-1)^n 2^23 of each value, two per 64-bit word
-    const uint64_t b01 = (uint64_t(0x4B000000u | (ng[1] << 31)) << 32) | (0x4B000000u | (ng[0] << 31));
-    const uint64_t b23 = (uint64_t(0x4B000000u | (ng[3] << 31)) << 32) | (0x4B000000u | (ng[2] << 31));
+    const uint64_t b01 = signed_bias(ng[0], ng[1]), b23 = signed_bias(ng[2], ng[3]);
 #pragma unroll
     for (int t = 1; t <= S; ++t) {
         uint32_t d[4];
 #pragma unroll
         for (int c = 0; c < 4; ++c) d[c] = uint32_t(F[c] >> (BITS * (S - t))) & MASK;
         put4(out + int64_t(t - 1) * slice_stride, bf16x2_of_digits(d[0], d[1], b01), bf16x2_of_digits(d[2], d[3], b23),
-             vec, valid);
+             full, valid);
     }
 }
 
 // BITS = 0: digit width and count from the arguments; else the compile-time form
 template <int BITS, int S>
+__device__ __forceinline__ void slice_store4_as(const double (&x)[4], int e, int bits, int s, uint16_t* out,
+                                                int64_t slice_stride, bool full, int valid) {
+    if constexpr (BITS > 0) slice_store4_fixed<BITS, S>(x, e, out, slice_stride, full, valid);
+    else slice_store4(x, e, bits, s, out, slice_stride, full, valid);
+}
+// The choice of stores made once for all digits: inside the digit loop it cost 4 to 8% of a v-contiguous
+// real split (in the complex one, with its four groups of places, two unrolled forms cost more, 3%)
+template <int BITS, int S>
 __device__ __forceinline__ void slice_store4_any(const double (&x)[4], int e, int bits, int s, uint16_t* out,
-                                                 int64_t slice_stride, bool vec, int valid = 4) {
-    if constexpr (BITS > 0) slice_store4_fixed<BITS, S>(x, e, out, slice_stride, vec, valid);
-    else slice_store4(x, e, bits, s, out, slice_stride, vec, valid);
+                                                 int64_t slice_stride, bool vec) {
+    if (vec) slice_store4_as<BITS, S>(x, e, bits, s, out, slice_stride, true, 4);
+    else slice_store4_as<BITS, S>(x, e, bits, s, out, slice_stride, false, 4);
 }
 
 // ---------------------------------------------------------------------------
@@ -207,7 +211,7 @@ __device__ __forceinline__ void slice_store4_any(const double (&x)[4], int e, in
 //  * w contiguous: one to eight warps hold a line in registers (real, up to 8 x 4 values a
 //    thread), or a CTA in shared memory (complex), take its exponent and slice it.  Longer lines
 //    are read again, from L2.
-//  * v contiguous: a cluster of 1 to 8 CTAs shares 32 lines and scans a part of w each; the maxima
+//  * v contiguous: a cluster of 1 to 8 CTAs shares 32 or 128 lines and scans a part of w each; the maxima
 //    meet in distributed shared memory.  A second kernel slices tiles of 64 w x 32 lines, transposed
 //    through shared memory.  (As a programmatic dependent it was slower, 14.2 against 10.4 us at
 //    1000 x 900.  Slicing in the scanning cluster, the lines read again from L2, was slower
@@ -221,10 +225,10 @@ __device__ __forceinline__ void slice_store4_any(const double (&x)[4], int e, in
 // scan read everything once more, and complex rows of odd length were stored two bytes at a
 // time.  Before -> now, seven slices of seven bits, us in a row in a CUDA graph: w contiguous
 // 8192^2 298 -> 261 (5.6 TB/s), 4096^2 82 -> 71, 1000 x 900 9.2 -> 6.4; v contiguous 1000 x 900
-// 15.5 -> 10.5, 5000 x 300 22.8 -> 15.2, 4096^2 91 -> 92, 8192^2 323 -> 350 (the scan's short
-// pieces of a row); both operands of a complex 1500 x 1100 x 2301 product 190 -> 76.
+// 15.6 -> 9.9, 5000 x 300 14.2 -> 12.3, 4096^2 91 -> 93, 8192^2 326 -> 333, 20000 x 2000 197 -> 206
+// (1256 scanning CTAs are two waves and a bit); both operands of a complex 1500 x 1100 x 2301 product 190 -> 76.
 // ---------------------------------------------------------------------------
-constexpr int SPLIT_CLUSTER = 8;   // most CTAs that share 32 v-contiguous lines
+constexpr int SPLIT_CLUSTER = 8;   // most CTAs that share 32 or 128 v-contiguous lines
 constexpr int SPLIT_HELD = 8;      // chunks of four values a thread holds (real, w contiguous)
 
 struct SplitJob {
@@ -240,6 +244,8 @@ struct SplitJob {
     int vec_in, vec_out;           // 16-byte loads (real, w contiguous); 8-byte stores
     int warps;                     // w contiguous, real: warps per line (1, 2, 4 or 8)
     int cached;                    // w contiguous, complex: the line fits shared memory
+    unsigned pieces;               // v contiguous: slicing CTAs along w (a block index divides in 32 bits: with 64
+                                   // the slicing took 4 to 8% longer)
     unsigned blocks;
 };
 
@@ -416,7 +422,7 @@ __device__ __forceinline__ void split_w_complex(const SplitJob& j, int64_t v, in
                     }
                 }
             }
-            slice_store4_any<BITS, S>(x, e, bits, s, out.at(p), j.plane, j.vec_out != 0);
+            slice_store4_as<BITS, S>(x, e, bits, s, out.at(p), j.plane, true, 4);    // a workspace's slices are aligned
         }
     }
 }
@@ -436,7 +442,7 @@ __device__ __forceinline__ void emit_tile_row(const SplitJob& j, const double (*
             const double y = c < valid ? tile[r & 63][(vl + ((r & 63) >> 2)) & 31] : 0.0;
             x[c] = flip ? -y : y;
         }
-        slice_store4_any<BITS, S>(x, e, bits, s, row.at(pos + first), j.plane, j.vec_out != 0, valid);
+        slice_store4_as<BITS, S>(x, e, bits, s, row.at(pos + first), j.plane, j.vec_out && valid == 4, valid);
     };
     const int first = lead + 4 * wq;
     if (first < n) group(first, min(4, n - first));
@@ -445,10 +451,11 @@ __device__ __forceinline__ void emit_tile_row(const SplitJob& j, const double (*
 
 // Exponents of 2 LX v-contiguous lines: a cluster shares them, each CTA scans its part of w, LX
 // lanes with two lines each by 256 / LX entries at a time.  Loads come in batches, the last one
-// predicated (a remainder loop would take them one by one).
+// predicated (a remainder loop would take them one by one).  Six real loads a batch let four CTAs share
+// an SM; with eight (78 registers, three CTAs) the 512 CTAs of 8192 lines took two waves, 96 -> 79 us.
 template <int LX, bool CPLX>
 __device__ __forceinline__ void scan_v(const SplitJob& j, int64_t block) {
-    constexpr int R = 256 / LX, U = CPLX ? 4 : 8;
+    constexpr int R = 256 / LX, U = CPLX ? 4 : 6;
     __shared__ uint64_t red[R][2 * LX], cmax[2 * LX];
     const int rank = int(cluster_ctarank()), CS = int(cluster_nctarank());
     const int tx = int(threadIdx.x) % LX, ty = int(threadIdx.x) / LX;
@@ -456,16 +463,18 @@ __device__ __forceinline__ void scan_v(const SplitJob& j, int64_t block) {
     const int64_t part = (j.nw + CS - 1) / CS, w0 = rank * part, w1 = min(j.nw, w0 + part);
     const bool two = v + 1 < j.nv, vec = two && j.vec_in;
     uint64_t ma = 0, mb = 0;
+    const int64_t step = R * j.ld;
     if (v < j.nv) {
-        for (int64_t w = w0 + ty; w < w1; w += R * U) {
+        const auto batch = [&](auto full, int64_t w) {
+            constexpr bool FULL = decltype(full)::value;
+            const double* p = j.M + (CPLX ? 2 : 1) * (v + w * j.ld);
             if constexpr (CPLX) {
                 double2 x[U], y[U];
 #pragma unroll
-                for (int u = 0; u < U; ++u) {
-                    const bool in = w + R * u < w1;
-                    const double2* p = reinterpret_cast<const double2*>(j.M) + v + (w + R * u) * j.ld;
-                    x[u] = in ? p[0] : make_double2(0.0, 0.0);
-                    y[u] = in && two ? p[1] : make_double2(0.0, 0.0);
+                for (int u = 0; u < U; ++u, p += 2 * step) {
+                    const bool in = FULL || w + R * u < w1;
+                    x[u] = in ? reinterpret_cast<const double2*>(p)[0] : make_double2(0.0, 0.0);
+                    y[u] = in && two ? reinterpret_cast<const double2*>(p)[1] : make_double2(0.0, 0.0);
                 }
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
@@ -475,9 +484,8 @@ __device__ __forceinline__ void scan_v(const SplitJob& j, int64_t block) {
             } else {
                 double2 x[U];
 #pragma unroll
-                for (int u = 0; u < U; ++u) {
-                    const bool in = w + R * u < w1;
-                    const double* p = j.M + v + (w + R * u) * j.ld;
+                for (int u = 0; u < U; ++u, p += step) {
+                    const bool in = FULL || w + R * u < w1;
                     if (in && vec) x[u] = *reinterpret_cast<const double2*>(p);
                     else x[u] = make_double2(in ? p[0] : 0.0, in && two ? p[1] : 0.0);
                 }
@@ -487,7 +495,10 @@ __device__ __forceinline__ void scan_v(const SplitJob& j, int64_t block) {
                     mb = mag_max(mb, mag_bits(x[u].y));
                 }
             }
-        }
+        };
+        int64_t w = w0 + ty;
+        for (; w + R * (U - 1) < w1; w += R * U) batch(std::true_type{}, w);
+        if (w < w1) batch(std::false_type{}, w);
     }
     red[ty][2 * tx] = ma;
     red[ty][2 * tx + 1] = mb;
@@ -516,14 +527,14 @@ __device__ __forceinline__ void scan_v(const SplitJob& j, int64_t block) {
 
 // one tile of 64 w x 32 v-contiguous lines, transposed through shared memory
 template <int BITS, int S, bool CPLX, bool BLOCKED>
-__device__ __forceinline__ void slice_v(const SplitJob& j, int64_t block, int bits, int s) {
+__device__ __forceinline__ void slice_v(const SplitJob& j, unsigned block, int bits, int s) {
     // column v of row w at (v + w / 4) % 32: conflict-free both along v and for the four
     // consecutive w a thread slices
     __shared__ double tile[CPLX ? 2 : 1][64][32];
     const int tx = int(threadIdx.x) & 31, ty = int(threadIdx.x) >> 5;   // 32 x 8
     const int64_t len = CPLX ? j.nw : j.ldq;        // a real row's padding belongs to its last entries
-    const int64_t tiles_w = (len + 63) / 64;
-    const int64_t w0 = block % tiles_w * 64, v0 = block / tiles_w * 32, v = v0 + tx;
+    const unsigned row = block / j.pieces;
+    const int64_t w0 = int64_t(block - row * j.pieces) * 64, v0 = int64_t(row) * 32, v = v0 + tx;
     const int n = int(min(int64_t(64), len - w0));
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
@@ -591,7 +602,7 @@ __global__ void __launch_bounds__(256) ozaki_scan_v_kernel(SplitJob j0, SplitJob
     scan_v<LX, CPLX>(first ? j0 : j1, first ? blockIdx.x : blockIdx.x - j0.blocks);
 }
 template <int BITS, int S, bool CPLX, bool BLOCKED>
-__global__ void __launch_bounds__(256, CPLX ? 5 : BITS > 0 ? 8 : 6) ozaki_slice_v_kernel(SplitJob j0, SplitJob j1, int bits, int s) {
+__global__ void __launch_bounds__(256, CPLX ? 5 : BITS > 0 ? 8 : 5) ozaki_slice_v_kernel(SplitJob j0, SplitJob j1, int bits, int s) {
     pdl_trigger();
     const bool first = blockIdx.x < j0.blocks;
     slice_v<BITS, S, CPLX, BLOCKED>(first ? j0 : j1, first ? blockIdx.x : blockIdx.x - j0.blocks, bits, s);
@@ -816,7 +827,9 @@ hsmm_status_t launch_split(SplitJob a, SplitJob b, int bits, int slices, cudaStr
         unsigned cs = 1;
         while (cs < unsigned(SPLIT_CLUSTER) && nw > int64_t(128) * cs) cs *= 2;
         const auto scan_blocks = [cs, lines](const SplitJob& j) { return unsigned((j.nv + lines - 1) / lines * cs); };
-        const auto slice_blocks = [](const SplitJob& j) { return (j.nv + 31) / 32 * (((CPLX ? j.nw : j.ldq) + 63) / 64); };
+        a.pieces = unsigned(((CPLX ? a.nw : a.ldq) + 63) / 64);
+        b.pieces = unsigned(((CPLX ? b.nw : b.ldq) + 63) / 64);
+        const auto slice_blocks = [](const SplitJob& j) { return (j.nv + 31) / 32 * int64_t(j.pieces); };
         if (slice_blocks(a) + slice_blocks(b) > INT32_MAX) return HSMM_STATUS_NOT_SUPPORTED;
         a.blocks = scan_blocks(a);
         b.blocks = scan_blocks(b);
