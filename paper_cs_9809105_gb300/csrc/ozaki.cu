@@ -10,8 +10,7 @@
 // op(B)), w = the contraction index, contiguous, row pitch ldq (a multiple of 8 so
 // that the TMA row stride is a multiple of 16 bytes).
 //
-// One launch splits both operands of a product (or one): every CTA finds the exponents of its
-// lines and slices them while they are still on the chip.
+// One or two launches split both operands of a product (or one).
 #include <algorithm>
 #include <atomic>
 #include <climits>
@@ -207,16 +206,20 @@ __device__ __forceinline__ void slice_store4_any(const double (&x)[4], int e, in
 // nw entries fills row v with [Re, Im] (A') or row v with [Re, -Im] and row nv + v with [Im, Re]
 // (B''), 2 nw values and zeros up to ldq.
 //
-// Two schedules:
-//  * w contiguous: one to eight warps hold a line in registers (real, up to 8 x 4 values a
-//    thread), or a CTA in shared memory (complex), take its exponent and slice it.  Longer lines
-//    are read again, from L2.
-//  * v contiguous: a cluster of 1 to 8 CTAs shares 32 or 128 lines and scans a part of w each; the maxima
-//    meet in distributed shared memory.  A second kernel slices tiles of 64 w x 32 lines, transposed
-//    through shared memory.  (As a programmatic dependent it was slower, 14.2 against 10.4 us at
-//    1000 x 900.  Slicing in the scanning cluster, the lines read again from L2, was slower
-//    from 2048 x 4096 on: 339 against 323 us at 8192^2, four CTAs per SM.)
-// All kernels of the form but the slicing one and long products are programmatic dependents of the one
+// Three schedules:
+//  * w contiguous, one pass: one to eight warps hold a line in registers (real, seven digits of seven
+//    bits, up to 8 x 4 values a thread), or a CTA in shared memory (complex, three CTAs an SM), take
+//    its exponent and slice it.
+//  * w contiguous, two passes (scan_w, slice_w): other digits, and longer lines.  In one pass the
+//    shifts of general digits ran at two CTAs an SM, and a line that did not fit was read again in one
+//    serial chain: us, one pass -> two: 8192^2, eight digits of six bits 739 -> 448, 12000^2 964 -> 638,
+//    1024^2 six bits 23.9 -> 11.5; complex 16 x 4096 x 8000 (whole product) 1880 -> 1520.
+//  * v contiguous: a cluster of 1 to 8 CTAs shares 32 or 128 lines and scans a part of w each; the
+//    maxima meet in distributed shared memory.  A second kernel slices tiles of 64 w x 32 lines,
+//    transposed through shared memory.  (As a programmatic dependent it was slower, 14.2 against 10.4 us
+//    at 1000 x 900.  Slicing in the scanning cluster, the lines read again from L2, was slower from
+//    2048 x 4096 on: 339 against 323 us at 8192^2.)
+// All kernels of the form but the slicing ones and long products are programmatic dependents of the one
 // before them (pdl_launch), and the products let theirs start only at their end (from the start on:
 // 2 us more at 300 x 400 x 500).  Us a call, eager, before -> now: 128^3 23.2 -> 17.4 (op(A) = T) and 37.4 -> 25.7
 // (N), 300 x 400 x 500 33.3 -> 25.4 and 46.0 -> 34, 1000 x 1200 x 900 77.6 -> 69.5 and 89.8 -> 79.
@@ -224,11 +227,12 @@ __device__ __forceinline__ void slice_store4_any(const double (&x)[4], int e, in
 // ones: an operand took four launches before (initialise the exponents, scan, slice, fix up), the
 // scan read everything once more, and complex rows of odd length were stored two bytes at a
 // time.  Before -> now, seven slices of seven bits, us in a row in a CUDA graph: w contiguous
-// 8192^2 298 -> 261 (5.6 TB/s), 4096^2 82 -> 71, 1000 x 900 9.2 -> 6.4; v contiguous 1000 x 900
+// 8192^2 300 -> 247 (6.0 TB/s), 4096^2 81 -> 68, 1000 x 900 8.9 -> 5.3; v contiguous 1000 x 900
 // 15.6 -> 9.9, 5000 x 300 14.2 -> 12.3, 4096^2 91 -> 93, 8192^2 326 -> 333, 20000 x 2000 197 -> 206
-// (1256 scanning CTAs are two waves and a bit); both operands of a complex 1500 x 1100 x 2301 product 190 -> 76.
+// (1256 scanning CTAs are two waves and a bit); both operands of a complex 1500 x 1100 x 2301
+// product 190 -> 76.
 // ---------------------------------------------------------------------------
-constexpr int SPLIT_CLUSTER = 8;   // most CTAs that share 32 or 128 v-contiguous lines
+constexpr int SPLIT_CLUSTER = 8;   // most CTAs that share 32 or 128 v-contiguous lines, or a w-contiguous one
 constexpr int SPLIT_HELD = 8;      // chunks of four values a thread holds (real, w contiguous)
 
 struct SplitJob {
@@ -243,9 +247,9 @@ struct SplitJob {
     int v_contig, conj, role_b;
     int vec_in, vec_out;           // 16-byte loads (real, w contiguous); 8-byte stores
     int warps;                     // w contiguous, real: warps per line (1, 2, 4 or 8)
-    int cached;                    // w contiguous, complex: the line fits shared memory
-    unsigned pieces;               // v contiguous: slicing CTAs along w (a block index divides in 32 bits: with 64
-                                   // the slicing took 4 to 8% longer)
+    int two_pass, group;           // w contiguous, real: scan and slice (scan_w, slice_w), threads of a line there
+    unsigned pieces;               // slicing kernels: CTAs along w (a block index divides in 32 bits: with 64 the
+                                   // slicing took 4 to 8% longer)
     unsigned blocks;
 };
 
@@ -277,6 +281,12 @@ __device__ __forceinline__ int stored_exponent(uint64_t mx) {
     return e == INT_MIN ? 0 : e;
 }
 
+__device__ __forceinline__ uint64_t ld_cluster_u64(uint32_t addr) {
+    uint64_t v;
+    asm volatile("ld.shared::cluster.u64 %0, [%1];" : "=l"(v) : "r"(addr) : "memory");
+    return v;
+}
+
 // four values w .. w+3 of a w-contiguous real line, zero from nw on
 __device__ __forceinline__ void load4(const double* line, int64_t w, int64_t nw, bool vec, double (&x)[4]) {
     if (vec && w + 4 <= nw) {
@@ -289,6 +299,19 @@ __device__ __forceinline__ void load4(const double* line, int64_t w, int64_t nw,
     }
 }
 
+// exponent of the line from the halfwise maxima of the 32 WL threads that share it (a CTA of eight
+// warps holds 8 / WL lines; `red` has eight entries)
+__device__ __forceinline__ uint64_t line_mag_max(uint64_t mx, int WL, uint64_t* red) {
+    mx = warp_mag_max(mx);
+    if (WL > 1) {
+        if (lane_id() == 0) red[warp_id()] = mx;
+        __syncthreads();
+        const int w0 = int(warp_id()) / WL * WL;
+        for (int i = 0; i < WL; ++i) mx = mag_max(mx, red[w0 + i]);
+    }
+    return mx;
+}
+
 template <int BITS, int S, bool BLOCKED>
 __device__ __forceinline__ void split_w_real(const SplitJob& j, int64_t block, int bits, int s) {
     __shared__ uint64_t red[8];
@@ -298,64 +321,96 @@ __device__ __forceinline__ void split_w_real(const SplitJob& j, int64_t block, i
     if (WL == 1 && !live) return;
     const double* line = j.M + (live ? v : 0) * j.ld;
     const int64_t step = 4 * G;
-    const bool held = j.ldq <= SPLIT_HELD * step, vec = j.vec_in != 0;
+    const bool vec = j.vec_in != 0;
     double x[SPLIT_HELD][4];
     uint64_t mx = 0;
-    if (held) {
 #pragma unroll
-        for (int c = 0; c < SPLIT_HELD; ++c)
-            if (c * step < j.nw) load4(line, c * step + 4 * t, j.nw, vec, x[c]);
+    for (int c = 0; c < SPLIT_HELD; ++c)
+        if (c * step < j.nw) load4(line, c * step + 4 * t, j.nw, vec, x[c]);
 #pragma unroll
-        for (int c = 0; c < SPLIT_HELD; ++c)
-            if (c * step < j.nw) {
+    for (int c = 0; c < SPLIT_HELD; ++c)
+        if (c * step < j.nw) {
 #pragma unroll
-                for (int i = 0; i < 4; ++i) mx = mag_max(mx, mag_bits(x[c][i]));
-            }
-    } else {
-#pragma unroll 4
-        for (int64_t w = 4 * t; w < j.nw; w += step) {
-            double y[4];
-            load4(line, w, j.nw, vec, y);
-#pragma unroll
-            for (int i = 0; i < 4; ++i) mx = mag_max(mx, mag_bits(y[i]));
+            for (int i = 0; i < 4; ++i) mx = mag_max(mx, mag_bits(x[c][i]));
         }
-    }
-    mx = warp_mag_max(mx);
-    if (WL > 1) {
-        if (lane_id() == 0) red[warp_id()] = mx;
-        __syncthreads();
-        const int w0 = int(warp_id()) / WL * WL;
-        for (int i = 0; i < WL; ++i) mx = mag_max(mx, red[w0 + i]);
-        if (!live) return;
-    }
+    mx = line_mag_max(mx, WL, red);
+    if (!live) return;
     const int e = stored_exponent(mx);
     if (t == 0) j.expo[v] = e;
     const SliceRow<BLOCKED> out(j, v);
-    if (held) {
 #pragma unroll
-        for (int c = 0; c < SPLIT_HELD; ++c) {
-            const int64_t w = c * step + 4 * t;
-            if (c * step >= j.nw) {
+    for (int c = 0; c < SPLIT_HELD; ++c) {
+        const int64_t w = c * step + 4 * t;
+        if (c * step >= j.nw) {
 #pragma unroll
-                for (int i = 0; i < 4; ++i) x[c][i] = 0.0;
-            }
-            if (w < j.ldq) slice_store4_any<BITS, S>(x[c], e, bits, s, out.at(w), j.plane, j.vec_out != 0);
+            for (int i = 0; i < 4; ++i) x[c][i] = 0.0;
         }
-    } else {
-        for (int64_t w = 4 * t; w < j.ldq; w += step) {
-            double y[4];
-            load4(line, w, j.nw, vec, y);
-            slice_store4_any<BITS, S>(y, e, bits, s, out.at(w), j.plane, j.vec_out != 0);
-        }
+        if (w < j.ldq) slice_store4_any<BITS, S>(x[c], e, bits, s, out.at(w), j.plane, j.vec_out != 0);
     }
 }
 
-// part 0 / 1 of complex entry (v, w): real, imaginary (conjugated for op = C)
-__device__ __forceinline__ double zpart(const SplitJob& j, int64_t idx, int part) {
-    const double y = j.M[2 * idx + part];
-    return part == 1 && j.conj ? -y : y;
+// Exponents of w-contiguous lines, 1 to 8 warps each (complex: 8), or all warps of the CTAs of a cluster
+template <bool CPLX>
+__device__ __forceinline__ void scan_w(const SplitJob& j, int64_t block) {
+    __shared__ uint64_t red[8], cmax;
+    const int rank = int(cluster_ctarank()), CS = int(cluster_nctarank());
+    const int WL = CPLX ? 8 : j.warps, t = int(threadIdx.x) & (32 * WL - 1);
+    const int64_t v = block / CS * (8 / WL) + warp_id() / WL;
+    const bool live = v < j.nv;
+    const double* line = j.M + (CPLX ? 2 : 1) * (live ? v : 0) * j.ld;
+    const int64_t part = ((j.nw + CS - 1) / CS + 3) / 4 * 4, w0 = rank * part, w1 = live ? min(j.nw, w0 + part) : 0;
+    uint64_t mx = 0;
+    if constexpr (CPLX) {
+        for (int64_t w = w0 + t; w < w1; w += 256 * 8) {
+            double2 x[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u)
+                x[u] = w + 256 * u < w1 ? reinterpret_cast<const double2*>(line)[w + 256 * u] : make_double2(0.0, 0.0);
+#pragma unroll
+            for (int u = 0; u < 8; ++u) mx = mag_max(mx, mag_max(mag_bits(x[u].x), mag_bits(x[u].y)));
+        }
+    } else {
+        const int64_t step = 128 * WL;
+        for (int64_t w = w0 + 4 * t; w < w1; w += 4 * step) {
+            double x[4][4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) load4(line, w + u * step, w1, j.vec_in != 0, x[u]);
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+#pragma unroll
+                for (int i = 0; i < 4; ++i) mx = mag_max(mx, mag_bits(x[u][i]));
+        }
+    }
+    mx = line_mag_max(mx, WL, red);
+    if (CS == 1) {
+        if (t == 0 && live) j.expo[v] = stored_exponent(mx);
+        return;
+    }
+    if (threadIdx.x == 0) cmax = mx;        // WL = 8: the CTA's part of one line
+    __syncwarp();
+    cluster_sync_all();
+    if (rank == 0 && threadIdx.x == 0) {
+        for (int r = 1; r < CS; ++r) mx = mag_max(mx, ld_cluster_u64(mapa_shared(smem_u32(&cmax), uint32_t(r))));
+        j.expo[v] = stored_exponent(mx);
+    }
+    __syncwarp();
+    cluster_sync_all();                     // no CTA leaves while rank 0 may still read its maximum
 }
-// which part of which entry stands at position p < 2 nw of row kind `second` (B'' rows nv + v)
+
+// digits of four entries a thread, j.group threads to a line (of up to 1024 entries of it)
+template <int BITS, int S, bool BLOCKED>
+__device__ __forceinline__ void slice_w(const SplitJob& j, unsigned block, int bits, int s) {
+    const int t = int(threadIdx.x) & (j.group - 1), lines = 256 / j.group;
+    const unsigned row = block / j.pieces, piece = block - row * j.pieces;
+    const int64_t v = int64_t(row) * lines + int(threadIdx.x) / j.group, w = (int64_t(piece) * j.group + t) * 4;
+    if (v >= j.nv || w >= j.ldq) return;
+    double x[4];
+    load4(j.M + v * j.ld, w, j.nw, j.vec_in != 0, x);
+    slice_store4_any<BITS, S>(x, j.expo[v], bits, s, SliceRow<BLOCKED>(j, v).at(w), j.plane, j.vec_out != 0);
+}
+
+// which part (0 real, 1 imaginary) of which entry stands at position p < 2 nw of row kind `second`
+// (B'' rows nv + v), and whether negated
 __device__ __forceinline__ int zpart_at(const SplitJob& j, int64_t p, bool second, int64_t& w, bool& flip) {
     const bool right = p >= j.nw;
     w = right ? p - j.nw : p;
@@ -371,7 +426,7 @@ __device__ __forceinline__ void split_w_complex(const SplitJob& j, int64_t v, in
     __shared__ uint64_t red[8];
     const int t = int(threadIdx.x);
     const double2* line = reinterpret_cast<const double2*>(j.M) + v * j.ld;
-    const int half = j.cached ? cache_at(int(j.nw)) + 1 : 0;      // imaginary parts from here on
+    const int half = cache_at(int(j.nw)) + 1;                     // imaginary parts from here on
     uint64_t mx = 0;
     for (int64_t w0 = t; w0 < j.nw; w0 += 256 * 8) {
         double2 a[8];
@@ -381,19 +436,13 @@ __device__ __forceinline__ void split_w_complex(const SplitJob& j, int64_t v, in
         for (int u = 0; u < 8; ++u) {
             const int64_t w = w0 + 256 * u;
             mx = mag_max(mx, mag_max(mag_bits(a[u].x), mag_bits(a[u].y)));
-            if (j.cached && w < j.nw) {
+            if (w < j.nw) {
                 cache[cache_at(int(w))] = a[u].x;
                 cache[half + cache_at(int(w))] = j.conj ? -a[u].y : a[u].y;
             }
         }
     }
-    mx = warp_mag_max(mx);
-    if (lane_id() == 0) red[warp_id()] = mx;
-    __syncthreads();
-    mx = red[0];
-#pragma unroll
-    for (int i = 1; i < 8; ++i) mx = mag_max(mx, red[i]);
-    const int e = stored_exponent(mx);
+    const int e = stored_exponent(line_mag_max(mx, 8, red));
     if (t == 0) j.expo[v] = e;
     const int64_t nw = j.nw;
     for (int second = 0; second <= (j.role_b ? 1 : 0); ++second) {
@@ -401,7 +450,7 @@ __device__ __forceinline__ void split_w_complex(const SplitJob& j, int64_t v, in
         for (int64_t p = 4 * t; p < j.ldq; p += 1024) {
             double x[4];
             const bool left = p + 4 <= nw, right = p >= nw && p + 4 <= 2 * nw;
-            if (j.cached && (left || right)) {              // all four from one half of the row
+            if (left || right) {                            // all four from one half of the row
                 const int part = int(right) ^ second, w = int(right ? p - nw : p);
                 const bool flip = right && j.role_b && second == 0;
 #pragma unroll
@@ -417,7 +466,7 @@ __device__ __forceinline__ void split_w_complex(const SplitJob& j, int64_t v, in
                         int64_t w;
                         bool flip;
                         const int part = zpart_at(j, p + c, second != 0, w, flip);
-                        const double y = j.cached ? cache[part * half + cache_at(int(w))] : zpart(j, v * j.ld + w, part);
+                        const double y = cache[part * half + cache_at(int(w))];
                         x[c] = flip ? -y : y;
                     }
                 }
@@ -425,6 +474,54 @@ __device__ __forceinline__ void split_w_complex(const SplitJob& j, int64_t v, in
             slice_store4_as<BITS, S>(x, e, bits, s, out.at(p), j.plane, true, 4);    // a workspace's slices are aligned
         }
     }
+}
+
+// digits of up to 1024 entries of a complex line, in the two places (A') or four (B'') they occupy
+template <int BITS, int S, bool BLOCKED>
+__device__ __forceinline__ void slice_w_complex(const SplitJob& j, unsigned block, int bits, int s) {
+    __shared__ double part[2][1024 + 64];
+    const unsigned row = block / j.pieces;
+    const int64_t v = row, w0 = int64_t(block - row * j.pieces) * 1024;
+    const int n = int(min(int64_t(1024), j.nw - w0)), t = int(threadIdx.x);
+    const double2* line = reinterpret_cast<const double2*>(j.M) + v * j.ld + w0;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        const int w = t + 256 * u;
+        const double2 a = w < n ? __ldcs(line + w) : make_double2(0.0, 0.0);
+        part[0][cache_at(w)] = a.x;
+        part[1][cache_at(w)] = j.conj ? -a.y : a.y;
+    }
+    __syncthreads();
+    const int e = j.expo[v];
+    const SliceRow<BLOCKED> row1(j, v), row2(j, j.role_b ? j.nv + v : v);
+    // part q to positions pos .. of a row, four at a time from the first multiple of four on
+    const auto emit = [&](int q, const SliceRow<BLOCKED>& out, int64_t pos, bool flip) {
+        const int lead = j.vec_out ? min(n, int(-pos & 3)) : 0;
+        const auto group = [&](int first, int valid) {
+            double x[4];
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                const double y = c < valid ? part[q][cache_at(first + c)] : 0.0;
+                x[c] = flip ? -y : y;
+            }
+            slice_store4_as<BITS, S>(x, e, bits, s, out.at(pos + first), j.plane, j.vec_out && valid == 4, valid);
+        };
+        const int first = lead + 4 * t;
+        if (first < n) group(first, min(4, n - first));
+        if (lead > 0 && t == 255) group(0, lead);
+    };
+    emit(0, row1, w0, false);
+    emit(1, row1, j.nw + w0, j.role_b != 0);
+    if (j.role_b) {
+        emit(1, row2, w0, false);
+        emit(0, row2, j.nw + w0, false);
+    }
+    if (w0 == 0)                   // zeros from 2 nw to ldq
+        for (int64_t p = 2 * j.nw + t; p < j.ldq; p += 256)
+            for (int q = 0; q < s; ++q) {
+                row1.at(p)[int64_t(q) * j.plane] = 0;
+                if (j.role_b) row2.at(p)[int64_t(q) * j.plane] = 0;
+            }
 }
 
 // entries [w0, w0 + n) of line vl of a tile (n <= 64, column v of row w at (v + w / 4) % 32) to
@@ -513,12 +610,7 @@ __device__ __forceinline__ void scan_v(const SplitJob& j, int64_t block) {
     __syncwarp();
     cluster_sync_all();
     if (rank == 0 && t < 2 * LX) {
-        for (int r = 1; r < CS; ++r) {
-            uint64_t y;
-            asm volatile("ld.shared::cluster.u64 %0, [%1];" : "=l"(y) : "r"(mapa_shared(smem_u32(&cmax[t]), uint32_t(r)))
-                         : "memory");
-            mx = mag_max(mx, y);
-        }
+        for (int r = 1; r < CS; ++r) mx = mag_max(mx, ld_cluster_u64(mapa_shared(smem_u32(&cmax[t]), uint32_t(r))));
         if (v0 + t < j.nv) j.expo[v0 + t] = stored_exponent(mx);
     }
     __syncwarp();
@@ -594,6 +686,21 @@ __global__ void __launch_bounds__(256, CPLX ? 4 : 2) ozaki_split_w_kernel(SplitJ
     const int64_t block = first ? blockIdx.x : blockIdx.x - j0.blocks;
     if constexpr (CPLX) split_w_complex<BITS, S, BLOCKED>(j, block, bits, s, cache);
     else split_w_real<BITS, S, BLOCKED>(j, block, bits, s);
+}
+template <bool CPLX>
+__global__ void __launch_bounds__(256) ozaki_scan_w_kernel(SplitJob j0, SplitJob j1) {
+    pdl_wait();
+    const bool first = blockIdx.x < j0.blocks;
+    scan_w<CPLX>(first ? j0 : j1, first ? blockIdx.x : blockIdx.x - j0.blocks);
+}
+template <int BITS, int S, bool CPLX, bool BLOCKED>
+__global__ void __launch_bounds__(256) ozaki_slice_w_kernel(SplitJob j0, SplitJob j1, int bits, int s) {
+    pdl_trigger();
+    const bool first = blockIdx.x < j0.blocks;
+    const SplitJob& j = first ? j0 : j1;
+    const unsigned block = first ? blockIdx.x : blockIdx.x - j0.blocks;
+    if constexpr (CPLX) slice_w_complex<BITS, S, BLOCKED>(j, block, bits, s);
+    else slice_w<BITS, S, BLOCKED>(j, block, bits, s);
 }
 template <int LX, bool CPLX>
 __global__ void __launch_bounds__(256) ozaki_scan_v_kernel(SplitJob j0, SplitJob j1) {
@@ -782,10 +889,10 @@ hsmm_status_t ozaki_recombine(int64_t m, int64_t n, int slices, int bits, const 
 
 namespace {
 
-constexpr size_t SPLIT_CACHE = 200 * 1024;     // shared memory for a complex line
+constexpr size_t SPLIT_CACHE = 72 * 1024;      // shared memory for a complex line: three CTAs an SM
 size_t split_cache_bytes(int64_t nw) { return size_t(16) * (size_t(nw) + size_t(nw) / 16 + 1); }
 
-hsmm_status_t make_split_job(const SplitOperand& o, bool cplx, SplitJob* j) {
+hsmm_status_t make_split_job(const SplitOperand& o, bool cplx, bool fixed, SplitJob* j) {
     if (o.nv > SPLIT_MAX_LINES) return fail(HSMM_STATUS_NOT_SUPPORTED, "ozaki: an operand of more than %lld lines",
                                             static_cast<long long>(SPLIT_MAX_LINES));
     j->M = static_cast<const double*>(o.M);
@@ -810,7 +917,12 @@ hsmm_status_t make_split_job(const SplitOperand& o, bool cplx, SplitJob* j) {
     j->vec_out = q.ldq % 4 == 0 && q.plane % 4 == 0 && aligned_to(q.q, 8);
     j->warps = 1;                  // as many warps per line as hold it in their registers
     while (j->warps < 8 && q.ldq > int64_t(SPLIT_HELD) * 128 * j->warps) j->warps *= 2;
-    j->cached = cplx && !o.v_contig && split_cache_bytes(o.nw) <= SPLIT_CACHE;
+    j->two_pass = !o.v_contig && (cplx ? split_cache_bytes(o.nw) > SPLIT_CACHE : !fixed || q.ldq > int64_t(SPLIT_HELD) * 1024);
+    if (cplx) j->warps = 8;
+    else if (j->two_pass)          // more where there are few lines
+        while (j->warps < 8 && o.nv * j->warps < int64_t(num_sms()) * 16 && q.ldq > int64_t(128) * j->warps) j->warps *= 2;
+    j->group = 32;
+    while (j->group < 256 && q.ldq > int64_t(4) * j->group) j->group *= 2;
     const int lines = cplx ? 1 : 8 / j->warps;     // lines of a CTA (w contiguous)
     j->blocks = unsigned((o.nv + lines - 1) / lines);
     return HSMM_STATUS_SUCCESS;
@@ -818,7 +930,7 @@ hsmm_status_t make_split_job(const SplitOperand& o, bool cplx, SplitJob* j) {
 
 template <int BITS, int S, bool CPLX, bool BLOCKED>
 hsmm_status_t launch_split(SplitJob a, SplitJob b, int bits, int slices, cudaStream_t st) {
-    cudaError_t e;
+    cudaError_t e = cudaSuccess;
     if (a.v_contig) {
         // 128 lines per scanning CTA (1 KiB of a row of w), 32 where that leaves SMs idle; clusters
         // so that a CTA has a batch of loads and more
@@ -840,7 +952,29 @@ hsmm_status_t launch_split(SplitJob a, SplitJob b, int bits, int slices, cudaStr
         a.blocks = unsigned(slice_blocks(a));
         b.blocks = unsigned(slice_blocks(b));
         ozaki_slice_v_kernel<BITS, S, CPLX, BLOCKED><<<a.blocks + b.blocks, 256, 0, st>>>(a, b, bits, slices);
-    } else {
+    } else if (a.two_pass) {
+        // a CTA to a line (or to some), or up to eight while there are under two CTAs an SM
+        unsigned cs = 1;
+        while (a.warps == 8 && (b.nv == 0 || b.warps == 8) && cs < unsigned(SPLIT_CLUSTER) &&
+               (a.nv + b.nv) * cs < num_sms() * 2 && a.nw > int64_t(4096) * cs)
+            cs *= 2;
+        const auto slice_blocks = [](SplitJob& j) {
+            if (j.nv == 0) return int64_t(0);
+            const int64_t lines = CPLX ? 1 : 256 / j.group;
+            j.pieces = unsigned(CPLX ? (j.nw + 1023) / 1024 : (j.ldq + 4 * j.group - 1) / (4 * j.group));
+            return (j.nv + lines - 1) / lines * int64_t(j.pieces);
+        };
+        const int64_t na = slice_blocks(a), nb = slice_blocks(b);
+        if (na + nb > INT32_MAX) return HSMM_STATUS_NOT_SUPPORTED;
+        a.blocks *= cs;
+        b.blocks *= cs;
+        e = pdl_launch(ozaki_scan_w_kernel<CPLX>, dim3(a.blocks + b.blocks), 256, 0, cs, st, a, b);
+        count_launches(1);
+        if (e != cudaSuccess) return record_cuda(e);
+        a.blocks = unsigned(na);
+        b.blocks = unsigned(nb);
+        ozaki_slice_w_kernel<BITS, S, CPLX, BLOCKED><<<a.blocks + b.blocks, 256, 0, st>>>(a, b, bits, slices);
+    } else if constexpr (BITS > 0 || CPLX) {
         auto kern = ozaki_split_w_kernel<BITS, S, CPLX, BLOCKED>;
         size_t smem = 0;
         if (CPLX) {
@@ -849,7 +983,7 @@ hsmm_status_t launch_split(SplitJob a, SplitJob b, int bits, int slices, cudaStr
                 return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(SPLIT_CACHE));
             });
             if (as != HSMM_STATUS_SUCCESS) return as;
-            smem = std::max(a.cached ? split_cache_bytes(a.nw) : 0, b.cached ? split_cache_bytes(b.nw) : 0);
+            smem = std::max(split_cache_bytes(a.nw), split_cache_bytes(b.nw));
         }
         e = pdl_launch(kern, dim3(a.blocks + b.blocks), 256, smem, 1, st, a, b, bits, slices);
     }
@@ -873,10 +1007,11 @@ hsmm_status_t launch_split(bool cplx, const SplitJob& a, const SplitJob& b, int 
 hsmm_status_t ozaki_split(bool cplx, const SplitOperand* ops, int count, int bits, int slices, cudaStream_t st) {
     SplitJob j[2] = {};
     for (int i = 0; i < count; ++i) {
-        const hsmm_status_t r = make_split_job(ops[i], cplx, &j[i]);
+        const hsmm_status_t r = make_split_job(ops[i], cplx, bits == 7 && slices == 7, &j[i]);
         if (r != HSMM_STATUS_SUCCESS) return r;
     }
-    if (count == 1 || (j[0].v_contig == j[1].v_contig && j[0].blocked == j[1].blocked)) return launch_split(cplx, j[0], j[1], bits, slices, st);
+    if (count == 1 || (j[0].v_contig == j[1].v_contig && j[0].blocked == j[1].blocked && j[0].two_pass == j[1].two_pass))
+        return launch_split(cplx, j[0], j[1], bits, slices, st);
     const hsmm_status_t r = launch_split(cplx, j[0], SplitJob{}, bits, slices, st);
     return r != HSMM_STATUS_SUCCESS ? r : launch_split(cplx, j[1], SplitJob{}, bits, slices, st);
 }
