@@ -72,6 +72,8 @@ def build(force: bool = False, verbose: bool = False) -> str:
     if r.returncode != 0:
         raise RuntimeError(f"link failed:\n{r.stderr}")
     os.replace(tmp, LIB)
+    for old in glob.glob(os.path.join(OUT, "_hsmmcall*.so")):     # of another interpreter or an older library
+        os.remove(old)
     if with_call:
         tmp = CALL + f".tmp{os.getpid()}"
         cmd = [os.environ.get("CC", "gcc"), "-O2", "-shared", "-fPIC", f"-I{headers}", f"-I{INCLUDE}",

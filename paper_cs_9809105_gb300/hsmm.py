@@ -13,14 +13,16 @@ column-major product C^T = op(B)^T op(A)^T without copies.
 from __future__ import annotations
 
 import ctypes
-import glob
 import importlib.util
 import os
+import sysconfig
 
 import torch
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "_build", "libhsmm.so")
+# the call module that build.py compiles for this interpreter, no other
+CALL_PATH = os.path.join(_HERE, "_build", "_hsmmcall" + (sysconfig.get_config_var("EXT_SUFFIX") or ".so"))
 
 # status codes (hsmm_status_t)
 SUCCESS, INVALID_VALUE, NOT_SUPPORTED, WORKSPACE_TOO_SMALL, CUDA_ERROR, TIMEOUT = range(6)
@@ -115,16 +117,16 @@ _call = None      # the CPython module of the per-step calls, or None
 
 def _bind_calls(L) -> None:
     global _call
-    for path in glob.glob(os.path.join(os.path.dirname(LIB_PATH), "_hsmmcall*.so")):
-        spec = importlib.util.spec_from_file_location("_hsmmcall", path)
-        try:
-            mod = importlib.util.module_from_spec(spec)
-            spec.loader.exec_module(mod)
-        except ImportError:       # built for another Python
-            continue
-        mod.bind(*(ctypes.cast(f, ctypes.c_void_p).value for f in (L.hsmm_gemm, L.hsmm_gemv)))
-        _call = mod
+    if not os.path.exists(CALL_PATH):
         return
+    spec = importlib.util.spec_from_file_location("_hsmmcall", CALL_PATH)
+    try:
+        mod = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(mod)
+    except ImportError:
+        return
+    mod.bind(*(ctypes.cast(f, ctypes.c_void_p).value for f in (L.hsmm_gemm, L.hsmm_gemv)))
+    _call = mod
 
 
 def status_string(s: int) -> str:
