@@ -9,6 +9,7 @@ import concurrent.futures as cf
 import glob
 import hashlib
 import os
+import shlex
 import subprocess
 import sys
 import sysconfig
@@ -41,6 +42,15 @@ def _fingerprint() -> str:
     h.update(" ".join(ARCH + FLAGS).encode())
     h.update((os.uname().machine + CALL).encode())
     return h.hexdigest()
+
+
+def compile_call(headers: str, out: str) -> None:
+    """The Python binding's call module, with the compiler (and options) of $CC."""
+    cmd = shlex.split(os.environ.get("CC") or "gcc") + ["-O2", "-shared", "-fPIC", f"-I{headers}", f"-I{INCLUDE}",
+                                                        os.path.join(CSRC, "pycall.c"), "-o", out]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    if r.returncode != 0:
+        raise RuntimeError(f"compiling pycall.c failed:\n{r.stderr}")
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
@@ -76,11 +86,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
         os.remove(old)
     if with_call:
         tmp = CALL + f".tmp{os.getpid()}"
-        cmd = [os.environ.get("CC", "gcc"), "-O2", "-shared", "-fPIC", f"-I{headers}", f"-I{INCLUDE}",
-               os.path.join(CSRC, "pycall.c"), "-o", tmp]
-        r = subprocess.run(cmd, capture_output=True, text=True)
-        if r.returncode != 0:
-            raise RuntimeError(f"compiling pycall.c failed:\n{r.stderr}")
+        compile_call(headers, tmp)
         os.replace(tmp, CALL)
     with open(stamp, "w") as f:
         f.write(fp)
