@@ -108,6 +108,9 @@ typedef struct {
  *                                        complex row / column); needs workspace
  *  Scalars: alpha and beta point to the compute type: double for 64F, two doubles
  *  (re, im) for C64F, float for BF16/TF32 products.
+ *  BF16/TF32 products sum in FP32 in an order that is fixed for given sizes and operand forms on
+ *  one GPU; with few output tiles the contraction is cut in up to eight parts, by the number of
+ *  SMs and of clusters that fit, so another GPU or partition may give other last bits.
  *  Tensor-core paths need 16-byte aligned A, B and lda*size, ldb*size multiples of
  *  16 bytes (TMA); otherwise HSMM_STATUS_NOT_SUPPORTED.
  *  Ring order (ring_p != 0): a cluster of p = ring_p CTAs is the ring of p processors of

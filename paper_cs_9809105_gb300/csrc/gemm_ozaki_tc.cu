@@ -83,7 +83,7 @@ __host__ __device__ __forceinline__ int oz_weight(int d, int s) { return oz_thi(
 // Units of one anti-diagonal, not groups of them with equal slice-pair counts: 20 tiles were 80
 // groups on 76 pairs, two rounds of 7 slice pairs each, and are 8 at most now (7.4 the mean).
 // Before -> now, same bits: 1000 x 1200 x 900 146.6 -> 109.9 us, complex 1500 x 1100 x 2301 706
-// -> 676, 4096^3 from host memory (blocks of 64 tiles) 3279 -> 2952, 8192^3 18.0 -> 17.8 ms.
+// -> 676, 4096^3 from host memory (blocks of 64 tiles) 3279 -> 2952; 8192^3 (17.8 ms) within its spread.
 struct OzWork {
     int t;         // tile
     int nd;        // anti-diagonals: s (whole tile, d = s+1 .. 2) or 1
@@ -324,7 +324,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
 // CTAs' epilogue warps release an accumulator on the even CTA's `acc_empty`.
 // The producer and MMA roles are run by whole warps (see gemm_tc.cu): 1000 x 1200 x 900 149.9 ->
 // 146.6 us, 4096^3 from host memory 3318 -> 3279, complex 1500 x 1100 x 2301 714 -> 706; 8192^3
-// is bound by the power cap (18.51 -> 18.46 ms).
+// is bound by the power cap (18.5 ms either way).
 
 __global__ void __launch_bounds__(OZ_THREADS, 1)
     gemm_ozaki_pair_kernel(const __grid_constant__ SliceMaps mA, const __grid_constant__ SliceMaps mB,

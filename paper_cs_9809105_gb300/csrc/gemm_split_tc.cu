@@ -25,6 +25,11 @@
 // 8.2 -> 5.3, 256 x 256 x 8192 39.4 -> 6.7, 1024^3 10.0 -> 5.8, 64 x 4392 x 5520 39.1 -> 13.9;
 // 2048^3 15.5 on whole tiles and 16.6 here (whole tiles stay).
 //
+// The tile and the split follow from the sizes, the number of SMs and how many clusters fit the GPU (see
+// split_plan): the order of the FP32 sums, and so their last bits, is the same in every call on one GPU
+// but not on every GPU.  The error does not grow: the FP32 result of 16 x 4096 x 6144 is 2.1e-6 off its
+// 64-bit value (norm) in eight parts, 4.4e-6 in one; over 51 shapes it was nowhere larger.
+//
 // When every CTA has an SM to itself it takes the whole shared memory for stages; else two share
 // an SM, and one's prologue and epilogue overlap the other's main loop.
 #include <algorithm>
